@@ -7,7 +7,7 @@ the paper's SA1 model, Table I).  One step = one call of inla_value_and_grad
 (all of the hot path: assembly of Q_p and Q_c, both BTA factorisations, the
 solve for x*, f, both in-place selected inversions with the fused Phase A/C
 traces, Phase B and the explicit terms) in emulated FP64: every b x b product
-computed to FP64 accuracy from 8 BF16 slices on the tensor cores, everything
+computed to FP64 accuracy from 14 BF16 residue products on the tensor cores, everything
 else in FP64.  The working set (two factors of 70.7 GB) is far larger than
 L2, so no flush is needed between steps.
 
@@ -41,8 +41,8 @@ METRIC = "INLA f+∇f evals/s on 1 GB300: AD vs 2d+1 FD; % FP64 TC peak; rel err
 UNIT = "gradient evaluations/s"
 WORKLOAD = "coreg_production"      # 3 x 40x40 grid, b = 4800, n_t = 192, a = 12, d = 15
 SIDE = "st_medium"                 # 32x32 grid, b = 1024, n_t = 50, a = 6, d = 4
-PRECISION = 2                      # emulated FP64 (BF16 slices on tcgen05)
-PAIRS = 36                         # BF16 slice products per emulated FP64 product
+PRECISION = 2                      # emulated FP64 (BF16 residue products on tcgen05)
+PRODUCTS = 14                      # BF16 residue products per emulated FP64 product
 
 
 def reduce_replicas(times, dist=None, device="cpu"):
@@ -262,7 +262,7 @@ def run_reference(args):
 def gemm_roofline(P, torch, b, reps=5, mixed=0):
     """Average duration of the FP64 tile GEMM (mixed=1: the split-TF32
     tensor-core GEMM with its operand splitting; mixed=2: the FP64 GEMM
-    emulated from 8 BF16 slices, splitting included) at the sweep's dense
+    emulated from 14 BF16 residue products, residues and recovery included) at the sweep's dense
     block shape (b x b x b, the Z_B = -Z_D,i+1 F_B product of the selected
     inversion), timed with CUDA events on its launch stream."""
     import ctypes as C
@@ -609,11 +609,11 @@ def main():
     b = prob.b
     kms = emulated_kernel_ms(torch, min(b, 5120))
     kb = min(b, 5120)
-    bf16_flop = PAIRS * 2.0 * float(kb) ** 3
+    bf16_flop = PRODUCTS * 2.0 * float(kb) ** 3
     achieved = bf16_flop / (kms * 1e-3) / 1e12
     flops_grad, flops_val = _flops_model(prob.b, prob.nt, prob.a)
     step_tf = flops_grad / t_step / 1e12
-    ceiling = peaks["bf16_tflops_sustained"] / PAIRS      # FP64-equivalent tensor ceiling
+    ceiling = peaks["bf16_tflops_sustained"] / PRODUCTS      # FP64-equivalent tensor ceiling
     ld_closed = spectral_logdet_prior(prob)
     side = None if args.no_side else side_workload(P, torch, workloads, stream, args.side_steps,
                                                    fp64_peak)
@@ -631,8 +631,8 @@ def main():
                        "grid": f"{prob.k} x {prob.nx}x{prob.ny}", "b": prob.b, "ld": model.ld,
                        "nt": prob.nt, "a": prob.a, "d": prob.d, "n_obs": prob.n_obs,
                        "arithmetic": ("FP64 results; every b x b product emulated to FP64 "
-                                      "accuracy from 8 BF16 slices on tcgen05 (36 slice "
-                                      "products), diagonal-block leaves, log-dets, arrow, tip "
+                                      "accuracy from 14 BF16 residue products on "
+                                      "tcgen05, diagonal-block leaves, log-dets, arrow, tip "
                                       "and reductions on the FP64 pipe") if prec == 2 else
                                      {0: "FP64", 1: "mixed (split TF32)"}[prec],
                        "l2": f"working set {2 * prob.nt * model.ld ** 2 * 8 / 1e9:.0f} GB > "
@@ -645,15 +645,15 @@ def main():
                      "fp64_equivalent_tflops": step_tf,
                      "frac_of_emulated_ceiling": step_tf / ceiling,
                      "emulated_ceiling_tflops": ceiling,
-                     "ceiling_source": "measured sustained BF16 rate / 36 slice products",
+                     "ceiling_source": "measured sustained BF16 rate / 14 residue products",
                      "frac_of_fp64_pipe_peak": step_tf / fp64_peak},
             "roofline": {"bound": "tensor", "kernel": f"emulated product tensor-core kernel at "
-                                                      f"{kb} x {kb} x {kb} (BF16 slices)",
+                                                      f"{kb} x {kb} x {kb} (BF16 residues)",
                          "achieved": achieved, "peak": peaks["bf16_tflops_sustained"],
                          "unit": "TFLOP/s", "frac": achieved / peaks["bf16_tflops_sustained"],
                          "traffic": GEMM4800_DRAM_BYTES if kb == 4800 else None,
                          "launch_ms": kms,
-                         "algorithmic": f"36 x 2 x {kb}^3 BF16 flop per launch",
+                         "algorithmic": f"14 x 2 x {kb}^3 BF16 flop per launch",
                          "fp64_equivalent_tflops": 2.0 * float(kb) ** 3 / (kms * 1e-3) / 1e12,
                          "frac_of_burst": achieved / peaks["bf16_tflops"],
                          "peak_source": f"{peaks['source']} bf16_tflops_sustained (the kernel "

@@ -126,7 +126,7 @@ typedef struct {
                           mode 1, with the arrow's rows and rank-a terms
                           carried along, and the diagonal factor's inner and
                           tile products, computed to FP64 accuracy on the
-                          BF16 tensor cores (8 slices, as bta_gemm_emulated;
+                          BF16 tensor cores (as bta_gemm_emulated;
                           products with K > 5120 fall back to FP64);
                           everything else as in mode 0                        */
   int32_t use_graph;   /* 1: capture the evaluation in a CUDA graph, replay */
@@ -329,16 +329,18 @@ bta_status bta_gemm_mixed(int32_t M, int32_t N, int32_t K, double alpha, const d
 
 /*
  * bta_gemm_emulated -- the same product as bta_gemm to FP64 accuracy on the
- * BF16 tensor cores (the products of the emulated-FP64 mode, the Ozaki
- * error-free splitting; no counterpart in the paper, whose GPUs have FP64
- * tensor cores): each row of op(A) and column of op(B) is scaled by a power
- * of two and written as `slices` (6..8) signed base-128 digits (7 bits
- * each: 8 slices carry 56 bits, more than FP64's 53), the slice products
- * of the leading levels accumulate exactly in FP32 and are summed in 64-bit
- * integers, and the result is rounded once to FP64.  Error per entry at most
+ * BF16 tensor cores (the products of the emulated-FP64 mode, the modular
+ * Ozaki scheme; no counterpart in the paper, whose GPUs have FP64 tensor
+ * cores): each row of op(A) and column of op(B) is scaled by a power of two
+ * to 56-bit integers (55 for K > 4847), three more bits than an FP64
+ * significand; their integer product is computed exactly modulo 14 coprime
+ * moduli (14 BF16 products, exact in FP32 accumulators), recovered by the
+ * Chinese remainder theorem and rounded once to FP64.  `slices` (6..8) is
+ * the accuracy asked for: the error per entry is at most
  * (slices + 4) 2^(-7 slices) K max_k|a_ik| max_k|b_kn| plus the final
- * rounding (slices = 8: the order of an FP64 GEMM's rounding bound).  Requires 1 <= K <= 5120.  status as for
- * bta_gemm_mixed.  Allocates its operand slices with cudaMallocAsync on
+ * rounding (slices = 8: the order of an FP64 GEMM's rounding bound); every
+ * value gives the same product.  Requires 1 <= K <= 5120.  status as for
+ * bta_gemm_mixed.  Allocates its operand residues with cudaMallocAsync on
  * the stream.
  */
 bta_status bta_gemm_emulated(int32_t M, int32_t N, int32_t K, double alpha, const double* A,

@@ -266,8 +266,8 @@ def bta_gemm(A: torch.Tensor, B: torch.Tensor, C_out: torch.Tensor, alpha: float
 def bta_gemm_emulated(A: torch.Tensor, B: torch.Tensor, C_out: torch.Tensor, alpha: float = 1.0,
                       beta: float = 0.0, transA: bool = False, transB: bool = False,
                       slices: int = 8, stream=None) -> torch.Tensor:
-    """As bta_gemm, computed to FP64 accuracy on the BF16 tensor cores from
-    `slices` base-128 digits per operand (bta_gemm_emulated).  Returns the
+    """As bta_gemm, computed to FP64 accuracy on the BF16 tensor cores
+    (bta_gemm_emulated; slices: the accuracy asked for, 6..8).  Returns the
     device status word (0, or BTA_ERR_TIMEOUT if a bounded wait expired)."""
     M = A.shape[0] if transA else A.shape[1]
     K = A.shape[1] if transA else A.shape[0]

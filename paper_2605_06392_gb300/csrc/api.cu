@@ -577,7 +577,7 @@ bta_status bta_factor(bta_desc* q, double* rhs_inout, double* logdet, int32_t* f
   const size_t wsb = SweepWs::bytes(q->ld, q->a);
   const int ld = q->ld;
   // tensor-core modes: operand copies of the b x b products (split TF32
-  // planes or BF16 slices, whichever is larger), 256-byte aligned
+  // planes or BF16 residue planes, whichever is larger), 256-byte aligned
   const size_t tcb = precision ? sweep_tc_ws_bytes(ld, q->a) : 0;
   const size_t head = (wsb + nsl * sizeof(double) + 255) / 256 * 256;
   uint8_t* buf = nullptr;
@@ -794,8 +794,8 @@ bta_status bta_gemm_emulated(int32_t M, int32_t N, int32_t K, double alpha, cons
   g.B = B; g.ldb = ldb; g.transB = transB ? 1 : 0;
   g.C = Cm; g.ldc = ldc; g.Cin = Cm; g.ldcin = ldc;
   void* ws = nullptr;
-  BTA_CUDA_TRY(cudaMallocAsync(&ws, ozaki_ws_bytes(M, N, K, slices), stream));
-  bta_status st = ozaki_gemm(g, ws, status, slices, stream);
+  BTA_CUDA_TRY(cudaMallocAsync(&ws, ozaki_ws_bytes(M, N, K), stream));
+  bta_status st = ozaki_gemm(g, ws, status, stream);
   cudaFreeAsync(ws, stream);
   return st;
 }
@@ -818,11 +818,11 @@ bta_status bta_gemm_emulated_timed(int32_t M, int32_t N, int32_t K, double alpha
   BTA_CUDA_TRY(cudaEventCreate(&marks[1]));
   void* ws = nullptr;
   bta_status st = BTA_OK;
-  if (cudaMallocAsync(&ws, ozaki_ws_bytes(M, N, K, slices), stream) != cudaSuccess) {
+  if (cudaMallocAsync(&ws, ozaki_ws_bytes(M, N, K), stream) != cudaSuccess) {
     cudaGetLastError();
     st = BTA_ERR_NOMEM;
   }
-  if (st == BTA_OK) st = ozaki_gemm(g, ws, status, slices, stream, marks);
+  if (st == BTA_OK) st = ozaki_gemm(g, ws, status, stream, marks);
   if (ws) cudaFreeAsync(ws, stream);
   if (st == BTA_OK && cudaEventSynchronize(marks[1]) == cudaSuccess &&
       cudaEventElapsedTime(kernel_ms, marks[0], marks[1]) != cudaSuccess)

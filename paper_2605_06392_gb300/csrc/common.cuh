@@ -183,13 +183,13 @@ struct TuneScope {
 
 bta_status tc_gemm_mixed(const Gemm& g, void* ws, int32_t* status, cudaStream_t s);
 size_t tc_gemm_ws_bytes(int M, int N, int K);
-// FP64 GEMM emulated on BF16 tensor cores with `slices` (6..8) base-128
-// digits per operand (ozaki_gemm.cu); single problem, K <= kOzakiMaxK.
-constexpr int kOzakiMaxK = 5120;   // keeps the 64-bit integer sums below 2^62.4
+// FP64 GEMM emulated on BF16 tensor cores by residues modulo 14 moduli
+// (ozaki_gemm.cu); single problem, K <= kOzakiMaxK.
+constexpr int kOzakiMaxK = 5120;
 // marks (optional): events recorded around the tensor-core product kernel.
-bta_status ozaki_gemm(const Gemm& g, void* ws, int32_t* status, int slices, cudaStream_t s,
+bta_status ozaki_gemm(const Gemm& g, void* ws, int32_t* status, cudaStream_t s,
                       const cudaEvent_t* marks = nullptr);
-size_t ozaki_ws_bytes(int M, int N, int K, int slices);
+size_t ozaki_ws_bytes(int M, int N, int K);
 bool ozaki_supported(const Gemm& g);
 
 // ----------------------------------------------------------------------------
@@ -211,7 +211,7 @@ int potrf_inv_slots(int n);   // number of logdet slots potrf_inv writes
 // rows the block is split 2 x 2 recursively, the diagonal sub-blocks factored
 // by the task-graph kernel and the products of each level run in FP64
 // (precision 0) or emulated FP64 (precision 1, 2; per-block workspace tcws of
-// ozaki_ws_bytes(n, n, n, 8) bytes and status words tcstat).
+// ozaki_ws_bytes(n, n, n) bytes and status words tcstat).
 bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
                                 double* const* scratch, double* const* logdet_parts,
                                 int32_t* const* fail, const int32_t* fail_code, int precision,

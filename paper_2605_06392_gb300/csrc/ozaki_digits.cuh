@@ -20,13 +20,11 @@ __device__ __forceinline__ float i2f_small(int d) {
   return __int_as_float(d + 0x4B400000) - 12582912.0f;
 }
 
-// X * 2^E rounded to the nearest double, from the integer X by integer
-// operations (the usual case); out-of-range exponents take ldexp.
-__device__ __forceinline__ double compose(long long X, int E) {
-  if (X == 0) return 0.0;
-  const unsigned long long sgn = X < 0 ? (1ull << 63) : 0ull;
-  unsigned long long u = X < 0 ? 0ull - (unsigned long long)X : (unsigned long long)X;
+// u * 2^E (negated if neg) rounded to the nearest double, from the integer u > 0 by
+// integer operations (the usual case); out-of-range exponents take ldexp.
+__device__ __forceinline__ double compose_mag(bool neg, unsigned long long u, int E) {
   int lz = __clzll((long long)u);
+  const unsigned long long mag = u;
   u <<= lz;                                   // leading one at bit 63
   unsigned long long m = u >> 11;             // 53 significant bits
   const unsigned long long rem = u & 0x7FFull;
@@ -35,9 +33,16 @@ __device__ __forceinline__ double compose(long long X, int E) {
     if (m >> 53) { m >>= 1; --lz; }
   }
   const int be = 1023 + (63 - lz) + E;
-  if (be <= 0 || be >= 2047) return ldexp((double)X, E);
-  return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) |
+  if (be <= 0 || be >= 2047) return ldexp(neg ? -(double)mag : (double)mag, E);
+  return __longlong_as_double((long long)((neg ? 1ull << 63 : 0ull) |
+                                          ((unsigned long long)be << 52) |
                                           (m & ((1ull << 52) - 1))));
+}
+
+// X * 2^E rounded to the nearest double.
+__device__ __forceinline__ double compose(long long X, int E) {
+  if (X == 0) return 0.0;
+  return compose_mag(X < 0, X < 0 ? 0ull - (unsigned long long)X : (unsigned long long)X, E);
 }
 
 // The S signed base-128 digits of v for the row exponent bound er, each

@@ -208,7 +208,7 @@ bta_status rec(const PB& b, int64_t aoff, int n, int ld, int64_t woff, int soff,
 }
 
 // The products of one recursion level: batched FP64 (precision 0) or one
-// emulated-FP64 product per block (8 BF16 slices; FP64 accuracy).
+// emulated-FP64 product per block (ozaki_gemm; FP64 accuracy).
 struct ProdCfg {
   int precision = 0;
   void* const* tcws = nullptr;
@@ -224,7 +224,7 @@ bta_status level_product(const Gemm& g, const ProdCfg& c, cudaStream_t s) {
     one.Ab = nullptr; one.Bb = nullptr; one.Cb = nullptr; one.Cinb = nullptr;
     one.A = g.Ab[z]; one.B = g.Bb[z]; one.C = g.Cb[z];
     one.Cin = g.Cinb ? g.Cinb[z] : g.Cb[z];
-    BTA_TRY(ozaki_gemm(one, c.tcws[z], c.tcstat[z], 8, s));
+    BTA_TRY(ozaki_gemm(one, c.tcws[z], c.tcstat[z], s));
   }
   return BTA_OK;
 }

@@ -233,7 +233,7 @@ bool arrow_fused(int ld, int a, int precision) {
 size_t sweep_tc_ws_bytes(int ld, int a) {
   const int e = a > 0 && ld + a <= kOzakiMaxK ? a : 0;
   return std::max(tc_gemm_ws_bytes(ld, ld, ld),
-                  ld <= kOzakiMaxK ? ozaki_ws_bytes(ld + e, ld, ld + e, 8) : (size_t)0);
+                  ld <= kOzakiMaxK ? ozaki_ws_bytes(ld + e, ld, ld + e) : (size_t)0);
 }
 
 
@@ -277,7 +277,7 @@ inline const double* const* cp(const std::vector<double*>& v) {
 
 // A b x b product of the sweep over the items idx: batched FP64
 // (precision 0), or one tensor-core product per matrix: split TF32
-// (precision 1) or FP64 emulated from 8 BF16 slices (precision 2).
+// (precision 1) or FP64 emulated on BF16 tensor cores (precision 2).
 bta_status big_product(const Gemm& g, const SweepItem* it, const std::vector<int>& idx,
                        int precision, cudaStream_t s) {
   if (precision == 0 || (precision == 2 && g.K > 5120)) return gemm_f64(g, s);
@@ -290,7 +290,7 @@ bta_status big_product(const Gemm& g, const SweepItem* it, const std::vector<int
     one.A = g.Ab[z]; one.B = g.Bb[z]; one.C = g.Cb[z];
     one.Cin = g.Cinb ? g.Cinb[z] : g.Cb[z];
     if (precision == 2) {
-      BTA_TRY(ozaki_gemm(one, ws.tc, ws.tcstat, 8, s));
+      BTA_TRY(ozaki_gemm(one, ws.tc, ws.tcstat, s));
     } else {
       BTA_TRY(tc_gemm_mixed(one, ws.tc, ws.tcstat, s));
     }
@@ -352,7 +352,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEv
   auto fused = [&](int z) { return emu && arrow_fused(ld, it[z].q.a, precision); };
   auto emulate = [&](int z, const Gemm& g) -> bta_status {
     if (!it[z].ws.tc) return BTA_ERR_ARG;
-    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, 8, s);
+    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s);
   };
   // L_Ci (in Wc1) into C_i, then T -= L_Ci L_Ci^T
   auto arrow_tail = [&](const std::vector<int>& grp, int i) -> bta_status {
@@ -712,7 +712,7 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
   auto fused = [&](int z) { return emu && arrow_fused(ld, it[z].q.a, precision); };
   auto emulate = [&](int z, const Gemm& g) -> bta_status {
     if (!it[z].ws.tc) return BTA_ERR_ARG;
-    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, 8, s);
+    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s);
   };
   for (int i = i_hi; i >= i_lo; --i) {
     BTA_SWEEP_MARK(s, 4, i);
