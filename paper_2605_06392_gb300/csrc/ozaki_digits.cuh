@@ -1,5 +1,4 @@
-// Digit split and integer-to-FP64 composition of the emulated FP64 products
-// (Ozaki scheme, fixed-point slices): shared by the emulated GEMM
+// Integer conversions of the emulated FP64 products: the emulated GEMM
 // (ozaki_gemm.cu) and the task-graph leaves' 32 x 32 tile products
 // (potrf_dag.cu).
 #pragma once
@@ -45,10 +44,9 @@ __device__ __forceinline__ double compose(long long X, int E) {
   return compose_mag(X < 0, X < 0 ? 0ull - (unsigned long long)X : (unsigned long long)X, E);
 }
 
-// The S signed base-128 digits of v for the row exponent bound er, each
-// times its power of two (exact in BF16).
-template <int S>
-__device__ __forceinline__ void digits(double v, int er, float (&out)[S]) {
+// The 8 signed base-128 digits of v for the row exponent bound er, as integers
+// in FP32 (|d_0| <= 128, |d_j| <= 64 otherwise): v = sum_j d_j 2^(er - 1029 - 7 j).
+__device__ __forceinline__ void digits(double v, int er, float (&out)[8]) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
   const int E = (int)((bits >> 52) & 0x7FF);
   long long F = 0;   // v 2^(1078 - er): |F| < 2^56
@@ -62,28 +60,20 @@ __device__ __forceinline__ void digits(double v, int er, float (&out)[S]) {
     }
     if (bits >> 63) F = -F;
   }
-  // F = G 2^28 + R, R in [-2^27, 2^27): digits 1..4 from G, 5..8 from R,
+  // F = G 2^28 + R, R in [-2^27, 2^27): digits 0..3 from G, 4..7 from R,
   // each taken with round-half-up so that every remainder stays within
-  // half a digit (|d_1| <= 128, |d_j| <= 64 otherwise); 32-bit arithmetic.
+  // half a digit; 32-bit arithmetic
   const int G0 = (int)((F + (1ll << 27)) >> 28);
-  const int R0 = (int)(F - (long long)G0 * (1ll << 28));
-  int parts[2] = {G0, R0};
+  const int parts[2] = {G0, (int)(F - (long long)G0 * (1ll << 28))};
 #pragma unroll
-  for (int hpart = 0; hpart < 2; ++hpart) {
-    int x = parts[hpart];
+  for (int h = 0; h < 2; ++h) {
+    int x = parts[h];
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int j = 4 * hpart + jj;
-      if (j >= S) break;
-      int d;
-      if (jj < 3) {
-        const int sh = 21 - 7 * jj;
-        d = (x + (1 << (sh - 1))) >> sh;
-        x -= d * (1 << sh);
-      } else {
-        d = x;
-      }
-      out[j] = i2f_small(d) * __int_as_float((127 - 7 * j) << 23);
+    for (int j = 0; j < 4; ++j) {
+      const int sh = 21 - 7 * j;
+      const int d = j < 3 ? (x + (1 << (sh - 1))) >> sh : x;
+      x -= d * (1 << sh);
+      out[4 * h + j] = i2f_small(d);
     }
   }
 }

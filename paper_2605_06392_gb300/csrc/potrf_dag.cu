@@ -26,7 +26,8 @@
 // so the graph always drains.  Per-tile counters (W updates applied, R
 // updates applied, F/S/G done) are published with release stores after the
 // tile is written and read with acquire loads; tile data are read through
-// L2 (ld.global.cg).  Every wait is bounded by a globaltimer limit (2 s); on
+// L2 (ld.global.cg).  A tile is written by the whole CTA, then a barrier, then one
+// thread's release store, which the barrier makes cumulative.  Every wait is bounded by a globaltimer limit (2 s); on
 // expiry the CTA raises a shared abort flag, writes BTA_ERR_TIMEOUT into the
 // block's failure word (which otherwise holds -1 or the index of a block with
 // a non-positive pivot) and returns, and every other CTA returns at its next
@@ -208,14 +209,14 @@ __device__ __forceinline__ void tile_syrk_lower(double (*L)[T + 1], double (*W)[
 // accuracy from 8 BF16 digit slices per operand on warp-level tensor-core
 // MMAs (mma.sync m16n8k16): on GB300 these run ~1900 BF16 flop per clock per
 // SM against ~1.6 FP64 FMAs, so the 36 slice-pair products of a tile cost
-// ~1.2 k clocks where its 32^3 FP64 FMAs cost ~20 k.  The digits are those
-// of the emulated GEMM (fixed point on each row's exponent bound, 7 bits a
-// digit); a level L = i + j of slice pairs sums to |S_L| < 2^21 digit units
-// over K = 32, exact in FP32; levels 0..5 are added as 64-bit integers in
-// units of 2^-35 of level 0, levels 6 and 7 rounded to that unit, and the
-// FP64 result assembled by integer operations.  Levels from 8 on are dropped,
-// the bound of the emulated GEMM with K = 32.  ylower: Y is lower triangular
-// (its upper part is not read).
+// ~1.2 k clocks where its 32^3 FP64 FMAs cost ~20 k.  A row is scaled to
+// 56-bit integers by its exponent bound and written in signed base-128 digits
+// (Ozaki's error-free splitting, fixed point); a level L = i + j of slice pairs
+// sums to an integer |S_L| < 2^21 over K = 32, exact in FP32; levels 0..5 are
+// added as 64-bit integers in units of level 5, levels 6 and 7 rounded to that
+// unit, and the FP64 result assembled by integer operations.  Levels from 8 on
+// are dropped, below the 56th bit of the operands' products.  ylower: Y is lower
+// triangular (its upper part is not read).
 constexpr int kOzPitch = 40;                      // bf16 a slice row: 80 bytes, conflict-free ldmatrix
 constexpr int kOzPlane = T * kOzPitch;            // one 32 x 32 slice
 constexpr int kOzTileSmem = 2 * 8 * kOzPlane * 2 + 2 * T * 4;   // both operands' slices, exponents
@@ -227,28 +228,40 @@ struct OzTile {
   int* ey;             // [32] row exponents of op(Y)^T
 };
 
-// Slices of a 32 x 32 matrix (element (r, k) = get(r, k)) into planes[8][r][k]
-// and its row exponent bounds e[r]: warp w takes rows w, w + 8, w + 16, w + 24.
+// Slices of a 32 x 32 matrix (element (r, k) = get(r, k)) into planes[8][r][.]
+// and its row exponent bounds e[r].  A half-warp takes a row, a lane its elements
+// k and k + 16, which sit side by side in the slice row (both operands of a
+// product use this order of k); the two rows of a warp are four apart, so that
+// their 4-byte stores fall on different banks.
 template <class Get>
 __device__ __forceinline__ void oz_split(Get get, __nv_bfloat16* planes, int* e) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double v[4];
-  int er[4];
+  const int k = lane & 15;
+  const int r0 = (warp & 3) + 16 * (warp >> 2) + 4 * (lane >> 4);
+  double v[2][2];
+  int er[2];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    v[q] = get(warp + 8 * q, lane);
-    const int ef = (int)((__double_as_longlong(v[q]) >> 52) & 0x7FF);
-    er[q] = (int)__reduce_max_sync(0xffffffffu, (unsigned)ef);
+  for (int q = 0; q < 2; ++q) {
+    v[q][0] = get(r0 + 8 * q, k);
+    v[q][1] = get(r0 + 8 * q, k + 16);
+    er[q] = max((int)((__double_as_longlong(v[q][0]) >> 52) & 0x7FF),
+                (int)((__double_as_longlong(v[q][1]) >> 52) & 0x7FF));
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = warp + 8 * q;
-    float d[8];
-    oz::digits<8>(v[q], er[q], d);
+  for (int o = 8; o; o >>= 1)
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      planes[j * kOzPlane + r * kOzPitch + lane] = __float2bfloat16_rn(d[j]);
-    if (lane == 0) e[r] = er[q];
+    for (int q = 0; q < 2; ++q) er[q] = max(er[q], __shfl_xor_sync(0xffffffffu, er[q], o));
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int r = r0 + 8 * q;
+    float d0[8], d1[8];
+    oz::digits(v[q][0], er[q], d0);
+    oz::digits(v[q][1], er[q], d1);
+    uint32_t* y = reinterpret_cast<uint32_t*>(planes + r * kOzPitch) + k;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)   // |digit| <= 128: its BF16 pattern is the upper half
+      y[j * (kOzPlane / 2)] = __byte_perm(__float_as_uint(d0[j]), __float_as_uint(d1[j]), 0x7632);
+    if (k == 0) e[r] = er[q];
   }
 }
 
@@ -258,55 +271,37 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
                : "r"(addr)
                : "memory");
 }
-__device__ __forceinline__ void ldsm_x2(uint32_t addr, uint32_t (&r)[2]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
-               : "=r"(r[0]), "=r"(r[1])
-               : "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4],
-                                         const uint32_t (&b)[2]) {
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
       "{%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// All 256 threads; out must not alias X or Y.  Warp w computes the 16 x 8
-// output block (rows 16 (w / 4).., columns 8 (w % 4)..).
-__device__ void tile_mm_oz(double (*X)[T + 1], double (*Y)[T + 1], bool ytrans, bool ylower,
-                           double (*out)[T + 1], double sign, bool accumulate,
-                           const OzTile& z) {
-  const bool same = X == Y && ytrans && !ylower;   // X op(Y) = X X^T: one split
-  oz_split([&](int r, int k) { return X[r][k]; }, z.xp, z.ex);
-  if (!same)
-    oz_split(
-        [&](int n, int k) {
-          const double v = ytrans ? Y[n][k] : Y[k][n];
-          return ylower && (ytrans ? k > n : n > k) ? 0.0 : v;
-        },
-        z.yp, z.ey);
-  __syncthreads();
-  const __nv_bfloat16* yp = same ? z.xp : z.yp;
-  const int* ey = same ? z.ex : z.ey;
+// The products of the slices and their combination: warp w computes the
+// 16 x 8 output block (rows 16 (w / 4).., columns 8 (w % 4)..).
+__device__ __forceinline__ void oz_combine(const __nv_bfloat16* xp, const __nv_bfloat16* yp,
+                                           const int* ex, const int* ey, double (*out)[T + 1],
+                                           double sign, bool accumulate) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int mt = warp >> 2, nt = warp & 3;
-  uint32_t a[8][2][4], b[8][2][2];
+  uint32_t a[8][2][4], b[8][4];
   {
-    const uint32_t xb = (uint32_t)__cvta_generic_to_shared(z.xp);
+    const uint32_t xb = (uint32_t)__cvta_generic_to_shared(xp);
     const uint32_t yb = (uint32_t)__cvta_generic_to_shared(yp);
-    // ldmatrix rows: A's four 8 x 8 blocks (rows 0-7 / 8-15 by k 0-7 / 8-15),
-    // B's two (columns 0-7 by k 0-7 / 8-15), from lanes 0-31 / 0-15
+    // ldmatrix rows: A's four 8 x 8 blocks (rows 0-7 / 8-15 by k 0-7 / 8-15) of one
+    // 16-wide K step; B's four (columns 0-7 by k 0-7 / 8-15 / 16-23 / 24-31)
     const int ar = 16 * mt + (lane & 7) + ((lane >> 3) & 1) * 8, ac = (lane >> 4) * 8;
-    const int br = 8 * nt + (lane & 7), bc = ((lane >> 3) & 1) * 8;
+    const int br = 8 * nt + (lane & 7), bc = (lane >> 3) * 8;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+    for (int j = 0; j < 8; ++j) {
+      ldsm_x4(yb + 2u * (uint32_t)(j * kOzPlane + br * kOzPitch + bc), b[j]);
 #pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
+      for (int ks = 0; ks < 2; ++ks)
         ldsm_x4(xb + 2u * (uint32_t)(j * kOzPlane + ar * kOzPitch + 16 * ks + ac), a[j][ks]);
-        ldsm_x2(yb + 2u * (uint32_t)(j * kOzPlane + br * kOzPitch + 16 * ks + bc), b[j][ks]);
-      }
+    }
   }
   // one accumulator per level, the pairs issued slice by slice of A so that
   // consecutive MMAs go to different accumulators (no dependent chain)
@@ -320,24 +315,41 @@ __device__ void tile_mm_oz(double (*X)[T + 1], double (*Y)[T + 1], bool ytrans, 
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; i + j < 8; ++j) mma_bf16(c[i + j], a[i][ks], b[j][ks]);
-  // S_L = c[L] 2^(7 L), |S_L| < 2^21: to integers by the exact FP32 rounding
-  // against 1.5 2^23 (no 64-bit conversions, which GB300 runs at its FP64
-  // rate); two levels 7 bits apart share one 32-bit integer, then
+      for (int j = 0; i + j < 8; ++j) mma_bf16(c[i + j], a[i][ks], b[j][2 * ks], b[j][2 * ks + 1]);
+  // |S_L| < 2^21: to integers by the exact FP32 rounding against 1.5 2^23 (no
+  // 64-bit conversions, which GB300 runs at its FP64 rate); two levels 7 bits
+  // apart share one 32-bit integer, then
   // tot = S_0 2^35 + S_1 2^28 + ... + S_5 + round(S_6 2^-7 + S_7 2^-14).
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     int sl[6];
 #pragma unroll
-    for (int L = 0; L < 6; ++L) sl[L] = oz::f2i_small(c[L][q] * __int_as_float((127 + 7 * L) << 23));
-    const int r67 = oz::f2i_small((c[6][q] + c[7][q]) * 34359738368.0f);
+    for (int L = 0; L < 6; ++L) sl[L] = oz::f2i_small(c[L][q]);
+    const int r67 = oz::f2i_small(fmaf(c[6][q], 0.0078125f, c[7][q] * 0.00006103515625f));
     const long long tot = ((long long)(sl[0] * 128 + sl[1]) << 28) +
-                          ((long long)(sl[2] * 128 + sl[3]) << 14) + (sl[4] * 128 + sl[5]) + r67;
-    const int r = 16 * mt + g + (q >> 1) * 8, c = 8 * nt + 2 * t + (q & 1);
-    const double v = oz::compose(tot, z.ex[r] + ey[c] - 2093);
-    out[r][c] = accumulate ? fma(sign, v, out[r][c]) : sign * v;
+                          ((long long)(sl[2] * 128 + sl[3]) << 14) + (sl[4] * 128 + sl[5] + r67);
+    const int r = 16 * mt + g + (q >> 1) * 8, cc = 8 * nt + 2 * t + (q & 1);
+    // a = sum_j d_j 2^(ex - 1029 - 7 j): the integer's unit is level 5's
+    double v = oz::compose(tot, ex[r] + ey[cc] - 2093);
+    if (sign < 0.0) v = -v;
+    out[r][cc] = accumulate ? out[r][cc] + v : v;
   }
+}
+
+// All 256 threads; out must not alias X or Y.
+__device__ void tile_mm_oz(double (*X)[T + 1], double (*Y)[T + 1], bool ytrans, bool ylower,
+                           double (*out)[T + 1], double sign, bool accumulate,
+                           const OzTile& z) {
+  oz_split([&](int r, int k) { return X[r][k]; }, z.xp, z.ex);
+  oz_split(
+      [&](int n, int k) {
+        if (ylower && (ytrans ? k > n : n > k)) return 0.0;
+        return ytrans ? Y[n][k] : Y[k][n];
+      },
+      z.yp, z.ey);
+  __syncthreads();
+  oz_combine(z.xp, z.yp, z.ex, z.ey, out, sign, accumulate);
 }
 
 struct Task {
@@ -387,27 +399,42 @@ __device__ Task decode(const DagArgs& g, int l) {
   return t;
 }
 
-// 1 / v to FP64 accuracy.  Seed: the FP32 reciprocal of v's leading bits,
-// with v narrowed and the result widened by integer operations (a GB300 FP64
-// instruction, conversions included, has ~64 clock cycles of latency).  With
-// r = (1 + eps) / v, e = 1 - v r = -eps, the correction r (1 + e + e^2) has
-// relative error eps^3 (~2^-66) plus rounding: three dependent FP64 FMAs.
+// 1 / v to FP64 accuracy by one third-order step (Householder's iteration,
+// r (1 + e + e^2) with e = 1 - v r) from the FP32 reciprocal of v's leading
+// bits, all of it in integers: a GB300 FP64 instruction, conversions included,
+// has ~72 clocks of latency, a dependent 32 x 32 -> 64 bit multiply ~10.  With
+// the significand M = v 2^52 (53 bits) and the seed R = r 2^24 (24 bits),
+// e 2^76 = 2^76 - M R fits 64 bits (|e| <= 2^-22), so its low word is exact;
+// the result is rounded once from 56 bits (error within 0.53 of the last place).
 // Values outside the seed's exponent range use the division.
 __device__ __forceinline__ double recip(double v) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int e = (int)((b >> 52) & 0x7FF);
-  if (e < 1023 - 100 || e > 1023 + 100) return 1.0 / v;
-  const unsigned f = (unsigned)((b >> 32) & 0x80000000u) | ((unsigned)(e - 1023 + 127) << 23) |
-                     (unsigned)((b >> 29) & 0x7FFFFFu);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const int ef = (int)((hi >> 20) & 0x7FF);
+  if (ef < 1023 - 100 || ef > 1023 + 100) return 1.0 / v;
+  const unsigned mh = (hi & 0xFFFFFu) | 0x100000u;   // M = mh 2^32 + lo
+  // seed in [1/2, 1): of the significand's leading 24 bits
   float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(__uint_as_float(f)));
-  const unsigned rb = __float_as_uint(rf);
-  const unsigned long long db = ((unsigned long long)(rb & 0x80000000u) << 32) |
-                                ((unsigned long long)(((rb >> 23) & 0xFF) - 127 + 1023) << 52) |
-                                ((unsigned long long)(rb & 0x7FFFFFu) << 29);
-  const double r = __longlong_as_double((long long)db);
-  const double err = fma(-v, r, 1.0);
-  return fma(r, fma(err, err, err), r);
+  asm("rcp.approx.ftz.f32 %0, %1;"
+      : "=f"(rf)
+      : "f"(__uint_as_float(0x3F800000u | ((hi & 0xFFFFFu) << 3) | (lo >> 29))));
+  const unsigned R = (min(max(__float_as_uint(rf), 0x3F000000u), 0x3F7FFFFFu) & 0x7FFFFFu) |
+                     0x800000u;
+  const unsigned long long mr =
+      (unsigned long long)lo * R + ((unsigned long long)(mh * R) << 32);   // M R mod 2^64
+  long long e = (long long)(0ull - mr);                                    // e 2^76
+  const int eh = (int)(e >> 24);                                           // |eh| <= 2^30
+  e += ((long long)eh * eh) >> 28;                                         // e + e^2
+  const int th = (int)(e >> 24);
+  const unsigned tl = (unsigned)e & 0xFFFFFFu;
+  // r (1 + e + e^2) 2^56, in [2^55, 2^56]
+  const long long corr = (long long)th * (int)R + (long long)(((unsigned long long)tl * R) >> 24);
+  const unsigned long long q = ((unsigned long long)R << 32) + (unsigned long long)(corr >> 20);
+  const unsigned long long m = (q + 4) >> 3;   // 53 bits, or 2^53
+  // v = M 2^(ef - 1075): 1 / v = m 2^-53 2^(1023 - ef)
+  return __longlong_as_double((long long)((b & 0x8000000000000000ull) |
+                                          ((((unsigned long long)(2045 - ef)) << 52) +
+                                           (m - (1ull << 52)))));
 }
 
 // d^{-1/2} to FP64 accuracy: FP32 seed of the narrowed value widened by
@@ -431,108 +458,130 @@ __device__ __forceinline__ double rsqrt_fp64(double d) {
 
 // Leaf on smem tile S (lower, W_kk): D / unit-L elimination carrying the
 // inverse of the unit-L factor in X, then X = D^{-1/2} (unit L)^{-1} =
-// L_kk^{-1}; the pivots d_i stay in piv[] (leaf_logdet sums their logs, off
-// the critical path).
+// L_kk^{-1} (lower part; its upper part is not written); the pivots d_i stay in
+// piv[] (leaf_logdet sums their logs, off the critical path).
 //
 // Pivot j eliminates column j with the multipliers l_ij = S_ij / d_j:
 // S_ik -= l_ij S_kj (j < k <= i) and X_ik -= l_ij X_jk (k <= j < i).  Warp 0
 // runs one pivot ahead: while warps 1-3 and 5-7 apply pivot j to columns
 // k >= j+2 and to X, it applies pivot j to column j+1, takes d_{j+1}, its
-// reciprocal and the next multipliers, so each pivot costs one barrier and
-// the serial chain per pivot is one FMA, the reciprocal and one multiply.
-// Warp 4 shares warp 0's scheduler and FP64 unit and stays idle, so the
-// chain's instructions do not queue behind bulk ones.
-__device__ void leaf(double (*S)[T + 1], double (*X)[T + 1], double (*lcol)[T], double* piv,
-                     double* rs) {
+// reciprocal and the next multipliers.  A position (i, k) belongs to one thread
+// for the whole leaf, which holds S_ik and, from pivot k on, X_ik in a register;
+// only what others read goes through shared memory, double buffered by the
+// pivot's parity: the multipliers and the column of the pivot (from warp 0),
+// column j+2 (for warp 0) and row j+1 of X.  So each pivot costs one barrier of
+// these seven warps, and the serial chain is one FMA, the integer reciprocal and
+// one multiply.  An SM sub-partition issues one FP64 warp instruction per 64
+// clocks: warp 4 shares warp 0's and takes no part (see service).
+// Measured alone: 20.6 k clocks (10 us; 15 us with the FP64 reciprocal, positions in
+// shared memory and the log-det between the steps), bound by the bulk warps (~520 clocks
+// a pivot) ahead of the chain (~440).  512-row factor in the tensor-core modes 0.41 ->
+// 0.31 ms (a diagonal step 25.5 -> 18.8 us).
+struct LeafBuf {
+  double l[2][T], v[2][T], x[2][T], s[2][T];
+};
+
+__device__ __forceinline__ void leaf_bar() {   // warps 0-3 and 5-7
+  asm volatile("bar.sync 1, 224;" ::: "memory");
+}
+
+// service: run by warp 4 alongside the pivots.
+template <class Service>
+__device__ __forceinline__ void leaf(double (*S)[T + 1], double (*X)[T + 1], LeafBuf& B,
+                                     double* piv, double* rs, Service service) {
   constexpr int kPos = T * (T + 1) / 2;   // lower-triangle positions, row by row
   constexpr int kBulk = kDagThreads - 64;   // warps 1-3 and 5-7
   constexpr int kPer = (kPos + kBulk - 1) / kBulk;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool bulk = warp != 0 && warp != 4;
   const int bt = warp < 4 ? tid - 32 : tid - 64;   // 0..kBulk-1 over the bulk warps
   int pi[kPer], pk[kPer];
-  if (bulk) {
+  double val[kPer];
+  if (warp == 0) {
+    double v = S[lane][0];
+    double d = __shfl_sync(0xffffffffu, v, 0);
+    double l = v * recip(d);
+    B.l[0][lane] = l;
+    B.v[0][lane] = v;
+    B.s[0][lane] = S[lane][1];
+    if (lane == 0) {
+      B.x[0][0] = 1.0;
+      piv[0] = d;
+    }
+    leaf_bar();
+    for (int j = 0; j < T - 1; ++j) {
+      // column c = j+1 with pivot j, then pivot c and its multipliers
+      const int c = j + 1, p = c & 1;
+      const double vc = __shfl_sync(0xffffffffu, v, c);
+      v = fma(-l, vc, B.s[j & 1][lane]);
+      d = __shfl_sync(0xffffffffu, v, c);
+      l = v * recip(d);
+      B.l[p][lane] = l;
+      B.v[p][lane] = v;
+      if (lane == 0) piv[c] = d;
+      leaf_bar();
+    }
+    rs[lane] = rsqrt_fp64(piv[lane]);   // rows scale by d_i^{-1/2}
+    leaf_bar();
+  } else if (warp == 4) {
+    service();
+  } else {
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
       const int q = bt + kBulk * r;
-      if (q < kPos) {
-        int i = 0;
-        while ((i + 1) * (i + 2) / 2 <= q) ++i;
-        pi[r] = i;
-        pk[r] = q - i * (i + 1) / 2;
-      } else {
-        pi[r] = -1;
-        pk[r] = 0;
-      }
+      int i = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
+      if (i * (i + 1) / 2 > q) --i;
+      if ((i + 1) * (i + 2) / 2 <= q) ++i;
+      pi[r] = q < kPos ? i : -1;
+      pk[r] = q < kPos ? q - i * (i + 1) / 2 : 0;
+      val[r] = q < kPos ? S[i][pk[r]] : 0.0;
     }
-  }
-  for (int e = tid; e < T * T; e += kDagThreads) X[e % T][e / T] = (e % T == e / T) ? 1.0 : 0.0;
-  if (tid < 32) {   // pivot 0 and its multipliers
-    const double d = S[0][0];
-    const double r = recip(d);
-    if (lane > 0) lcol[0][lane] = S[lane][0] * r;
-    if (lane == 0) piv[0] = d;
-  }
-  __syncthreads();
-  for (int j = 0; j < T - 1; ++j) {
-    const double* lj = lcol[j & 1];
-    if (tid < 32) {
-      // column j+1 with pivot j, then pivot j+1 and its multipliers
-      const int c = j + 1;
-      double v = 0.0;
-      if (lane >= c) {
-        v = fma(-lj[lane], S[c][j], S[lane][c]);
-        S[lane][c] = v;
-      }
-      const double d = __shfl_sync(0xffffffffu, v, c);
-      const double r = recip(d);
-      if (lane > c) lcol[c & 1][lane] = v * r;
-      if (lane == 0) piv[c] = d;
-    } else if (bulk) {
-      // k > j+1: trailing S_ik -= l_ij S_kj; k <= j: X_ik -= l_ij X_jk.  The
-      // positions are distinct and none is a source of this pivot (column j of
-      // S, row j of X), so all loads go first and the FMAs overlap.
-      double* dst[kPer];
-      double dv[kPer], sv[kPer], lv[kPer];
-      bool act[kPer];
+    leaf_bar();
+    for (int j = 0; j < T - 1; ++j) {
+      const int p = j & 1;
+      double src[kPer], lv[kPer];
 #pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        const int i = pi[q], k = pk[q];
-        act[q] = i > j && k != j + 1;
-        if (act[q]) {
-          dst[q] = k > j ? &S[i][k] : &X[i][k];
-          sv[q] = k > j ? S[k][j] : X[j][k];
-          dv[q] = *dst[q];
-          lv[q] = lj[i];
+      for (int r = 0; r < kPer; ++r) {
+        if (pi[r] > j) {
+          src[r] = pk[r] > j ? B.v[p][pk[r]] : B.x[p][pk[r]];
+          lv[r] = B.l[p][pi[r]];
         }
       }
 #pragma unroll
-      for (int q = 0; q < kPer; ++q)
-        if (act[q]) *dst[q] = fma(-lv[q], sv[q], dv[q]);
+      for (int r = 0; r < kPer; ++r) {
+        const int i = pi[r], k = pk[r];
+        if (i > j) {
+          // (k == j+1, warp 0's column, is computed here too but not used: at
+          // pivot k the position turns into X_ik, which starts from 0)
+          val[r] = fma(-lv[r], src[r], k == j ? 0.0 : val[r]);
+          if (k == j + 2) B.s[p ^ 1][i] = val[r];
+          if (i == j + 1) B.x[p ^ 1][k] = k == i ? 1.0 : val[r];
+        }
+      }
+      leaf_bar();
     }
-    __syncthreads();
-  }
-  if (tid < 32) rs[tid] = rsqrt_fp64(piv[tid]);   // rows scale by d_i^{-1/2}
-  __syncthreads();
-  for (int e = tid; e < T * T; e += kDagThreads) {
-    const int i = e % T, k = e / T;
-    X[i][k] = i >= k ? X[i][k] * rs[i] : 0.0;
+    leaf_bar();
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+      const int i = pi[r], k = pk[r];
+      if (i >= 0) X[i][k] = k == i ? rs[i] : val[r] * rs[i];
+    }
   }
   __syncthreads();
 }
 
 // Log-det slot of a leaf: sum of log d_i over its pivots, and the failure
-// code on a non-positive or non-finite pivot (warp 0).
+// code on a non-positive or non-finite pivot (one warp).
 __device__ __forceinline__ void leaf_logdet(const double* piv, double* slot, int32_t* fail,
                                             int32_t code) {
-  if (threadIdx.x < 32) {
-    const double dj = piv[threadIdx.x];
+  {
+    const int lane = threadIdx.x & 31;
+    const double dj = piv[lane];
     const bool b = !(dj > 0.0) || !isfinite(dj);
     double l = b ? 0.0 : log(dj);
 #pragma unroll
     for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     const unsigned anyb = __ballot_sync(0xffffffffu, b);
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
       *slot = l;
       if (anyb) atomicCAS(fail, -1, code);
     }
@@ -543,7 +592,7 @@ __device__ __forceinline__ void leaf_logdet(const double* piv, double* slot, int
 // the tensor-core modes); otherwise FP64 FMAs.
 template <bool TC>
 __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
-  // three tiles (~26 KB with the leaf's vectors); TC adds the slices of two
+  // three tiles (~28 KB with the leaf's vectors); TC adds the slices of two
   // tiles (40 KB of dynamic shared memory)
   __shared__ double S0[T][T + 1], S1[T][T + 1], S2[T][T + 1];
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -562,7 +611,8 @@ __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
     if constexpr (TC) tile_mm_oz(W, Y, true, true, o, 1.0, false, ozs);
     else tile_mm_lt(W, Y, o);
   };
-  __shared__ double lcol[2][T], piv[T], rs[T];
+  __shared__ LeafBuf lbuf;
+  __shared__ double piv[2][T], rs[T];
   __shared__ int s_task, s_ok;
   const int p = g.p, ld = g.ld, pp = p * p;
   int* busy = &g.smbusy[sm_id() & 255];
@@ -639,29 +689,42 @@ __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
             S0[e % T][e / T] = wcc[q];
           }
           store_tile(Lt(c, c - 1), T, S2, false);
-          __syncthreads();
-          if (threadIdx.x == 0) { __threadfence(); st_release(&doneS[c * p + c - 1], 1); }
-          if constexpr (TC) tile_mm_oz(S2, S2, true, false, S0, -1.0, true, ozs);   // W_cc -= L L^T
-          else tile_syrk_lower(S2, S0);           // W_cc -= L L^T (lower)
+          // W_cc -= L L^T (lower); a thread of a warp that has no part in it publishes L
+          if constexpr (TC) {
+            oz_split([&](int r, int k) { return S2[r][k]; }, ozs.xp, ozs.ex);
+            __syncthreads();
+            const int warp = threadIdx.x >> 5;
+            if (warp != 2 && warp != 3)           // output rows 0-15 by columns 16-31
+              oz_combine(ozs.xp, ozs.xp, ozs.ex, ozs.ex, S0, -1.0, true);
+            else if (threadIdx.x == 96)
+              st_release(&doneS[c * p + c - 1], 1);
+          } else {
+            __syncthreads();
+            tile_syrk_lower(S2, S0);
+            if (threadIdx.x == 224) st_release(&doneS[c * p + c - 1], 1);
+          }
           __syncthreads();
           if (threadIdx.x == 0 && z == 0) DAG_TRACE(2, c);
         } else {
           load_tile(S0, tile(I.A, ld, 0, 0), ld);
           __syncthreads();
         }
-        leaf(S0, S1, lcol, piv, rs);              // S1 = X_cc = L_cc^{-1}
+        // S1 = X_cc = L_cc^{-1}; warp 4 meanwhile sums the logs of the last step's pivots
+        leaf(S0, S1, lbuf, piv[c & 1], rs, [&]() {
+          if (c > 0) leaf_logdet(piv[(c - 1) & 1], &I.slots[c - 1], I.fail, I.code);
+        });
         if (threadIdx.x == 0 && z == 0) DAG_TRACE(3, c);
         store_tile(tile(I.A, ld, c, c), ld, S1, true);
         __syncthreads();
-        if (threadIdx.x == 0) {
-          __threadfence();
+        // thread 0 goes on to the next step's waits
+        if (threadIdx.x == 224) {
           st_release(&cntW[c * p + c], c);
           st_release(&doneF[c], 1);
           if (z == 0) DAG_TRACE(4, c);
         }
-        leaf_logdet(piv, &I.slots[c], I.fail, I.code);   // after the release: off the chain
-        __syncthreads();
       }
+      if (threadIdx.x < 32) leaf_logdet(piv[(p - 1) & 1], &I.slots[p - 1], I.fail, I.code);
+      __syncthreads();
       if (threadIdx.x == 0 && g.yield) atomicSub(busy, 1);
       continue;
     }
@@ -703,7 +766,7 @@ __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
         __syncthreads();
         store_tile(Lt(t.i, t.k), T, S2, false);
         __syncthreads();
-        if (threadIdx.x == 0) { __threadfence(); st_release(&doneS[t.i * p + t.k], 1); }
+        if (threadIdx.x == 0) { st_release(&doneS[t.i * p + t.k], 1); }
         break;
       }
       case TK_G: {   // X_kj = X_kk R_kj  (t.i = k)
@@ -718,7 +781,7 @@ __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
         __syncthreads();
         store_tile(tile(I.A, ld, t.i, t.j), ld, S2, false);
         __syncthreads();
-        if (threadIdx.x == 0) { __threadfence(); st_release(&doneG[t.i * p + t.j], 1); }
+        if (threadIdx.x == 0) { st_release(&doneG[t.i * p + t.j], 1); }
         break;
       }
       case TK_U: {   // W_ij -= L_ik L_jk^T
@@ -730,7 +793,7 @@ __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
         __syncthreads();
         store_tile(tile(I.A, ld, t.i, t.j), ld, S2, t.i == t.j);
         __syncthreads();
-        if (threadIdx.x == 0) { __threadfence(); st_release(&cntW[t.i * p + t.j], t.k + 1); }
+        if (threadIdx.x == 0) { st_release(&cntW[t.i * p + t.j], t.k + 1); }
         break;
       }
       default: {     // TK_V: R_ij -= L_ik X_kj
@@ -748,7 +811,6 @@ __global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
         store_tile(tile(I.A, ld, t.i, t.j), ld, S2, false);
         __syncthreads();
         if (threadIdx.x == 0) {
-          __threadfence();
           st_release(&cntR[t.i * p + t.j], t.k - t.j + 1);
         }
       }
