@@ -316,20 +316,21 @@ int env_int(const char* name, int dflt) {
 
 int potrf_hybrid_leaf(int precision) {
   // Largest block the task-graph kernel factors whole below the top level
-  // (0: always whole).  Up to 1024 rows its serial chain of 32-row pivots
+  // (0: always whole).  FP64: up to 1024 rows its serial chain of 32-row pivots
   // costs about as much as the split's extra products; above, the split wins
-  // (measured on GB300: b = 2025 1.6x (emulated) and 1.9x (mixed) faster per
-  // gradient, b = 4800 2.2x; FP64 b = 2025 1.4 %).
+  // (b = 2025 1.4 %).  Tensor-core modes: the emulated products of a split cost
+  // little, while a 1024-row leaf waits ~30 us a step for its bulk tasks; leaves
+  // of up to 640 rows keep them off the chain.  Measured on GB300 per gradient,
+  // leaves 1024 / 640 / 512 / 256: b = 2025 104.7 / 83.5 / 83.3 / 90.0 ms,
+  // b = 4800 226 / 226 / 235 / 250 ms, b = 768..3072 104 / 96.8 / 97.0 / 93.3 ms.
   static const int fp64 = env_int("BTA_POTRF_LEAF_FP64", 1024);
-  static const int tc = env_int("BTA_POTRF_LEAF_TC", 1024);
+  static const int tc = env_int("BTA_POTRF_LEAF_TC", 640);
   return precision == 0 ? fp64 : tc;
 }
 
 namespace {
-// Blocks above this many rows are split at least once (tensor-core modes):
-// with the emulated products a 1024-row block is faster as two 512-row
-// task graphs (GB300: 157 -> 154 ms emulated, 142 -> 130 ms mixed per
-// gradient of the b = 1024 model), while deeper splits of larger blocks lose.
+// Blocks above this many rows are split at least once (tensor-core modes): a
+// 1024-row block is faster as two 512-row task graphs than as one.
 int potrf_hybrid_top(int precision) {
   static const int tc = env_int("BTA_POTRF_SPLIT_TC", 512);
   return precision == 0 ? 0 : tc;
