@@ -39,7 +39,7 @@ struct EvalCtx {
   SweepWs wsc, wsp;
   SelinvFuse fc, fp;
   double* dr = nullptr;         // mixed mode: refinement residual / correction
-  double *w4c = nullptr, *w4p = nullptr;   // low memory: second L_B buffer per sweep
+  double* red = nullptr;        // sums of the final combination
   int have_factors = 0;         // last evaluation was value-only: factors still held
 };
 
@@ -125,8 +125,6 @@ bta_status ctx_alloc(inla_model* m, EvalCtx& c) {
     BTA_TRY(dmalloc(m, &c.qp.B, std::max(nt - 1, 1) * blk));
   } else {
     c.qp.B = nullptr;
-    BTA_TRY(dmalloc(m, &c.w4c, blk));
-    BTA_TRY(dmalloc(m, &c.w4p, blk));
   }
   BTA_TRY(dmalloc(m, &c.x, (size_t)nt * ld + a));
   BTA_TRY(dmalloc(m, &c.slots_c, m->nslots));
@@ -143,6 +141,7 @@ bta_status ctx_alloc(inla_model* m, EvalCtx& c) {
   // residual_kernel writes kMaxK rows
   BTA_TRY(dmalloc(m, &c.RS, (size_t)kMaxK * resid_chunks(md)));
   BTA_TRY(dmalloc(m, &c.out, out_size(md.d)));
+  BTA_TRY(dmalloc(m, &c.red, kRedDoubles));
   const size_t wsb = SweepWs::bytes(ld, a) / sizeof(double);
   double* wsbuf = nullptr;
   BTA_TRY(dmalloc(m, &wsbuf, 2 * wsb));
@@ -215,8 +214,6 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
     ic.md = ip.md = &md;
     ic.lay = ip.lay = &m->L;
     ic.coef = ip.coef = c.coefbuf;
-    ic.W4 = c.w4c;
-    ip.W4 = c.w4p;
   }
   // set-up on s0, the fork, and (mode < 2) the assembly of both sets
   steps.push_back([=]() -> bta_status {
@@ -256,8 +253,10 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
           EvalCtx& c = m->ctx[e];
           BTA_TRY(launch_rhs(md, m->L, c.coefbuf, c.dr, m->s1));
           BTA_TRY(launch_qc_residual(md, m->L, c.coefbuf, c.x, c.dr, m->s1));
-          BTA_TRY(lower_solve(c.qc, c.dr, c.wsc, m->s1));
-          BTA_TRY(upper_solve(c.qc, c.dr, c.wsc, m->s1));
+          SweepItem dx = sets->ic[e];
+          dx.vec = c.dr;
+          BTA_TRY(lower_solve(dx, m->s1));
+          BTA_TRY(upper_solve_multi(&dx, 1, m->s1));
           BTA_TRY(launch_axpy((int64_t)md.nt * md.ld + md.a, 1.0, c.dr, c.x, m->s1));
         }
       }
@@ -278,6 +277,10 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
       });
   // join and combine
   steps.push_back([=]() -> bta_status {
+    if (grad) {
+      BTA_TRY(selinv_sums(sets->ic.data(), cnt, m->s1));
+      BTA_TRY(selinv_sums(sets->ip.data(), cnt, m->s2));
+    }
     BTA_CUDA_TRY(cudaEventRecord(m->ev1, m->s1));
     BTA_CUDA_TRY(cudaEventRecord(m->ev2, m->s2));
     BTA_CUDA_TRY(cudaStreamWaitEvent(s0, m->ev1, 0));
@@ -288,7 +291,7 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
       r.PDc = c.PDc; r.PBc = c.PBc; r.PCc = c.PCc; r.ZTc = c.qc.T;
       r.PDp = c.PDp; r.PBp = c.PBp; r.QD = c.QD; r.QB = c.QB; r.RS = c.RS;
       r.ldc = c.slots_c; r.nldc = m->nslots; r.ldp = c.slots_p; r.nldp = m->nslots;
-      r.failc = c.fail; r.failp = c.fail + 1; r.x = c.x; r.grad = grad;
+      r.failc = c.fail; r.failp = c.fail + 1; r.x = c.x; r.red = c.red; r.grad = grad;
       BTA_TRY(launch_finalize(md, m->L, c.coefbuf, r, c.out, s0));
     }
     return BTA_OK;
@@ -618,16 +621,20 @@ bta_status bta_solve(const bta_desc* L, double* z_inout, int32_t lower, int32_t 
   double* dx = r + nv;
   bta_status st = BTA_OK;
   if (refine)
-    st = copy_block(z_inout, (int)nv, r, (int)nv, (int)nv, 1, 1.0, 0, stream);
-  if (st == BTA_OK && lower) st = lower_solve(*L, z_inout, ws, stream);
-  if (st == BTA_OK) st = upper_solve(*L, z_inout, ws, stream);
+    st = copy_block(z_inout, (int)nv, r, (int)nv, (int)nv, 1, 1.0, stream);
+  SweepItem it, di;
+  it.q = *L; it.ws = ws; it.vec = z_inout;
+  di = it;
+  di.vec = dx;
+  if (st == BTA_OK && lower) st = lower_solve(it, stream);
+  if (st == BTA_OK) st = upper_solve_multi(&it, 1, stream);
   if (st == BTA_OK && refine) {
     // one step of iterative refinement in FP64 (Eqs. 3-5 on the residual):
     // x += Q^{-1} (r - Q x) with the factor L of Q
-    st = copy_block(r, (int)nv, dx, (int)nv, (int)nv, 1, 1.0, 0, stream);
-    if (st == BTA_OK) st = bta_residual(*Q_or_null, z_inout, dx, ws.gv, stream);
-    if (st == BTA_OK) st = lower_solve(*L, dx, ws, stream);
-    if (st == BTA_OK) st = upper_solve(*L, dx, ws, stream);
+    st = copy_block(r, (int)nv, dx, (int)nv, (int)nv, 1, 1.0, stream);
+    if (st == BTA_OK) st = bta_residual(*Q_or_null, z_inout, dx, stream);
+    if (st == BTA_OK) st = lower_solve(di, stream);
+    if (st == BTA_OK) st = upper_solve_multi(&di, 1, stream);
     if (st == BTA_OK) st = launch_axpy((int64_t)nv, 1.0, dx, z_inout, stream);
   }
   cudaFreeAsync(buf, stream);
@@ -668,7 +675,7 @@ bta_status bta_selinv(bta_desc* L, inla_model* m, const double* theta, int32_t w
     const size_t nRS = (size_t)kMaxK * resid_chunks(md);
     double* rb = nullptr;
     const size_t nZ0 = std::max(nPD + nPB, (size_t)md.nt * md.ld + md.a);
-    size_t total = m->L.total + nPD + nPB + nPC + nZ0 + nRS + out_size(md.d) + 4;
+    size_t total = m->L.total + nPD + nPB + nPC + nZ0 + nRS + kRedDoubles + out_size(md.d) + 4;
     BTA_CUDA_TRY(cudaMallocAsync(&rb, total * sizeof(double), stream));
     double* cb = rb;
     double* PD = cb + m->L.total;
@@ -676,7 +683,8 @@ bta_status bta_selinv(bta_desc* L, inla_model* m, const double* theta, int32_t w
     double* PC = PB + nPB;
     double* Z0 = PC + nPC;           // zero reductions for the other matrix / quad forms
     double* RS = Z0 + nZ0;
-    double* o = RS + nRS;
+    double* red = RS + nRS;
+    double* o = red + kRedDoubles;
     int32_t* fl = reinterpret_cast<int32_t*>(o + out_size(md.d));
     BTA_CUDA_TRY(cudaMemsetAsync(rb, 0, total * sizeof(double), stream));
     BTA_CUDA_TRY(cudaMemsetAsync(fl, 0xff, 2 * sizeof(int32_t), stream));
@@ -695,7 +703,7 @@ bta_status bta_selinv(bta_desc* L, inla_model* m, const double* theta, int32_t w
       r.PDp = which ? Z0 : PD; r.PBp = which ? Z0 + nPD : PB;
       r.QD = Z0; r.QB = Z0 + nPD; r.RS = RS;
       r.ldc = Z0; r.nldc = 1; r.ldp = Z0; r.nldp = 1; r.failc = fl; r.failp = fl + 1;
-      r.x = Z0; r.grad = 1;
+      r.x = Z0; r.red = red; r.grad = 1;
       ModelDev mz = md;
       mz.a = which ? md.a : 0;
       st = launch_finalize(mz, m->L, cb, r, o, stream);
@@ -703,7 +711,7 @@ bta_status bta_selinv(bta_desc* L, inla_model* m, const double* theta, int32_t w
         // phases at o + 1 + d + kOutParts: A (d), B (d), C (d)
         const double* ph = o + 1 + md.d + kOutParts;
         st = copy_block(which ? ph : ph + 2 * md.d, md.d, trace_terms, md.d, md.d, 1,
-                        which ? -2.0 : 2.0, 0, stream);
+                        which ? -2.0 : 2.0, stream);
       }
     }
     cudaFreeAsync(rb, stream);

@@ -150,24 +150,28 @@ struct Gemm {
 };
 bta_status gemm_f64(const Gemm& g, cudaStream_t s);
 
-// y[M] = alpha * op(A) x + beta * yin ; A column-major lda; tri masks A.
-// Batched like Gemm: per-problem A, x, y, yin and GEMV work areas.
+// y[M] = alpha * (op(A) x + A2^T x2) + beta * yin ; A column-major lda; tri masks A.
+// The second part (K2 > 0) only with transA.  y must not alias x or x2 (it may alias
+// yin).  Batched like Gemm.
 struct Gemv {
   int M = 0, K = 0;
   const double* A = nullptr; int lda = 0; int transA = 0; int triA = TRI_NONE;
   const double* x = nullptr;
   double* y = nullptr;
-  const double* yin = nullptr;    // may alias y
+  const double* yin = nullptr;    // null: y
+  int K2 = 0;
+  const double* A2 = nullptr; int lda2 = 0;
+  const double* x2 = nullptr;
   double alpha = 1.0, beta = 0.0;
   int batch = 1;
   const double* const* Ab = nullptr;
   const double* const* xb = nullptr;
   double* const* yb = nullptr;
   const double* const* yinb = nullptr;   // null: yin = y
-  double* const* workb = nullptr;
+  const double* const* A2b = nullptr;
+  const double* const* x2b = nullptr;
 };
-bta_status gemv_f64(const Gemv& g, double* work, cudaStream_t s);
-constexpr int kGemvSplit = 16;      // K splits; work needs kGemvSplit * M doubles
+bta_status gemv_f64(const Gemv& g, cudaStream_t s);
 
 // Split-precision (3xTF32) tensor-core GEMM (tc_gemm.cu): same contract as
 // gemm_f64 for a single problem; ws holds tc_gemm_ws_bytes(M, N, K) bytes;
@@ -230,9 +234,12 @@ extern int g_potrf_recursive;
 
 // Small helpers (sweep.cu)
 bta_status copy_block(const double* src, int lds, double* dst, int ldd, int rows, int cols,
-                      double alpha, int mode, cudaStream_t s);  // mode 0 copy, 1 mirror lower->full
+                      double alpha, cudaStream_t s);
 bta_status copy_block_batch(int count, const double* const* src, int lds, double* const* dst,
-                            int ldd, int rows, int cols, double alpha, int mode, cudaStream_t s);
+                            int ldd, int rows, int cols, double alpha, cudaStream_t s);
+// dst = the symmetric n x n matrix whose lower triangle src holds (in place when src == dst)
+bta_status mirror_batch(int count, const double* const* src, int lds, double* const* dst, int ldd,
+                        int n, cudaStream_t s);
 bta_status fill_value(double* p, int64_t n, double v, cudaStream_t s);
 bta_status sum_slots(const double* parts, int nparts, double* out, int accumulate,
                      cudaStream_t s);

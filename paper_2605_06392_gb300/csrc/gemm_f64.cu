@@ -7,6 +7,8 @@
 // idle tails), not to save bandwidth.  A 16x16 thread grid computes a
 // BM x BN tile with DFMA from shared-memory stages of BK = 16, prefetching
 // the next stage into registers while the current one is consumed.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstdlib>
 #include <map>
@@ -196,64 +198,111 @@ __global__ void splitk_reduce(SplitDev d) {
 }
 
 struct GemvDev {
-  int M, K, lda, triA, nsplit;
+  int M, K, lda, triA, K2, lda2;
   double alpha, beta;
   const double* A[kMaxBatch];
   const double* x[kMaxBatch];
   double* y[kMaxBatch];
   const double* yin[kMaxBatch];
-  double* work[kMaxBatch];
+  const double* A2[kMaxBatch];
+  const double* x2[kMaxBatch];
 };
 
-// y = op(A) x with op(A) = A: thread per output row, partial sums over a K
-// split written to a fixed slot (summed in order by gemv_finish).
-__global__ void gemv_n_partial(GemvDev g) {
-  const int z = blockIdx.z;
+// y = alpha A x + beta yin.  A matrix-vector product is FP64-pipe bound on one SM
+// long before its bytes matter (one 32-lane FMA per 64 clocks and sub-partition),
+// so it is spread thinly: a cluster of 8 CTAs owns 32 rows (lane = row, coalesced
+// columns), its 64 warps take every 64th column, and the CTAs' partial sums meet in
+// the first one's registers through distributed shared memory, in a fixed order: one
+// launch, no workspace.  1024 x 1024: 20 us and a second launch before (one warp per
+// 32 rows and 64 columns, dependent FMAs), 12 us now (cold cache).
+constexpr int kGemvThreads = 256;
+constexpr int kGemvCluster = 8;
+__global__ void __cluster_dims__(kGemvCluster, 1, 1) __launch_bounds__(kGemvThreads)
+    gemv_n_kernel(GemvDev g) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
+  const int z = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = (int)cl.block_rank();
   const double* __restrict__ A = g.A[z];
   const double* __restrict__ x = g.x[z];
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  int split = blockIdx.y;
-  int kc = (g.K + gridDim.y - 1) / gridDim.y;
-  int kb = split * kc, ke = min(g.K, kb + kc);
-  if (g.triA == TRI_LOWER) ke = min(ke, m + 1);
-  if (g.triA == TRI_UPPER) kb = max(kb, m);
-  double s = 0.0;
-  if (m < g.M)
-    for (int k = kb; k < ke; ++k) s = fma(A[m + (int64_t)k * g.lda], x[k], s);
-  if (m < g.M) g.work[z][(int64_t)split * g.M + m] = s;
+  const int m0 = (int)(blockIdx.x / kGemvCluster) * 32, m = m0 + lane;
+  int kb = 0, ke = g.K;
+  if (g.triA == TRI_LOWER) ke = min(ke, m0 + 32);
+  if (g.triA == TRI_UPPER) kb = m0;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  const int first = kb + rank * (kGemvThreads / 32) + warp;
+  constexpr int kStep = kGemvCluster * kGemvThreads / 32;
+  if (m < g.M) {
+    for (int k = first; k < ke; k += 4 * kStep) {
+      double a[4], v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kq = k + q * kStep;
+        const bool in = kq < ke && !(g.triA == TRI_LOWER && kq > m) &&
+                        !(g.triA == TRI_UPPER && kq < m);
+        a[q] = in ? A[m + (int64_t)kq * g.lda] : 0.0;
+        v[q] = in ? x[kq] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s[q] = fma(a[q], v[q], s[q]);
+    }
+  }
+  __shared__ double part[kGemvThreads / 32][32];
+  part[warp][lane] = (s[0] + s[1]) + (s[2] + s[3]);
+  __syncthreads();
+  if (warp == 0) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kGemvThreads / 32; ++w) t += part[w][lane];
+    part[0][lane] = t;
+  }
+  cl.sync();
+  if (rank == 0 && warp == 0) {
+    double p[kGemvCluster];
+#pragma unroll
+    for (int r = 0; r < kGemvCluster; ++r) p[r] = cl.map_shared_rank(&part[0][0], r)[lane];
+    double t = 0.0;
+#pragma unroll
+    for (int r = 0; r < kGemvCluster; ++r) t += p[r];
+    if (m < g.M) {
+      double v = g.alpha * t;
+      if (g.beta != 0.0) v = fma(g.beta, g.yin[z][m], v);
+      g.y[z][m] = v;
+    }
+  }
+  cl.sync();   // the parts stay until they have been read
 }
 
-// y[m] = sum_k A[k, m] x[k] (op(A) = A^T), one warp per output, lanes over K.
-__global__ void gemv_t_partial(GemvDev g) {
-  const int z = blockIdx.z;
+// y = alpha (A^T x + A2^T x2) + beta yin (A2 optional): one warp per output, lanes
+// over K.
+__global__ void __launch_bounds__(kGemvThreads) gemv_t_kernel(GemvDev g) {
+  const int z = blockIdx.y;
   const double* __restrict__ A = g.A[z];
   const double* __restrict__ x = g.x[z];
-  int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  int split = blockIdx.y;
+  const int m = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (m >= g.M) return;
-  int kc = (g.K + gridDim.y - 1) / gridDim.y;
-  int kb = split * kc, ke = min(g.K, kb + kc);
+  int kb = 0, ke = g.K;
   // op(A)[m,k] = A[k,m]; op(A) lower -> zero for k > m
   if (g.triA == TRI_LOWER) ke = min(ke, m + 1);
-  if (g.triA == TRI_UPPER) kb = max(kb, m);
-  double s = 0.0;
-  for (int k = kb + lane; k < ke; k += 32) s = fma(A[k + (int64_t)m * g.lda], x[k], s);
+  if (g.triA == TRI_UPPER) kb = m;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int k = kb + lane; k < ke; k += 128) {
 #pragma unroll
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) g.work[z][(int64_t)split * g.M + m] = s;
-}
-
-__global__ void gemv_finish(GemvDev g) {
-  const int z = blockIdx.y;
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= g.M) return;
-  const double* part = g.work[z];
-  double s = 0.0;
-  for (int j = 0; j < g.nsplit; ++j) s += part[(int64_t)j * g.M + m];
-  double v = g.alpha * s;
-  if (g.beta != 0.0) v = fma(g.beta, g.yin[z][m], v);
-  g.y[z][m] = v;
+    for (int q = 0; q < 4; ++q) {
+      const int kq = k + 32 * q;
+      if (kq < ke) s[q] = fma(A[kq + (int64_t)m * g.lda], x[kq], s[q]);
+    }
+  }
+  for (int k = lane; k < g.K2; k += 32)
+    s[0] = fma(g.A2[z][k + (int64_t)m * g.lda2], g.x2[z][k], s[0]);
+  double t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) {
+    double v = g.alpha * t;
+    if (g.beta != 0.0) v = fma(g.beta, g.yin[z][m], v);
+    g.y[z][m] = v;
+  }
 }
 
 // ---- measured tile choice ---------------------------------------------------
@@ -465,37 +514,32 @@ bta_status gemm_f64(const Gemm& g, cudaStream_t s) {
   return BTA_OK;
 }
 
-bta_status gemv_f64(const Gemv& g, double* work, cudaStream_t s) {
+bta_status gemv_f64(const Gemv& g, cudaStream_t s) {
   if (g.M <= 0 || g.batch <= 0) return BTA_OK;
-  if (g.Ab ? !(g.xb && g.yb && g.workb) : (g.batch != 1 || !g.A || !g.x || !g.y || !work))
-    return BTA_ERR_ARG;
-  const int nb = g.batch;
-  int nsplit = g.K >= 512 ? kGemvSplit : 1;
-  if (g.K <= 0) nsplit = 1;
+  if (g.Ab ? !(g.xb && g.yb) : (g.batch != 1 || !g.A || !g.x || !g.y)) return BTA_ERR_ARG;
+  if (g.K2 > 0 && (!g.transA || (g.Ab ? !(g.A2b && g.x2b) : !(g.A2 && g.x2)))) return BTA_ERR_ARG;
   GemvDev d;
-  d.M = g.M; d.K = g.K > 0 ? g.K : 0; d.lda = g.lda; d.triA = g.triA; d.nsplit = nsplit;
+  d.M = g.M; d.K = std::max(g.K, 0); d.lda = g.lda; d.triA = g.triA;
+  d.K2 = std::max(g.K2, 0); d.lda2 = g.lda2;
   d.alpha = g.alpha; d.beta = g.beta;
-  for (int z0 = 0; z0 < nb; z0 += kMaxBatch) {
-    const int cnt = std::min(kMaxBatch, nb - z0);
+  for (int z0 = 0; z0 < g.batch; z0 += kMaxBatch) {
+    const int cnt = std::min(kMaxBatch, g.batch - z0);
     for (int z = 0; z < cnt; ++z) {
-      if (!g.Ab) {   // single problem given by the scalar pointers
-        d.A[z] = g.A; d.x[z] = g.x; d.y[z] = g.y; d.yin[z] = g.yin ? g.yin : g.y;
-        d.work[z] = work;
-      } else {
-        d.A[z] = g.Ab[z0 + z]; d.x[z] = g.xb[z0 + z]; d.y[z] = g.yb[z0 + z];
-        d.yin[z] = g.yinb ? g.yinb[z0 + z] : g.yb[z0 + z];
-        d.work[z] = g.workb[z0 + z];
-      }
+      const int q = z0 + z;
+      d.A[z] = g.Ab ? g.Ab[q] : g.A;
+      d.x[z] = g.Ab ? g.xb[q] : g.x;
+      d.y[z] = g.Ab ? g.yb[q] : g.y;
+      const double* yin = g.Ab ? (g.yinb ? g.yinb[q] : nullptr) : g.yin;
+      d.yin[z] = yin ? yin : d.y[z];
+      d.A2[z] = g.K2 > 0 ? (g.Ab ? g.A2b[q] : g.A2) : nullptr;
+      d.x2[z] = g.K2 > 0 ? (g.Ab ? g.x2b[q] : g.x2) : nullptr;
+      // an output is written while others still read x
+      if (d.x[z] == d.y[z] || (d.x2[z] && d.x2[z] == d.y[z])) return BTA_ERR_ARG;
     }
-    if (!g.transA) {
-      dim3 grid(cdiv(g.M, 128), nsplit, cnt);
-      gemv_n_partial<<<grid, 128, 0, s>>>(d);
-    } else {
-      dim3 grid(cdiv((int64_t)g.M * 32, 256), nsplit, cnt);
-      gemv_t_partial<<<grid, 256, 0, s>>>(d);
-    }
-    BTA_LAUNCHED();
-    gemv_finish<<<dim3(cdiv(g.M, 256), cnt), 256, 0, s>>>(d);
+    if (!g.transA)
+      gemv_n_kernel<<<dim3(kGemvCluster * cdiv(g.M, 32), cnt), kGemvThreads, 0, s>>>(d);
+    else
+      gemv_t_kernel<<<dim3(cdiv((int64_t)g.M * 32, kGemvThreads), cnt), kGemvThreads, 0, s>>>(d);
     BTA_LAUNCHED();
   }
   return BTA_OK;

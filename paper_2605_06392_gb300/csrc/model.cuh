@@ -69,17 +69,19 @@ bta_status launch_assemble_b(const ModelDev& md, const CoefLayout& L, const doub
 // Sizes of the per-block partial-sum arrays.
 int pattern_chunks(const ModelDev& md);
 int arrow_chunks(const ModelDev& md);
-// Pattern inner products <Z^(pq), S> of one dense b x b block (Phase A/C).
-// out: [k*k][chunks][kNP]
-bta_status launch_pattern_dot(const ModelDev& md, const double* Z, int with_counts, int t,
-                              double* out, cudaStream_t s);
-// <Z_C, craw_t restricted to variable m> for all m.  out: [k][achunks]
-bta_status launch_arrow_dot(const ModelDev& md, const double* ZC, int t, double* out,
+// Pattern inner products <Z^(pq), S> of `count` dense b x b blocks (ld x ld, one after
+// the other; time blocks t0 ..), Phase A/C.  out: [count][k*k][chunks][kNP]
+bta_status launch_pattern_dot(const ModelDev& md, const double* Z, int with_counts, int t0,
+                              int count, double* out, cudaStream_t s);
+inline size_t pattern_doubles(const ModelDev& md) {   // of one block
+  return (size_t)md.k * md.k * pattern_chunks(md) * kNP;
+}
+// <Z_C, craw_t restricted to variable m> for all m of `count` arrow blocks from the
+// first on.  out: [count][k][achunks]
+bta_status launch_arrow_dot(const ModelDev& md, const double* ZC, int count, double* out,
                             cudaStream_t s);
-// Stencil quadratic forms x_t^(p)T S x_u^(q).  out: [k*k][chunks][kNP]
-bta_status launch_pattern_quad(const ModelDev& md, const double* xr, const double* xc,
-                               double* out, cudaStream_t s);
-// All of them for one mode x: QD[t] = x_t x_t forms, QB[t] = x_{t+1} x_t forms.
+// Stencil quadratic forms x_t^(p)T S x_u^(q) of one mode x: QD[t] = x_t x_t forms,
+// QB[t] = x_{t+1} x_t forms, each [k*k][chunks][kNP].
 bta_status launch_pattern_quad_all(const ModelDev& md, const double* x, double* QD, double* QB,
                                   cudaStream_t s);
 // Squared residuals per response.  out: [k][rchunks]
@@ -113,11 +115,14 @@ struct Reductions {
   const int32_t* failc;
   const int32_t* failp;
   const double* x;     // mode (for beta part of x^T Q_p x)
+  double* red;         // work: kRedDoubles
   int grad;
 };
 // out: [0] f, [1..d] grad, then parts (8) and phases (4*d).
 bta_status launch_finalize(const ModelDev& md, const CoefLayout& L, const double* coefbuf,
                            const Reductions& r, double* out, cudaStream_t s);
+// sums over the blocks: [3][kNJ][k*k][kNS] pattern sums, [4][k] per response, [2] log-dets
+constexpr int kRedDoubles = 3 * kNJ * kMaxK * kMaxK * kNS + 4 * kMaxK + 2;
 constexpr int kOutParts = 8;
 inline int out_size(int d) { return 1 + d + kOutParts + 4 * d; }
 

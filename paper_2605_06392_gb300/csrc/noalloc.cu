@@ -41,10 +41,10 @@ constexpr int kNoAllocMaxLd = 256;
 constexpr int kNoAllocMaxA = 32;
 constexpr int kNoAllocMaxSlots = 16384;
 // Work area of one sweep at the maximum sizes, in doubles (see SweepWs):
-// 4 ld^2 + 2 a ld + kGemvSplit ld + a + 64.
+// 4 ld^2 + a ld + ld + a + 64, rounded up to a multiple of 32.
 constexpr size_t kWorkDoubles = 4 * (size_t)kNoAllocMaxLd * kNoAllocMaxLd +
-                                2 * (size_t)kNoAllocMaxA * kNoAllocMaxLd +
-                                (size_t)kGemvSplit * kNoAllocMaxLd + kNoAllocMaxA + 64;
+                                (size_t)kNoAllocMaxA * kNoAllocMaxLd + kNoAllocMaxLd +
+                                kNoAllocMaxA + 64 + 31;
 constexpr size_t kScratchDoubles = kWorkDoubles + kNoAllocMaxSlots;
 
 static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];

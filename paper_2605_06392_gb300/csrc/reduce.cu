@@ -44,12 +44,15 @@ struct PatArgs {
   const int32_t* row_of;
   const int32_t* col;
   const double* val;
-  const double* cnt;   // [ld] of this block, or null
+  const double* cnt;   // [ld] of the first block, or null
 };
 
-// out[((pq * chunks) + chunk) * kNP + s]
-__global__ void __launch_bounds__(RT) pattern_dot_kernel(PatArgs a, const double* __restrict__ Z,
-                                                         double* out) {
+// out[((t * kk + pq) * chunks + chunk) * kNP + s], block t = blockIdx.z.  One launch for
+// all blocks: 2 launches of ~5 us a block stood between the blocks of a small model.
+__global__ void __launch_bounds__(RT) pattern_dot_kernel(PatArgs a, const double* __restrict__ Zs,
+                                                         double* outs) {
+  const double* __restrict__ Z = Zs + (int64_t)blockIdx.z * a.ld * a.ld;
+  double* out = outs + (int64_t)blockIdx.z * gridDim.y * gridDim.x * kNP;
   const int chunk = blockIdx.x, pq = blockIdx.y;
   const int p = pq / a.k, q = pq % a.k;
   const int e = chunk * RT + threadIdx.x;
@@ -61,24 +64,7 @@ __global__ void __launch_bounds__(RT) pattern_dot_kernel(PatArgs a, const double
     v[0] = z * a.val[e];
     v[1] = z * a.val[a.nnz + e];
     v[2] = z * a.val[2 * a.nnz + e];
-    if (a.cnt && p == q && s1 == s2) v[3] = z * a.cnt[r];
-  }
-  block_sum<kNP>(v, out + ((int64_t)pq * gridDim.x + chunk) * kNP, 1);
-}
-
-__global__ void __launch_bounds__(RT) pattern_quad_kernel(PatArgs a, const double* __restrict__ xr,
-                                                          const double* __restrict__ xc,
-                                                          double* out) {
-  const int chunk = blockIdx.x, pq = blockIdx.y;
-  const int p = pq / a.k, q = pq % a.k;
-  const int e = chunk * RT + threadIdx.x;
-  double v[kNP] = {0.0, 0.0, 0.0, 0.0};
-  if (e < a.nnz) {
-    int s2 = a.row_of[e], s1 = a.col[e];
-    double z = xr[p * a.ns + s1] * xc[q * a.ns + s2];
-    v[0] = z * a.val[e];
-    v[1] = z * a.val[a.nnz + e];
-    v[2] = z * a.val[2 * a.nnz + e];
+    if (a.cnt && p == q && s1 == s2) v[3] = z * a.cnt[(int64_t)blockIdx.z * a.ld + r];
   }
   block_sum<kNP>(v, out + ((int64_t)pq * gridDim.x + chunk) * kNP, 1);
 }
@@ -111,11 +97,14 @@ __global__ void __launch_bounds__(RT) pattern_quad_all_kernel(PatArgs a,
   block_sum<kNP>(v, out + ((int64_t)pq * gridDim.x + chunk) * kNP, 1);
 }
 
-// <Z_C, craw> restricted to variable m: rows m*a_r.., columns m*ns..
-__global__ void __launch_bounds__(RT) arrow_dot_kernel(int ns, int a, int a_r,
-                                                       const double* __restrict__ ZC,
-                                                       const double* __restrict__ craw,
-                                                       double* out) {
+// <Z_C, craw> of block blockIdx.z restricted to variable m: rows m*a_r.., columns m*ns..
+__global__ void __launch_bounds__(RT) arrow_dot_kernel(int ns, int a, int a_r, int64_t stride,
+                                                       const double* __restrict__ ZCs,
+                                                       const double* __restrict__ craws,
+                                                       double* outs) {
+  const double* __restrict__ ZC = ZCs + blockIdx.z * stride;
+  const double* __restrict__ craw = craws + blockIdx.z * stride;
+  double* out = outs + (int64_t)blockIdx.z * gridDim.y * gridDim.x;
   const int chunk = blockIdx.x, m = blockIdx.y;
   const int i = chunk * RT + threadIdx.x;
   double v[1] = {0.0};
@@ -167,30 +156,22 @@ __device__ __forceinline__ double warp_total(double v) {
   return v;
 }
 
-constexpr int kFinThreads = 1024;
-
-// The combination of Eq. 1 and Eq. 6 from the per-block partial sums.  On
-// GB300 every dependent FP64 add costs ~64 cycles, so each sum is split over
-// the lanes of a warp (fixed order: the result is deterministic) and the
-// warps take different sums.
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a, const double* coefbuf,
-                                                               double* out) {
-  // R[j][pq][s] sums for Q_c (RDc), Q_p (RDp) and the mode's quadratic form (RX).
-  __shared__ double RDc[kNJ][kMaxK * kMaxK][kNS], RDp[kNJ][kMaxK * kMaxK][kNS],
-      RX[kNJ][kMaxK * kMaxK][kNS];
-  __shared__ double CNT[kMaxK], PC[kMaxK], TT[kMaxK], RS[kMaxK], SL[2];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int kk = a.kk, nt = a.nt, pch = a.pch, k = a.k;
+// The sums over the blocks' partial sums (Reductions) into r.red, one CTA each in a
+// fixed order: the pattern sums of (array, pq, s) against the kNJ temporal matrices, then
+// per response the counts, arrow and tip traces and squared residuals, then the two
+// log-determinants.  (One CTA for all of them was FP64-bound: 90 us of a production
+// call at 8 time blocks, 2 ms at 192.)
+__global__ void __launch_bounds__(RT) reduce_kernel(FinArgs a) {
+  const int kk = a.kk, nt = a.nt, pch = a.pch, k = a.k, np = 3 * kk * kNS;
   const Reductions& r = a.r;
-  // (1) pattern sums: one warp per (array, pq, s), lanes over (block, chunk)
-  for (int w = warp; w < 3 * kk * kNS; w += nw) {
-    const int which = w / (kk * kNS), pq = (w / kNS) % kk, s = w % kNS;
+  if ((int)blockIdx.x < np) {
+    const int w = blockIdx.x, which = w / (kk * kNS), pq = (w / kNS) % kk, s = w % kNS;
     const double* PD = which == 0 ? r.PDc : which == 1 ? r.PDp : r.QD;
     const double* PB = which == 0 ? r.PBc : which == 1 ? r.PBp : r.QB;
     double acc[kNJ] = {0.0, 0.0, 0.0};
     if (which == 2 || a.grad) {
       const int nd = nt * pch, nb = (nt - 1) * pch;
-      for (int u = lane; u < nd + nb; u += 32) {
+      for (int u = threadIdx.x; u < nd + nb; u += RT) {
         const bool isb = u >= nd;
         const int uu = isb ? u - nd : u, t = uu / pch, c = uu % pch;
         const double v = (isb ? PB : PD)[(((int64_t)t * kk + pq) * pch + c) * kNP + s];
@@ -200,56 +181,57 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a, const 
           acc[j] = fma(m, v, acc[j]);
         }
       }
-#pragma unroll
-      for (int j = 0; j < kNJ; ++j) acc[j] = warp_total(acc[j]);
     }
-    if (lane == 0)
-      for (int j = 0; j < kNJ; ++j) {
-        if (which == 0) RDc[j][pq][s] = acc[j];
-        else if (which == 1) RDp[j][pq][s] = acc[j];
-        else RX[j][pq][s] = acc[j];
-      }
+    block_sum<kNJ>(acc, r.red + ((int64_t)which * kNJ * kk + pq) * kNS + s, kk * kNS);
+    return;
   }
-  // (2) per response: counts, arrow and tip traces, residual sums; the two
-  // log-determinant slot sums
-  for (int w = warp; w < 4 * k + 2; w += nw) {
-    double v = 0.0;
-    if (w < 4 * k) {
-      const int q = w / k, m = w % k;
-      if (q == 0 && a.grad) {          // sum of the count-diagonal pattern term
-        const int mm = m * k + m;
-        for (int u = lane; u < nt * pch; u += 32) {
-          const int t = u / pch, c = u % pch;
-          v += r.PDc[(((int64_t)t * kk + mm) * pch + c) * kNP + 3];
-        }
-      } else if (q == 1 && a.grad && a.a > 0) {
-        for (int u = lane; u < nt * a.ach; u += 32) {
-          const int t = u / a.ach, c = u % a.ach;
-          v += r.PCc[((int64_t)t * k + m) * a.ach + c];
-        }
-      } else if (q == 2 && a.grad && a.a > 0) {
-        const double* tr = a.traw + (int64_t)m * a.a * a.a;
-        for (int i = lane; i < a.a * a.a; i += 32) v = fma(r.ZTc[i], tr[i], v);
-      } else if (q == 3) {
-        for (int c = lane; c < a.rch; c += 32) v += r.RS[(int64_t)m * a.rch + c];
+  const int w = blockIdx.x - np;
+  double v[1] = {0.0};
+  if (w < 4 * k) {
+    const int q = w / k, m = w % k;
+    if (q == 0 && a.grad) {          // sum of the count-diagonal pattern term
+      const int mm = m * k + m;
+      for (int u = threadIdx.x; u < nt * pch; u += RT) {
+        const int t = u / pch, c = u % pch;
+        v[0] += r.PDc[(((int64_t)t * kk + mm) * pch + c) * kNP + 3];
       }
-      v = warp_total(v);
-      if (lane == 0) {
-        if (q == 0) CNT[m] = v;
-        else if (q == 1) PC[m] = v;
-        else if (q == 2) TT[m] = v;
-        else RS[m] = v;
+    } else if (q == 1 && a.grad && a.a > 0) {
+      for (int u = threadIdx.x; u < nt * a.ach; u += RT) {
+        const int t = u / a.ach, c = u % a.ach;
+        v[0] += r.PCc[((int64_t)t * k + m) * a.ach + c];
       }
-    } else {
-      const bool cond = w == 4 * k;
-      const double* sl = cond ? r.ldc : r.ldp;
-      const int ns = cond ? a.nldc : a.nldp;
-      for (int i = lane; i < ns; i += 32) v += sl[i];
-      v = warp_total(v);
-      if (lane == 0) SL[cond ? 0 : 1] = v;
+    } else if (q == 2 && a.grad && a.a > 0) {
+      const double* tr = a.traw + (int64_t)m * a.a * a.a;
+      for (int i = threadIdx.x; i < a.a * a.a; i += RT) v[0] = fma(r.ZTc[i], tr[i], v[0]);
+    } else if (q == 3) {
+      for (int c = threadIdx.x; c < a.rch; c += RT) v[0] += r.RS[(int64_t)m * a.rch + c];
     }
+  } else {
+    const bool cond = w == 4 * k;
+    const double* sl = cond ? r.ldc : r.ldp;
+    const int ns = cond ? a.nldc : a.nldp;
+    for (int i = threadIdx.x; i < ns; i += RT) v[0] += sl[i];
   }
-  __syncthreads();
+  block_sum<1>(v, r.red + np * kNJ + w, 1);
+}
+
+constexpr int kFinThreads = 1024;
+
+// The combination of Eq. 1 and Eq. 6 from the sums of reduce_kernel.  On
+// GB300 every dependent FP64 add costs ~72 cycles, so each sum is split over
+// the lanes of a warp (fixed order: the result is deterministic) and the
+// warps take different sums.
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a, const double* coefbuf,
+                                                               double* out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int kk = a.kk, nt = a.nt, k = a.k;
+  const Reductions& r = a.r;
+  // pattern sums [kNJ][kk][kNS] of Q_c, Q_p and the mode's quadratic form
+  const double* RDc = r.red;
+  const double* RDp = RDc + kNJ * kk * kNS;
+  const double* RX = RDp + kNJ * kk * kNS;
+  const double* CNT = RX + kNJ * kk * kNS;
+  const double *PC = CNT + k, *TT = PC + k, *RS = TT + k, *SL = RS + k;
   const CoefLayout& L = a.L;
   const double* th = coefbuf + L.theta;
   const double* tau = coefbuf + L.tau;
@@ -265,7 +247,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a, const 
     double quad = 0.0;
     for (int i = lane; i < nterm; i += 32) {
       const int pq = i / (kNJ * kNS), j = (i / kNS) % kNJ, s = i % kNS;
-      quad = fma(coef[i], RX[j][pq][s], quad);
+      quad = fma(coef[i], RX[(j * kk + pq) * kNS + s], quad);
     }
     const double* beta = r.x + (int64_t)nt * a.ld;
     for (int i = lane; i < a.a; i += 32) quad += a.tip * beta[i] * beta[i];
@@ -290,9 +272,9 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinArgs a, const 
       for (int i = lane; i < nterm; i += 32) {
         const int pq = i / (kNJ * kNS), j = (i / kNS) % kNJ, s = i % kNS;
         const double w = dc[i];
-        trc = fma(w, RDc[j][pq][s], trc);
-        trp = fma(w, RDp[j][pq][s], trp);
-        qx = fma(w, RX[j][pq][s], qx);
+        trc = fma(w, RDc[(j * kk + pq) * kNS + s], trc);
+        trp = fma(w, RDp[(j * kk + pq) * kNS + s], trp);
+        qx = fma(w, RX[(j * kk + pq) * kNS + s], qx);
       }
       trc = warp_total(trc);
       trp = warp_total(trp);
@@ -324,20 +306,16 @@ int resid_chunks(const ModelDev& md) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(2048, (md.n_obs + RT - 1) / RT));
 }
 
-bta_status launch_pattern_dot(const ModelDev& md, const double* Z, int with_counts, int t,
-                              double* out, cudaStream_t s) {
-  PatArgs a{md.k, md.ns, md.ld, md.nnz, md.row_of, md.col, md.val,
-            with_counts ? md.cnt + (int64_t)t * md.ld : nullptr};
-  pattern_dot_kernel<<<dim3(pattern_chunks(md), md.k * md.k), RT, 0, s>>>(a, Z, out);
-  BTA_LAUNCHED();
-  return BTA_OK;
-}
-
-bta_status launch_pattern_quad(const ModelDev& md, const double* xr, const double* xc,
-                               double* out, cudaStream_t s) {
-  PatArgs a{md.k, md.ns, md.ld, md.nnz, md.row_of, md.col, md.val, nullptr};
-  pattern_quad_kernel<<<dim3(pattern_chunks(md), md.k * md.k), RT, 0, s>>>(a, xr, xc, out);
-  BTA_LAUNCHED();
+bta_status launch_pattern_dot(const ModelDev& md, const double* Z, int with_counts, int t0,
+                              int count, double* out, cudaStream_t s) {
+  for (int z0 = 0; z0 < count; z0 += 65535) {
+    const int cnt = std::min(65535, count - z0);
+    PatArgs a{md.k, md.ns, md.ld, md.nnz, md.row_of, md.col, md.val,
+              with_counts ? md.cnt + (int64_t)(t0 + z0) * md.ld : nullptr};
+    pattern_dot_kernel<<<dim3(pattern_chunks(md), md.k * md.k, cnt), RT, 0, s>>>(
+        a, Z + (int64_t)z0 * md.ld * md.ld, out + z0 * pattern_doubles(md));
+    BTA_LAUNCHED();
+  }
   return BTA_OK;
 }
 
@@ -350,11 +328,16 @@ bta_status launch_pattern_quad_all(const ModelDev& md, const double* x, double* 
   return BTA_OK;
 }
 
-bta_status launch_arrow_dot(const ModelDev& md, const double* ZC, int t, double* out,
+bta_status launch_arrow_dot(const ModelDev& md, const double* ZC, int count, double* out,
                             cudaStream_t s) {
-  arrow_dot_kernel<<<dim3(arrow_chunks(md), md.k), RT, 0, s>>>(
-      md.ns, md.a, md.a_r, ZC, md.craw + (int64_t)t * md.a * md.ld, out);
-  BTA_LAUNCHED();
+  const int64_t stride = (int64_t)md.a * md.ld;
+  for (int z0 = 0; z0 < count; z0 += 65535) {
+    const int cnt = std::min(65535, count - z0);
+    arrow_dot_kernel<<<dim3(arrow_chunks(md), md.k, cnt), RT, 0, s>>>(
+        md.ns, md.a, md.a_r, stride, ZC + z0 * stride, md.craw + z0 * stride,
+        out + (int64_t)z0 * md.k * arrow_chunks(md));
+    BTA_LAUNCHED();
+  }
   return BTA_OK;
 }
 
@@ -377,6 +360,8 @@ bta_status launch_finalize(const ModelDev& md, const CoefLayout& L, const double
   a.m_diag = md.m_diag; a.m_sub = md.m_sub; a.traw = md.traw;
   for (int m = 0; m < kMaxK; ++m) a.n_var[m] = m < md.k ? md.n_per_var[m] : 0.0;
   a.L = L; a.r = r;
+  reduce_kernel<<<3 * a.kk * kNS + 4 * md.k + 2, RT, 0, s>>>(a);
+  BTA_LAUNCHED();
   finalize_kernel<<<1, kFinThreads, 0, s>>>(a, coefbuf, out);
   BTA_LAUNCHED();
   return BTA_OK;

@@ -25,89 +25,100 @@ namespace {
 // Tip block (a x a, a <= kMaxTip) in one CTA: Cholesky, solves, inverse.
 constexpr int kMaxTip = 32;
 
+// One CTA of 128 threads.  FP64 latency (72 clocks an operation, several hundred a
+// division or square root) bounds it, so the columns of an update go to different
+// threads and each pivot's reciprocal is taken once.  Measured a = 9: 35 us with one
+// thread, 10 us.
 // mode 0: factor T in place (lower L_T, upper zeroed), logdet slot, and if
-//         r != null: z_T = L_T^{-1} (r_T - v_T)  (written to r)
+//         r != null: z_T = L_T^{-1} (r_T - v_T)  (written to r); T2, vT2 (or null):
+//         another leg's shares, added to T and v_T
 // mode 1: x_T = L_T^{-T} z_T in place (z)
 // mode 2: T <- Z_T = L_T^{-T} L_T^{-1} (full)
-__global__ void tip_kernel(int mode, int a, double* T, double* r, const double* vT,
-                           double* logdet_slot, int32_t* fail, int32_t fail_code) {
+constexpr int kTipThreads = 128;
+__global__ void __launch_bounds__(kTipThreads)
+    tip_kernel(int mode, int a, double* T, double* r, const double* vT, const double* T2,
+               const double* vT2, double* logdet_slot, int32_t* fail, int32_t fail_code) {
   __shared__ double L[kMaxTip][kMaxTip + 1];
-  __shared__ double v[kMaxTip];
-  __shared__ int bad;
-  if (threadIdx.x != 0) return;   // a is small; one thread keeps it exact and simple
-  for (int j = 0; j < a; ++j)
-    for (int i = 0; i < a; ++i) L[i][j] = T[i + j * a];
-  bad = 0;
+  __shared__ double rp[kMaxTip];   // reciprocal pivots
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int e = tid; e < a * a; e += kTipThreads)
+    L[e % a][e / a] = T2 ? T[e] + T2[e] : T[e];
+  __syncthreads();
   if (mode == 0) {
-    double ld = 0.0;
+    bool bad = false;
+    double ld = 0.0;   // lane j of warp 0: log of pivot j
     for (int j = 0; j < a; ++j) {
-      double dsum = L[j][j];
-      for (int k = 0; k < j; ++k) dsum -= L[j][k] * L[j][k];
-      if (!(dsum > 0.0) || !isfinite(dsum)) { bad = 1; dsum = 1.0; }
-      double piv = sqrt(dsum);
-      L[j][j] = piv;
-      ld += log(piv);
-      for (int i = j + 1; i < a; ++i) {
-        double s = L[i][j];
-        for (int k = 0; k < j; ++k) s -= L[i][k] * L[j][k];
-        L[i][j] = s / piv;
+      double d = L[j][j];
+      if (!(d > 0.0) || !isfinite(d)) { bad = true; d = 1.0; }
+      const double piv = sqrt(d), inv = 1.0 / piv;   // every thread: the same value
+      __syncthreads();
+      if (tid < a - j) {
+        L[j + tid][j] = tid == 0 ? piv : L[j + tid][j] * inv;
+        if (tid == 0) rp[j] = inv;
+      }
+      if (warp == 0 && lane == j) ld = log(piv);
+      __syncthreads();
+      for (int k = j + 1 + warp; k < a; k += kTipThreads / 32)   // column k, lane = row
+        if (lane >= k && lane < a) L[lane][k] = fma(-L[lane][j], L[k][j], L[lane][k]);
+      __syncthreads();
+    }
+    for (int e = tid; e < a * a; e += kTipThreads)
+      T[e] = e % a >= e / a ? L[e % a][e / a] : 0.0;
+    if (warp == 0) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) ld += __shfl_xor_sync(0xffffffffu, ld, o);
+      if (lane == 0) {
+        *logdet_slot = 2.0 * ld;
+        if (bad) atomicCAS(fail, -1, fail_code);
+      }
+      if (r) {   // lane = row
+        double s = lane < a ? r[lane] - vT[lane] : 0.0;
+        if (vT2 && lane < a) s -= vT2[lane];
+        for (int k = 0; k < a; ++k) {
+          const double v = __shfl_sync(0xffffffffu, s, k) * rp[k];
+          if (lane == k) s = v;
+          else if (lane > k && lane < a) s = fma(-L[lane][k], v, s);
+        }
+        if (lane < a) r[lane] = s;
       }
     }
-    for (int j = 0; j < a; ++j)
-      for (int i = 0; i < a; ++i) T[i + j * a] = i >= j ? L[i][j] : 0.0;
-    *logdet_slot = 2.0 * ld;
-    if (bad) atomicCAS(fail, -1, fail_code);
-    if (r) {
-      for (int i = 0; i < a; ++i) {
-        double s = r[i] - vT[i];
-        for (int k = 0; k < i; ++k) s -= L[i][k] * v[k];
-        v[i] = s / L[i][i];
-      }
-      for (int i = 0; i < a; ++i) r[i] = v[i];
-    }
-  } else if (mode == 1) {
-    for (int i = a - 1; i >= 0; --i) {
-      double s = r[i];
-      for (int k = i + 1; k < a; ++k) s -= L[k][i] * v[k];
-      v[i] = s / L[i][i];
-    }
-    for (int i = 0; i < a; ++i) r[i] = v[i];
-  } else {
-    // W = L^{-1} (lower), then Z = W^T W
-    __shared__ double W[kMaxTip][kMaxTip + 1];
-    for (int c = 0; c < a; ++c) {
-      for (int i = 0; i < c; ++i) W[i][c] = 0.0;
-      W[c][c] = 1.0 / L[c][c];
-      for (int i = c + 1; i < a; ++i) {
-        double s = 0.0;
-        for (int k = c; k < i; ++k) s += L[i][k] * W[k][c];
-        W[i][c] = -s / L[i][i];
-      }
-    }
-    for (int j = 0; j < a; ++j)
-      for (int i = 0; i < a; ++i) {
-        double s = 0.0;
-        for (int k = (i > j ? i : j); k < a; ++k) s += W[k][i] * W[k][j];
-        T[i + j * a] = s;
-      }
+    return;
   }
-}
-
-__global__ void copy_kernel(const double* __restrict__ src, int lds, double* __restrict__ dst,
-                            int ldd, int rows, int cols, double alpha, int mode) {
-  int64_t n = (int64_t)rows * cols;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int i = (int)(e % rows), j = (int)(e / rows);
-    double v;
-    if (mode == 1 && i < j) v = src[j + (int64_t)i * lds];
-    else v = src[i + (int64_t)j * lds];
-    dst[i + (int64_t)j * ldd] = alpha * v;
+  if (tid < a) rp[tid] = 1.0 / L[tid][tid];
+  __syncthreads();
+  if (mode == 1) {
+    if (warp == 0) {
+      double s = lane < a ? r[lane] : 0.0;
+      for (int k = a - 1; k >= 0; --k) {
+        const double v = __shfl_sync(0xffffffffu, s, k) * rp[k];
+        if (lane == k) s = v;
+        else if (lane < k) s = fma(-L[k][lane], v, s);
+      }
+      if (lane < a) r[lane] = s;
+    }
+    return;
+  }
+  // W = L^{-1} (lower): thread = column; then Z = W^T W
+  __shared__ double W[kMaxTip][kMaxTip + 1];
+  if (tid < a) {
+    for (int i = 0; i < a; ++i) W[i][tid] = i == tid ? rp[i] : 0.0;
+    for (int i = tid + 1; i < a; ++i) {
+      double s = 0.0;
+      for (int k = tid; k < i; ++k) s = fma(L[i][k], W[k][tid], s);
+      W[i][tid] = -s * rp[i];
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < a * a; e += kTipThreads) {
+    const int i = e % a, j = e / a;
+    double s = 0.0;
+    for (int k = i > j ? i : j; k < a; ++k) s = fma(W[k][i], W[k][j], s);
+    T[e] = s;
   }
 }
 
 struct CopyDev {
-  int lds, ldd, rows, cols, mode;
+  int lds, ldd, rows, cols;
   double alpha;
   const double* src[kMaxBatch];
   double* dst[kMaxBatch];
@@ -120,10 +131,35 @@ __global__ void copy_batch_kernel(CopyDev d) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
     int i = (int)(e % d.rows), j = (int)(e / d.rows);
-    double v;
-    if (d.mode == 1 && i < j) v = src[j + (int64_t)i * d.lds];
-    else v = src[i + (int64_t)j * d.lds];
-    dst[i + (int64_t)j * d.ldd] = d.alpha * v;
+    dst[i + (int64_t)j * d.ldd] = d.alpha * src[i + (int64_t)j * d.lds];
+  }
+}
+
+// A pair of 32 x 32 tiles (bi, bj) and (bj, bi), bi >= bj, per CTA: the lower one is read
+// once, coalesced, and its transpose written through shared memory (src == dst: only
+// the upper triangle is written).
+__global__ void __launch_bounds__(256) mirror_kernel(CopyDev d) {
+  const int bi = blockIdx.x, bj = blockIdx.y;
+  if (bi < bj) return;
+  const double* src = d.src[blockIdx.z];
+  double* dst = d.dst[blockIdx.z];
+  __shared__ double t[32][33];   // t[column][row]
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = bi * 32 + x, c = bj * 32 + y + 8 * q;
+    if (r < d.rows && c < d.rows) t[y + 8 * q][x] = src[r + (int64_t)c * d.lds];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int k = y + 8 * q;
+    int r = bi * 32 + x, c = bj * 32 + k;
+    if (src != dst && r >= c && r < d.rows && c < d.rows) dst[r + (int64_t)c * d.ldd] = t[k][x];
+    // element (c2, r2) of the upper triangle = (r2, c2) of the lower one
+    r = bj * 32 + x;
+    c = bi * 32 + k;
+    if (r < c && c < d.rows) dst[r + (int64_t)c * d.ldd] = t[x][k];
   }
 }
 
@@ -160,22 +196,12 @@ int sm_count() {
   return v;
 }
 
-bta_status copy_block(const double* src, int lds, double* dst, int ldd, int rows, int cols,
-                      double alpha, int mode, cudaStream_t s) {
-  int64_t n = (int64_t)rows * cols;
-  if (n <= 0) return BTA_OK;
-  int grid = (int)std::min<int64_t>(cdiv(n, 256), 32 * sm_count());
-  copy_kernel<<<grid, 256, 0, s>>>(src, lds, dst, ldd, rows, cols, alpha, mode);
-  BTA_LAUNCHED();
-  return BTA_OK;
-}
-
 bta_status copy_block_batch(int count, const double* const* src, int lds, double* const* dst,
-                            int ldd, int rows, int cols, double alpha, int mode, cudaStream_t s) {
+                            int ldd, int rows, int cols, double alpha, cudaStream_t s) {
   const int64_t n = (int64_t)rows * cols;
   if (n <= 0 || count <= 0) return BTA_OK;
   CopyDev d;
-  d.lds = lds; d.ldd = ldd; d.rows = rows; d.cols = cols; d.mode = mode; d.alpha = alpha;
+  d.lds = lds; d.ldd = ldd; d.rows = rows; d.cols = cols; d.alpha = alpha;
   for (int z0 = 0; z0 < count; z0 += kMaxBatch) {
     const int cnt = std::min(kMaxBatch, count - z0);
     for (int z = 0; z < cnt; ++z) {
@@ -184,6 +210,28 @@ bta_status copy_block_batch(int count, const double* const* src, int lds, double
     }
     int gx = (int)std::min<int64_t>(cdiv(n, 256), std::max(1, 32 * sm_count() / cnt));
     copy_batch_kernel<<<dim3(gx, cnt), 256, 0, s>>>(d);
+    BTA_LAUNCHED();
+  }
+  return BTA_OK;
+}
+
+bta_status copy_block(const double* src, int lds, double* dst, int ldd, int rows, int cols,
+                      double alpha, cudaStream_t s) {
+  return copy_block_batch(1, &src, lds, &dst, ldd, rows, cols, alpha, s);
+}
+
+bta_status mirror_batch(int count, const double* const* src, int lds, double* const* dst, int ldd,
+                        int n, cudaStream_t s) {
+  if (n <= 0 || count <= 0) return BTA_OK;
+  CopyDev d;
+  d.lds = lds; d.ldd = ldd; d.rows = n; d.cols = n; d.alpha = 1.0;
+  for (int z0 = 0; z0 < count; z0 += kMaxBatch) {
+    const int cnt = std::min(kMaxBatch, count - z0);
+    for (int z = 0; z < cnt; ++z) {
+      d.src[z] = src[z0 + z];
+      d.dst[z] = dst[z0 + z];
+    }
+    mirror_kernel<<<dim3(cdiv(n, 32), cdiv(n, 32), cnt), 256, 0, s>>>(d);
     BTA_LAUNCHED();
   }
   return BTA_OK;
@@ -208,7 +256,7 @@ size_t SweepWs::bytes(int ld, int a) {
   size_t m = (size_t)ld * ld;
   // a multiple of 256 bytes: a second workspace carved right after this one
   // keeps its blocks aligned for vector access
-  const size_t d = 4 * m + 2 * (size_t)a * ld + (size_t)kGemvSplit * ld + a + 64;
+  const size_t d = 4 * m + (size_t)a * ld + (size_t)ld + a + 64;
   return sizeof(double) * ((d + 31) / 32 * 32);
 }
 
@@ -219,9 +267,8 @@ void SweepWs::carve(double* base, int ld, int a) {
   W3 = W2 + m;
   pot = W3 + m;
   Wc1 = pot + m;
-  Wc2 = Wc1 + (size_t)a * ld;
-  gv = Wc2 + (size_t)a * ld;
-  vT = gv + (size_t)kGemvSplit * ld;
+  gv = Wc1 + (size_t)a * ld;
+  vT = gv + ld;
 }
 
 int logdet_slots(int n, int ld) { return n * potrf_inv_slots(ld) + 1; }
@@ -298,24 +345,50 @@ bta_status big_product(const Gemm& g, const SweepItem* it, const std::vector<int
   return BTA_OK;
 }
 
+// Whether a product's output may overwrite one of its operands: the tensor-core
+// products first copy their operands into planes; the FP64 tiles read them throughout.
+bool in_place(int precision, int ld) {
+  return precision == 1 || (precision == 2 && ld <= kOzakiMaxK);
+}
+
 bta_status check_set(const SweepItem* it, int m) {
   if (m < 1) return BTA_ERR_ARG;
   const bool low = it[0].q.B == nullptr;
   for (int z = 0; z < m; ++z) {
     if (it[z].q.n != it[0].q.n || it[z].q.ld != it[0].q.ld) return BTA_ERR_ARG;
+    if (it[z].rev != it[0].rev || it[z].blocks() != it[0].blocks()) return BTA_ERR_ARG;
     if (it[z].q.a > kMaxTip) return BTA_ERR_ARG;
     if ((it[z].q.B == nullptr) != low) return BTA_ERR_ARG;
-    if (low && it[z].q.n > 1 && (!it[z].md || !it[z].lay || !it[z].coef || !it[z].W4))
-      return BTA_ERR_ARG;
+    if (low && it[z].q.n > 1 && (!it[z].md || !it[z].lay || !it[z].coef)) return BTA_ERR_ARG;
   }
   return BTA_OK;
 }
 
-// Low-memory sweeps: B_i of every item of idx into the item's W2.
+// Where block i of a leg lives (SweepItem): its diagonal and arrow block, vector part and
+// slots at block(i) of the matrix, the coupling to block i + 1 in B slot coupling(i),
+// which holds Q[i+1, i] of a forward leg and the transpose of a reverse one's.
+inline int block_of(const SweepItem& it, int i) { return it.rev ? it.q.n - 1 - i : i; }
+inline int coupling_of(const SweepItem& it, int i) { return it.rev ? it.q.n - 2 - i : i; }
+inline double* D_of(const SweepItem& it, int i) {
+  return it.q.D + block_of(it, i) * (int64_t)it.q.ld * it.q.ld;
+}
+inline double* B_of(const SweepItem& it, int i) {
+  return it.q.B + coupling_of(it, i) * (int64_t)it.q.ld * it.q.ld;
+}
+inline double* C_of(const SweepItem& it, int i) {
+  return it.q.C + block_of(it, i) * (int64_t)it.q.a * it.q.ld;
+}
+inline double* vec_of(const SweepItem& it, int i) {
+  return it.vec + block_of(it, i) * (int64_t)it.q.ld;
+}
+inline double* tip_vec(const SweepItem& it) { return it.vec + (int64_t)it.q.n * it.q.ld; }
+
+// Low-memory sweeps: the coupling i of every item of idx into the item's W2.
 bta_status assemble_b_items(const SweepItem* it, const std::vector<int>& idx, int i,
                             cudaStream_t s) {
   for (int z : idx)
-    BTA_TRY(launch_assemble_b(*it[z].md, *it[z].lay, it[z].coef, i, it[z].ws.W2, s));
+    BTA_TRY(launch_assemble_b(*it[z].md, *it[z].lay, it[z].coef, coupling_of(it[z], i),
+                              it[z].ws.W2, s));
   return BTA_OK;
 }
 
@@ -327,7 +400,8 @@ bta_status assemble_b_items(const SweepItem* it, const std::vector<int>& idx, in
 bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEvent_t mark,
                               int precision, int i0, int i1) {
   BTA_TRY(check_set(it, m));
-  const int n = it[0].q.n, ld = it[0].q.ld;
+  const int n = it[0].blocks(), ld = it[0].q.ld;
+  const bool rev = it[0].rev;
   if (i1 < 0) i1 = n;
   if (i0 < 0 || i0 > i1 || i1 > n) return BTA_ERR_ARG;
   const int64_t blk = (int64_t)ld * ld;
@@ -336,40 +410,47 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEv
   const int M = (int)G.all.size();
   if (i0 == 0)
     for (int z = 0; z < m; ++z) {
-      if (it[z].q.a > 0 && it[z].vec) BTA_TRY(fill_value(it[z].ws.vT, it[z].q.a, 0.0, s));
-      BTA_TRY(fill_value(it[z].slots + (int64_t)n * p, 1, 0.0, s));
+      const int a = it[z].q.a;
+      if (a > 0 && it[z].vec)
+        BTA_CUDA_TRY(cudaMemsetAsync(it[z].ws.vT, 0, a * sizeof(double), s));
+      if (a > 0 && it[z].tip)   // the reverse leg's share of the tip
+        BTA_CUDA_TRY(cudaMemsetAsync(it[z].tip, 0, (size_t)a * a * sizeof(double), s));
+      if (a == 0 && !rev)
+        BTA_CUDA_TRY(cudaMemsetAsync(it[z].slots + (int64_t)it[z].q.n * p, 0, sizeof(double), s));
     }
-  auto D = [&](int z, int i) { return it[z].q.D + i * blk; };
-  auto B = [&](int z, int i) { return it[z].q.B + i * blk; };
-  auto Cb = [&](int z, int i) { return it[z].q.C + (int64_t)i * it[z].q.a * ld; };
+  auto D = [&](int z, int i) { return D_of(it[z], i); };
+  auto B = [&](int z, int i) { return B_of(it[z], i); };
+  auto Cb = [&](int z, int i) { return C_of(it[z], i); };
+  auto tip = [&](int z) { return it[z].tip ? it[z].tip : it[z].q.T; };
   const bool low = it[0].q.B == nullptr;
-  // where L_Bi lives: in place of B_i, or (low memory) in W1 / W4 by parity
-  auto LB = [&](int z, int i) {
-    return low ? ((i & 1) ? it[z].W4 : it[z].ws.W1) : B(z, i);
-  };
+  // where the factor's coupling L_Bi lives: in place of B_i, or (low memory) in W1 until
+  // block i + 1 has been updated with it
+  auto LB = [&](int z, int i) { return low ? it[z].ws.W1 : B(z, i); };
   // Emulated FP64: one product per matrix; the arrow rides along (arrow_fused).
   const bool emu = precision == 2 && ld <= kOzakiMaxK;
+  const bool over = in_place(precision, ld);
   auto fused = [&](int z) { return emu && arrow_fused(ld, it[z].q.a, precision); };
   auto emulate = [&](int z, const Gemm& g) -> bta_status {
     if (!it[z].ws.tc) return BTA_ERR_ARG;
     return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s);
   };
-  // L_Ci (in Wc1) into C_i, then T -= L_Ci L_Ci^T
-  auto arrow_tail = [&](const std::vector<int>& grp, int i) -> bta_status {
-    const int a = it[grp[0]].q.a, c = (int)grp.size();
+  // T -= L_Ci L_Ci^T
+  auto tip_update = [&](const std::vector<int>& grp, int i) -> bta_status {
+    const int a = it[grp[0]].q.a;
     auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
-    auto W = ptrs(grp, [&](int z) { return it[z].ws.Wc1; });
-    auto T = ptrs(grp, [&](int z) { return it[z].q.T; });
+    auto T = ptrs(grp, tip);
     auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });
-    BTA_TRY(copy_block_batch(c, cp(W), a, Ci.data(), a, a, ld, 1.0, 0, s));
-    Gemm h; h.M = a; h.N = a; h.K = ld; h.batch = c;
+    Gemm h; h.M = a; h.N = a; h.K = ld; h.batch = (int)grp.size();
     h.Ab = cp(Ci); h.lda = a; h.Bb = cp(Ci); h.ldb = a; h.transB = 1;
     h.Cb = T.data(); h.ldc = a; h.Cinb = cp(T); h.ldcin = a; h.alpha = -1.0; h.beta = 1.0;
     h.sk_wsb = SK.data(); h.sk_cap = blk;
     return gemm_f64(h, s);
   };
-  for (int i = i0; i < i1; ++i) {
-    BTA_SWEEP_MARK(s, 0, i);
+  for (int i = i0; i <= i1 && i < n; ++i) {
+    // the range's end: a reverse leg's last coupling updates the block the legs share
+    const bool join = i == i1;
+    if (join && !(rev && i1 == n - 1)) break;
+    if (!join) BTA_SWEEP_MARK(s, 0, i);
     if (i > 0) {
       if (emu) {  // D_i -= L_B,i-1 L_B,i-1^T (lower); rows below: C_i -= L_C,i-1 L_B,i-1^T
         for (int z : G.all) {
@@ -407,13 +488,33 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEv
         BTA_TRY(gemm_f64(g, s));
       }
     }
+    if (!G.vec.empty()) {
+      // t = r_i - L_B,i-1 z_{i-1} into gv (r_0 itself for the first block; into r_i where
+      // the legs join)
+      const int c = (int)G.vec.size();
+      auto ri = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
+      auto gv = ptrs(G.vec, [&](int z) { return join ? vec_of(it[z], i) : it[z].ws.gv; });
+      if (i == 0) {
+        BTA_TRY(copy_block_batch(c, cp(ri), ld, gv.data(), ld, ld, 1, 1.0, s));
+      } else {
+        auto Bp = ptrs(G.vec, [&](int z) { return LB(z, i - 1); });
+        auto rp = ptrs(G.vec, [&](int z) { return vec_of(it[z], i - 1); });
+        Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.alpha = -1.0; g.beta = 1.0; g.batch = c;
+        g.Ab = cp(Bp); g.xb = cp(rp); g.yb = gv.data(); g.yinb = cp(ri);
+        BTA_TRY(gemv_f64(g, s));
+      }
+    }
+    if (join) return BTA_OK;
     {  // L_Di^{-1} in place, log-det slots
       auto Di = ptrs(G.all, [&](int z) { return D(z, i); });
       auto W = ptrs(G.all, [&](int z) { return it[z].ws.pot; });
-      auto sl = ptrs(G.all, [&](int z) { return it[z].slots + (int64_t)i * p; });
+      auto sl = ptrs(G.all, [&](int z) { return it[z].slots + (int64_t)block_of(it[z], i) * p; });
       std::vector<int32_t*> fl;
-      std::vector<int32_t> code(M, i);
-      for (int z : G.all) fl.push_back(it[z].fail);
+      std::vector<int32_t> code;
+      for (int z : G.all) {
+        fl.push_back(it[z].fail);
+        code.push_back(block_of(it[z], i));
+      }
       std::vector<void*> tw;
       std::vector<int32_t*> ts;
       for (int z : G.all) {
@@ -439,57 +540,50 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEv
       g.Cb = W.data(); g.ldc = a;
       g.sk_wsb = SK.data(); g.sk_cap = blk;
       BTA_TRY(gemm_f64(g, s));
-      BTA_TRY(arrow_tail(grp, i));
+      BTA_TRY(copy_block_batch(c, cp(W), a, Ci.data(), a, a, ld, 1.0, s));
+      BTA_TRY(tip_update(grp, i));
     }
-    if (i < n - 1) {  // L_Bi = B_i L_Di^{-T}
+    if (i < n - 1) {  // L_Bi = Q[i+1, i] L_Di^{-T}
       if (low) BTA_TRY(assemble_b_items(it, G.all, i, s));
       auto Bi = ptrs(G.all, [&](int z) { return low ? it[z].ws.W2 : B(z, i); });
       auto Di = ptrs(G.all, [&](int z) { return D(z, i); });
-      auto W = ptrs(G.all, [&](int z) { return low ? LB(z, i) : it[z].ws.W1; });
-      if (emu) {  // rows below: L_Ci = C_i L_Di^{-T} into Wc1
+      auto W = ptrs(G.all, [&](int z) { return low || !over ? it[z].ws.W1 : B(z, i); });
+      if (emu) {  // rows below: L_Ci = C_i L_Di^{-T}
         for (size_t q = 0; q < G.all.size(); ++q) {
           const int z = G.all[q];
           Gemm g; g.M = ld; g.N = ld; g.K = ld;
-          g.A = Bi[q]; g.lda = ld; g.B = Di[q]; g.ldb = ld; g.transB = 1; g.triB = TRI_UPPER;
-          g.C = W[q]; g.ldc = ld;
+          g.A = Bi[q]; g.lda = ld; g.transA = rev; g.B = Di[q]; g.ldb = ld; g.transB = 1;
+          g.triB = TRI_UPPER; g.C = W[q]; g.ldc = ld;
           if (fused(z)) {
             const int a = it[z].q.a;
             g.M = ld + a; g.a_rows = ld; g.A21 = {Cb(z, i), a, 0};
-            g.c_rows = ld; g.C2 = it[z].ws.Wc1; g.ldc2 = a;
+            g.c_rows = ld; g.C2 = Cb(z, i); g.ldc2 = a;
           }
           BTA_TRY(emulate(z, g));
         }
       } else {
         Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
-        g.Ab = cp(Bi); g.lda = ld; g.Bb = cp(Di); g.ldb = ld; g.transB = 1; g.triB = TRI_UPPER;
-        g.Cb = W.data(); g.ldc = ld;
+        g.Ab = cp(Bi); g.lda = ld; g.transA = rev; g.Bb = cp(Di); g.ldb = ld; g.transB = 1;
+        g.triB = TRI_UPPER; g.Cb = W.data(); g.ldc = ld;
         BTA_TRY(big_product(g, it, G.all, precision, s));
       }
-      if (!low) BTA_TRY(copy_block_batch(M, cp(W), ld, Bi.data(), ld, ld, ld, 1.0, 0, s));
+      if (!low && !over) BTA_TRY(copy_block_batch(M, cp(W), ld, Bi.data(), ld, ld, ld, 1.0, s));
       if (with_b)
         for (const auto& grp : G.arrow)
-          if (fused(grp[0])) BTA_TRY(arrow_tail(grp, i));
+          if (fused(grp[0])) BTA_TRY(tip_update(grp, i));
     }
-    if (!G.vec.empty()) {  // z_i = L_Di^{-1} (r_i - L_B,i-1 z_{i-1});  v_T += L_Ci z_i
-      const int c = (int)G.vec.size();
-      auto ri = ptrs(G.vec, [&](int z) { return it[z].vec + (int64_t)i * ld; });
+    if (!G.vec.empty()) {  // z_i = L_Di^{-1} t;  v_T += L_Ci z_i
+      auto zi = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
       auto gv = ptrs(G.vec, [&](int z) { return it[z].ws.gv; });
-      if (i > 0) {
-        auto Bp = ptrs(G.vec, [&](int z) { return LB(z, i - 1); });
-        auto rp = ptrs(G.vec, [&](int z) { return it[z].vec + (int64_t)(i - 1) * ld; });
-        Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.alpha = -1.0; g.beta = 1.0; g.batch = c;
-        g.Ab = cp(Bp); g.xb = cp(rp); g.yb = ri.data(); g.yinb = cp(ri); g.workb = gv.data();
-        BTA_TRY(gemv_f64(g, nullptr, s));
-      }
       auto Di = ptrs(G.vec, [&](int z) { return D(z, i); });
-      Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.triA = TRI_LOWER; g.batch = c;
-      g.Ab = cp(Di); g.xb = cp(ri); g.yb = ri.data(); g.workb = gv.data();
-      BTA_TRY(gemv_f64(g, nullptr, s));
+      Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.triA = TRI_LOWER; g.batch = (int)G.vec.size();
+      g.Ab = cp(Di); g.xb = cp(gv); g.yb = zi.data();
+      BTA_TRY(gemv_f64(g, s));
       for (int z : G.vec) {
         if (it[z].q.a == 0) continue;
         Gemv h; h.M = it[z].q.a; h.K = ld; h.A = Cb(z, i); h.lda = it[z].q.a;
-        h.x = it[z].vec + (int64_t)i * ld; h.y = it[z].ws.vT; h.yin = it[z].ws.vT; h.beta = 1.0;
-        BTA_TRY(gemv_f64(h, it[z].ws.gv, s));
+        h.x = vec_of(it[z], i); h.y = it[z].ws.vT; h.beta = 1.0;
+        BTA_TRY(gemv_f64(h, s));
       }
     }
     BTA_SWEEP_MARK(s, 3, i);
@@ -498,8 +592,10 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEv
   for (int z = 0; z < m; ++z) {
     const int a = it[z].q.a;
     if (a == 0) continue;
-    tip_kernel<<<1, 32, 0, s>>>(0, a, it[z].q.T, it[z].vec ? it[z].vec + (int64_t)n * ld : nullptr,
-                                it[z].ws.vT, it[z].slots + (int64_t)n * p, it[z].fail, n);
+    tip_kernel<<<1, kTipThreads, 0, s>>>(0, a, it[z].q.T, it[z].vec ? tip_vec(it[z]) : nullptr,
+                                         it[z].ws.vT, it[z].tip2, it[z].vT2,
+                                         it[z].slots + (int64_t)it[z].q.n * p, it[z].fail,
+                                         it[z].q.n);
     BTA_LAUNCHED();
   }
   return BTA_OK;
@@ -525,8 +621,7 @@ __global__ void diag_axpy_kernel(const double* __restrict__ D, int ld, const dou
 }
 }  // namespace
 
-bta_status bta_residual(const bta_desc& q, const double* x, double* d, double* gv,
-                        cudaStream_t s) {
+bta_status bta_residual(const bta_desc& q, const double* x, double* d, cudaStream_t s) {
   const int n = q.n, ld = q.ld, a = q.a;
   const int64_t blk = (int64_t)ld * ld;
   const double* xT = x + (int64_t)n * ld;
@@ -538,8 +633,8 @@ bta_status bta_residual(const bta_desc& q, const double* x, double* d, double* g
     auto minus = [&](const double* A, int lda, int M, int K, int trans, int tri,
                      const double* v, double* y) {
       Gemv g; g.M = M; g.K = K; g.A = A; g.lda = lda; g.transA = trans; g.triA = tri;
-      g.x = v; g.y = y; g.yin = y; g.alpha = -1.0; g.beta = 1.0;
-      return gemv_f64(g, gv, s);
+      g.x = v; g.y = y; g.alpha = -1.0; g.beta = 1.0;
+      return gemv_f64(g, s);
     };
     BTA_TRY(minus(Di, ld, ld, ld, 0, TRI_LOWER, xi, di));          // - L x
     BTA_TRY(minus(Di, ld, ld, ld, 1, TRI_UPPER, xi, di));          // - L^T x
@@ -555,10 +650,10 @@ bta_status bta_residual(const bta_desc& q, const double* x, double* d, double* g
   }
   if (a > 0) {   // - T x_T (lower triangle referenced, as D)
     Gemv g; g.M = a; g.K = a; g.A = q.T; g.lda = a; g.triA = TRI_LOWER;
-    g.x = xT; g.y = dT; g.yin = dT; g.alpha = -1.0; g.beta = 1.0;
-    BTA_TRY(gemv_f64(g, gv, s));
+    g.x = xT; g.y = dT; g.alpha = -1.0; g.beta = 1.0;
+    BTA_TRY(gemv_f64(g, s));
     g.transA = 1; g.triA = TRI_UPPER;
-    BTA_TRY(gemv_f64(g, gv, s));
+    BTA_TRY(gemv_f64(g, s));
     diag_axpy_kernel<<<1, 32, 0, s>>>(q.T, a, xT, dT);
     BTA_LAUNCHED();
   }
@@ -566,121 +661,138 @@ bta_status bta_residual(const bta_desc& q, const double* x, double* d, double* g
 }
 
 // ----------------------------------------------------------------------------
-// Lower solve alone (L z = r) on one matrix, for bta_solve(lower = 1)
+// Lower solve alone (L z = r) with a factor: blocks i0 <= i < i1 of a leg, the set-up
+// with the first and the tip with a forward leg's last (see factor_sweep_multi)
 // ----------------------------------------------------------------------------
 namespace {
-__global__ void tip_fwd_kernel(int a, const double* T, double* r, const double* vT) {
-  if (threadIdx.x || blockIdx.x) return;
-  double v[kMaxTip];
-  for (int i = 0; i < a; ++i) {
-    double s = r[i] - vT[i];
-    for (int k = 0; k < i; ++k) s -= T[i + k * a] * v[k];
-    v[i] = s / T[i + i * a];
+// z_T = L_T^{-1} (r_T - v_T - v2_T) with the factored tip: one warp, lane = row.
+__global__ void tip_fwd_kernel(int a, const double* T, double* r, const double* vT,
+                               const double* vT2) {
+  const int lane = threadIdx.x;
+  double s = 0.0, inv = 0.0;
+  if (lane < a) {
+    s = r[lane] - vT[lane];
+    if (vT2) s -= vT2[lane];
+    inv = 1.0 / T[lane + lane * a];
   }
-  for (int i = 0; i < a; ++i) r[i] = v[i];
+  for (int k = 0; k < a; ++k) {
+    const double v = __shfl_sync(0xffffffffu, s * inv, k);
+    if (lane == k) s = v;
+    else if (lane > k && lane < a) s = fma(-T[lane + k * a], v, s);
+  }
+  if (lane < a) r[lane] = s;
 }
 }  // namespace
 
-bta_status tip_forward(const bta_desc& q, double* rT, const double* vT, cudaStream_t s) {
-  tip_fwd_kernel<<<1, 32, 0, s>>>(q.a, q.T, rT, vT);
-  BTA_LAUNCHED();
-  return BTA_OK;
-}
-
-bta_status lower_solve(const bta_desc& q, double* z, const SweepWs& ws, cudaStream_t s) {
-  const int n = q.n, ld = q.ld, a = q.a;
-  const int64_t blk = (int64_t)ld * ld;
-  if (a > 0) BTA_TRY(fill_value(ws.vT, a, 0.0, s));
-  for (int i = 0; i < n; ++i) {
-    double* ri = z + (int64_t)i * ld;
-    if (i > 0) {
-      Gemv g; g.M = ld; g.K = ld; g.A = q.B + (i - 1) * blk; g.lda = ld;
-      g.x = ri - ld; g.y = ri; g.yin = ri; g.alpha = -1.0; g.beta = 1.0;
-      BTA_TRY(gemv_f64(g, ws.gv, s));
+bta_status lower_solve(const SweepItem& it, cudaStream_t s, int i0, int i1) {
+  const int n = it.blocks(), ld = it.q.ld, a = it.q.a;
+  const bool rev = it.rev;
+  if (i1 < 0) i1 = n;
+  if (i0 < 0 || i0 > i1 || i1 > n || !it.vec || (n > 1 && !it.q.B)) return BTA_ERR_ARG;
+  if (a > 0 && i0 == 0)
+    BTA_CUDA_TRY(cudaMemsetAsync(it.ws.vT, 0, a * sizeof(double), s));
+  for (int i = i0; i <= i1 && i < n; ++i) {
+    const bool join = i == i1;
+    if (join && !(rev && i1 == n - 1)) break;
+    double* ri = vec_of(it, i);
+    if (i == 0) {
+      BTA_TRY(copy_block(ri, ld, it.ws.gv, ld, ld, 1, 1.0, s));
+    } else {
+      Gemv g; g.M = ld; g.K = ld; g.A = B_of(it, i - 1); g.lda = ld;
+      g.x = vec_of(it, i - 1); g.y = join ? ri : it.ws.gv; g.yin = ri;
+      g.alpha = -1.0; g.beta = 1.0;
+      BTA_TRY(gemv_f64(g, s));
     }
-    Gemv g; g.M = ld; g.K = ld; g.A = q.D + i * blk; g.lda = ld; g.triA = TRI_LOWER;
-    g.x = ri; g.y = ri;
-    BTA_TRY(gemv_f64(g, ws.gv, s));
+    if (join) return BTA_OK;
+    Gemv g; g.M = ld; g.K = ld; g.A = D_of(it, i); g.lda = ld; g.triA = TRI_LOWER;
+    g.x = it.ws.gv; g.y = ri;
+    BTA_TRY(gemv_f64(g, s));
     if (a > 0) {
-      Gemv h; h.M = a; h.K = ld; h.A = q.C + (int64_t)i * a * ld; h.lda = a; h.x = ri;
-      h.y = ws.vT; h.yin = ws.vT; h.beta = 1.0;
-      BTA_TRY(gemv_f64(h, ws.gv, s));
+      Gemv h; h.M = a; h.K = ld; h.A = C_of(it, i); h.lda = a; h.x = ri;
+      h.y = it.ws.vT; h.beta = 1.0;
+      BTA_TRY(gemv_f64(h, s));
     }
   }
-  if (a > 0) BTA_TRY(tip_forward(q, z + (int64_t)n * ld, ws.vT, s));
+  if (i1 == n && a > 0) {
+    tip_fwd_kernel<<<1, 32, 0, s>>>(a, it.q.T, tip_vec(it), it.ws.vT, it.vT2);
+    BTA_LAUNCHED();
+  }
   return BTA_OK;
 }
 
 // ----------------------------------------------------------------------------
 // Eqs. 3-5 on a set of matrices (items with a vector)
 // ----------------------------------------------------------------------------
-bta_status upper_solve_multi(const SweepItem* it, int m, cudaStream_t s) {
+bta_status upper_solve_multi(const SweepItem* it, int m, cudaStream_t s, int i_hi, int i_lo) {
   BTA_TRY(check_set(it, m));
-  const int n = it[0].q.n, ld = it[0].q.ld;
-  const int64_t blk = (int64_t)ld * ld;
+  const int n = it[0].blocks(), ld = it[0].q.ld;
+  if (i_hi < 0) i_hi = n - 1;
+  if (i_lo < 0 || i_hi >= n || i_lo > i_hi + 1) return BTA_ERR_ARG;
   const Groups G = make_groups(it, m);
   if (G.vec.empty()) return BTA_OK;
   const int c = (int)G.vec.size();
-  for (int z : G.vec) {
-    const int a = it[z].q.a;
-    if (a == 0) continue;
-    tip_kernel<<<1, 32, 0, s>>>(1, a, it[z].q.T, it[z].vec + (int64_t)n * ld, nullptr, nullptr,
-                                nullptr, 0);
-    BTA_LAUNCHED();
-  }
-  auto gv = ptrs(G.vec, [&](int z) { return it[z].ws.gv; });
-  for (int i = n - 1; i >= 0; --i) {
-    auto zi = ptrs(G.vec, [&](int z) { return it[z].vec + (int64_t)i * ld; });
-    for (int z : G.vec) {  // z_i -= L_Ci^T x_T
+  if (i_hi == n - 1)
+    for (int z : G.vec) {
       const int a = it[z].q.a;
       if (a == 0) continue;
-      double* zz = it[z].vec + (int64_t)i * ld;
-      Gemv g; g.M = ld; g.K = a; g.A = it[z].q.C + (int64_t)i * a * ld; g.lda = a; g.transA = 1;
-      g.x = it[z].vec + (int64_t)n * ld; g.y = zz; g.yin = zz; g.alpha = -1.0; g.beta = 1.0;
-      BTA_TRY(gemv_f64(g, it[z].ws.gv, s));
+      tip_kernel<<<1, kTipThreads, 0, s>>>(1, a, it[z].q.T, tip_vec(it[z]), nullptr, nullptr,
+                                           nullptr, nullptr, nullptr, 0);
+      BTA_LAUNCHED();
     }
-    if (i < n - 1 && it[0].q.B) {  // z_i -= L_Bi^T x_{i+1}
-      auto Bi = ptrs(G.vec, [&](int z) { return it[z].q.B + i * blk; });
-      auto xn = ptrs(G.vec, [&](int z) { return it[z].vec + (int64_t)(i + 1) * ld; });
-      Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.transA = 1; g.alpha = -1.0; g.beta = 1.0;
-      g.batch = c; g.Ab = cp(Bi); g.xb = cp(xn); g.yb = zi.data(); g.yinb = cp(zi);
-      g.workb = gv.data();
-      BTA_TRY(gemv_f64(g, nullptr, s));
-    } else if (i < n - 1) {
-      // low memory: L_Bi^T x_{i+1} = L_Di^{-1} (B_i^T x_{i+1}), B_i assembled into W2,
-      // the product into W3's first ld entries
+  bool same_a = true;   // one launch over the set: the arrow rides along
+  for (int z : G.vec) same_a = same_a && it[z].q.a == it[G.vec[0]].q.a;
+  if (!same_a) return BTA_ERR_ARG;
+  const int a = it[G.vec[0]].q.a;
+  const bool low = it[0].q.B == nullptr;
+  auto gv = ptrs(G.vec, [&](int z) { return it[z].ws.gv; });
+  auto xT = ptrs(G.vec, [&](int z) { return tip_vec(it[z]); });
+  for (int i = i_hi; i >= i_lo; --i) {
+    auto zi = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
+    auto Di = ptrs(G.vec, [&](int z) { return D_of(it[z], i); });
+    std::vector<double*> Ci;
+    if (a > 0) Ci = ptrs(G.vec, [&](int z) { return C_of(it[z], i); });
+    const bool hasB = i < n - 1;
+    std::vector<double*> xn;
+    if (hasB) xn = ptrs(G.vec, [&](int z) { return vec_of(it[z], i + 1); });
+    // gv = z_i - L_Bi^T x_{i+1} - L_Ci^T x_T
+    Gemv g; g.M = ld; g.transA = 1; g.alpha = -1.0; g.beta = 1.0; g.batch = c;
+    g.yb = gv.data(); g.yinb = cp(zi);
+    if (hasB && !low) {
+      auto Bi = ptrs(G.vec, [&](int z) { return B_of(it[z], i); });
+      g.K = ld; g.lda = ld; g.Ab = cp(Bi); g.xb = cp(xn);
+      if (a > 0) { g.K2 = a; g.lda2 = a; g.A2b = cp(Ci); g.x2b = cp(xT); }
+      BTA_TRY(gemv_f64(g, s));
+    } else if (a > 0) {
+      g.K = a; g.lda = a; g.Ab = cp(Ci); g.xb = cp(xT);
+      BTA_TRY(gemv_f64(g, s));
+    } else {
+      BTA_TRY(copy_block_batch(c, cp(zi), ld, gv.data(), ld, ld, 1, 1.0, s));
+    }
+    if (hasB && low) {
+      // low memory: L_Bi^T x_{i+1} = L_Di^{-1} (Q[i+1, i]^T x_{i+1}), the coupling assembled
+      // into W2, the product into W3's first ld entries
       BTA_TRY(assemble_b_items(it, G.vec, i, s));
       auto W2 = ptrs(G.vec, [&](int z) { return it[z].ws.W2; });
       auto t = ptrs(G.vec, [&](int z) { return it[z].ws.W3; });
-      auto xn = ptrs(G.vec, [&](int z) { return it[z].vec + (int64_t)(i + 1) * ld; });
-      Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.transA = 1; g.batch = c;
-      g.Ab = cp(W2); g.xb = cp(xn); g.yb = t.data(); g.workb = gv.data();
-      BTA_TRY(gemv_f64(g, nullptr, s));
-      auto Di = ptrs(G.vec, [&](int z) { return it[z].q.D + i * blk; });
+      Gemv b; b.M = ld; b.K = ld; b.lda = ld; b.transA = !it[0].rev; b.batch = c;
+      b.Ab = cp(W2); b.xb = cp(xn); b.yb = t.data();
+      BTA_TRY(gemv_f64(b, s));
       Gemv h; h.M = ld; h.K = ld; h.lda = ld; h.triA = TRI_LOWER; h.alpha = -1.0; h.beta = 1.0;
-      h.batch = c; h.Ab = cp(Di); h.xb = cp(t); h.yb = zi.data(); h.yinb = cp(zi);
-      h.workb = gv.data();
-      BTA_TRY(gemv_f64(h, nullptr, s));
+      h.batch = c; h.Ab = cp(Di); h.xb = cp(t); h.yb = gv.data();
+      BTA_TRY(gemv_f64(h, s));
     }
-    {  // x_i = L_Di^{-T} z_i
-      auto Di = ptrs(G.vec, [&](int z) { return it[z].q.D + i * blk; });
-      Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.transA = 1; g.triA = TRI_UPPER;
-      g.batch = c; g.Ab = cp(Di); g.xb = cp(zi); g.yb = zi.data(); g.workb = gv.data();
-      BTA_TRY(gemv_f64(g, nullptr, s));
+    {  // x_i = L_Di^{-T} gv
+      Gemv h; h.M = ld; h.K = ld; h.lda = ld; h.transA = 1; h.triA = TRI_UPPER;
+      h.batch = c; h.Ab = cp(Di); h.xb = cp(gv); h.yb = zi.data();
+      BTA_TRY(gemv_f64(h, s));
     }
   }
   return BTA_OK;
 }
 
-bta_status upper_solve(const bta_desc& q, double* z, const SweepWs& ws, cudaStream_t s) {
-  SweepItem item;
-  item.q = q; item.vec = z; item.ws = ws;
-  return upper_solve_multi(&item, 1, s);
-}
-
 // ----------------------------------------------------------------------------
-// Selected inversion, in place, on a set of matrices, with the fused Eq. 7
-// reductions.  With F_Bi = L_Bi L_Di^{-1}, F_Ci = L_Ci L_Di^{-1}:
+// Selected inversion, in place, on a set of matrices.  With F_Bi = L_Bi
+// L_Di^{-1}, F_Ci = L_Ci L_Di^{-1}:
 //   Z_Ci = -Z_T F_Ci - Z_C,i+1 F_Bi
 //   Z_Bi = -Z_D,i+1 F_Bi - Z_C,i+1^T F_Ci
 //   Z_Di = L_Di^{-T} L_Di^{-1} - Z_Bi^T F_Bi - Z_Ci^T F_Ci
@@ -688,27 +800,28 @@ bta_status upper_solve(const bta_desc& q, double* z, const SweepWs& ws, cudaStre
 bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int precision,
                               int i_hi, int i_lo) {
   BTA_TRY(check_set(it, m));
-  const int n = it[0].q.n, ld = it[0].q.ld;
+  const int n = it[0].blocks(), ld = it[0].q.ld;
+  const bool rev = it[0].rev;
   if (i_hi < 0) i_hi = n - 1;
   if (i_lo < 0 || i_hi >= n || i_lo > i_hi + 1) return BTA_ERR_ARG;
   const int64_t blk = (int64_t)ld * ld;
   const Groups G = make_groups(it, m);
   const int M = (int)G.all.size();
-  auto D = [&](int z, int i) { return it[z].q.D + i * blk; };
-  auto B = [&](int z, int i) { return it[z].q.B + i * blk; };
-  auto Cb = [&](int z, int i) { return it[z].q.C + (int64_t)i * it[z].q.a * ld; };
-  if (i_hi == n - 1)
+  auto D = [&](int z, int i) { return D_of(it[z], i); };
+  auto B = [&](int z, int i) { return B_of(it[z], i); };
+  auto Cb = [&](int z, int i) { return C_of(it[z], i); };
+  if (i_hi == n - 1 && !rev)
     for (int z = 0; z < m; ++z) {
       if (it[z].q.a == 0) continue;
-      tip_kernel<<<1, 32, 0, s>>>(2, it[z].q.a, it[z].q.T, nullptr, nullptr, nullptr, nullptr, 0);
+      tip_kernel<<<1, kTipThreads, 0, s>>>(2, it[z].q.a, it[z].q.T, nullptr, nullptr, nullptr,
+                                           nullptr, nullptr, nullptr, 0);
       BTA_LAUNCHED();
     }
   auto W1 = ptrs(G.all, [&](int z) { return it[z].ws.W1; });
-  auto W2 = ptrs(G.all, [&](int z) { return it[z].ws.W2; });
-  auto W3 = ptrs(G.all, [&](int z) { return it[z].ws.W3; });
   const bool low = it[0].q.B == nullptr;
   // Emulated FP64: one product per matrix; the arrow rides along (arrow_fused).
   const bool emu = precision == 2 && ld <= kOzakiMaxK;
+  const bool over = in_place(precision, ld);
   auto fused = [&](int z) { return emu && arrow_fused(ld, it[z].q.a, precision); };
   auto emulate = [&](int z, const Gemm& g) -> bta_status {
     if (!it[z].ws.tc) return BTA_ERR_ARG;
@@ -718,11 +831,18 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
     BTA_SWEEP_MARK(s, 4, i);
     const bool hasB = i < n - 1;
     auto Di = ptrs(G.all, [&](int z) { return D(z, i); });
-    if (hasB && low) {  // low memory: W3 = L_Bi = B_i L_Di^{-T}, B_i assembled into W2
+    // Z_B in place of L_Bi, free once F_B is formed (low memory: in W2)
+    std::vector<double*> ZB;
+    if (hasB) ZB = ptrs(G.all, [&](int z) { return low ? it[z].ws.W2 : B(z, i); });
+    // Z_D is built in place, or (FP64 products) in W3
+    auto ZD = ptrs(G.all, [&](int z) { return over ? D(z, i) : it[z].ws.W3; });
+    if (hasB && low) {  // low memory: W3 = L_Bi = Q[i+1, i] L_Di^{-T}, assembled into W2
       BTA_TRY(assemble_b_items(it, G.all, i, s));
+      auto W2 = ptrs(G.all, [&](int z) { return it[z].ws.W2; });
+      auto W3 = ptrs(G.all, [&](int z) { return it[z].ws.W3; });
       Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
-      g.Ab = cp(W2); g.lda = ld; g.Bb = cp(Di); g.ldb = ld; g.transB = 1; g.triB = TRI_UPPER;
-      g.Cb = W3.data(); g.ldc = ld;
+      g.Ab = cp(W2); g.lda = ld; g.transA = rev; g.Bb = cp(Di); g.ldb = ld; g.transB = 1;
+      g.triB = TRI_UPPER; g.Cb = W3.data(); g.ldc = ld;
       BTA_TRY(big_product(g, it, G.all, precision, s));
     }
     if (hasB) {  // W1 = F_B = L_Bi L_Di^{-1}
@@ -755,7 +875,6 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
       auto Dg = ptrs(grp, [&](int z) { return D(z, i); });
       auto Wc1 = ptrs(grp, [&](int z) { return it[z].ws.Wc1; });
-      auto Wc2 = ptrs(grp, [&](int z) { return it[z].ws.Wc2; });
       auto T = ptrs(grp, [&](int z) { return it[z].q.T; });
       auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });   // W3 is free until LAUUM
       {  // Wc1 = F_C = L_Ci L_Di^{-1}
@@ -765,18 +884,18 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         g.sk_wsb = SK.data(); g.sk_cap = blk;
         BTA_TRY(gemm_f64(g, s));
       }
-      {  // Wc2 = -Z_T F_C
+      {  // Z_C = -Z_T F_C, in place of L_Ci
         Gemm g; g.M = a; g.N = ld; g.K = a; g.batch = c;
         g.Ab = cp(T); g.lda = a; g.Bb = cp(Wc1); g.ldb = a;
-        g.Cb = Wc2.data(); g.ldc = a; g.alpha = -1.0;
+        g.Cb = Ci.data(); g.ldc = a; g.alpha = -1.0;
         BTA_TRY(gemm_f64(g, s));
       }
-      if (hasB) {  // Wc2 -= Z_C,i+1 F_B
+      if (hasB) {  // Z_C -= Z_C,i+1 F_B
         auto Cn = ptrs(grp, [&](int z) { return Cb(z, i + 1); });
         auto W1g = ptrs(grp, [&](int z) { return it[z].ws.W1; });
         Gemm g; g.M = a; g.N = ld; g.K = ld; g.batch = c;
         g.Ab = cp(Cn); g.lda = a; g.Bb = cp(W1g); g.ldb = ld;
-        g.Cb = Wc2.data(); g.ldc = a; g.Cinb = cp(Wc2); g.ldcin = a; g.alpha = -1.0;
+        g.Cb = Ci.data(); g.ldc = a; g.Cinb = cp(Ci); g.ldcin = a; g.alpha = -1.0;
         g.beta = 1.0;
         g.sk_wsb = SK.data(); g.sk_cap = blk;
         BTA_TRY(gemm_f64(g, s));
@@ -785,36 +904,36 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
     if (hasB) {
       auto Dn = ptrs(G.all, [&](int z) { return D(z, i + 1); });
       if (emu) {
-        // W2 = Z_B = -Z_D,i+1 F_B; an arrow carried along as a 2 x 2 block
-        // product: [W2; Wc2] = -[Z_D,i+1, Z_C,i+1^T; Z_C,i+1, Z_T] [F_B; F_C],
-        // i.e. also W2 -= Z_C,i+1^T F_C and Wc2 = Z_C = -Z_C,i+1 F_B - Z_T F_C
+        // Z_B = -Z_D,i+1 F_B; an arrow carried along as a 2 x 2 block product:
+        // [Z_B; Z_C] = -[Z_D,i+1, Z_C,i+1^T; Z_C,i+1, Z_T] [F_B; F_C],
+        // i.e. also Z_B -= Z_C,i+1^T F_C and Z_C = -Z_C,i+1 F_B - Z_T F_C
         for (size_t q = 0; q < G.all.size(); ++q) {
           const int z = G.all[q];
           Gemm g; g.M = ld; g.N = ld; g.K = ld;
           g.A = Dn[q]; g.lda = ld; g.B = W1[q]; g.ldb = ld;
-          g.C = W2[q]; g.ldc = ld; g.alpha = -1.0;
+          g.C = ZB[q]; g.ldc = ld; g.alpha = -1.0;
           if (fused(z)) {
             const int a = it[z].q.a;
             const double* Cn = Cb(z, i + 1);
             g.M = ld + a; g.K = ld + a; g.a_rows = ld; g.a_k = ld;
             g.A12 = {Cn, a, 1}; g.A21 = {Cn, a, 0}; g.A22 = {it[z].q.T, a, 0};
             g.b_k = ld; g.B21 = {it[z].ws.Wc1, a, 0};
-            g.c_rows = ld; g.C2 = it[z].ws.Wc2; g.ldc2 = a;
+            g.c_rows = ld; g.C2 = Cb(z, i); g.ldc2 = a;
           }
           BTA_TRY(emulate(z, g));
         }
-      } else {  // W2 = Z_B = -Z_D,i+1 F_B
+      } else {  // Z_B = -Z_D,i+1 F_B
         Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
         g.Ab = cp(Dn); g.lda = ld; g.Bb = cp(W1); g.ldb = ld;
-        g.Cb = W2.data(); g.ldc = ld; g.alpha = -1.0;
+        g.Cb = ZB.data(); g.ldc = ld; g.alpha = -1.0;
         BTA_TRY(big_product(g, it, G.all, precision, s));
       }
-      for (const auto& grp : G.arrow) {  // W2 -= Z_C,i+1^T F_C
+      for (const auto& grp : G.arrow) {  // Z_B -= Z_C,i+1^T F_C
         if (fused(grp[0])) continue;
         const int a = it[grp[0]].q.a, c = (int)grp.size();
         auto Cn = ptrs(grp, [&](int z) { return Cb(z, i + 1); });
         auto Wc1 = ptrs(grp, [&](int z) { return it[z].ws.Wc1; });
-        auto W2g = ptrs(grp, [&](int z) { return it[z].ws.W2; });
+        auto W2g = ptrs(grp, [&](int z) { return low ? it[z].ws.W2 : B(z, i); });
         Gemm g; g.M = ld; g.N = ld; g.K = a; g.batch = c;
         g.Ab = cp(Cn); g.lda = a; g.transA = 1; g.Bb = cp(Wc1); g.ldb = a;
         g.Cb = W2g.data(); g.ldc = ld; g.Cinb = cp(W2g); g.ldcin = ld; g.alpha = -1.0;
@@ -822,74 +941,71 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         BTA_TRY(gemm_f64(g, s));
       }
     }
-    {  // W3 = L_Di^{-T} L_Di^{-1} (lower part)
+    {  // Z_D = L_Di^{-T} L_Di^{-1} (lower part)
       Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
       g.Ab = cp(Di); g.lda = ld; g.transA = 1; g.triA = TRI_UPPER;
       g.Bb = cp(Di); g.ldb = ld; g.triB = TRI_LOWER;
-      g.Cb = W3.data(); g.ldc = ld; g.out_lower = 1;
+      g.Cb = ZD.data(); g.ldc = ld; g.out_lower = 1;
       BTA_TRY(big_product(g, it, G.all, precision, s));
     }
-    if (hasB) {  // W3 -= Z_B^T F_B
-      if (emu) {  // an arrow carried along extends K: W3 -= [Z_B; Z_C]^T [F_B; F_C]
+    if (hasB) {  // Z_D -= Z_B^T F_B
+      if (emu) {  // an arrow carried along extends K: Z_D -= [Z_B; Z_C]^T [F_B; F_C]
         for (size_t q = 0; q < G.all.size(); ++q) {
           const int z = G.all[q];
           Gemm g; g.M = ld; g.N = ld; g.K = ld;
-          g.A = W2[q]; g.lda = ld; g.transA = 1; g.B = W1[q]; g.ldb = ld;
-          g.C = W3[q]; g.ldc = ld; g.Cin = W3[q]; g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
+          g.A = ZB[q]; g.lda = ld; g.transA = 1; g.B = W1[q]; g.ldb = ld;
+          g.C = ZD[q]; g.ldc = ld; g.Cin = ZD[q]; g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
           g.out_lower = 1;
           if (fused(z)) {
             const int a = it[z].q.a;
-            g.K = ld + a; g.a_k = ld; g.A12 = {it[z].ws.Wc2, a, 1};
+            g.K = ld + a; g.a_k = ld; g.A12 = {Cb(z, i), a, 1};
             g.b_k = ld; g.B21 = {it[z].ws.Wc1, a, 0};
           }
           BTA_TRY(emulate(z, g));
         }
       } else {
         Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
-        g.Ab = cp(W2); g.lda = ld; g.transA = 1; g.Bb = cp(W1); g.ldb = ld;
-        g.Cb = W3.data(); g.ldc = ld; g.Cinb = cp(W3); g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
+        g.Ab = cp(ZB); g.lda = ld; g.transA = 1; g.Bb = cp(W1); g.ldb = ld;
+        g.Cb = ZD.data(); g.ldc = ld; g.Cinb = cp(ZD); g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
         g.out_lower = 1;
         BTA_TRY(big_product(g, it, G.all, precision, s));
       }
     }
-    for (const auto& grp : G.arrow) {  // W3 -= Z_C^T F_C
+    for (const auto& grp : G.arrow) {  // Z_D -= Z_C^T F_C
       if (hasB && fused(grp[0])) continue;
       const int a = it[grp[0]].q.a, c = (int)grp.size();
       auto Wc1 = ptrs(grp, [&](int z) { return it[z].ws.Wc1; });
-      auto Wc2 = ptrs(grp, [&](int z) { return it[z].ws.Wc2; });
-      auto W3g = ptrs(grp, [&](int z) { return it[z].ws.W3; });
+      auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
+      auto ZDg = ptrs(grp, [&](int z) { return over ? D(z, i) : it[z].ws.W3; });
       Gemm g; g.M = ld; g.N = ld; g.K = a; g.batch = c;
-      g.Ab = cp(Wc2); g.lda = a; g.transA = 1; g.Bb = cp(Wc1); g.ldb = a;
-      g.Cb = W3g.data(); g.ldc = ld; g.Cinb = cp(W3g); g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
+      g.Ab = cp(Ci); g.lda = a; g.transA = 1; g.Bb = cp(Wc1); g.ldb = a;
+      g.Cb = ZDg.data(); g.ldc = ld; g.Cinb = cp(ZDg); g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
       g.out_lower = 1;
       BTA_TRY(gemm_f64(g, s));
     }
-    BTA_TRY(copy_block_batch(M, cp(W3), ld, Di.data(), ld, ld, ld, 1.0, 1, s));   // Z_D (full)
-    if (hasB && !low) {   // Z_B in place of L_Bi (low memory: reduced from W2 below)
-      auto Bi = ptrs(G.all, [&](int z) { return B(z, i); });
-      BTA_TRY(copy_block_batch(M, cp(W2), ld, Bi.data(), ld, ld, ld, 1.0, 0, s));
-    }
-    for (const auto& grp : G.arrow) {
-      const int a = it[grp[0]].q.a, c = (int)grp.size();
-      auto Wc2 = ptrs(grp, [&](int z) { return it[z].ws.Wc2; });
-      auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
-      BTA_TRY(copy_block_batch(c, cp(Wc2), a, Ci.data(), a, a, ld, 1.0, 0, s));
-    }
-    for (int z = 0; z < m; ++z) {
-      const SelinvFuse* fz = it[z].fuse;
-      if (!fz) continue;
-      const ModelDev& md = *fz->md;
-      const int kk = md.k * md.k, pch = pattern_chunks(md);
-      BTA_TRY(launch_pattern_dot(md, D(z, i), fz->counts, i,
-                                 fz->PD + (int64_t)i * kk * pch * kNP, s));
-      if (hasB)
-        BTA_TRY(launch_pattern_dot(md, low ? it[z].ws.W2 : B(z, i), 0, i,
-                                   fz->PB + (int64_t)i * kk * pch * kNP, s));
-      if (it[z].q.a > 0 && fz->PC)
-        BTA_TRY(launch_arrow_dot(md, Cb(z, i), i, fz->PC + (int64_t)i * md.k * arrow_chunks(md),
-                                 s));
-    }
+    BTA_TRY(mirror_batch(M, cp(ZD), ld, Di.data(), ld, ld, s));   // Z_D (full)
+    if (hasB && low)   // Z_B is not kept: reduce it here
+      for (int z = 0; z < m; ++z) {
+        const SelinvFuse* fz = it[z].fuse;
+        if (!fz) continue;
+        const int b = coupling_of(it[z], i);
+        BTA_TRY(launch_pattern_dot(*fz->md, it[z].ws.W2, 0, b, 1,
+                                   fz->PB + (int64_t)b * pattern_doubles(*fz->md), s));
+      }
     BTA_SWEEP_MARK(s, 5, i);
+  }
+  return BTA_OK;
+}
+
+bta_status selinv_sums(const SweepItem* it, int m, cudaStream_t s) {
+  for (int z = 0; z < m; ++z) {
+    const SelinvFuse* fz = it[z].fuse;
+    if (!fz) continue;
+    const ModelDev& md = *fz->md;
+    const bta_desc& q = it[z].q;
+    BTA_TRY(launch_pattern_dot(md, q.D, fz->counts, 0, q.n, fz->PD, s));
+    if (q.B && q.n > 1) BTA_TRY(launch_pattern_dot(md, q.B, 0, 0, q.n - 1, fz->PB, s));
+    if (q.a > 0 && fz->PC) BTA_TRY(launch_arrow_dot(md, q.C, q.n, fz->PC, s));
   }
   return BTA_OK;
 }
@@ -898,7 +1014,8 @@ bta_status selinv_sweep(const bta_desc& q, const SweepWs& ws, const SelinvFuse* 
                         cudaStream_t s) {
   SweepItem item;
   item.q = q; item.ws = ws; item.fuse = fuse;
-  return selinv_sweep_multi(&item, 1, s);
+  BTA_TRY(selinv_sweep_multi(&item, 1, s));
+  return selinv_sums(&item, 1, s);
 }
 
 }  // namespace bta
