@@ -4,15 +4,16 @@
 //   stream 0 : theta -> coefficients (closed-form Kronecker coefficients and
 //              their theta-derivatives)
 //   stream 1 : assemble Q_c, r -> Algorithm 1 with fused lower solve ->
-//              Eqs. 3-5 -> x*, residuals ->  [grad] selected inversion of Q_c
-//              with Phase A fused
+//              Eqs. 3-5 -> x*, residuals ->  [grad] selected inversion of Q_c, Phase A sums
 //   stream 2 : assemble Q_p -> block Cholesky -> (after x*) stencil quadratic
-//              forms (Phase B, x*^T Q_p x*) -> [grad] selected inversion of Q_p
-//              with Phase C fused
+//              forms (Phase B, x*^T Q_p x*) -> [grad] selected inversion of Q_p,
+//              Phase C sums
+//   streams 3, 4 : the reverse legs of Q_c and Q_p (three time blocks or more)
 //   stream 0 : join, final combination into f and grad.
-// The two factorisations and the two selected inversions are independent, so
-// they run concurrently and fill each other's idle SMs.  The whole evaluation
-// is captured once into a CUDA graph per (value / value+grad) and replayed.
+// Both matrices are eliminated from both ends towards the middle block (see SweepItem), so
+// four chains of dependent block steps run concurrently and fill each other's idle SMs.
+// The whole evaluation is captured once into a CUDA graph per (value / value+grad)
+// and replayed.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -36,7 +37,8 @@ struct EvalCtx {
   double *PDc = nullptr, *PBc = nullptr, *PCc = nullptr, *PDp = nullptr, *PBp = nullptr;
   double *QD = nullptr, *QB = nullptr, *RS = nullptr;
   double* out = nullptr;
-  SweepWs wsc, wsp;
+  SweepWs wsc, wsp, wsc2, wsp2;   // forward and reverse legs
+  double* tip2 = nullptr;         // the reverse leg's share of Q_c's tip
   SelinvFuse fc, fp;
   double* dr = nullptr;         // mixed mode: refinement residual / correction
   double* red = nullptr;        // sums of the final combination
@@ -63,11 +65,16 @@ struct inla_model {
   std::vector<double> last;     // output of the last single evaluation
   std::vector<GraphKey> graphs;
   int64_t launched = 0;         // kernels this model ran (graph replays included)
-  // the Q_c set and the Q_p set are swept on two streams (fork/join by events)
-  cudaStream_t s1 = nullptr, s2 = nullptr;
+  // the legs of the Q_c set and of the Q_p set are swept on four streams (fork/join by events)
+  cudaStream_t s1 = nullptr, s2 = nullptr, s3 = nullptr, s4 = nullptr;
   cudaStream_t s0 = nullptr;    // the model's own root stream inside a multi-model graph
-  cudaEvent_t ev0 = nullptr, evx = nullptr, ev1 = nullptr, ev2 = nullptr, evd = nullptr;
+  cudaEvent_t ev0 = nullptr, evx = nullptr, ev1 = nullptr, ev2 = nullptr;
+  // reverse legs: assembled, ready for the shared block, shared block done, finished
+  cudaEvent_t evac = nullptr, evap = nullptr, evjc = nullptr, evjp = nullptr, evmc = nullptr,
+              evmp = nullptr, ev3 = nullptr, ev4 = nullptr;
   cudaEvent_t evj = nullptr;    // join event of a multi-model graph
+  // blocks of the reverse legs: both ends meet in the middle
+  int reverse_blocks() const { return n >= 3 ? (n - 1) / 2 : 0; }
 };
 
 // Several models evaluated by one CUDA graph (see inla_batch_value_and_grad).
@@ -142,19 +149,21 @@ bta_status ctx_alloc(inla_model* m, EvalCtx& c) {
   BTA_TRY(dmalloc(m, &c.RS, (size_t)kMaxK * resid_chunks(md)));
   BTA_TRY(dmalloc(m, &c.out, out_size(md.d)));
   BTA_TRY(dmalloc(m, &c.red, kRedDoubles));
+  const int legs = m->reverse_blocks() > 0 ? 4 : 2;
+  SweepWs* const ws[4] = {&c.wsc, &c.wsp, &c.wsc2, &c.wsp2};
   const size_t wsb = SweepWs::bytes(ld, a) / sizeof(double);
   double* wsbuf = nullptr;
-  BTA_TRY(dmalloc(m, &wsbuf, 2 * wsb));
-  c.wsc.carve(wsbuf, ld, a);
-  c.wsp.carve(wsbuf + wsb, ld, a);
-  // tensor-core modes: operand copies of the tensor-core products, one per sweep
+  BTA_TRY(dmalloc(m, &wsbuf, legs * wsb));
+  // tensor-core modes: operand copies of the tensor-core products, one per leg
   const size_t tcb = sweep_tc_ws_bytes(ld, a);
   uint8_t* tcbuf = nullptr;
-  BTA_TRY(dmalloc(m, &tcbuf, 2 * tcb));
-  c.wsc.tc = tcbuf;
-  c.wsp.tc = tcbuf + tcb;
-  c.wsc.tcstat = c.fail + 2;
-  c.wsp.tcstat = c.fail + 2;
+  BTA_TRY(dmalloc(m, &tcbuf, legs * tcb));
+  for (int q = 0; q < legs; ++q) {
+    ws[q]->carve(wsbuf + q * wsb, ld, a);
+    ws[q]->tc = tcbuf + q * tcb;
+    ws[q]->tcstat = c.fail + 2;
+  }
+  BTA_TRY(dmalloc(m, &c.tip2, std::max(a * a, 1)));
   BTA_TRY(dmalloc(m, &c.dr, (size_t)nt * ld + a));
   c.fc.md = &m->md; c.fc.counts = 1; c.fc.PD = c.PDc; c.fc.PB = c.PBc; c.fc.PC = c.PCc;
   c.fp.md = &m->md; c.fp.counts = 0; c.fp.PD = c.PDp; c.fp.PB = c.PBp; c.fp.PC = nullptr;
@@ -181,32 +190,34 @@ bta_status ensure_ctx(inla_model* m, int count) {
 //   mode 0: f only; 1: f and gradient; 2: reverse pass of a preceding mode-0
 //   evaluation (the factors are still in place).
 // The conditional matrices Q_c of all contexts form one set and the priors
-// Q_p another; each set is swept with one batched launch per block step, and
-// the two sets run on two streams.  They are independent until the final
-// combination (the stencil quadratic forms on the Q_p stream wait for x*), so
-// the serial diagonal steps of one set overlap the wide products of the other.
-// Each step issues one block of both sweeps (Q_c's, then Q_p's), so the two
-// streams' operations, and the nodes of a captured graph, are created in
-// alternation: the driver submits a graph's kernels in creation order into a
-// bounded queue, and a whole Q_c sweep created first (~1600 launches a block)
-// held the Q_p stream back until the GPU had drained most of it.
+// Q_p another; each set is swept with one batched launch per block step.  Each set
+// is eliminated from both ends towards the middle block (SweepItem: a forward and a
+// reverse leg with workspaces of their own), so that a value takes half as many dependent
+// diagonal factors, and the four legs run on four streams: a chain of small kernels
+// leaves most of the GPU idle, and the serial diagonal steps of one leg overlap the wide
+// products of the others.  Per call, one leg per matrix / two: b = 1024, 50 blocks emulated
+// gradient 75.8 / 58.6 ms, value 55.2 / 38.7 ms; b = 4800, 8 blocks 215 / 205 ms; b = 64,
+// 4 blocks FP64 0.92 / 0.72 ms; the FP64-bound b = 1024 gradient 68.6 / 67.4 ms.
+// Each step issues one block of every leg, so the streams' operations, and the nodes of
+// a captured graph, are created in alternation: the driver submits a graph's kernels in
+// creation order into a bounded queue, and a whole sweep created first (~1600 launches a
+// block) held the others back until the GPU had drained most of it.
 using IssueStep = std::function<bta_status()>;
 
 struct GroupSets {
-  std::vector<SweepItem> ic, ip;
+  std::vector<SweepItem> ic, ip;   // forward legs
+  std::vector<SweepItem> jc, jp;   // reverse legs (empty below three blocks)
 };
 
 bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_t s0,
                          std::vector<IssueStep>& steps) {
   const ModelDev& md = m->md;
   const int grad = mode >= 1, nt = md.nt;
+  const int nb = m->reverse_blocks(), mid = nt - 1 - nb;
   auto sets = std::make_shared<GroupSets>();
-  sets->ic.resize(cnt);
-  sets->ip.resize(cnt);
   for (int e = 0; e < cnt; ++e) {
     EvalCtx& c = m->ctx[e];
-    SweepItem& ic = sets->ic[e];
-    SweepItem& ip = sets->ip[e];
+    SweepItem ic, ip;
     ic.q = c.qc; ic.vec = c.x; ic.slots = c.slots_c; ic.fail = c.fail;
     ic.ws = c.wsc; ic.fuse = &c.fc;
     ip.q = c.qp; ip.vec = nullptr; ip.slots = c.slots_p; ip.fail = c.fail + 1;
@@ -214,6 +225,23 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
     ic.md = ip.md = &md;
     ic.lay = ip.lay = &m->L;
     ic.coef = ip.coef = c.coefbuf;
+    if (nb > 0) {
+      SweepItem jc = ic, jp = ip;
+      ic.len = ip.len = mid + 1;
+      jc.rev = jp.rev = 1;
+      jc.len = jp.len = nb + 1;
+      jc.ws = c.wsc2;
+      jp.ws = c.wsp2;
+      if (md.a > 0) {
+        jc.tip = c.tip2;
+        ic.tip2 = c.tip2;
+        ic.vT2 = c.wsc2.vT;
+      }
+      sets->jc.push_back(jc);
+      sets->jp.push_back(jp);
+    }
+    sets->ic.push_back(ic);
+    sets->ip.push_back(ip);
   }
   // set-up on s0, the fork, and (mode < 2) the assembly of both sets
   steps.push_back([=]() -> bta_status {
@@ -234,29 +262,75 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
                                 m->s1));
         BTA_TRY(launch_assemble(md, m->L, m->ctx[e].coefbuf, 0, m->ctx[e].qp, nullptr, m->s2));
       }
+    if (nb > 0) {
+      BTA_CUDA_TRY(cudaEventRecord(m->evac, m->s1));
+      BTA_CUDA_TRY(cudaEventRecord(m->evap, m->s2));
+      BTA_CUDA_TRY(cudaStreamWaitEvent(m->s3, m->evac, 0));
+      BTA_CUDA_TRY(cudaStreamWaitEvent(m->s4, m->evap, 0));
+    }
     return BTA_OK;
   });
   if (mode < 2) {
-    for (int i = 0; i < nt; ++i)
+    for (int i = 0; i <= mid; ++i)
       steps.push_back([=]() -> bta_status {
-        BTA_TRY(factor_sweep_multi(sets->ic.data(), cnt, m->s1, m->evd, prec, i, i + 1));
-        // the Q_p sweep starts one diagonal step behind the Q_c sweep: the two
-        // then alternate their latency-bound diagonal factors with wide products
-        if (i == 0) BTA_CUDA_TRY(cudaStreamWaitEvent(m->s2, m->evd, 0));
-        return factor_sweep_multi(sets->ip.data(), cnt, m->s2, nullptr, prec, i, i + 1);
+        if (nb > 0 && i == mid) {   // the reverse legs have updated the shared block
+          BTA_CUDA_TRY(cudaStreamWaitEvent(m->s1, m->evjc, 0));
+          BTA_CUDA_TRY(cudaStreamWaitEvent(m->s2, m->evjp, 0));
+        }
+        BTA_TRY(factor_sweep_multi(sets->ic.data(), cnt, m->s1, prec, i, i + 1));
+        BTA_TRY(factor_sweep_multi(sets->ip.data(), cnt, m->s2, prec, i, i + 1));
+        if (i >= nb) return BTA_OK;
+        BTA_TRY(factor_sweep_multi(sets->jc.data(), cnt, m->s3, prec, i, i + 1));
+        BTA_TRY(factor_sweep_multi(sets->jp.data(), cnt, m->s4, prec, i, i + 1));
+        if (i == nb - 1) {
+          BTA_CUDA_TRY(cudaEventRecord(m->evjc, m->s3));
+          BTA_CUDA_TRY(cudaEventRecord(m->evjp, m->s4));
+        }
+        return BTA_OK;
       });
+    // the upper solve from the shared block outwards, both legs at once; then s1 has x
+    auto upper = [=](const SweepItem* it, const SweepItem* jt, int count) -> bta_status {
+      BTA_TRY(upper_solve_multi(it, count, m->s1, mid, mid));
+      if (nb > 0) {
+        BTA_CUDA_TRY(cudaEventRecord(m->evmc, m->s1));
+        BTA_CUDA_TRY(cudaStreamWaitEvent(m->s3, m->evmc, 0));
+      }
+      for (int t = 0; t < mid; ++t) {
+        BTA_TRY(upper_solve_multi(it, count, m->s1, mid - 1 - t, mid - 1 - t));
+        if (t < nb) BTA_TRY(upper_solve_multi(jt, count, m->s3, nb - 1 - t, nb - 1 - t));
+      }
+      if (nb > 0) {
+        BTA_CUDA_TRY(cudaEventRecord(m->ev3, m->s3));
+        BTA_CUDA_TRY(cudaStreamWaitEvent(m->s1, m->ev3, 0));
+      }
+      return BTA_OK;
+    };
     steps.push_back([=]() -> bta_status {
-      BTA_TRY(upper_solve_multi(sets->ic.data(), cnt, m->s1));
+      BTA_TRY(upper(sets->ic.data(), sets->jc.data(), cnt));
       if (prec == 1) {
         // one step of iterative refinement in FP64: x += Q_c^{-1} (r - Q_c x)
         for (int e = 0; e < cnt; ++e) {
           EvalCtx& c = m->ctx[e];
           BTA_TRY(launch_rhs(md, m->L, c.coefbuf, c.dr, m->s1));
           BTA_TRY(launch_qc_residual(md, m->L, c.coefbuf, c.x, c.dr, m->s1));
-          SweepItem dx = sets->ic[e];
+          SweepItem dx = sets->ic[e], dj;
           dx.vec = c.dr;
-          BTA_TRY(lower_solve(dx, m->s1));
-          BTA_TRY(upper_solve_multi(&dx, 1, m->s1));
+          if (nb > 0) {
+            dj = sets->jc[e];
+            dj.vec = c.dr;
+            BTA_CUDA_TRY(cudaEventRecord(m->evac, m->s1));
+            BTA_CUDA_TRY(cudaStreamWaitEvent(m->s3, m->evac, 0));
+            for (int i = 0; i < mid; ++i) {
+              BTA_TRY(lower_solve(dx, m->s1, i, i + 1));
+              if (i < nb) BTA_TRY(lower_solve(dj, m->s3, i, i + 1));
+            }
+            BTA_CUDA_TRY(cudaEventRecord(m->evjc, m->s3));
+            BTA_CUDA_TRY(cudaStreamWaitEvent(m->s1, m->evjc, 0));
+            BTA_TRY(lower_solve(dx, m->s1, mid, mid + 1));
+          } else {
+            BTA_TRY(lower_solve(dx, m->s1));
+          }
+          BTA_TRY(upper(&dx, &dj, 1));
           BTA_TRY(launch_axpy((int64_t)md.nt * md.ld + md.a, 1.0, c.dr, c.x, m->s1));
         }
       }
@@ -270,13 +344,31 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
     });
   }
   if (grad)
-    for (int i = nt - 1; i >= 0; --i)
+    for (int t = 0; t <= mid; ++t)
       steps.push_back([=]() -> bta_status {
+        const int i = mid - t, r = nb - t;   // the reverse legs follow the shared block
         BTA_TRY(selinv_sweep_multi(sets->ic.data(), cnt, m->s1, prec, i, i));
-        return selinv_sweep_multi(sets->ip.data(), cnt, m->s2, prec, i, i);
+        BTA_TRY(selinv_sweep_multi(sets->ip.data(), cnt, m->s2, prec, i, i));
+        if (nb == 0) return BTA_OK;
+        if (t == 0) {
+          BTA_CUDA_TRY(cudaEventRecord(m->evmc, m->s1));
+          BTA_CUDA_TRY(cudaEventRecord(m->evmp, m->s2));
+          BTA_CUDA_TRY(cudaStreamWaitEvent(m->s3, m->evmc, 0));
+          BTA_CUDA_TRY(cudaStreamWaitEvent(m->s4, m->evmp, 0));
+        } else if (r >= 0) {
+          BTA_TRY(selinv_sweep_multi(sets->jc.data(), cnt, m->s3, prec, r, r));
+          BTA_TRY(selinv_sweep_multi(sets->jp.data(), cnt, m->s4, prec, r, r));
+        }
+        return BTA_OK;
       });
   // join and combine
   steps.push_back([=]() -> bta_status {
+    if (nb > 0) {
+      BTA_CUDA_TRY(cudaEventRecord(m->ev3, m->s3));
+      BTA_CUDA_TRY(cudaEventRecord(m->ev4, m->s4));
+      BTA_CUDA_TRY(cudaStreamWaitEvent(m->s1, m->ev3, 0));
+      BTA_CUDA_TRY(cudaStreamWaitEvent(m->s2, m->ev4, 0));
+    }
     if (grad) {
       BTA_TRY(selinv_sums(sets->ic.data(), cnt, m->s1));
       BTA_TRY(selinv_sums(sets->ip.data(), cnt, m->s2));
@@ -415,8 +507,11 @@ void inla_model_destroy(inla_model* m) {
   if (m->htheta) cudaFreeHost(m->htheta);
   if (m->s1) cudaStreamDestroy(m->s1);
   if (m->s2) cudaStreamDestroy(m->s2);
+  if (m->s3) cudaStreamDestroy(m->s3);
+  if (m->s4) cudaStreamDestroy(m->s4);
   if (m->s0) cudaStreamDestroy(m->s0);
-  for (cudaEvent_t e : {m->ev0, m->evx, m->ev1, m->ev2, m->evd, m->evj})
+  for (cudaEvent_t e : {m->ev0, m->evx, m->ev1, m->ev2, m->evac, m->evap, m->evjc, m->evjp,
+                        m->evmc, m->evmp, m->ev3, m->ev4, m->evj})
     if (e) cudaEventDestroy(e);
   delete m;
 }
@@ -511,8 +606,11 @@ static bta_status model_create_impl(const inla_model_spec* sp, inla_model* m) {
   BTA_CUDA_TRY(cudaMallocHost(&m->htheta, (size_t)kMaxBatch * kMaxD * sizeof(double)));
   BTA_CUDA_TRY(cudaStreamCreateWithFlags(&m->s1, cudaStreamNonBlocking));
   BTA_CUDA_TRY(cudaStreamCreateWithFlags(&m->s2, cudaStreamNonBlocking));
+  BTA_CUDA_TRY(cudaStreamCreateWithFlags(&m->s3, cudaStreamNonBlocking));
+  BTA_CUDA_TRY(cudaStreamCreateWithFlags(&m->s4, cudaStreamNonBlocking));
   BTA_CUDA_TRY(cudaStreamCreateWithFlags(&m->s0, cudaStreamNonBlocking));
-  for (cudaEvent_t* e : {&m->ev0, &m->evx, &m->ev1, &m->ev2, &m->evd, &m->evj})
+  for (cudaEvent_t* e : {&m->ev0, &m->evx, &m->ev1, &m->ev2, &m->evac, &m->evap, &m->evjc,
+                         &m->evjp, &m->evmc, &m->evmp, &m->ev3, &m->ev4, &m->evj})
     BTA_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   BTA_CUDA_TRY(cudaDeviceSynchronize());
   return BTA_OK;

@@ -397,8 +397,8 @@ bta_status assemble_b_items(const SweepItem* it, const std::vector<int>& idx, in
 // ----------------------------------------------------------------------------
 // Algorithm 1 on a set of matrices
 // ----------------------------------------------------------------------------
-bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEvent_t mark,
-                              int precision, int i0, int i1) {
+bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int precision, int i0,
+                              int i1) {
   BTA_TRY(check_set(it, m));
   const int n = it[0].blocks(), ld = it[0].q.ld;
   const bool rev = it[0].rev;
@@ -525,7 +525,6 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, cudaEv
       BTA_TRY(potrf_inv_batch_prec(M, Di.data(), ld, ld, W.data(), sl.data(), fl.data(),
                                    code.data(), precision, tw.data(), ts.data(), s));
       BTA_SWEEP_MARK(s, 2, i);
-      if (i == 0 && mark) BTA_CUDA_TRY(cudaEventRecord(mark, s));
     }
     const bool with_b = emu && i < n - 1;   // L_Ci as extra rows of L_Bi's product
     for (const auto& grp : G.arrow) {  // L_Ci = C_i L_Di^{-T};  T -= L_Ci L_Ci^T
@@ -605,7 +604,7 @@ bta_status factor_sweep(const bta_desc& q, double* rhs, double* slots, int32_t* 
                         const SweepWs& ws, cudaStream_t s, int precision) {
   SweepItem item;
   item.q = q; item.vec = rhs; item.slots = slots; item.fail = fail; item.ws = ws;
-  return factor_sweep_multi(&item, 1, s, nullptr, precision);
+  return factor_sweep_multi(&item, 1, s, precision);
 }
 
 // ----------------------------------------------------------------------------

@@ -70,8 +70,6 @@ struct SweepItem {
   const double* coef = nullptr;
   int blocks() const { return len > 0 ? len : q.n; }
 };
-// mark (optional): recorded on s right after block 0's diagonal factor, so a
-// concurrent sweep can start one diagonal step behind this one.
 // precision 0: every product in FP64; 1: the b x b off-diagonal Schur
 // products (and the selected-inversion products) in split precision on the
 // tensor cores, the diagonal-block factorisation, arrow and log-det in FP64.
@@ -85,9 +83,8 @@ struct SweepItem {
 // range: the forward leg's step of that block, the tip and the shared block's x and Z must
 // be ordered after it, and the reverse leg's solve and selected inversion (from
 // block len - 2) after theirs.
-bta_status factor_sweep_multi(const SweepItem* items, int m, cudaStream_t s,
-                              cudaEvent_t mark = nullptr, int precision = 0, int i0 = 0,
-                              int i1 = -1);
+bta_status factor_sweep_multi(const SweepItem* items, int m, cudaStream_t s, int precision = 0,
+                              int i0 = 0, int i1 = -1);
 bta_status upper_solve_multi(const SweepItem* items, int m, cudaStream_t s, int i_hi = -1,
                              int i_lo = 0);
 bta_status selinv_sweep_multi(const SweepItem* items, int m, cudaStream_t s, int precision = 0,
