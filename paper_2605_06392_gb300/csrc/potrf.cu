@@ -14,6 +14,7 @@
 //                   A22 <- A22 - L21 L21^T,  L22^{-1} (recursive)
 //                   (L^{-1})21 = -L22^{-1} L21 L11^{-1}
 // with a single-CTA shared-memory kernel for 32 x 32 leaves.
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 
@@ -213,7 +214,6 @@ struct ProdCfg {
   int precision = 0;
   void* const* tcws = nullptr;
   int32_t* const* tcstat = nullptr;
-  int leaf_ctas = 0;   // cap on the task-graph grid of the leaves (0: one CTA per SM)
 };
 
 bta_status level_product(const Gemm& g, const ProdCfg& c, cudaStream_t s) {
@@ -245,8 +245,13 @@ bta_status rec_hybrid(const PB& b, int64_t aoff, int n, int ld, int64_t woff, in
       W[z] = b.W[z] + woff;
       sl[z] = b.slots[z] + soff;
     }
-    return potrf_dag_batch(cnt, A, n, ld, W, sl, b.fail, b.code, s, pc.leaf_ctas,
-                           pc.precision != 0);
+    // In the tensor-core modes the other legs' products run on the SMs the leaves leave
+    // free: a CTA per 16 rows keeps the bulk tasks off the chain (512 rows, 65 / 40 / 32
+    // / 24 CTAs: 0.289 / 0.287 / 0.299 / 0.334 ms alone; the b = 1024 gradient of 50 blocks
+    // 57.2 / 54.2 / 53.9 / 55.3 ms).  The FP64 mode, whose bulk tasks need the SMs, keeps
+    // them all.
+    const int ctas = pc.precision ? std::max(2, n / 16) : 0;
+    return potrf_dag_batch(cnt, A, n, ld, W, sl, b.fail, b.code, s, ctas, pc.precision != 0);
   }
   const int p = n / T;
   const int n1 = (p / 2) * T, n2 = n - n1;
@@ -352,11 +357,6 @@ bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
   PriorityScope prio(highest_priority());
   ProdCfg pc;
   pc.precision = precision;
-  // In the tensor-core modes the other sweep's products run on the SMs the
-  // leaves leave free: ~3/7 of the SMs keep the leaves' bulk tasks off their
-  // chain (GB300, b = 1024: mixed 126 -> 114 ms, emulated 134 -> 127 ms per
-  // gradient; the FP64 mode, whose bulk tasks need the SMs, keeps them all).
-  pc.leaf_ctas = precision ? std::max(2, sm_count() * 3 / 7) : 0;
   for (int z0 = 0; z0 < count; z0 += kMaxBatch) {
     PB b;
     b.cnt = count - z0 < kMaxBatch ? count - z0 : kMaxBatch;

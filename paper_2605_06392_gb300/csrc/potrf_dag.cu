@@ -26,13 +26,23 @@
 // so the graph always drains.  Per-tile counters (W updates applied, R
 // updates applied, F/S/G done) are published with release stores after the
 // tile is written and read with acquire loads; tile data are read through
-// L2 (ld.global.cg).  A tile is written by the whole CTA, then a barrier, then one
-// thread's release store, which the barrier makes cumulative.  Every wait is bounded by a globaltimer limit (2 s); on
-// expiry the CTA raises a shared abort flag, writes BTA_ERR_TIMEOUT into the
-// block's failure word (which otherwise holds -1 or the index of a block with
-// a non-positive pivot) and returns, and every other CTA returns at its next
-// wait.  A test switch (bta_set_wait_limit) lowers the limit and makes the
-// chain wait on a counter nothing sets, so that this path runs without a fault.
+// L2 (cp.async.cg).
+//
+// A CTA is three parties.  Warp 8 fetches: it takes a ticket, waits for the tiles the
+// task reads and loads them into one of two stages, so that the next task's ticket,
+// waits (three L2 round trips) and loads run behind the current task's products.  Warps
+// 0-7 compute, and store the result.  Warp 9 publishes: its release store waits for
+// the stores to be visible (~900 clocks) while the others go on; the compute warps'
+// barrier makes it cumulative.  On the chain the fetcher brings the next step's W tiles
+// while the leaf runs (in the tensor-core modes split into slices) and the publisher
+// sums the pivots' logs.  Stages change hands through mbarriers.
+//
+// Every wait is bounded by a globaltimer limit (2 s); on expiry the CTA raises a shared
+// abort flag, writes BTA_ERR_TIMEOUT into the block's failure word (which otherwise
+// holds -1 or the index of a block with a non-positive pivot) and returns, and every
+// other CTA returns at its next wait.  A test switch (bta_set_wait_limit) lowers the
+// limit and makes the chain wait on a counter nothing sets, so that this path runs
+// without a fault.
 #include <algorithm>
 #include <cstdlib>
 #include <vector>
@@ -46,7 +56,10 @@
 // measurement build that includes this file may define DAG_TRACE(event, step)
 // before the include to stamp the chain's phases of each diagonal step:
 // 0 the step's inputs are final (waits done), 1 the triangular product done,
-// 2 the symmetric update done, 3 the leaf done, 4 the step published.
+// 2 the symmetric update done, 3 the leaf done, 4 the step published; and of the two bulk
+// tasks that the chain's step k + 2 waits for, S(k+2,k) and U(k+2,k+1,k): 5 / 8 the task's
+// tiles are final, 6 / 9 in place, 7 / 10 its result published, 11 the fetcher has seen
+// step c's tiles final.
 #ifndef DAG_TRACE
 #define DAG_TRACE(event, step) ((void)0)
 #endif
@@ -55,10 +68,13 @@ namespace bta {
 namespace {
 
 constexpr int T = kPad;                 // tile size
-constexpr int kDagThreads = 256;
+constexpr int kTP = T + 2;              // column pitch of a tile in shared memory (16-byte columns)
+constexpr int kDagThreads = 256;        // compute threads (warps 0-7)
+constexpr int kDagFetch = 8, kDagPublish = 9;   // service warps
+constexpr int kDagAllThreads = kDagThreads + 64;
 constexpr int kMaxP = 160;              // tile rows supported (ld <= 5120)
 
-enum : int { TK_H = 0, TK_S = 1, TK_G = 2, TK_U = 3, TK_V = 4 };
+enum : int { TK_H = 0, TK_S = 1, TK_G = 2, TK_U = 3, TK_V = 4, TK_END = 5 };
 
 struct DagInst {
   double* A;       // n x n block, ld
@@ -76,6 +92,7 @@ struct DagArgs {
   int* abort;               // shared abort flag
   int* smbusy;              // per SM: chain tasks running there (see TK_H)
   int yield;                // bulk tasks wait while a chain task holds their SM
+  int vec;                  // the blocks are 16-byte aligned
   int stall;                // test switch: the chain waits on a counter nothing sets
   unsigned long long wait_ns;   // bound of every wait
   int off[kMaxP + 1];       // task offset of each step within one instance
@@ -121,72 +138,113 @@ __device__ __forceinline__ double* tile(double* A, int ld, int r, int c) {
   return A + (int64_t)c * T * ld + (int64_t)r * T;
 }
 
-// Load a 32 x 32 tile (column-major, ld) into smem S[row][col] through L2.
-__device__ __forceinline__ void load_tile(double (*S)[T + 1], const double* src, int ld) {
+// A tile in shared memory: column-major, element (r, c) at S[c][r].
+using Tile = double (*)[kTP];
+__device__ __forceinline__ double& at(Tile S, int r, int c) { return S[c][r]; }
+
+// One warp starts the load of a 32 x 32 tile (column-major, ld) through L2: 16
+// asynchronous copies a lane, so that every tile of a task takes one round trip together
+// (load_wait) and no registers.  A block that is not 16-byte aligned (a caller's; vec = 0)
+// goes through registers.
+__device__ __forceinline__ void load_tile(Tile S, const double* src, int ld, int vec) {
+  const int lane = threadIdx.x & 31, r = 2 * (lane & 15);
+  if (!vec) {
+    for (int c = 0; c < T; ++c) S[c][lane] = __ldcg(src + (int64_t)c * ld + lane);
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int c = 2 * q + (lane >> 4);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(&S[c][r])),
+                 "l"(src + (int64_t)c * ld + r)
+                 : "memory");
+  }
+}
+__device__ __forceinline__ void load_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
+}
+// Zeros above the diagonal (one warp).
+__device__ __forceinline__ void zero_upper(Tile S) {
+  const int r = threadIdx.x & 31;
+  for (int c = r + 1; c < T; ++c) S[c][r] = 0.0;
+}
+
+// Barrier of the compute warps.
+__device__ __forceinline__ void compute_bar() {
+  asm volatile("bar.sync 2, 256;" ::: "memory");
+}
+// ... which also tells them whether v holds in all of them: a decision that all share.
+__device__ __forceinline__ bool compute_all(bool v) {
+  int r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n"
+      " barrier.cta.red.and.pred q, 2, 256, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((int)v)
+      : "memory");
+  return r != 0;
+}
+
+__device__ __forceinline__ void store_tile(double* dst, int ld, Tile S, bool lower) {
   for (int e = threadIdx.x; e < T * T; e += kDagThreads) {
     const int r = e % T, c = e / T;
-    S[r][c] = __ldcg(src + (int64_t)c * ld + r);
+    if (!lower || r >= c) dst[(int64_t)c * ld + r] = at(S, r, c);
   }
 }
 
-__device__ __forceinline__ void store_tile(double* dst, int ld, double (*S)[T + 1], bool lower) {
-  for (int e = threadIdx.x; e < T * T; e += kDagThreads) {
-    const int r = e % T, c = e / T;
-    if (!lower || r >= c) dst[(int64_t)c * ld + r] = S[r][c];
-  }
-}
-
-// out[r][c] (+)= sign * sum_m X[r][m] * Y'[m][c], with Y' = Y^T when ytrans.
+// at(out, r, c) (+)= sign * sum_m at(X, r, m) * Y'[m][c], with Y' = Y^T when ytrans.
 // 256 threads, each 2 x 2 outputs.
-__device__ __forceinline__ void tile_mm(double (*X)[T + 1], double (*Y)[T + 1], bool ytrans,
-                                        double (*out)[T + 1], double sign, bool accumulate) {
+__device__ __forceinline__ void tile_mm(Tile X, Tile Y, bool ytrans,
+                                        Tile out, double sign, bool accumulate) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   double a00 = 0.0, a01 = 0.0, a10 = 0.0, a11 = 0.0;
 #pragma unroll 8
   for (int m = 0; m < T; ++m) {
-    const double x0 = X[tx][m], x1 = X[tx + 16][m];
-    const double y0 = ytrans ? Y[ty][m] : Y[m][ty];
-    const double y1 = ytrans ? Y[ty + 16][m] : Y[m][ty + 16];
+    const double x0 = at(X, tx, m), x1 = at(X, tx + 16, m);
+    const double y0 = ytrans ? at(Y, ty, m) : at(Y, m, ty);
+    const double y1 = ytrans ? at(Y, ty + 16, m) : at(Y, m, ty + 16);
     a00 = fma(x0, y0, a00); a01 = fma(x0, y1, a01);
     a10 = fma(x1, y0, a10); a11 = fma(x1, y1, a11);
   }
   if (accumulate) {
-    out[tx][ty] += sign * a00; out[tx][ty + 16] += sign * a01;
-    out[tx + 16][ty] += sign * a10; out[tx + 16][ty + 16] += sign * a11;
+    at(out, tx, ty) += sign * a00; at(out, tx, ty + 16) += sign * a01;
+    at(out, tx + 16, ty) += sign * a10; at(out, tx + 16, ty + 16) += sign * a11;
   } else {
-    out[tx][ty] = sign * a00; out[tx][ty + 16] = sign * a01;
-    out[tx + 16][ty] = sign * a10; out[tx + 16][ty + 16] = sign * a11;
+    at(out, tx, ty) = sign * a00; at(out, tx, ty + 16) = sign * a01;
+    at(out, tx + 16, ty) = sign * a10; at(out, tx + 16, ty + 16) = sign * a11;
   }
 }
 
-// out[r][c] = sum_{m <= c} W[r][m] Y[c][m] = (W Y^T)[r][c] for lower-triangular Y
+// at(out, r, c) = sum_{m <= c} at(W, r, m) at(Y, c, m) = (W Y^T)[r][c] for lower-triangular Y
 // (its upper part is not read).  Same thread layout as tile_mm; the m range
 // of a thread's columns (ty, ty + 16) is uniform within a warp, so the
 // skipped half of the products issues no instructions.
-__device__ __forceinline__ void tile_mm_lt(double (*W)[T + 1], double (*Y)[T + 1],
-                                           double (*out)[T + 1]) {
+__device__ __forceinline__ void tile_mm_lt(Tile W, Tile Y,
+                                           Tile out) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   double a00 = 0.0, a01 = 0.0, a10 = 0.0, a11 = 0.0;
   for (int m = 0; m <= ty; ++m) {
-    const double x0 = W[tx][m], x1 = W[tx + 16][m];
-    const double y0 = Y[ty][m], y1 = Y[ty + 16][m];
+    const double x0 = at(W, tx, m), x1 = at(W, tx + 16, m);
+    const double y0 = at(Y, ty, m), y1 = at(Y, ty + 16, m);
     a00 = fma(x0, y0, a00); a01 = fma(x0, y1, a01);
     a10 = fma(x1, y0, a10); a11 = fma(x1, y1, a11);
   }
   for (int m = ty + 1; m <= ty + 16; ++m) {
-    const double y1 = Y[ty + 16][m];
-    a01 = fma(W[tx][m], y1, a01);
-    a11 = fma(W[tx + 16][m], y1, a11);
+    const double y1 = at(Y, ty + 16, m);
+    a01 = fma(at(W, tx, m), y1, a01);
+    a11 = fma(at(W, tx + 16, m), y1, a11);
   }
-  out[tx][ty] = a00; out[tx][ty + 16] = a01;
-  out[tx + 16][ty] = a10; out[tx + 16][ty + 16] = a11;
+  at(out, tx, ty) = a00; at(out, tx, ty + 16) = a01;
+  at(out, tx + 16, ty) = a10; at(out, tx + 16, ty + 16) = a11;
 }
 
-// W[r][c] -= sum_m L[r][m] L[c][m] on the lower triangle (r >= c): threads
+// at(W, r, c) -= sum_m at(L, r, m) at(L, c, m) on the lower triangle (r >= c): threads
 // 0..135 each own one 2 x 2 block of the 16 x 16 block triangle, so only 5
 // of the 8 warps issue FMAs.  Upper entries of diagonal blocks get the same
 // update (W is symmetric; only its lower part is read afterwards).
-__device__ __forceinline__ void tile_syrk_lower(double (*L)[T + 1], double (*W)[T + 1]) {
+__device__ __forceinline__ void tile_syrk_lower(Tile L, Tile W) {
   const int b = threadIdx.x;
   if (b >= 136) return;
   int bi = 0;
@@ -196,12 +254,12 @@ __device__ __forceinline__ void tile_syrk_lower(double (*L)[T + 1], double (*W)[
   double a00 = 0.0, a01 = 0.0, a10 = 0.0, a11 = 0.0;
 #pragma unroll 8
   for (int m = 0; m < T; ++m) {
-    const double x0 = L[r][m], x1 = L[r + 1][m], y0 = L[c][m], y1 = L[c + 1][m];
+    const double x0 = at(L, r, m), x1 = at(L, r + 1, m), y0 = at(L, c, m), y1 = at(L, c + 1, m);
     a00 = fma(x0, y0, a00); a01 = fma(x0, y1, a01);
     a10 = fma(x1, y0, a10); a11 = fma(x1, y1, a11);
   }
-  W[r][c] -= a00; W[r][c + 1] -= a01;
-  W[r + 1][c] -= a10; W[r + 1][c + 1] -= a11;
+  at(W, r, c) -= a00; at(W, r, c + 1) -= a01;
+  at(W, r + 1, c) -= a10; at(W, r + 1, c + 1) -= a11;
 }
 
 // ---- emulated-FP64 tile products (tensor-core modes) -----------------------
@@ -233,11 +291,12 @@ struct OzTile {
 // k and k + 16, which sit side by side in the slice row (both operands of a
 // product use this order of k); the two rows of a warp are four apart, so that
 // their 4-byte stores fall on different banks.
+// part 0..7: the eighth of the rows the calling warp takes.
 template <class Get>
-__device__ __forceinline__ void oz_split(Get get, __nv_bfloat16* planes, int* e) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void oz_split(Get get, __nv_bfloat16* planes, int* e, int part) {
+  const int lane = threadIdx.x & 31;
   const int k = lane & 15;
-  const int r0 = (warp & 3) + 16 * (warp >> 2) + 4 * (lane >> 4);
+  const int r0 = (part & 3) + 16 * (part >> 2) + 4 * (lane >> 4);
   double v[2][2];
   int er[2];
 #pragma unroll
@@ -283,39 +342,38 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 // The products of the slices and their combination: warp w computes the
 // 16 x 8 output block (rows 16 (w / 4).., columns 8 (w % 4)..).
 __device__ __forceinline__ void oz_combine(const __nv_bfloat16* xp, const __nv_bfloat16* yp,
-                                           const int* ex, const int* ey, double (*out)[T + 1],
+                                           const int* ex, const int* ey, Tile out,
                                            double sign, bool accumulate) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int mt = warp >> 2, nt = warp & 3;
-  uint32_t a[8][2][4], b[8][4];
-  {
-    const uint32_t xb = (uint32_t)__cvta_generic_to_shared(xp);
-    const uint32_t yb = (uint32_t)__cvta_generic_to_shared(yp);
-    // ldmatrix rows: A's four 8 x 8 blocks (rows 0-7 / 8-15 by k 0-7 / 8-15) of one
-    // 16-wide K step; B's four (columns 0-7 by k 0-7 / 8-15 / 16-23 / 24-31)
-    const int ar = 16 * mt + (lane & 7) + ((lane >> 3) & 1) * 8, ac = (lane >> 4) * 8;
-    const int br = 8 * nt + (lane & 7), bc = (lane >> 3) * 8;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      ldsm_x4(yb + 2u * (uint32_t)(j * kOzPlane + br * kOzPitch + bc), b[j]);
-#pragma unroll
-      for (int ks = 0; ks < 2; ++ks)
-        ldsm_x4(xb + 2u * (uint32_t)(j * kOzPlane + ar * kOzPitch + 16 * ks + ac), a[j][ks]);
-    }
-  }
   // one accumulator per level, the pairs issued slice by slice of A so that
-  // consecutive MMAs go to different accumulators (no dependent chain)
+  // consecutive MMAs go to different accumulators (no dependent chain); one 16-wide
+  // K step at a time, which keeps the kernel at two CTAs an SM
   float c[8][4];
 #pragma unroll
   for (int L = 0; L < 8; ++L)
 #pragma unroll
     for (int q = 0; q < 4; ++q) c[L][q] = 0.f;
+  // ldmatrix rows: A's four 8 x 8 blocks (rows 0-7 / 8-15 by k 0-7 / 8-15); B's two
+  // (columns 0-7 by k 0-7 / 8-15) of two slices
+  const int ar = 16 * mt + (lane & 7) + ((lane >> 3) & 1) * 8, ac = (lane >> 4) * 8;
+  const int br = 8 * nt + (lane & 7), bc = ((lane >> 3) & 1) * 8, bs = lane >> 4;
+  const uint32_t xb = (uint32_t)__cvta_generic_to_shared(xp) + 2u * (ar * kOzPitch + ac);
+  const uint32_t yb =
+      (uint32_t)__cvta_generic_to_shared(yp) + 2u * (bs * kOzPlane + br * kOzPitch + bc);
 #pragma unroll
-  for (int ks = 0; ks < 2; ++ks)
+  for (int ks = 0; ks < 2; ++ks) {
+    uint32_t a[8][4], b[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ldsm_x4(yb + 2u * (2 * j * kOzPlane + 16 * ks), b[j]);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) ldsm_x4(xb + 2u * (j * kOzPlane + 16 * ks), a[j]);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; i + j < 8; ++j) mma_bf16(c[i + j], a[i][ks], b[j][2 * ks], b[j][2 * ks + 1]);
+      for (int j = 0; i + j < 8; ++j)
+        mma_bf16(c[i + j], a[i], b[j >> 1][2 * (j & 1)], b[j >> 1][2 * (j & 1) + 1]);
+  }
   // |S_L| < 2^21: to integers by the exact FP32 rounding against 1.5 2^23 (no
   // 64-bit conversions, which GB300 runs at its FP64 rate); two levels 7 bits
   // apart share one 32-bit integer, then
@@ -333,22 +391,23 @@ __device__ __forceinline__ void oz_combine(const __nv_bfloat16* xp, const __nv_b
     // a = sum_j d_j 2^(ex - 1029 - 7 j): the integer's unit is level 5's
     double v = oz::compose(tot, ex[r] + ey[cc] - 2093);
     if (sign < 0.0) v = -v;
-    out[r][cc] = accumulate ? out[r][cc] + v : v;
+    at(out, r, cc) = accumulate ? at(out, r, cc) + v : v;
   }
 }
 
-// All 256 threads; out must not alias X or Y.
-__device__ void tile_mm_oz(double (*X)[T + 1], double (*Y)[T + 1], bool ytrans, bool ylower,
-                           double (*out)[T + 1], double sign, bool accumulate,
-                           const OzTile& z) {
-  oz_split([&](int r, int k) { return X[r][k]; }, z.xp, z.ex);
+// All compute threads; out must not alias X or Y.
+__device__ __forceinline__ void tile_mm_oz(Tile X, Tile Y, bool ytrans,
+                                           bool ylower, Tile out, double sign,
+                                           bool accumulate, const OzTile& z) {
+  const int warp = threadIdx.x >> 5;
+  oz_split([&](int r, int k) { return at(X, r, k); }, z.xp, z.ex, warp);
   oz_split(
       [&](int n, int k) {
         if (ylower && (ytrans ? k > n : n > k)) return 0.0;
-        return ytrans ? Y[n][k] : Y[k][n];
+        return ytrans ? at(Y, n, k) : at(Y, k, n);
       },
-      z.yp, z.ey);
-  __syncthreads();
+      z.yp, z.ey, warp);
+  compute_bar();
   oz_combine(z.xp, z.yp, z.ex, z.ey, out, sign, accumulate);
 }
 
@@ -463,51 +522,39 @@ __device__ __forceinline__ double rsqrt_fp64(double d) {
 //
 // Pivot j eliminates column j with the multipliers l_ij = S_ij / d_j:
 // S_ik -= l_ij S_kj (j < k <= i) and X_ik -= l_ij X_jk (k <= j < i).  Warp 0
-// runs one pivot ahead: while warps 1-3 and 5-7 apply pivot j to columns
+// runs one pivot ahead: while warps 1-7 apply pivot j to columns
 // k >= j+2 and to X, it applies pivot j to column j+1, takes d_{j+1}, its
 // reciprocal and the next multipliers.  A position (i, k) belongs to one thread
 // for the whole leaf, which holds S_ik and, from pivot k on, X_ik in a register;
 // only what others read goes through shared memory, double buffered by the
 // pivot's parity: the multipliers and the column of the pivot (from warp 0),
-// column j+2 (for warp 0) and row j+1 of X.  So each pivot costs one barrier of
-// these seven warps, and the serial chain is one FMA, the integer reciprocal and
-// one multiply.  An SM sub-partition issues one FP64 warp instruction per 64
-// clocks: warp 4 shares warp 0's and takes no part (see service).
-// Measured alone: 20.6 k clocks (10 us; 15 us with the FP64 reciprocal, positions in
-// shared memory and the log-det between the steps), bound by the bulk warps (~520 clocks
-// a pivot) ahead of the chain (~440).  512-row factor in the tensor-core modes 0.41 ->
-// 0.31 ms (a diagonal step 25.5 -> 18.8 us).
+// column j+2 (for warp 0) and row j+1 of X.  So each pivot costs one barrier, and the
+// serial chain is one FMA, the integer reciprocal and one multiply.  An SM sub-partition
+// issues one FP64 warp instruction per 64 clocks, so of the 17 warps' worth of
+// positions warp 4, which shares warp 0's, takes two and each other sub-partition five.
+// Measured: 10.4 us of a chain step's 17.4 (512 rows, tensor-core modes).
 struct LeafBuf {
   double l[2][T], v[2][T], x[2][T], s[2][T];
 };
 
-__device__ __forceinline__ void leaf_bar() {   // warps 0-3 and 5-7
-  asm volatile("bar.sync 1, 224;" ::: "memory");
-}
-
-// service: run by warp 4 alongside the pivots.
-template <class Service>
-__device__ __forceinline__ void leaf(double (*S)[T + 1], double (*X)[T + 1], LeafBuf& B,
-                                     double* piv, double* rs, Service service) {
+__device__ __forceinline__ void leaf(Tile S, Tile X, LeafBuf& B,
+                                     double* piv, double* rs) {
   constexpr int kPos = T * (T + 1) / 2;   // lower-triangle positions, row by row
-  constexpr int kBulk = kDagThreads - 64;   // warps 1-3 and 5-7
+  constexpr int kBulk = kDagThreads - 32;   // warps 1-7
   constexpr int kPer = (kPos + kBulk - 1) / kBulk;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int bt = warp < 4 ? tid - 32 : tid - 64;   // 0..kBulk-1 over the bulk warps
-  int pi[kPer], pk[kPer];
-  double val[kPer];
   if (warp == 0) {
-    double v = S[lane][0];
+    double v = at(S, lane, 0);
     double d = __shfl_sync(0xffffffffu, v, 0);
     double l = v * recip(d);
     B.l[0][lane] = l;
     B.v[0][lane] = v;
-    B.s[0][lane] = S[lane][1];
+    B.s[0][lane] = at(S, lane, 1);
     if (lane == 0) {
       B.x[0][0] = 1.0;
       piv[0] = d;
     }
-    leaf_bar();
+    compute_bar();
     for (int j = 0; j < T - 1; ++j) {
       // column c = j+1 with pivot j, then pivot c and its multipliers
       const int c = j + 1, p = c & 1;
@@ -518,13 +565,15 @@ __device__ __forceinline__ void leaf(double (*S)[T + 1], double (*X)[T + 1], Lea
       B.l[p][lane] = l;
       B.v[p][lane] = v;
       if (lane == 0) piv[c] = d;
-      leaf_bar();
+      compute_bar();
     }
     rs[lane] = rsqrt_fp64(piv[lane]);   // rows scale by d_i^{-1/2}
-    leaf_bar();
-  } else if (warp == 4) {
-    service();
+    compute_bar();
   } else {
+    // warps 1-3, 5-7 and then 4: the last positions go to the first three
+    const int bt = (warp < 4 ? warp - 1 : warp == 4 ? 6 : warp - 2) * 32 + lane;
+    int pi[kPer], pk[kPer];
+    double val[kPer];
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
       const int q = bt + kBulk * r;
@@ -533,9 +582,9 @@ __device__ __forceinline__ void leaf(double (*S)[T + 1], double (*X)[T + 1], Lea
       if ((i + 1) * (i + 2) / 2 <= q) ++i;
       pi[r] = q < kPos ? i : -1;
       pk[r] = q < kPos ? q - i * (i + 1) / 2 : 0;
-      val[r] = q < kPos ? S[i][pk[r]] : 0.0;
+      val[r] = q < kPos ? at(S, i, pk[r]) : 0.0;
     }
-    leaf_bar();
+    compute_bar();
     for (int j = 0; j < T - 1; ++j) {
       const int p = j & 1;
       double src[kPer], lv[kPer];
@@ -557,265 +606,400 @@ __device__ __forceinline__ void leaf(double (*S)[T + 1], double (*X)[T + 1], Lea
           if (i == j + 1) B.x[p ^ 1][k] = k == i ? 1.0 : val[r];
         }
       }
-      leaf_bar();
+      compute_bar();
     }
-    leaf_bar();
+    compute_bar();
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
       const int i = pi[r], k = pk[r];
-      if (i >= 0) X[i][k] = k == i ? rs[i] : val[r] * rs[i];
+      if (i >= 0) at(X, i, k) = k == i ? rs[i] : val[r] * rs[i];
     }
   }
-  __syncthreads();
+  compute_bar();
 }
 
 // Log-det slot of a leaf: sum of log d_i over its pivots, and the failure
-// code on a non-positive or non-finite pivot (one warp).
-__device__ __forceinline__ void leaf_logdet(const double* piv, double* slot, int32_t* fail,
+// code on a non-positive or non-finite pivot (one warp, d its lane's pivot).
+__device__ __forceinline__ void leaf_logdet(double d, double* slot, int32_t* fail,
                                             int32_t code) {
-  {
-    const int lane = threadIdx.x & 31;
-    const double dj = piv[lane];
-    const bool b = !(dj > 0.0) || !isfinite(dj);
-    double l = b ? 0.0 : log(dj);
+  const bool b = !(d > 0.0) || !isfinite(d);
+  double l = b ? 0.0 : log(d);
 #pragma unroll
-    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    const unsigned anyb = __ballot_sync(0xffffffffu, b);
-    if (lane == 0) {
-      *slot = l;
-      if (anyb) atomicCAS(fail, -1, code);
+  for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  const unsigned anyb = __ballot_sync(0xffffffffu, b);
+  if ((threadIdx.x & 31) == 0) {
+    *slot = l;
+    if (anyb) atomicCAS(fail, -1, code);
+  }
+}
+
+struct Slot {
+  int type, i, j, k, z;
+};
+
+// Shared memory of a CTA: two stages of three tiles (first and second operand,
+// accumulator and result), and in the tensor-core modes the slices of two tiles.
+struct DagSmem {
+  alignas(16) double t[2][3][T][kTP];
+  LeafBuf lbuf;
+  double piv[2][T], rs[T];
+  Slot slot[2];
+  // mbarriers: stage filled / result stored / stage free, chain step's tiles in place,
+  // chain step's L / X stored (by parity of the step)
+  unsigned long long full[2], done[2], free[2], ch[2], lst[2], xst[2];
+  int abort;
+};
+template <bool TC>
+constexpr int dag_smem() {
+  return (int)((sizeof(DagSmem) + 15) / 16 * 16) + (TC ? kOzTileSmem : 0);
+}
+
+__device__ __forceinline__ void mb_init(unsigned long long* b) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(b))
+               : "memory");
+}
+__device__ __forceinline__ void mb_arrive(unsigned long long* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(b))
+               : "memory");
+}
+// Waits for the phase of the given parity; false after an abort in the CTA, or after
+// four times the limit of a wait on another CTA (which ends first).
+__device__ __forceinline__ bool mb_wait(unsigned long long* b, int parity, volatile int* abort,
+                                        unsigned long long wait_ns) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(b);
+  unsigned long long t0 = 0;
+  for (unsigned it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (*abort) return false;
+    if ((it & 63) == 63) {
+      const unsigned long long t = now_ns();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > 4 * wait_ns) {
+        *abort = 1;
+        return false;
+      }
     }
   }
 }
 
 // TC: the tile products emulated in FP64 on the tensor cores (tile_mm_oz,
-// the tensor-core modes); otherwise FP64 FMAs.
+// the tensor-core modes); otherwise FP64 FMAs.  Two CTAs fit an SM, or one beside a
+// product of another leg.
 template <bool TC>
-__global__ void __launch_bounds__(kDagThreads) potrf_dag_kernel(DagArgs g) {
-  // three tiles (~28 KB with the leaf's vectors); TC adds the slices of two
-  // tiles (40 KB of dynamic shared memory)
-  __shared__ double S0[T][T + 1], S1[T][T + 1], S2[T][T + 1];
+__global__ void __launch_bounds__(kDagAllThreads, 2) potrf_dag_kernel(DagArgs g) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  OzTile ozs;
-  ozs.xp = reinterpret_cast<__nv_bfloat16*>(dsm);
-  ozs.yp = ozs.xp + 8 * kOzPlane;
-  ozs.ex = reinterpret_cast<int*>(ozs.yp + 8 * kOzPlane);
-  ozs.ey = ozs.ex + T;
-  // out (+)= sign X op(Y), and the product with a lower-triangular Y^T
-  auto mm = [&](double (*X)[T + 1], double (*Y)[T + 1], bool ytrans, double (*o)[T + 1],
-                double sign, bool acc) {
-    if constexpr (TC) tile_mm_oz(X, Y, ytrans, false, o, sign, acc, ozs);
-    else tile_mm(X, Y, ytrans, o, sign, acc);
-  };
-  auto mm_lt = [&](double (*W)[T + 1], double (*Y)[T + 1], double (*o)[T + 1]) {
-    if constexpr (TC) tile_mm_oz(W, Y, true, true, o, 1.0, false, ozs);
-    else tile_mm_lt(W, Y, o);
-  };
-  __shared__ LeafBuf lbuf;
-  __shared__ double piv[2][T], rs[T];
-  __shared__ int s_task, s_ok;
+  DagSmem& sm = *reinterpret_cast<DagSmem*>(dsm);
+  OzTile oz;
+  oz.xp = reinterpret_cast<__nv_bfloat16*>(dsm + (sizeof(DagSmem) + 15) / 16 * 16);
+  oz.yp = oz.xp + 8 * kOzPlane;
+  oz.ex = reinterpret_cast<int*>(oz.yp + 8 * kOzPlane);
+  oz.ey = oz.ex + T;
   const int p = g.p, ld = g.ld, pp = p * p;
-  int* busy = &g.smbusy[sm_id() & 255];
-  while (true) {
-    if (threadIdx.x == 0) {
-      // On an SM that runs a chain, take no task while the chain is there: it
-      // gets the SM's whole FP64 pipe.  Waiting before taking a ticket holds
-      // nothing another task needs.
-      if (g.yield && ld_acquire(busy) > 0) {
-        const unsigned long long t0 = now_ns();
-        while (ld_acquire(busy) > 0 && ld_acquire(g.counter) < g.total && !ld_acquire(g.abort)) {
-          __nanosleep(256);
-          if (now_ns() - t0 > g.wait_ns) {
-            atomicExch(g.abort, 1);
-            break;
-          }
-        }
-      }
-      s_task = atomicAdd(g.counter, 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 2; ++q) {
+      mb_init(&sm.full[q]);
+      mb_init(&sm.done[q]);
+      mb_init(&sm.free[q]);
+      mb_init(&sm.ch[q]);
+      mb_init(&sm.lst[q]);
+      mb_init(&sm.xst[q]);
     }
-    __syncthreads();
-    const int tg = s_task;
-    __syncthreads();
-    if (tg >= g.total) return;
-    const int z = tg % g.cnt;
-    const Task t = decode(g, tg / g.cnt);
-    const DagInst& I = g.inst[z];
-    int* cntW = I.st;
-    int* cntR = I.st + pp;
-    int* doneF = I.st + 2 * pp;
-    int* doneS = doneF + p;
-    int* doneG = doneS + pp;
-    auto Lt = [&](int i, int k) { return I.Lt + ((int64_t)i * (i - 1) / 2 + k) * T * T; };
-    if (t.type == TK_H) {
-      // ---- the chain: every diagonal step of this block on this CTA
-      if (threadIdx.x == 0 && g.yield) atomicAdd(busy, 1);
-      for (int c = 0; c < p; ++c) {
-        if (c > 0 || g.stall) {
-          // W_{c,c-1} and W_cc updated through step c-2 by the U tasks (the
-          // test switch instead waits for a count no task reaches)
-          if (threadIdx.x == 0)
-            s_ok = g.stall ? wait_ge(&cntW[c * p + c], 0x7fffffff, g.abort, g.wait_ns)
-                           : wait_ge(&cntW[c * p + c - 1], c - 1, g.abort, g.wait_ns) &&
-                             wait_ge(&cntW[c * p + c], c - 1, g.abort, g.wait_ns);
-          __syncthreads();
-          if (!s_ok) {
-            if (threadIdx.x == 0) {
-              atomicExch(I.fail, (int32_t)BTA_ERR_TIMEOUT);
-              if (g.yield) atomicSub(busy, 1);
+    sm.abort = 0;
+  }
+  __syncthreads();
+  volatile int* const abort = &sm.abort;
+  auto Lt = [&](const DagInst& I, int i, int k) {
+    return I.Lt + ((int64_t)i * (i - 1) / 2 + k) * T * T;
+  };
+  auto cntW = [&](const DagInst& I) { return I.st; };
+  auto cntR = [&](const DagInst& I) { return I.st + pp; };
+  auto doneF = [&](const DagInst& I) { return I.st + 2 * pp; };
+  auto doneS = [&](const DagInst& I) { return I.st + 2 * pp + p; };
+  auto doneG = [&](const DagInst& I) { return I.st + 3 * pp + p; };
+  // phase of a chain step's barriers (by parity of the step), hc chains before this one on
+  // this CTA (blocks of one or two tiles have no tasks that tie a chain to its CTA)
+  auto step_phase = [&](int c, int hc) { return hc * ((p + 1 - (c & 1)) / 2) + (c >> 1); };
+  auto l_phase = [&](int c, int hc) {   // steps from 1 on
+    return hc * (c & 1 ? p / 2 : (p - 1) / 2) + ((c - 1) >> 1);
+  };
+  int hc = 0;
+  auto wait = [&](unsigned long long* b, int parity) {
+    return mb_wait(b, parity & 1, abort, g.wait_ns);
+  };
+
+  if (warp == kDagFetch) {
+    // ---- fetcher: task n into stage n & 1
+    int* busy = &g.smbusy[sm_id() & 255];
+    for (int n = 0;; ++n) {
+      const int s = n & 1;
+      if (n >= 2 && !wait(&sm.free[s], (n >> 1) - 1)) return;
+      int tg = 0;
+      if (lane == 0) {
+        // On an SM that runs a chain, take no task while the chain is there: it
+        // gets the SM's whole FP64 pipe.  Waiting before taking a ticket holds
+        // nothing another task needs.
+        if (g.yield && ld_acquire(busy) > 0) {
+          const unsigned long long t0 = now_ns();
+          while (ld_acquire(busy) > 0 && ld_acquire(g.counter) < g.total &&
+                 !ld_acquire(g.abort)) {
+            __nanosleep(256);
+            if (now_ns() - t0 > g.wait_ns) {
+              atomicExch(g.abort, 1);
+              break;
             }
-            return;
           }
         }
-        if (threadIdx.x == 0 && z == 0) DAG_TRACE(0, c);
-        if (c > 0) {
-          load_tile(S0, tile(I.A, ld, c, c - 1), ld);
-          // W_cc into registers now, into S0 once the product has read it
-          double wcc[T * T / kDagThreads];
-          {
-            const double* src = tile(I.A, ld, c, c);
-#pragma unroll
-            for (int q = 0; q < T * T / kDagThreads; ++q) {
-              const int e = threadIdx.x + kDagThreads * q;
-              wcc[q] = __ldcg(src + (int64_t)(e / T) * ld + e % T);
-            }
-          }
-          __syncthreads();
-          mm_lt(S0, S1, S2);                      // L_{c,c-1} = W X_{c-1,c-1}^T (S1)
-          __syncthreads();
-          if (threadIdx.x == 0 && z == 0) DAG_TRACE(1, c);
-#pragma unroll
-          for (int q = 0; q < T * T / kDagThreads; ++q) {
-            const int e = threadIdx.x + kDagThreads * q;
-            S0[e % T][e / T] = wcc[q];
-          }
-          store_tile(Lt(c, c - 1), T, S2, false);
-          // W_cc -= L L^T (lower); a thread of a warp that has no part in it publishes L
+        tg = atomicAdd(g.counter, 1);
+      }
+      tg = __shfl_sync(0xffffffffu, tg, 0);
+      if (tg >= g.total) {
+        if (lane == 0) {
+          sm.slot[s].type = TK_END;
+          mb_arrive(&sm.full[s]);
+        }
+        return;
+      }
+      const int z = tg % g.cnt;
+      const Task t = decode(g, tg / g.cnt);
+      const DagInst& I = g.inst[z];
+      // lanes 0..2 wait for one counter each
+      auto wait_all = [&](const int* c0, int v0, const int* c1, int v1, const int* c2,
+                          int v2) -> bool {
+        const int* c = lane == 0 ? c0 : lane == 1 ? c1 : c2;
+        const int v = lane == 0 ? v0 : lane == 1 ? v1 : v2;
+        const bool ok = lane > 2 || !c || wait_ge(c, v, g.abort, g.wait_ns);
+        const bool all = __all_sync(0xffffffffu, ok);
+        __syncwarp();   // the acquires of lanes 0..2 hold for all lanes
+        if (!all && lane == 0) {
+          atomicExch(I.fail, (int32_t)BTA_ERR_TIMEOUT);
+          *abort = 1;
+        }
+        return all;
+      };
+      if (t.type == TK_H) {
+        // the chain takes both stages: the task before it has left the other one
+        if (n >= 1 && !wait(&sm.free[s ^ 1], (n - 1) >> 1)) return;
+        if (lane == 0) {
+          if (g.yield) atomicAdd(busy, 1);
+          sm.slot[s] = {TK_H, 0, 0, 0, z};
+          mb_arrive(&sm.full[s]);
+        }
+        bool ok = true;
+        for (int c = 0; c < p && ok; ++c) {
+          // W_{c,c-1} and W_cc updated through step c-2 by the U tasks (the test
+          // switch instead waits for a count no task reaches).  They imply that step
+          // c-2, and the product of step c-1, are done with this stage and the slices.
+          Tile W = sm.t[c & 1][0];
+          if (c > 0 || g.stall)
+            ok = wait_all(c > 0 ? cntW(I) + c * p + c - 1 : nullptr, c - 1, cntW(I) + c * p + c,
+                          g.stall ? 0x7fffffff : c - 1, nullptr, 0);
+          if (!ok) break;
+          if (lane == 0 && z == 0) DAG_TRACE(11, c);
+          if (c > 0) load_tile(W, tile(I.A, ld, c, c - 1), ld, g.vec);
+          load_tile(sm.t[c & 1][2], tile(I.A, ld, c, c), ld, g.vec);
+          load_wait();
           if constexpr (TC) {
-            oz_split([&](int r, int k) { return S2[r][k]; }, ozs.xp, ozs.ex);
-            __syncthreads();
-            const int warp = threadIdx.x >> 5;
-            if (warp != 2 && warp != 3)           // output rows 0-15 by columns 16-31
-              oz_combine(ozs.xp, ozs.xp, ozs.ex, ozs.ex, S0, -1.0, true);
-            else if (threadIdx.x == 96)
-              st_release(&doneS[c * p + c - 1], 1);
-          } else {
-            __syncthreads();
-            tile_syrk_lower(S2, S0);
-            if (threadIdx.x == 224) st_release(&doneS[c * p + c - 1], 1);
+            if (c > 0)
+#pragma unroll 1
+              for (int part = 0; part < 8; ++part)
+                oz_split([&](int r, int k) { return at(W, r, k); }, oz.xp, oz.ex, part);
           }
-          __syncthreads();
-          if (threadIdx.x == 0 && z == 0) DAG_TRACE(2, c);
-        } else {
-          load_tile(S0, tile(I.A, ld, 0, 0), ld);
-          __syncthreads();
+          __syncwarp();
+          if (lane == 0) mb_arrive(&sm.ch[c & 1]);
         }
-        // S1 = X_cc = L_cc^{-1}; warp 4 meanwhile sums the logs of the last step's pivots
-        leaf(S0, S1, lbuf, piv[c & 1], rs, [&]() {
-          if (c > 0) leaf_logdet(piv[(c - 1) & 1], &I.slots[c - 1], I.fail, I.code);
-        });
-        if (threadIdx.x == 0 && z == 0) DAG_TRACE(3, c);
-        store_tile(tile(I.A, ld, c, c), ld, S1, true);
-        __syncthreads();
-        // thread 0 goes on to the next step's waits
-        if (threadIdx.x == 224) {
-          st_release(&cntW[c * p + c], c);
-          st_release(&doneF[c], 1);
-          if (z == 0) DAG_TRACE(4, c);
-        }
+        ok = ok && wait(&sm.free[s], n >> 1);
+        if (lane == 0 && g.yield) atomicSub(busy, 1);
+        if (!ok) return;
+        continue;
       }
-      if (threadIdx.x < 32) leaf_logdet(piv[(p - 1) & 1], &I.slots[p - 1], I.fail, I.code);
-      __syncthreads();
-      if (threadIdx.x == 0 && g.yield) atomicSub(busy, 1);
-      continue;
-    }
-    // ---- bulk task: wait for the tiles it reads
-    if (threadIdx.x == 0) {
-      bool ok = true;
+      bool ok;
       switch (t.type) {
         case TK_S:
-          ok = wait_ge(&doneF[t.k], 1, g.abort, g.wait_ns) &&
-               wait_ge(&cntW[t.i * p + t.k], t.k, g.abort, g.wait_ns);
+          ok = wait_all(doneF(I) + t.k, 1, cntW(I) + t.i * p + t.k, t.k, nullptr, 0);
           break;
         case TK_G:
-          ok = wait_ge(&doneF[t.i], 1, g.abort, g.wait_ns) &&
-               wait_ge(&cntR[t.i * p + t.j], t.i - t.j, g.abort, g.wait_ns);
+          ok = wait_all(doneF(I) + t.i, 1, cntR(I) + t.i * p + t.j, t.i - t.j, nullptr, 0);
           break;
         case TK_U:
-          ok = wait_ge(&doneS[t.i * p + t.k], 1, g.abort, g.wait_ns) &&
-               wait_ge(&doneS[t.j * p + t.k], 1, g.abort, g.wait_ns) &&
-               wait_ge(&cntW[t.i * p + t.j], t.k, g.abort, g.wait_ns);
+          ok = wait_all(doneS(I) + t.i * p + t.k, 1, doneS(I) + t.j * p + t.k, 1,
+                        cntW(I) + t.i * p + t.j, t.k);
           break;
         default:   // TK_V
-          ok = wait_ge(&doneS[t.i * p + t.k], 1, g.abort, g.wait_ns) &&
-               (t.j == t.k ? wait_ge(&doneF[t.k], 1, g.abort, g.wait_ns)
-                           : wait_ge(&doneG[t.k * p + t.j], 1, g.abort, g.wait_ns)) &&
-               wait_ge(&cntR[t.i * p + t.j], t.k - t.j, g.abort, g.wait_ns);
+          ok = wait_all(doneS(I) + t.i * p + t.k, 1,
+                        t.j == t.k ? doneF(I) + t.k : doneG(I) + t.k * p + t.j, 1,
+                        cntR(I) + t.i * p + t.j, t.k - t.j);
       }
-      s_ok = ok;
-      if (!ok) atomicExch(I.fail, (int32_t)BTA_ERR_TIMEOUT);
+      if (!ok) return;
+      // (measurement builds) the tasks on the way to the chain's step k + 2
+      const bool crit = z == 0 && t.i == t.k + 2 &&
+                        (t.type == TK_S || (t.type == TK_U && t.j == t.k + 1));
+      if (crit && lane == 0) DAG_TRACE(t.type == TK_S ? 5 : 8, t.k);
+      auto st = sm.t[s];
+      switch (t.type) {
+        case TK_S:   // L_ik = W_ik X_kk^T
+          load_tile(st[0], tile(I.A, ld, t.i, t.k), ld, g.vec);
+          load_tile(st[1], tile(I.A, ld, t.k, t.k), ld, g.vec);
+          break;
+        case TK_G:   // X_kj = X_kk R_kj  (t.i = k)
+          load_tile(st[0], tile(I.A, ld, t.i, t.i), ld, g.vec);
+          load_tile(st[1], tile(I.A, ld, t.i, t.j), ld, g.vec);
+          break;
+        case TK_U:   // W_ij -= L_ik L_jk^T
+          load_tile(st[0], Lt(I, t.i, t.k), T, 1);
+          load_tile(st[1], Lt(I, t.j, t.k), T, 1);
+          load_tile(st[2], tile(I.A, ld, t.i, t.j), ld, g.vec);
+          break;
+        default:     // TK_V: R_ij -= L_ik X_kj (R_ij starts at 0 with k = j, X_jj lower)
+          load_tile(st[0], Lt(I, t.i, t.k), T, 1);
+          load_tile(st[1], tile(I.A, ld, t.k, t.j), ld, g.vec);
+          if (t.k != t.j) load_tile(st[2], tile(I.A, ld, t.i, t.j), ld, g.vec);
+      }
+      load_wait();
+      // a diagonal tile of the inverse is lower
+      if (t.type == TK_S || (t.type == TK_V && t.k == t.j)) zero_upper(st[1]);
+      if (t.type == TK_G) zero_upper(st[0]);
+      __syncwarp();
+      if (lane == 0) {
+        sm.slot[s] = {t.type, t.i, t.j, t.k, z};
+        mb_arrive(&sm.full[s]);
+        if (crit) DAG_TRACE(t.type == TK_S ? 6 : 9, t.k);
+      }
     }
-    __syncthreads();
-    if (!s_ok) return;
-    // ---- execute
-    switch (t.type) {
-      case TK_S: {   // L_ik = W_ik X_kk^T
-        load_tile(S0, tile(I.A, ld, t.i, t.k), ld);
-        load_tile(S1, tile(I.A, ld, t.k, t.k), ld);
-        __syncthreads();
-        mm_lt(S0, S1, S2);                        // X_kk lower: its upper part is not read
-        __syncthreads();
-        store_tile(Lt(t.i, t.k), T, S2, false);
-        __syncthreads();
-        if (threadIdx.x == 0) { st_release(&doneS[t.i * p + t.k], 1); }
-        break;
-      }
-      case TK_G: {   // X_kj = X_kk R_kj  (t.i = k)
-        load_tile(S0, tile(I.A, ld, t.i, t.i), ld);
-        load_tile(S1, tile(I.A, ld, t.i, t.j), ld);
-        __syncthreads();
-        // X_kk is lower: zero its upper part before use
-        for (int e = threadIdx.x; e < T * T; e += kDagThreads)
-          if (e % T < e / T) S0[e % T][e / T] = 0.0;
-        __syncthreads();
-        mm(S0, S1, false, S2, 1.0, false);
-        __syncthreads();
-        store_tile(tile(I.A, ld, t.i, t.j), ld, S2, false);
-        __syncthreads();
-        if (threadIdx.x == 0) { st_release(&doneG[t.i * p + t.j], 1); }
-        break;
-      }
-      case TK_U: {   // W_ij -= L_ik L_jk^T
-        load_tile(S0, Lt(t.i, t.k), T);
-        load_tile(S1, Lt(t.j, t.k), T);
-        load_tile(S2, tile(I.A, ld, t.i, t.j), ld);
-        __syncthreads();
-        mm(S0, S1, true, S2, -1.0, true);
-        __syncthreads();
-        store_tile(tile(I.A, ld, t.i, t.j), ld, S2, t.i == t.j);
-        __syncthreads();
-        if (threadIdx.x == 0) { st_release(&cntW[t.i * p + t.j], t.k + 1); }
-        break;
-      }
-      default: {     // TK_V: R_ij -= L_ik X_kj
-        load_tile(S0, Lt(t.i, t.k), T);
-        load_tile(S1, tile(I.A, ld, t.k, t.j), ld);
-        const bool first = t.k == t.j;
-        if (!first) load_tile(S2, tile(I.A, ld, t.i, t.j), ld);
-        __syncthreads();
-        if (first)   // X_jj is lower: zero its upper part
-          for (int e = threadIdx.x; e < T * T; e += kDagThreads)
-            if (e % T < e / T) S1[e % T][e / T] = 0.0;
-        __syncthreads();
-        mm(S0, S1, false, S2, -1.0, !first);
-        __syncthreads();
-        store_tile(tile(I.A, ld, t.i, t.j), ld, S2, false);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          st_release(&cntR[t.i * p + t.j], t.k - t.j + 1);
+  }
+
+  if (warp == kDagPublish) {
+    // ---- publisher
+    for (int n = 0;; ++n) {
+      const int s = n & 1;
+      if (!wait(&sm.full[s], n >> 1)) return;
+      const Slot t = sm.slot[s];
+      if (t.type == TK_END) return;
+      const DagInst& I = g.inst[t.z];
+      if (t.type == TK_H) {
+        for (int c = 0; c < p; ++c) {
+          if (c > 0) {
+            if (!wait(&sm.lst[c & 1], l_phase(c, hc))) return;
+            if (lane == 0) st_release(doneS(I) + c * p + c - 1, 1);
+          }
+          if (!wait(&sm.xst[c & 1], step_phase(c, hc))) return;
+          const double d = sm.piv[c & 1][lane];   // before the release lets step c+2 go on
+          if (lane == 0) {
+            st_release(cntW(I) + c * p + c, c);
+            st_release(doneF(I) + c, 1);
+            if (t.z == 0) DAG_TRACE(4, c);
+          }
+          __syncwarp();
+          leaf_logdet(d, &I.slots[c], I.fail, I.code);
         }
+        ++hc;
+      }
+      if (!wait(&sm.done[s], n >> 1)) return;
+      if (lane == 0) {
+        switch (t.type) {
+          case TK_H: break;
+          case TK_S: st_release(doneS(I) + t.i * p + t.k, 1); break;
+          case TK_G: st_release(doneG(I) + t.i * p + t.j, 1); break;
+          case TK_U: st_release(cntW(I) + t.i * p + t.j, t.k + 1); break;
+          default: st_release(cntR(I) + t.i * p + t.j, t.k - t.j + 1);
+        }
+        if (t.z == 0 && t.i == t.k + 2 && t.type == TK_S) DAG_TRACE(7, t.k);
+        if (t.z == 0 && t.i == t.k + 2 && t.type == TK_U && t.j == t.k + 1) DAG_TRACE(10, t.k);
+        mb_arrive(&sm.free[s]);
+      }
+      __syncwarp();
+    }
+  }
+
+  // ---- compute warps
+  auto mm = [&](Tile X, Tile Y, bool ytrans, Tile o,
+                double sign, bool acc) {
+    if constexpr (TC) tile_mm_oz(X, Y, ytrans, false, o, sign, acc, oz);
+    else tile_mm(X, Y, ytrans, o, sign, acc);
+  };
+  for (int n = 0;; ++n) {
+    const int s = n & 1;
+    if (!compute_all(wait(&sm.full[s], n >> 1))) return;
+    const Slot t = sm.slot[s];
+    if (t.type == TK_END) return;
+    const DagInst& I = g.inst[t.z];
+    auto st = sm.t[s];
+    if (t.type == TK_H) {
+      // ---- the chain: every diagonal step of this block on this CTA
+      for (int c = 0; c < p; ++c) {
+        Tile W = sm.t[c & 1][0];      // W_{c,c-1}, then X_cc
+        Tile L = sm.t[c & 1][1];      // L_{c,c-1}
+        Tile Wc = sm.t[c & 1][2];     // W_cc
+        Tile X = sm.t[(c & 1) ^ 1][0];   // X_{c-1,c-1}
+        if (c > 0) {
+          if constexpr (TC)                      // while the fetcher may still be at W
+            oz_split([&](int r, int k) { return k > r ? 0.0 : at(X, r, k); }, oz.yp, oz.ey, warp);
+        }
+        if (!compute_all(wait(&sm.ch[c & 1], step_phase(c, hc)))) return;
+        if (threadIdx.x == 0 && t.z == 0) DAG_TRACE(0, c);
+        if (c > 0) {
+          if constexpr (TC) oz_combine(oz.xp, oz.yp, oz.ex, oz.ey, L, 1.0, false);
+          else tile_mm_lt(W, X, L);              // L_{c,c-1} = W X_{c-1,c-1}^T
+          compute_bar();
+          if (threadIdx.x == 0 && t.z == 0) DAG_TRACE(1, c);
+          store_tile(Lt(I, c, c - 1), T, L, false);
+          // W_cc -= L L^T (lower)
+          if constexpr (TC) {
+            oz_split([&](int r, int k) { return at(L, r, k); }, oz.yp, oz.ey, warp);
+            compute_bar();
+            if (threadIdx.x == 0) mb_arrive(&sm.lst[c & 1]);
+            if (warp != 2 && warp != 3)           // output rows 0-15 by columns 16-31
+              oz_combine(oz.yp, oz.yp, oz.ey, oz.ey, Wc, -1.0, true);
+          } else {
+            compute_bar();
+            if (threadIdx.x == 0) mb_arrive(&sm.lst[c & 1]);
+            tile_syrk_lower(L, Wc);
+          }
+          compute_bar();
+          if (threadIdx.x == 0 && t.z == 0) DAG_TRACE(2, c);
+        }
+        leaf(Wc, W, sm.lbuf, sm.piv[c & 1], sm.rs);   // X_cc = L_cc^{-1}
+        if (threadIdx.x == 0 && t.z == 0) DAG_TRACE(3, c);
+        store_tile(tile(I.A, ld, c, c), ld, W, true);
+        compute_bar();
+        if (threadIdx.x == 0) mb_arrive(&sm.xst[c & 1]);
+      }
+      ++hc;
+    } else {
+      switch (t.type) {
+        case TK_S:
+          if constexpr (TC) tile_mm_oz(st[0], st[1], true, false, st[2], 1.0, false, oz);
+          else tile_mm_lt(st[0], st[1], st[2]);
+          compute_bar();
+          store_tile(Lt(I, t.i, t.k), T, st[2], false);
+          break;
+        case TK_G:
+          mm(st[0], st[1], false, st[2], 1.0, false);
+          compute_bar();
+          store_tile(tile(I.A, ld, t.i, t.j), ld, st[2], false);
+          break;
+        case TK_U:
+          mm(st[0], st[1], true, st[2], -1.0, true);
+          compute_bar();
+          store_tile(tile(I.A, ld, t.i, t.j), ld, st[2], t.i == t.j);
+          break;
+        default:
+          mm(st[0], st[1], false, st[2], -1.0, t.k != t.j);
+          compute_bar();
+          store_tile(tile(I.A, ld, t.i, t.j), ld, st[2], false);
       }
     }
-    __syncthreads();
+    compute_bar();
+    if (threadIdx.x == 0) mb_arrive(&sm.done[s]);
   }
 }
 
@@ -894,6 +1078,7 @@ bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* c
     }
     g.off[p] = acc;
     g.total = (acc + 1) * cnt;
+    g.vec = 1;
     for (int z = 0; z < cnt; ++z) {
       DagInst& I = g.inst[z];
       I.A = A[z0 + z];
@@ -902,6 +1087,8 @@ bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* c
       I.slots = logdet_parts[z0 + z];
       I.fail = fail[z0 + z];
       I.code = fail_code[z0 + z];
+      if (reinterpret_cast<uintptr_t>(I.A) % 16) g.vec = 0;
+      if (reinterpret_cast<uintptr_t>(I.Lt) % 16) return BTA_ERR_ARG;   // library workspace
       BTA_CUDA_TRY(cudaMemsetAsync(I.st, 0, potrf_dag_state_ints(p) * sizeof(int), s));
     }
     // ticket counter and abort flag live after instance 0's counters
@@ -914,18 +1101,23 @@ bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* c
     int grid = std::min(g.total, sm_count() * dag_ctas_per_sm());
     const int cap = dag_max_ctas() > 0 ? dag_max_ctas() : max_ctas;
     if (cap > 0) grid = std::min(grid, std::max(2, cap));   // the chain and a bulk CTA
-    if (tc) {
-      static bool attr = false;   // the slices take the dynamic shared memory above 48 KB
-      if (!attr) {
-        BTA_CUDA_TRY(cudaFuncSetAttribute(potrf_dag_kernel<true>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          kOzTileSmem));
-        attr = true;
-      }
-      launch_prio_smem(potrf_dag_kernel<true>, dim3(grid), dim3(kDagThreads), kOzTileSmem, s, g);
-    } else {
-      launch_prio(potrf_dag_kernel<false>, dim3(grid), dim3(kDagThreads), s, g);
+    grid = std::max(grid, std::min(g.total, cnt + 1));   // every chain, and a bulk CTA
+    static bool attr = false;   // above 48 KB of dynamic shared memory
+    if (!attr) {
+      BTA_CUDA_TRY(cudaFuncSetAttribute(potrf_dag_kernel<true>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        dag_smem<true>()));
+      BTA_CUDA_TRY(cudaFuncSetAttribute(potrf_dag_kernel<false>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        dag_smem<false>()));
+      attr = true;
     }
+    if (tc)
+      launch_prio_smem(potrf_dag_kernel<true>, dim3(grid), dim3(kDagAllThreads), dag_smem<true>(),
+                       s, g);
+    else
+      launch_prio_smem(potrf_dag_kernel<false>, dim3(grid), dim3(kDagAllThreads),
+                       dag_smem<false>(), s, g);
     BTA_LAUNCHED();
   }
   return BTA_OK;
