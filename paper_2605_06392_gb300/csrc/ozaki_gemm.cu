@@ -22,9 +22,9 @@
 // 2.6 times that: 4800^3 whole call 5.38 ms before, 2.95 ms now, at no larger
 // error (no digit products are dropped).
 //
-// Kernels: exponents of the rows (ozaki_exp_kernel), residue planes
-// (residue_kernel), the 14 products (crt_gemm_kernel), and the
-// recovery with alpha, beta (crt_compose_kernel).
+// Kernels: exponents of the rows (ozaki_exp_kernel), residue planes (residue_kernel),
+// the 14 products (crt_gemm_kernel, crt_gemm_small_kernel), and the recovery with alpha,
+// beta (crt_compose_kernel).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -282,6 +282,39 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// One chunk's sums of 16 columns into the running residues: per column t = S + acc
+// (|t| < 2^24, exact), acc = t mod p, two columns per instruction.
+struct CrtMod {
+  uint64_t np, inv, magic, nmagic;
+  __device__ __forceinline__ explicit CrtMod(int m) {
+    const float pf = -c_mod.p[m], invf = c_mod.inv[m];
+    np = pack2(pf, pf);
+    inv = pack2(invf, invf);
+    magic = pack2(kMagic, kMagic);
+    nmagic = pack2(-kMagic, -kMagic);
+  }
+  __device__ __forceinline__ void add(const float (&v)[16], uint64_t* acc) const {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const uint64_t s = add2(pack2(v[2 * q], v[2 * q + 1]), acc[q]);
+      const uint64_t k = add2(fma2(s, inv, magic), nmagic);
+      acc[q] = fma2(k, np, s);
+    }
+  }
+};
+// Residues of 2 n consecutive columns of a row (columns `ld` apart) as 16-bit integers: the
+// low half of x + kMagic is x.
+template <int N>
+__device__ __forceinline__ void crt_store(uint16_t* out, int ld, const uint64_t (&acc)[N]) {
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    float a0, a1;
+    unpack2(acc[q], a0, a1);
+    out[(int64_t)(2 * q) * ld] = (uint16_t)__float_as_uint(a0 + (kMagic + kBias));
+    out[(int64_t)(2 * q + 1) * ld] = (uint16_t)__float_as_uint(a1 + (kMagic + kBias));
+  }
+}
+
 struct CrtArgs {
   int Mp, Np, Ap, Bp;   // output rows / columns (padded); rows per A / B plane
   int nk;               // 64-wide K slabs
@@ -298,9 +331,10 @@ struct CrtUnit {
   int mod, m0, n0, ks0, ks1;
 };
 
-// Unit u: modulus-major, so that the resident pairs work on the planes of one
+// Unit u of CT x CT tiles: modulus-major, so that the resident pairs work on the planes of one
 // modulus (they fit in L2).  Within it groups of `group` tile rows, column by
 // column; or, for the lower triangle, rows of tiles up to the diagonal.
+template <int CT>
 __device__ __forceinline__ CrtUnit crt_unit(const CrtArgs& g, int u) {
   CrtUnit t;
   t.mod = u / g.tiles;
@@ -396,9 +430,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
       int r = 0;
       bool stop = false;
       for (int j = 0; j < units && !stop; ++j) {
-        const CrtUnit t = crt_unit(g, u0 + j * g.slots);
-        const int ya = t.mod * g.Ap + t.m0 + (int)rank * CH;
-        const int yb = t.mod * g.Bp + t.n0 + (int)rank * CH;
+        const CrtUnit t = crt_unit<CT>(g, u0 + j * g.slots);
+        const int ya = t.mod * g.nk * g.Ap + t.m0 + (int)rank * CH;
+        const int yb = t.mod * g.nk * g.Bp + t.n0 + (int)rank * CH;
         for (int kt = t.ks0; kt < t.ks1; ++kt, ++r) {
           const int s = r % kStages;
           if (r >= kStages && !mbar_wait(smem_u32(&bars[kEmpty + s]),
@@ -414,8 +448,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
           if (rank == 0) mbar_expect_tx(smem_u32(&bars[kLoaded + s]), 2u * kStage);
           const uint32_t full = loaded0 + 8u * (uint32_t)s;
           uint8_t* st = smem + s * kStage;
-          tma_load_pair(smem_u32(st), &mA, full, kt * CK, ya);
-          tma_load_pair(smem_u32(st + kHalfTile), &mB, full, kt * CK, yb);
+          tma_load_pair(smem_u32(st), &mA, full, 0, ya + kt * g.Ap);
+          tma_load_pair(smem_u32(st + kHalfTile), &mB, full, 0, yb + kt * g.Bp);
           *(volatile int*)&s_issued = r + 1;
         }
       }
@@ -428,7 +462,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
       bool stop = false;
       int r = 0, e = 0;   // slabs consumed, chunks begun
       for (int j = 0; j < units && !stop; ++j) {
-        const CrtUnit t = crt_unit(g, u0 + j * g.slots);
+        const CrtUnit t = crt_unit<CT>(g, u0 + j * g.slots);
         for (int kc = t.ks0; kc < t.ks1 && !stop; kc += kChunkSlabs, ++e) {
           const int b = e & 1;
           // both CTAs have drained this accumulator's last chunk
@@ -467,18 +501,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
     }
     __syncwarp();
   } else {
-    // ---- warps 0-7 (both CTAs): thread = output row (TMEM lane) x 128 columns.
-    // Per chunk and column: t = S + acc (|t| < 2^24, exact), acc = t mod p.
+    // ---- warps 0-7 (both CTAs): thread = output row (TMEM lane) x 128 columns
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const int row = (int)rank * CH + (warp & 3) * 32 + lane, col0 = (warp >> 2) * 128;
     const uint32_t acc_empty = cluster_addr(smem_u32(&bars[kAccEmpty]), 0);
-    const uint64_t magic = pack2(kMagic, kMagic), nmagic = pack2(-kMagic, -kMagic);
     bool failed = false;
     int e = 0;
     for (int j = 0; j < units && !failed; ++j) {
-      const CrtUnit t = crt_unit(g, u0 + j * g.slots);
-      const float pf = -c_mod.p[t.mod], invf = c_mod.inv[t.mod];
-      const uint64_t np = pack2(pf, pf), inv = pack2(invf, invf);
+      const CrtUnit t = crt_unit<CT>(g, u0 + j * g.slots);
+      const CrtMod mod(t.mod);
       uint64_t acc[64];
 #pragma unroll
       for (int q = 0; q < 64; ++q) acc[q] = 0ull;
@@ -501,25 +532,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive_pair(acc_empty + 8u * (uint32_t)b);
           }
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            uint64_t& a = acc[8 * h + q];
-            const uint64_t s = add2(pack2(v[2 * q], v[2 * q + 1]), a);
-            const uint64_t k = add2(fma2(s, inv, magic), nmagic);
-            a = fma2(k, np, s);
-          }
+          mod.add(v, acc + 8 * h);
         }
       }
       if (failed) break;
-      // a warp's lanes are 32 consecutive rows; the low half of x + kMagic is x
-      uint16_t* out = g.R + ((int64_t)t.mod * g.Np + t.n0 + col0) * g.Mp + t.m0 + row;
-#pragma unroll
-      for (int q = 0; q < 64; ++q) {
-        float a0, a1;
-        unpack2(acc[q], a0, a1);
-        out[(int64_t)(2 * q) * g.Mp] = (uint16_t)__float_as_uint(a0 + (kMagic + kBias));
-        out[(int64_t)(2 * q + 1) * g.Mp] = (uint16_t)__float_as_uint(a1 + (kMagic + kBias));
-      }
+      // a warp's lanes are 32 consecutive rows
+      crt_store(g.R + ((int64_t)t.mod * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp, acc);
     }
     if (failed && lane == 0) atomicExch(&s_abort, 1);
   }
@@ -556,6 +574,183 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
+                 : "memory");
+  }
+}
+
+// ---- the 14 products, small shapes -------------------------------------------
+//
+// The same with one 128 x 128 tile modulo one p_i per CTA (twice the loads of a pair's
+// tile per product): 98 KB of shared memory, half of tensor memory and at most 102 registers a thread, so that two CTAs share an SM,
+// or one runs beside a task-graph leaf of another leg, where a pair finds no place
+// until the leaves end.
+constexpr int ST = 128;
+constexpr int kSmallStages = 3;
+constexpr int kSmallStage = 2 * kHalfTile;
+constexpr int kSmallSmem = kSmallStages * kSmallStage + 1024 + 256;
+constexpr uint32_t kSmallIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
+                                 ((uint32_t)(ST >> 3) << 17) | ((uint32_t)(ST >> 4) << 24);
+
+__device__ __forceinline__ void small_mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+      "l"(a), "l"(b), "r"(kSmallIdesc), "r"(acc)
+      : "memory");
+}
+
+__global__ void __launch_bounds__(kCrtThreads, 2)
+    crt_gemm_small_kernel(const __grid_constant__ CUtensorMap mA,
+                          const __grid_constant__ CUtensorMap mB, CrtArgs g) {
+  const CrtUnit t = crt_unit<ST>(g, blockIdx.x);
+  const int slabs = t.ks1 - t.ks0, chunks = (slabs + kChunkSlabs - 1) / kChunkSlabs;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSmallStages * kSmallStage);
+  const int kLoaded = 0, kEmpty = kSmallStages, kAccFull = 2 * kSmallStages,
+            kAccEmpty = kAccFull + 2, kFinal = kAccFull + 4;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kAccFull + 5);
+  __shared__ int s_abort, s_issued, s_waited;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSmallStages; ++s) {
+      mbar_init(smem_u32(&bars[kLoaded + s]), 1);
+      mbar_init(smem_u32(&bars[kEmpty + s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&bars[kAccFull + b]), 1);
+      mbar_init(smem_u32(&bars[kAccEmpty + b]), kDrainWarps);
+    }
+    mbar_init(smem_u32(&bars[kFinal]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_abort = 0;
+    s_issued = 0;
+    s_waited = 0;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(2 * ST)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == kDrainWarps) {
+    if (lane == 0) {   // ---- TMA producer
+      for (int r = 0; r < slabs; ++r) {
+        const int s = r % kSmallStages;
+        if (r >= kSmallStages && !mbar_wait(smem_u32(&bars[kEmpty + s]),
+                                            (uint32_t)((r / kSmallStages - 1) & 1),
+                                            kCrtWaitLimit)) {
+          atomicExch(&s_abort, 1);
+          break;
+        }
+        if (*(volatile int*)&s_abort) break;
+        const uint32_t full = smem_u32(&bars[kLoaded + s]);
+        mbar_expect_tx(full, (uint32_t)kSmallStage);
+        uint8_t* st = smem + s * kSmallStage;
+        const int ks = t.mod * g.nk + t.ks0 + r;
+        tma_load_2d(smem_u32(st), &mA, full, 0, ks * g.Ap + t.m0);
+        tma_load_2d(smem_u32(st + kHalfTile), &mB, full, 0, ks * g.Bp + t.n0);
+        *(volatile int*)&s_issued = r + 1;
+      }
+    }
+    __syncwarp();
+  } else if (warp == kDrainWarps + 1) {
+    if (lane == 0) {   // ---- MMA issuer
+      const uint64_t dbase = sdesc128(smem_u32(smem));
+      bool stop = false;
+      int r = 0;
+      for (int e = 0; e < chunks && !stop; ++e) {
+        const int b = e & 1;
+        if (e >= 2 && !mbar_wait(smem_u32(&bars[kAccEmpty + b]), (uint32_t)((e / 2 - 1) & 1),
+                                 kCrtWaitLimit)) {
+          stop = true;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int re = min(slabs, (e + 1) * kChunkSlabs);
+        for (; r < re; ++r) {
+          const int s = r % kSmallStages;
+          if (!mbar_wait(smem_u32(&bars[kLoaded + s]), (uint32_t)((r / kSmallStages) & 1),
+                         kCrtWaitLimit)) {
+            stop = true;
+            break;
+          }
+          *(volatile int*)&s_waited = r + 1;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t da = dbase + (uint64_t)((s * kSmallStage) >> 4);
+#pragma unroll
+          for (int kk = 0; kk < CK / 16; ++kk)
+            small_mma(tmem + (uint32_t)(b * ST), da + 2 * kk, da + (kHalfTile >> 4) + 2 * kk,
+                      r > e * kChunkSlabs || kk > 0);
+          mma_commit(smem_u32(&bars[kEmpty + s]));
+        }
+        if (!stop) mma_commit(smem_u32(&bars[kAccFull + b]));
+      }
+      if (stop) {
+        atomicExch(&s_abort, 1);
+        // wait (bounded) for the MMAs this thread issued before leaving
+        mma_commit(smem_u32(&bars[kFinal]));
+        mbar_wait(smem_u32(&bars[kFinal]), 0, kCrtWaitLimit);
+      }
+    }
+    __syncwarp();
+  } else {
+    // ---- warps 0-7: thread = output row (TMEM lane) x 64 columns
+    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+    const int row = (warp & 3) * 32 + lane, col0 = (warp >> 2) * 64;
+    const CrtMod mod(t.mod);
+    bool failed = false;
+    uint64_t acc[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] = 0ull;
+    for (int e = 0; e < chunks; ++e) {
+      const int b = e & 1;
+      bool ok = mbar_wait(smem_u32(&bars[kAccFull + b]), (uint32_t)((e / 2) & 1), kCrtWaitLimit);
+      ok = ok && !*(volatile int*)&s_abort;
+      if (!__all_sync(0xffffffffu, ok)) {
+        failed = true;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        float v[16];
+        tmem_ld16(tmem + lane_off + (uint32_t)(b * ST + col0 + 16 * h), v);
+        if (h == 3) {
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
+                             smem_u32(&bars[kAccEmpty + b]))
+                         : "memory");
+        }
+        mod.add(v, acc + 8 * h);
+      }
+    }
+    if (!failed)
+      crt_store(g.R + ((int64_t)t.mod * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp, acc);
+    else if (lane == 0)
+      atomicExch(&s_abort, 1);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && s_abort) {
+    // loads issued but not seen complete: wait (bounded) for them to land
+    for (int r = s_waited; r < s_issued; ++r)
+      mbar_wait(smem_u32(&bars[kLoaded + r % kSmallStages]), (uint32_t)((r / kSmallStages) & 1),
+                kCrtWaitLimit);
+    if (g.status) atomicExch(g.status, (int)BTA_ERR_TIMEOUT);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * ST)
                  : "memory");
   }
 }
@@ -703,6 +898,7 @@ struct SplitOp {
   const double* X;
   int ldx, trans, tri, rows, rowsP;
   int* ex;
+  int* pm;   // [eblocks][rowsP] partial maxima of the exponents
   __nv_bfloat16* Y;
   int rc, kc;
   SplitPart P[3];
@@ -729,22 +925,27 @@ struct SplitArgs {
   SplitOp op[2];   // blockIdx.z selects the operand
   int K, Kp;
   int bits;   // of the integers F (see the file's head)
+  int eblocks;   // partial maxima per row (0: ex holds the exponents)
 };
 
-// ex[r] = max over k of the biased exponent field of op(X)[r][k] (ex zeroed
-// beforehand).  Block 256 threads over 32 rows x 64 columns of op(X), read
-// in the memory order of X, 8 independent loads per thread.
-__global__ void ozaki_exp_kernel(SplitArgs a) {
+// The row exponents: the biased exponent field's maximum over the 64 columns of block kb
+// of op(X)[r][k].  Up to kPartialK columns it goes to pm[kb][r], of which residue_kernel
+// takes the maximum (nothing to clear: two launches less on a short product's path);
+// above, to ex[r] by an atomic maximum (ex zeroed beforehand).  Block 256 threads over 32
+// rows x 64 columns, read in the memory order of X, 8 independent loads per thread.
+constexpr int kExpCols = 64;
+constexpr int kPartialK = 1024;
+__global__ void __launch_bounds__(256) ozaki_exp_kernel(SplitArgs a) {
   const SplitOp o = blockIdx.z == 0 ? a.op[0] : a.op[1];
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
+  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * kExpCols;
   if (r0 >= o.rows) return;
   __shared__ int smax[32];
   const int t = threadIdx.x;
   if (t < 32) smax[t] = 0;
   __syncthreads();
-  int e = 0;
   if (!o.trans) {
     const int rr = t & 31, r = r0 + rr;   // consecutive threads: consecutive rows
+    int e = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = k0 + (t >> 5) + 8 * i;
@@ -769,9 +970,10 @@ __global__ void ozaki_exp_kernel(SplitArgs a) {
     }
   }
   __syncthreads();
-  if (t < 32 && r0 + t < o.rows && smax[t] > 0) atomicMax(&o.ex[r0 + t], smax[t]);
+  if (t >= 32) return;
+  if (a.eblocks) o.pm[(int64_t)blockIdx.x * o.rowsP + r0 + t] = smax[t];
+  else if (r0 + t < o.rows && smax[t] > 0) atomicMax(&o.ex[r0 + t], smax[t]);
 }
-
 
 // F = v 2^(1022 + bits - er) rounded to an integer (see the file's head), as
 // four signed 14-bit digits F = d3 2^42 + d2 2^28 + d1 2^14 + d0.
@@ -822,8 +1024,11 @@ __device__ __forceinline__ void residue_planes(const uint64_t (&d)[4][4], __nv_b
   }
 }
 
-// Y[i][r][k] (i < kNumMod, r < rowsP, k < Kp; K contiguous) = residue of
-// op(X)[r][k] modulo p_i in BF16; zero in the padding.  Block 256 threads over
+// Y[i][k / 64][r][k % 64] (i < kNumMod, r < rowsP, k < Kp) = residue of op(X)[r][k] modulo
+// p_i in BF16; zero in the padding.  A 64-wide K slab of a plane is contiguous, so that
+// this block writes 4 KB in a row to each plane, and a TMA load of the products reads 16
+// KB (not 128-byte pieces a row apart; 4800^3 call
+// 3.05 -> 2.95 ms).  Block 256 threads over
 // 32 rows x 64 columns, staged through a swizzled shared tile: column c of
 // row q sits at c ^ ((q ^ (c >> 3)) & 15), which keeps both the transposing
 // writes (16 rows, one column) and the digit reads (2 rows x 8 column groups)
@@ -835,7 +1040,15 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
   const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
   if (r0 >= o.rowsP) return;
   __shared__ double tile[32][64];   // tile[r - r0][split_swz(r - r0, k - k0)]
+  __shared__ int s_er[8][32];
   const int t = threadIdx.x;
+  if (a.eblocks) {   // the rows' exponents: warp w takes every eighth partial maximum
+    const int r = r0 + (t & 31);
+    int e = 0;
+    if (r < o.rows)
+      for (int b = t >> 5; b < a.eblocks; b += 8) e = max(e, o.pm[(int64_t)b * o.rowsP + r]);
+    s_er[t >> 5][t & 31] = e;
+  }
   if (!o.trans) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -854,12 +1067,19 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
     }
   }
   __syncthreads();
-  const size_t plane = (size_t)o.rowsP * a.Kp;
+  const size_t plane = (size_t)o.rowsP * a.Kp;   // of one modulus
   // thread: row q = t >> 3 and columns 8 g .. 8 g + 7, g = t & 7, so that a
   // warp writes 4 rows x 128 contiguous bytes of each plane, one 16-byte
   // store per thread and plane
-  const int q = t >> 3, g = t & 7, r = r0 + q, k = k0 + 8 * g;
-  const int er = r < o.rows ? o.ex[r] : 0;
+  const int q = t >> 3, g = t & 7, r = r0 + q;
+  int er = 0;
+  if (a.eblocks) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) er = max(er, s_er[w][q]);
+    if (blockIdx.x == 0 && g == 0 && r < o.rows) o.ex[r] = er;
+  } else if (r < o.rows) {
+    er = o.ex[r];
+  }
   uint64_t d[4][4];   // [digit][pair of columns]
 #pragma unroll
   for (int e = 0; e < 8; e += 2) {
@@ -869,14 +1089,14 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) d[j][e / 2] = pack2(x[j], y[j]);
   }
-  residue_planes<0>(d, o.Y + (size_t)r * a.Kp + k, plane);
+  residue_planes<0>(d, o.Y + ((size_t)blockIdx.x * o.rowsP + r) * 64 + 8 * g, plane);
 }
 
-// 2D map over Y viewed as (kNumMod * rowsP) x Kp BF16, box 64 (K) x 128 rows.
+// 2D map over Y viewed as rowsAll = kNumMod * slabs * rowsP rows of 64 BF16, box 128 rows.
 bta_status make_map_bf16(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map,
-                         const __nv_bfloat16* base, int rowsAll, int Kp) {
-  cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)rowsAll};
-  cuuint64_t strides[1] = {(cuuint64_t)Kp * 2};
+                         const __nv_bfloat16* base, int rowsAll) {
+  cuuint64_t dims[2] = {(cuuint64_t)CK, (cuuint64_t)rowsAll};
+  cuuint64_t strides[1] = {(cuuint64_t)CK * 2};
   cuuint32_t box[2] = {(cuuint32_t)CK, (cuuint32_t)CH};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(base),
@@ -912,19 +1132,32 @@ int pair_slots() {
   return n;
 }
 
+// Tile size of a product: pairs of CTAs on 256 x 256 tiles, or, while all units of 128 x
+// 128 tiles fit the GPU about four times over, single CTAs on those.  There a product is
+// bound by latency and by finding free SMs beside the leaves of other legs, above by
+// operand loads, which the larger tile halves.  Product kernel alone, pairs / single CTAs:
+// 192^3 12.8 / 8.8 us, 512^3 15.1 / 11.9, 1024^3 35.9 / 35.4.
+int crt_tile(int M, int N) {
+  const int64_t units = (int64_t)cdiv(M, ST) * cdiv(N, ST) * kNumMod;
+  return units <= 8 * sm_count() ? ST : CT;
+}
+
 struct OzLayout {
-  int Mp, Np, Kp;
-  size_t a_off, b_off, ea_off, eb_off, r_off, total;
-  OzLayout(int M, int N, int K) {
-    Mp = cdiv(M, CT) * CT;
-    Np = cdiv(N, CT) * CT;
+  int Mp, Np, Kp, eblocks;
+  size_t a_off, b_off, ea_off, eb_off, pa_off, pb_off, r_off, total;
+  OzLayout(int M, int N, int K, int tile) {
+    Mp = cdiv(M, tile) * tile;
+    Np = cdiv(N, tile) * tile;
     Kp = cdiv(K, CK) * CK;
+    eblocks = K <= kPartialK ? cdiv(K, kExpCols) : 0;
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     a_off = 0;
     b_off = up((size_t)kNumMod * Mp * Kp * 2);
     ea_off = b_off + up((size_t)kNumMod * Np * Kp * 2);
     eb_off = ea_off + up((size_t)Mp * 4);
-    r_off = eb_off + up((size_t)Np * 4);
+    pa_off = eb_off + up((size_t)Np * 4);   // (one memset clears both ex)
+    pb_off = pa_off + up((size_t)eblocks * Mp * 4);
+    r_off = pb_off + up((size_t)eblocks * Np * 4);
     total = r_off + up((size_t)kNumMod * Mp * Np * 2) + 256;
   }
 };
@@ -936,7 +1169,8 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
   BTA_TRY(tensor_map_encoder(&enc));
   const int M = g.M, N = g.N, K = g.K;
-  const OzLayout L(M, N, K);
+  const int tile = crt_tile(M, N);
+  const OzLayout L(M, N, K, tile);
   __nv_bfloat16* YA = reinterpret_cast<__nv_bfloat16*>(ws + L.a_off);
   __nv_bfloat16* YB = reinterpret_cast<__nv_bfloat16*>(ws + L.b_off);
   int* exA = reinterpret_cast<int*>(ws + L.ea_off);
@@ -954,58 +1188,68 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   sa.K = K;
   sa.Kp = L.Kp;
   sa.bits = K <= kMaxK56 ? 56 : 55;
+  sa.eblocks = L.eblocks;
   auto cut = [](int c) { return c > 0 ? c : INT_MAX; };
-  sa.op[0] = {g.A, g.lda, g.transA, g.triA, M, L.Mp, exA, YA, cut(g.a_rows), cut(g.a_k),
+  sa.op[0] = {g.A, g.lda, g.transA, g.triA, M, L.Mp, exA,
+              reinterpret_cast<int*>(ws + L.pa_off), YA, cut(g.a_rows), cut(g.a_k),
               {{g.A12.X, g.A12.ld, g.A12.trans},
                {g.A21.X, g.A21.ld, g.A21.trans},
                {g.A22.X, g.A22.ld, g.A22.trans}}};
   // the B side holds op(B)^T: its row cut is op(B)'s column cut and each
   // part is the transpose of the matching block of op(B)
-  sa.op[1] = {g.B, g.ldb, !g.transB, trib, N, L.Np, exB, YB, cut(g.b_cols), cut(g.b_k),
+  sa.op[1] = {g.B, g.ldb, !g.transB, trib, N, L.Np, exB,
+              reinterpret_cast<int*>(ws + L.pb_off), YB, cut(g.b_cols), cut(g.b_k),
               {{g.B21.X, g.B21.ld, !g.B21.trans},
                {g.B12.X, g.B12.ld, !g.B12.trans},
                {g.B22.X, g.B22.ld, !g.B22.trans}}};
   const int nops = same ? 1 : 2;
-  BTA_CUDA_TRY(cudaMemsetAsync(exA, 0, (size_t)L.Mp * 4, s));
-  if (!same) BTA_CUDA_TRY(cudaMemsetAsync(exB, 0, (size_t)L.Np * 4, s));
-  ozaki_exp_kernel<<<dim3(cdiv(K, 64), cdiv(std::max(M, N), 32), nops), 256, 0, s>>>(sa);
+  if (!L.eblocks) BTA_CUDA_TRY(cudaMemsetAsync(exA, 0, L.pa_off - L.ea_off, s));
+  ozaki_exp_kernel<<<dim3(cdiv(K, kExpCols), cdiv(std::max(M, N), 32), nops), 256, 0, s>>>(sa);
   BTA_LAUNCHED();
   residue_kernel<<<dim3(L.Kp / 64, std::max(L.Mp, L.Np) / 32, nops), 256, 0, s>>>(sa);
   BTA_LAUNCHED();
   CUtensorMap mA, mB;
   CrtArgs q{};
   q.Mp = L.Mp; q.Np = L.Np; q.Ap = L.Mp; q.Bp = same ? L.Mp : L.Np;
-  BTA_TRY(make_map_bf16(enc, &mA, YA, kNumMod * q.Ap, L.Kp));
-  BTA_TRY(make_map_bf16(enc, &mB, same ? YA : YB, kNumMod * q.Bp, L.Kp));
   q.nk = L.Kp / CK;
-  q.mt = L.Mp / CT;
-  q.nt = L.Np / CT;
+  BTA_TRY(make_map_bf16(enc, &mA, YA, kNumMod * q.nk * q.Ap));
+  BTA_TRY(make_map_bf16(enc, &mB, same ? YA : YB, kNumMod * q.nk * q.Bp));
+  q.mt = L.Mp / tile;
+  q.nt = L.Np / tile;
   // tile row i holds columns up to i; a C2 row (row >= c_rows) needs every column, so
   // it must lie in a row of tiles that holds them all
-  q.lower = g.out_lower && !(g.C2 && g.c_rows / CT < q.nt - 1);
+  q.lower = g.out_lower && !(g.C2 && g.c_rows / tile < q.nt - 1);
   const int h = std::min(q.mt, q.nt);
   q.tiles = q.lower ? h * (h + 1) / 2 + (q.mt - h) * q.nt : q.mt * q.nt;
   q.tri_a = g.triA;
   q.tri_b = g.triB;
-  q.slots = pair_slots();
-  // A wave of pairs spans a near-square patch of tiles.  A pair takes several units
-  // (the store of one overlaps the next) but at most ~300 slabs, ~75 us, so that the
-  // launches of a concurrent sweep find free SMs.
-  q.group = std::min(q.mt, std::max(1, (int)std::lround(std::sqrt((double)q.slots))));
-  const int units = q.tiles * kNumMod;
-  q.slots = std::min(q.slots, units);
-  q.per = std::max(1, std::min(cdiv(units, q.slots), 300 / q.nk));
   q.R = R;
   q.status = status;
+  const int units = q.tiles * kNumMod;
   static bool attr = false;
   if (!attr) {
     BTA_CUDA_TRY(cudaFuncSetAttribute(crt_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       kCrtSmem));
+    BTA_CUDA_TRY(cudaFuncSetAttribute(crt_gemm_small_kernel,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem));
     attr = true;
   }
-  if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
-  crt_gemm_kernel<<<2 * q.slots * cdiv(units, q.slots * q.per), kCrtThreads, kCrtSmem, s>>>(mA, mB,
-                                                                                         q);
+  if (tile == ST) {
+    q.group = q.mt;
+    if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
+    crt_gemm_small_kernel<<<units, kCrtThreads, kSmallSmem, s>>>(mA, mB, q);
+  } else {
+    // A wave of pairs spans a near-square patch of tiles.  A pair takes several units
+    // (the store of one overlaps the next) but at most ~300 slabs, ~75 us, so that the
+    // launches of a concurrent sweep find free SMs.
+    q.slots = pair_slots();
+    q.group = std::min(q.mt, std::max(1, (int)std::lround(std::sqrt((double)q.slots))));
+    q.slots = std::min(q.slots, units);
+    q.per = std::max(1, std::min(cdiv(units, q.slots), 300 / q.nk));
+    if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
+    crt_gemm_kernel<<<2 * q.slots * cdiv(units, q.slots * q.per), kCrtThreads, kCrtSmem, s>>>(
+        mA, mB, q);
+  }
   BTA_LAUNCHED();
   if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[1], s));
   ComposeArgs c;
@@ -1028,7 +1272,11 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
 
 // An upper bound over every product of at most M x N x K: a sweep sizes one
 // workspace for all of its products.
-size_t ozaki_ws_bytes(int M, int N, int K) { return OzLayout(M, N, K).total; }
+// (the larger tile's layout, and the partial maxima of a smaller K).
+size_t ozaki_ws_bytes(int M, int N, int K) {
+  const size_t full = OzLayout(M, N, K, CT).total;
+  return K > kPartialK ? std::max(full, OzLayout(M, N, kPartialK, CT).total) : full;
+}
 
 bool ozaki_supported(const Gemm& g) {
   if (!(g.batch == 1 && !g.Ab && g.A && g.B && g.C && g.K >= 1 && g.K <= kOzakiMaxK && g.M >= 1 &&

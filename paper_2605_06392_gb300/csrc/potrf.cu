@@ -229,6 +229,13 @@ bta_status level_product(const Gemm& g, const ProdCfg& c, cudaStream_t s) {
   return BTA_OK;
 }
 
+// Cap on the task graph's grid in the tensor-core modes: the other legs' products run on
+// the SMs the leaves leave free, and a CTA per 16 rows keeps the bulk tasks off the chain
+// (512 rows, 65 / 40 / 32 / 24 CTAs: 0.289 / 0.287 / 0.299 / 0.334 ms alone; the b = 1024
+// gradient of 50 blocks 57.2 / 54.2 / 53.9 / 55.3 ms).  The FP64 mode, whose bulk tasks
+// need the SMs, keeps them all.
+int leaf_ctas(int n) { return std::max(2, n / 16); }
+
 // The 2 x 2 recursion of rec() above, stopped at blocks of at most `leaf`
 // rows, which the task-graph kernel factors and inverts.  Those blocks hold
 // a fraction (leaf / n)^2 of the b^3 / 3 + b^3 / 3 flops of the factor and
@@ -245,13 +252,8 @@ bta_status rec_hybrid(const PB& b, int64_t aoff, int n, int ld, int64_t woff, in
       W[z] = b.W[z] + woff;
       sl[z] = b.slots[z] + soff;
     }
-    // In the tensor-core modes the other legs' products run on the SMs the leaves leave
-    // free: a CTA per 16 rows keeps the bulk tasks off the chain (512 rows, 65 / 40 / 32
-    // / 24 CTAs: 0.289 / 0.287 / 0.299 / 0.334 ms alone; the b = 1024 gradient of 50 blocks
-    // 57.2 / 54.2 / 53.9 / 55.3 ms).  The FP64 mode, whose bulk tasks need the SMs, keeps
-    // them all.
-    const int ctas = pc.precision ? std::max(2, n / 16) : 0;
-    return potrf_dag_batch(cnt, A, n, ld, W, sl, b.fail, b.code, s, ctas, pc.precision != 0);
+    return potrf_dag_batch(cnt, A, n, ld, W, sl, b.fail, b.code, s,
+                           pc.precision ? leaf_ctas(n) : 0, pc.precision != 0);
   }
   const int p = n / T;
   const int n1 = (p / 2) * T, n2 = n - n1;
@@ -352,6 +354,13 @@ bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
   if (top <= 0 || top > leaf) top = leaf;   // the top-level split threshold
   bool tc_ok = precision == 0 || (tcws && tcstat && n <= 5120);
   for (int z = 0; tc_ok && precision != 0 && z < count; ++z) tc_ok = tcws[z] && tcstat[z];
+  if (precision != 0 && n <= std::min(top, leaf) && n / T <= 160 && !g_potrf_recursive) {
+    // one task graph, its tile products emulated like those of a larger block's leaves
+    // (b = 192: 150 -> 123 us a block)
+    PriorityScope prio(highest_priority());
+    return potrf_dag_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s,
+                           leaf_ctas(n), 1);
+  }
   if (leaf < T || top < T || n <= top || n < 2 * T || !tc_ok || n / T > 160 || g_potrf_recursive)
     return potrf_inv_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s);
   PriorityScope prio(highest_priority());
