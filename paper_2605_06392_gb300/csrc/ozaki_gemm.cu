@@ -19,7 +19,7 @@
 // the tensor core's FP32 accumulator; each 256 of K the accumulator is
 // reduced modulo p_i in FP32 (exactly).  So one FP64 product costs 14 BF16
 // products.  Splitting into 8 base-128 digits, with 36 digit products, cost
-// 2.6 times that: 4800^3 whole call 5.38 ms before, 2.95 ms now, at no larger
+// 2.6 times that: 4800^3 whole call 5.38 ms before, 2.79 ms now, at no larger
 // error (no digit products are dropped).
 //
 // Kernels: exponents of the rows (ozaki_exp_kernel), residue planes (residue_kernel),
@@ -144,7 +144,8 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 // of 256 of K, and the drain of one chunk (and the store of a finished unit)
 // overlaps the MMAs of the next.  320 threads: warps 0-7 drain (two per TMEM lane
 // quarter, 128 columns each; the tile's residues stay in their registers across the
-// chunks), warp 8 loads (TMA, 128-byte swizzle, 64-wide K slabs, 6-stage ring),
+// chunks), warp 8 loads (TMA, 128-byte swizzle, 64-wide K slabs, a ring of three stages
+// of two slabs: with a barrier round per slab 6 % slower),
 // warp 9 of the leader CTA issues the MMAs.
 //
 // Across the pair: both CTAs' loads of a slab complete on the leader's `loaded`
@@ -160,8 +161,10 @@ constexpr int CT = 256;                   // tile rows and columns of a pair
 constexpr int CH = 128;                   // rows of A, and of B, per CTA
 constexpr int CK = 64;                    // bf16 per K slab: 128-byte rows
 constexpr int kHalfTile = CH * CK * 2;    // 16 KB
-constexpr int kStage = 2 * kHalfTile;
-constexpr int kStages = 6;
+constexpr int kSlab = 2 * kHalfTile;
+constexpr int kStageSlabs = 2;            // K slabs a stage: one barrier round for 128 of K
+constexpr int kStage = kStageSlabs * kSlab;
+constexpr int kStages = 3;
 constexpr int kChunkSlabs = 4;            // 256 of K: the exactness limit of a sum
 constexpr int kDrainWarps = 8;
 constexpr int kCrtThreads = (kDrainWarps + 2) * 32;
@@ -266,24 +269,26 @@ __device__ __forceinline__ void pair_mma(uint32_t tmem, uint64_t a, uint64_t b, 
       : "memory");
 }
 
-// 16 consecutive fp32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
+// Start the load of 8 consecutive fp32 columns of this thread's TMEM lane; tmem_wait
+// completes every load started.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15}, [%16];\n"
-      " tcgen05.wait::ld.sync.aligned;"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        "=r"(r[7])
       : "r"(taddr)
       : "memory");
-#pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[8]) {   // r: not read before
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7])
+               :
+               : "memory");
 }
 
-// One chunk's sums of 16 columns into the running residues: per column t = S + acc
-// (|t| < 2^24, exact), acc = t mod p, two columns per instruction.
+// A chunk's sums into the running residues: per column t = S + acc (|t| < 2^24, exact),
+// acc = t mod p, two columns per instruction.
 struct CrtMod {
   uint64_t np, inv, magic, nmagic;
   __device__ __forceinline__ explicit CrtMod(int m) {
@@ -293,15 +298,42 @@ struct CrtMod {
     magic = pack2(kMagic, kMagic);
     nmagic = pack2(-kMagic, -kMagic);
   }
-  __device__ __forceinline__ void add(const float (&v)[16], uint64_t* acc) const {
+  __device__ __forceinline__ void add(const uint32_t (&v)[8], uint64_t* acc) const {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const uint64_t s = add2(pack2(v[2 * q], v[2 * q + 1]), acc[q]);
+    for (int q = 0; q < 4; ++q) {
+      const uint64_t s = add2(
+          pack2(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1])), acc[q]);
       const uint64_t k = add2(fma2(s, inv, magic), nmagic);
       acc[q] = fma2(k, np, s);
     }
   }
 };
+// Drain of 2 N columns from taddr on; loaded() once all are in registers.  Ahead: the loads
+// of the next 8 columns run behind the arithmetic of the last 8 (with one CTA per SM the
+// drain's latency is on the product's critical path: an accumulator is refilled two chunks
+// later).  With two CTAs per SM the other one fills the wait, and loads of 16 columns
+// without overlap are 3 to 8 % faster.
+template <bool Ahead, int N, class Loaded>
+__device__ __forceinline__ void crt_drain(uint32_t taddr, const CrtMod& mod, uint64_t (&acc)[N],
+                                          Loaded loaded) {
+  uint32_t v[2][8];
+  if constexpr (Ahead) tmem_ld8(taddr, v[0]);
+#pragma unroll
+  for (int h = 0; h < N / 4; ++h) {
+    if constexpr (Ahead) {
+      tmem_wait(v[h & 1]);
+      if (h + 1 < N / 4) tmem_ld8(taddr + 8 * (h + 1), v[(h + 1) & 1]);
+      else loaded();
+    } else if ((h & 1) == 0) {
+      tmem_ld8(taddr + 8 * h, v[0]);
+      tmem_ld8(taddr + 8 * (h + 1), v[1]);
+      tmem_wait(v[0]);
+      tmem_wait(v[1]);
+      if (h + 2 == N / 4) loaded();
+    }
+    mod.add(v[h & 1], acc + 4 * h);
+  }
+}
 // Residues of 2 n consecutive columns of a row (columns `ld` apart) as 16-bit integers: the
 // low half of x + kMagic is x.
 template <int N>
@@ -433,7 +465,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
         const CrtUnit t = crt_unit<CT>(g, u0 + j * g.slots);
         const int ya = t.mod * g.nk * g.Ap + t.m0 + (int)rank * CH;
         const int yb = t.mod * g.nk * g.Bp + t.n0 + (int)rank * CH;
-        for (int kt = t.ks0; kt < t.ks1; ++kt, ++r) {
+        for (int kt = t.ks0; kt < t.ks1; kt += kStageSlabs, ++r) {
           const int s = r % kStages;
           if (r >= kStages && !mbar_wait(smem_u32(&bars[kEmpty + s]),
                                          (uint32_t)((r / kStages - 1) & 1), kCrtWaitLimit)) {
@@ -445,11 +477,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
             stop = true;
             break;
           }
-          if (rank == 0) mbar_expect_tx(smem_u32(&bars[kLoaded + s]), 2u * kStage);
+          const int ns = min(kStageSlabs, t.ks1 - kt);
+          if (rank == 0) mbar_expect_tx(smem_u32(&bars[kLoaded + s]), 2u * kSlab * ns);
           const uint32_t full = loaded0 + 8u * (uint32_t)s;
-          uint8_t* st = smem + s * kStage;
-          tma_load_pair(smem_u32(st), &mA, full, 0, ya + kt * g.Ap);
-          tma_load_pair(smem_u32(st + kHalfTile), &mB, full, 0, yb + kt * g.Bp);
+          for (int u = 0; u < ns; ++u) {
+            uint8_t* st = smem + s * kStage + u * kSlab;
+            tma_load_pair(smem_u32(st), &mA, full, 0, ya + (kt + u) * g.Ap);
+            tma_load_pair(smem_u32(st + kHalfTile), &mB, full, 0, yb + (kt + u) * g.Bp);
+          }
           *(volatile int*)&s_issued = r + 1;
         }
       }
@@ -473,7 +508,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const int ke = min(t.ks1, kc + kChunkSlabs);
-          for (int kt = kc; kt < ke; ++kt, ++r) {
+          for (int kt = kc; kt < ke; kt += kStageSlabs, ++r) {
             const int s = r % kStages;
             const uint32_t par = (uint32_t)((r / kStages) & 1);
             if (!mbar_wait(smem_u32(&bars[kLoaded + s]), par, kCrtWaitLimit)) {
@@ -482,11 +517,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
             }
             *(volatile int*)&s_waited = r + 1;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t da = dbase + (uint64_t)((s * kStage) >> 4);
+            for (int u = 0; u < min(kStageSlabs, ke - kt); ++u) {
+              const uint64_t da = dbase + (uint64_t)((s * kStage + u * kSlab) >> 4);
 #pragma unroll
-            for (int kk = 0; kk < CK / 16; ++kk)   // 16 bf16 = 32 bytes along K
-              pair_mma(tmem + (uint32_t)(b * CT), da + 2 * kk, da + (kHalfTile >> 4) + 2 * kk,
-                       kt > kc || kk > 0);
+              for (int kk = 0; kk < CK / 16; ++kk)   // 16 bf16 = 32 bytes along K
+                pair_mma(tmem + (uint32_t)(b * CT), da + 2 * kk, da + (kHalfTile >> 4) + 2 * kk,
+                         kt + u > kc || kk > 0);
+            }
             pair_commit_both(smem_u32(&bars[kEmpty + s]), 1u);   // both halves free
           }
           if (!stop) pair_commit_both(smem_u32(&bars[kAccFull + b]), 1u);   // sums ready
@@ -523,17 +560,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-        for (int h = 0; h < 8; ++h) {
-          float v[16];
-          tmem_ld16(tmem + lane_off + (uint32_t)(b * CT + col0 + 16 * h), v);
-          if (h == 7) {   // this warp's loads are done: the accumulator may be refilled
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive_pair(acc_empty + 8u * (uint32_t)b);
-          }
-          mod.add(v, acc + 8 * h);
-        }
+        crt_drain<true>(tmem + lane_off + (uint32_t)(b * CT + col0), mod, acc, [&]() {
+          // this warp's loads are done: the accumulator may be refilled
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive_pair(acc_empty + 8u * (uint32_t)b);
+        });
       }
       if (failed) break;
       // a warp's lanes are 32 consecutive rows
@@ -719,20 +751,14 @@ __global__ void __launch_bounds__(kCrtThreads, 2)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        float v[16];
-        tmem_ld16(tmem + lane_off + (uint32_t)(b * ST + col0 + 16 * h), v);
-        if (h == 3) {
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
-                             smem_u32(&bars[kAccEmpty + b]))
-                         : "memory");
-        }
-        mod.add(v, acc + 8 * h);
-      }
+      crt_drain<false>(tmem + lane_off + (uint32_t)(b * ST + col0), mod, acc, [&]() {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
+                           smem_u32(&bars[kAccEmpty + b]))
+                       : "memory");
+      });
     }
     if (!failed)
       crt_store(g.R + ((int64_t)t.mod * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp, acc);
