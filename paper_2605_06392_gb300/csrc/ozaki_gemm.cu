@@ -19,7 +19,7 @@
 // the tensor core's FP32 accumulator; each 256 of K the accumulator is
 // reduced modulo p_i in FP32 (exactly).  So one FP64 product costs 14 BF16
 // products.  Splitting into 8 base-128 digits, with 36 digit products, cost
-// 2.6 times that: 4800^3 whole call 5.38 ms before, 2.79 ms now, at no larger
+// 2.6 times that: 4800^3 whole call 5.38 ms before, 2.63 ms now, at no larger
 // error (no digit products are dropped).
 //
 // Kernels: exponents of the rows (ozaki_exp_kernel), residue planes (residue_kernel),
@@ -67,15 +67,29 @@ constexpr unsigned __int128 mod_product() {
   for (int j = 0; j < kNumMod; ++j) p *= (unsigned)kMod[j];
   return p;
 }
-// round(2^96 w_i / p_i): X / P = sum_i r_i w_i / p_i modulo 1 in 96-bit fractions
-constexpr unsigned __int128 crt_fraction(int i) {
-  return (((unsigned __int128)cofactor_inverse(i) << 96) + kMod[i] / 2) / (unsigned)kMod[i];
+// Recovery from pairs of residues: X / P = sum_i r_i w_i / p_i modulo 1, w_i = the inverse
+// of P / p_i modulo p_i of smallest magnitude.  Moduli p = p_2q and p' = p_2q+1 together
+// give (r a + r' b) / (p p') with a = w p', b = w' p below 2^17, so a 32-bit integer y and
+// one product of it by round(2^113 / (p p')) < 2^96 stand for two residues (half the wide
+// multiplications of one 96-bit fraction per residue).
+constexpr int kFracBits = 113;
+// the residues are stored + 256 (non-negative 16-bit integers below kStored)
+constexpr int kBias = 256, kStored = 513;
+constexpr int pair_coef(int i, int j) { return sym_mod(cofactor_inverse(i), kMod[i]) * kMod[j]; }
+constexpr int pair_shift(int i, int j) {   // makes y non-negative
+  const int a = pair_coef(i, j), b = pair_coef(j, i);
+  return (a < 0 ? -a * (kStored - 1) : 0) + (b < 0 ? -b * (kStored - 1) : 0);
 }
-// the residues are stored + 256 (non-negative 16-bit integers)
-constexpr int kBias = 256;
-constexpr unsigned __int128 crt_bias() {
+constexpr unsigned __int128 pair_fraction(int i, int j) {
+  const unsigned pp = (unsigned)(kMod[i] * kMod[j]);
+  return (((unsigned __int128)1 << kFracBits) + pp / 2) / pp;
+}
+// minus the sum when every residue is 0, modulo 2^128
+constexpr unsigned __int128 crt_offset() {
   unsigned __int128 s = 0;
-  for (int j = 0; j < kNumMod; ++j) s += kBias * crt_fraction(j);
+  for (int j = 0; j < kNumMod; j += 2)
+    s -= (unsigned __int128)(kBias * (pair_coef(j, j + 1) + pair_coef(j + 1, j)) +
+                             pair_shift(j, j + 1)) * pair_fraction(j, j + 1);
   return s;
 }
 constexpr unsigned long long kPTop = (unsigned long long)(mod_product() >> 62);   // P 2^-62
@@ -89,9 +103,19 @@ struct Modulus {
   static constexpr float c1 = (float)sym_mod(1ll << 14, kMod[I]);
   static constexpr float c2 = (float)sym_mod(1ll << 28, kMod[I]);
   static constexpr float c3 = (float)sym_mod(1ll << 42, kMod[I]);
-  static constexpr uint32_t f0 = (uint32_t)crt_fraction(I);
-  static constexpr uint32_t f1 = (uint32_t)(crt_fraction(I) >> 32);
-  static constexpr uint32_t f2 = (uint32_t)(crt_fraction(I) >> 64);
+};
+template <int I>   // moduli I and I + 1
+struct ModPair {
+  static constexpr int a = pair_coef(I, I + 1), b = pair_coef(I + 1, I);
+  static constexpr int c = pair_shift(I, I + 1);
+  static constexpr uint32_t f0 = (uint32_t)pair_fraction(I, I + 1);
+  static constexpr uint32_t f1 = (uint32_t)(pair_fraction(I, I + 1) >> 32);
+  static constexpr uint32_t f2 = (uint32_t)(pair_fraction(I, I + 1) >> 64);
+};
+struct CrtOffset {
+  static constexpr uint32_t l0 = (uint32_t)crt_offset(), l1 = (uint32_t)(crt_offset() >> 32);
+  static constexpr unsigned long long l2 =   // modulo 2^113 like the sum: 49 bits
+      (unsigned long long)(crt_offset() >> 64) & ((1ull << (kFracBits - 64)) - 1);
 };
 
 struct ModTable {
@@ -790,19 +814,18 @@ inline int alpha_mode(double a) { return a == 1.0 ? 0 : a == -1.0 ? 1 : 2; }
 inline int beta_mode(double b) { return b == 0.0 ? 0 : b == 1.0 ? 1 : 2; }
 
 __device__ __forceinline__ double scale_add(double out, int am, double alpha, int bm, double beta,
-                                            const double* cin) {
+                                            double cin) {
   if (am == 1) out = -out;
   else if (am == 2) out *= alpha;
-  if (bm == 1) out += *cin;
-  else if (bm == 2) out = fma(beta, *cin, out);
+  if (bm == 1) out += cin;
+  else if (bm == 2) out = fma(beta, cin, out);
   return out;
 }
 
-
 // C = alpha X 2^(exA + exB + scale) + beta Cin with X recovered from its residues:
-// T = X / P 2^96 = sum_i (r_i + kBias) f_i - bias modulo 2^96 (signed; its error of
-// 14 * 513 / 2 units is 2^41 of X, where the operands' last bit is worth 2^56),
-// then |X| = |T| P 2^-96 by one 64-bit product of leading parts and one rounding.
+// T = X / P 2^113 modulo 2^113 (signed; the fractions' rounding errors, 2^27 / 2 for each
+// pair's y about its centre at most, are 2^40 of X, where the operands' last bit is worth
+// 2^56), then |X| = |T| P 2^-113 by one 64-bit product of leading parts and one rounding.
 // All residues zero give exactly zero.
 struct ComposeArgs {
   int M, N, Mp, Np, out_lower, scale;
@@ -827,75 +850,97 @@ template <int I>
 __device__ __forceinline__ void crt_add(const uint32_t (&r)[kNumMod], int half,
                                         unsigned long long (&l)[3]) {
   if constexpr (I < kNumMod) {
-    const unsigned long long x = half ? r[I] >> 16 : r[I] & 0xFFFFu;
-    l[0] += x * Modulus<I>::f0;
-    l[1] += x * Modulus<I>::f1;
-    l[2] += x * Modulus<I>::f2;
-    crt_add<I + 1>(r, half, l);
+    using Q = ModPair<I>;
+    const int x0 = half ? r[I] >> 16 : r[I] & 0xFFFFu;
+    const int x1 = half ? r[I + 1] >> 16 : r[I + 1] & 0xFFFFu;
+    const unsigned long long y = (uint32_t)(x1 * Q::b + (x0 * Q::a + Q::c));   // < 2^27
+    l[0] += y * Q::f0;
+    l[1] += y * Q::f1;
+    l[2] += y * Q::f2;
+    crt_add<I + 2>(r, half, l);
   }
 }
 
 __device__ __forceinline__ double crt_value(const uint32_t (&r)[kNumMod], int half, int E) {
-  unsigned long long l[3] = {0, 0, 0};
+  unsigned long long l[3] = {CrtOffset::l0, CrtOffset::l1, CrtOffset::l2};
   crt_add<0>(r, half, l);
-  // 96 bits, lo (64) and hi (32)
-  const unsigned __int128 t = ((unsigned __int128)l[2] << 64) + ((unsigned __int128)l[1] << 32) +
-                              l[0] - crt_bias();
-  unsigned long long lo = (unsigned long long)t;
-  uint32_t hi = (uint32_t)(t >> 64);
-  const bool neg = hi >> 31;
-  if (neg) {
-    lo = 0ull - lo;
-    hi = ~hi + (lo == 0 ? 1u : 0u);
+  // words of T modulo 2^113 (signed), then of |T|
+  uint32_t w[4];
+  unsigned long long c = (l[0] >> 32) + (uint32_t)l[1];
+  w[0] = (uint32_t)l[0];
+  w[1] = (uint32_t)c;
+  c = (c >> 32) + (l[1] >> 32) + l[2];
+  w[2] = (uint32_t)c;
+  w[3] = (uint32_t)((int)((uint32_t)(c >> 32) << (128 - kFracBits)) >> (128 - kFracBits));
+  const bool neg = (int)w[3] < 0;
+  if (neg)
+    asm("sub.cc.u32 %0, 0, %0;\n subc.cc.u32 %1, 0, %1;\n subc.cc.u32 %2, 0, %2;\n"
+        " subc.u32 %3, 0, %3;"
+        : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]));
+  // leading 64 bits u of the 128: |T| = u 2^(64 - lz)
+  int lz = 0;
+  while (w[3] == 0) {
+    if (lz == 96) return 0.0;
+    w[3] = w[2];
+    w[2] = w[1];
+    w[1] = w[0];
+    w[0] = 0;
+    lz += 32;
   }
-  if ((lo | hi) == 0) return 0.0;
-  // leading 64 bits u of the 96, T = u 2^(32 - lz)
-  int lz;
-  unsigned long long u;
-  if (hi) {
-    lz = __clz((int)hi);
-    u = ((unsigned long long)hi << 32 | lo >> 32) << lz;
-    if (lz) u |= (lo & 0xFFFFFFFFull) >> (32 - lz);
-  } else {
-    const int z = __clzll((long long)lo);
-    lz = 32 + z;
-    u = lo << z;
+  const int z = __clz((int)w[3]);
+  lz += z - (128 - kFracBits);
+  const unsigned long long u = (unsigned long long)__funnelshift_l(w[2], w[3], z) << 32 |
+                               __funnelshift_l(w[1], w[2], z);
+  // v 2^(E + 62 - lz) rounded to nearest even; v >= 2^62 as u and kPTop are >= 2^63
+  unsigned long long v = __umul64hi(u, kPTop);
+  int be = 1023 + 63 + 62 + E - lz;
+  if (!(v >> 63)) {
+    v <<= 1;
+    --be;
   }
-  return oz::compose_mag(neg, __umul64hi(u, kPTop), E + 62 - lz);
+  if (be <= 0 || be >= 2046) return oz::compose_mag(neg, v, be - (1023 + 63));
+  // may carry to 2^53, which the sum turns into the next exponent
+  const unsigned long long m = (v >> 11) + ((v & 0x7FFull) + ((v >> 11) & 1ull) > 0x400ull);
+  return __longlong_as_double(
+      (long long)((neg ? 1ull << 63 : 0ull) + ((unsigned long long)(be - 1) << 52) + m));
 }
 
-constexpr int kComposeCols = 2;
-
-// Thread: rows m, m + 1 and kComposeCols consecutive columns.
+// Thread: rows m, m + 1 of column n, whose residues (and the entries of Cin) are loaded
+// before the first is used; the padding of R makes the load beyond row M harmless.
+// Column bases are the same for a block, so a load's address is one 32-bit offset.
+// Bound by instruction issue (4800^3: 200 us with 96-bit fractions per residue, 179 now).
 __global__ void __launch_bounds__(256) crt_compose_kernel(ComposeArgs g) {
-  const int m = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  if (m >= g.M) return;
+  const unsigned m = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (m >= (unsigned)g.M) return;
   const int64_t plane = (int64_t)g.Mp * g.Np;
-  for (int n0 = blockIdx.y * kComposeCols; n0 < g.N; n0 += gridDim.y * kComposeCols) {
-    if (g.out_lower && m + 1 < n0 && m + 1 < g.c_rows) break;
+  for (int n = blockIdx.y; n < g.N; n += gridDim.y) {
+    if (g.out_lower && (int)m + 1 < n && (int)m + 1 < g.c_rows) break;
+    uint32_t r[kNumMod];
+    const uint16_t* col = g.R + (int64_t)n * g.Mp;
 #pragma unroll
-    for (int c = 0; c < kComposeCols; ++c) {
-      const int n = n0 + c;
-      if (n >= g.N) break;
-      uint32_t r[kNumMod];
-      const uint16_t* p = g.R + m + (int64_t)n * g.Mp;
+    for (int i = 0; i < kNumMod; ++i)
+      r[i] = __ldg(reinterpret_cast<const unsigned int*>(col + i * plane + m));
+    double ci[2];
+    bool out[2], top[2];
 #pragma unroll
-      for (int i = 0; i < kNumMod; ++i)
-        r[i] = __ldg(reinterpret_cast<const unsigned int*>(p + i * plane));
-      const int eb = g.exB[n] + g.scale;
+    for (int h = 0; h < 2; ++h) {
+      const int mm = (int)m + h;
+      top[h] = mm < g.c_rows;
+      out[h] = mm < g.M && !(g.out_lower && top[h] && mm < n);
+      ci[h] = 0.0;
+      if (out[h] && g.bmode)
+        ci[h] = top[h] ? (g.Cin + (int64_t)n * g.ldcin)[mm]
+                       : (g.Cin2 + (int64_t)n * g.ldcin2)[mm - g.c_rows];
+    }
+    const int eb = g.exB[n] + g.scale;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int mm = m + h;
-        if (mm >= g.M) break;
-        const bool top = mm < g.c_rows;
-        if (g.out_lower && top && mm < n) continue;
-        const double v = crt_value(r, h, g.exA[mm] + eb);
-        const double* cin = top ? g.Cin + mm + (int64_t)n * g.ldcin
-                                : g.Cin2 + (mm - g.c_rows) + (int64_t)n * g.ldcin2;
-        double* co = top ? g.C + mm + (int64_t)n * g.ldc
-                         : g.C2 + (mm - g.c_rows) + (int64_t)n * g.ldc2;
-        *co = scale_add(v, g.amode, g.alpha, g.bmode, g.beta, cin);
-      }
+    for (int h = 0; h < 2; ++h) {
+      const int mm = (int)m + h;
+      if (!out[h]) continue;
+      const double v = scale_add(crt_value(r, h, g.exA[mm] + eb), g.amode, g.alpha, g.bmode,
+                                 g.beta, ci[h]);
+      if (top[h]) (g.C + (int64_t)n * g.ldc)[mm] = v;
+      else (g.C2 + (int64_t)n * g.ldc2)[mm - g.c_rows] = v;
     }
   }
 }
@@ -952,7 +997,40 @@ struct SplitArgs {
   int K, Kp;
   int bits;   // of the integers F (see the file's head)
   int eblocks;   // partial maxima per row (0: ex holds the exponents)
+  int tile;      // of the products
 };
+
+// The 32 x 64 block of op(X) at (r0, k0), 8 elements a thread of 256: thread t holds
+// (r, k) = (t & 31, (t >> 5) + 8 i) with rows contiguous in memory, else ((t >> 6) + 4 i,
+// t & 63).  A block outside the triangle is not read, and one that lies wholly inside it
+// and the leading block takes 8 loads without tests between them: with the tests of the
+// general form in between, each load waited for the one before it (4800^3: exponents 127 ->
+// 61 us, residues 350 -> 272).
+template <int TR>
+__device__ __forceinline__ void load_block(const SplitOp& o, int K, int r0, int k0,
+                                           double (&v)[8]) {
+  const int t = threadIdx.x;
+  const int rr = TR ? t >> 6 : t & 31, kk = TR ? t & 63 : t >> 5;
+  const bool zero = (o.tri == TRI_LOWER && k0 > r0 + 31) || (o.tri == TRI_UPPER && k0 + 63 < r0);
+  const bool full = r0 + 32 <= min(o.rows, o.rc) && k0 + 64 <= min(K, o.kc) &&
+                    !(o.tri == TRI_LOWER && k0 + 63 > r0) && !(o.tri == TRI_UPPER && k0 < r0 + 31);
+  if (zero) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = 0.0;
+  } else if (full) {
+    const double* x = TR ? o.X + (k0 + kk) + (int64_t)(r0 + rr) * o.ldx
+                         : o.X + (r0 + rr) + (int64_t)(k0 + kk) * o.ldx;
+    const int64_t step = (int64_t)(TR ? 4 : 8) * o.ldx;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = x[i * step];
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = r0 + rr + (TR ? 4 * i : 0), k = k0 + kk + (TR ? 0 : 8 * i);
+      v[i] = r < o.rows && k < K ? op_get<TR>(o, r, k) : 0.0;
+    }
+  }
+}
 
 // The row exponents: the biased exponent field's maximum over the 64 columns of block kb
 // of op(X)[r][k].  Up to kPartialK columns it goes to pm[kb][r], of which residue_kernel
@@ -969,30 +1047,20 @@ __global__ void __launch_bounds__(256) ozaki_exp_kernel(SplitArgs a) {
   const int t = threadIdx.x;
   if (t < 32) smax[t] = 0;
   __syncthreads();
+  double v[8];
+  auto field = [](double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); };
   if (!o.trans) {
-    const int rr = t & 31, r = r0 + rr;   // consecutive threads: consecutive rows
+    load_block<0>(o, a.K, r0, k0, v);
     int e = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int k = k0 + (t >> 5) + 8 * i;
-      if (r < o.rows && k < a.K) {
-        const double v = op_get<0>(o, r, k);
-        e = max(e, (int)((__double_as_longlong(v) >> 52) & 0x7FF));
-      }
-    }
-    atomicMax(&smax[rr], e);
+    for (int i = 0; i < 8; ++i) e = max(e, field(v[i]));
+    atomicMax(&smax[t & 31], e);
   } else {
-    const int kk = t & 63, k = k0 + kk;   // consecutive threads: consecutive k
+    load_block<1>(o, a.K, r0, k0, v);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int rr = (t >> 6) + 4 * i, r = r0 + rr;
-      int ei = 0;
-      if (r < o.rows && k < a.K) {
-        const double v = op_get<1>(o, r, k);
-        ei = (int)((__double_as_longlong(v) >> 52) & 0x7FF);
-      }
-      ei = (int)__reduce_max_sync(0xffffffffu, (unsigned)ei);   // a warp shares rr
-      if ((t & 31) == 0) atomicMax(&smax[rr], ei);
+    for (int i = 0; i < 8; ++i) {   // a warp shares its row
+      const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)field(v[i]));
+      if ((t & 31) == 0) atomicMax(&smax[(t >> 6) + 4 * i], e);
     }
   }
   __syncthreads();
@@ -1053,9 +1121,8 @@ __device__ __forceinline__ void residue_planes(const uint64_t (&d)[4][4], __nv_b
 // Y[i][k / 64][r][k % 64] (i < kNumMod, r < rowsP, k < Kp) = residue of op(X)[r][k] modulo
 // p_i in BF16; zero in the padding.  A 64-wide K slab of a plane is contiguous, so that
 // this block writes 4 KB in a row to each plane, and a TMA load of the products reads 16
-// KB (not 128-byte pieces a row apart; 4800^3 call
-// 3.05 -> 2.95 ms).  Block 256 threads over
-// 32 rows x 64 columns, staged through a swizzled shared tile: column c of
+// KB (not 128-byte pieces a row apart; 4800^3 call 3.05 ->
+// 2.95 ms).  Block 256 threads over 32 rows x 64 columns, staged through a swizzled shared tile: column c of
 // row q sits at c ^ ((q ^ (c >> 3)) & 15), which keeps both the transposing
 // writes (16 rows, one column) and the digit reads (2 rows x 8 column groups)
 // of every half-warp on 16 distinct 8-byte banks.
@@ -1065,6 +1132,12 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
   const SplitOp o = blockIdx.z == 0 ? a.op[0] : a.op[1];
   const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
   if (r0 >= o.rowsP) return;
+  // slabs outside the triangle of the products' tile are never read (crt_unit); the first
+  // block of a row also writes the exponents
+  const int t0 = r0 / a.tile * a.tile;
+  if (blockIdx.x > 0 && ((o.tri == TRI_LOWER && k0 >= t0 + a.tile) ||
+                         (o.tri == TRI_UPPER && k0 + 64 <= t0)))
+    return;
   __shared__ double tile[32][64];   // tile[r - r0][split_swz(r - r0, k - k0)]
   __shared__ int s_er[8][32];
   const int t = threadIdx.x;
@@ -1075,21 +1148,17 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
       for (int b = t >> 5; b < a.eblocks; b += 8) e = max(e, o.pm[(int64_t)b * o.rowsP + r]);
     s_er[t >> 5][t & 31] = e;
   }
+  double v[8];
   if (!o.trans) {
+    load_block<0>(o, a.K, r0, k0, v);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int idx = t + 256 * i, rr = idx & 31, kk = idx >> 5;
-      const int r = r0 + rr, k = k0 + kk;
-      tile[rr][split_swz(rr, kk)] =
-          (r < o.rows && k < a.K) ? op_get<0>(o, r, k) : 0.0;
-    }
+    for (int i = 0; i < 8; ++i) tile[t & 31][split_swz(t & 31, (t >> 5) + 8 * i)] = v[i];
   } else {
+    load_block<1>(o, a.K, r0, k0, v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int idx = t + 256 * i, kk = idx & 63, rr = idx >> 6;
-      const int r = r0 + rr, k = k0 + kk;
-      tile[rr][split_swz(rr, kk)] =
-          (r < o.rows && k < a.K) ? op_get<1>(o, r, k) : 0.0;
+      const int rr = (t >> 6) + 4 * i;
+      tile[rr][split_swz(rr, t & 63)] = v[i];
     }
   }
   __syncthreads();
@@ -1215,6 +1284,7 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   sa.Kp = L.Kp;
   sa.bits = K <= kMaxK56 ? 56 : 55;
   sa.eblocks = L.eblocks;
+  sa.tile = tile;
   auto cut = [](int c) { return c > 0 ? c : INT_MAX; };
   sa.op[0] = {g.A, g.lda, g.transA, g.triA, M, L.Mp, exA,
               reinterpret_cast<int*>(ws + L.pa_off), YA, cut(g.a_rows), cut(g.a_k),
@@ -1289,7 +1359,7 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   c.C2 = g.C2; c.ldc2 = g.ldc2;
   c.Cin2 = g.Cin2 ? g.Cin2 : g.C2; c.ldcin2 = g.Cin2 ? g.ldcin2 : g.ldc2;
   c.exA = exA; c.exB = same ? exA : exB; c.R = R;
-  crt_compose_kernel<<<dim3(cdiv(M, 512), std::min(cdiv(N, kComposeCols), 65535)), 256, 0, s>>>(c);
+  crt_compose_kernel<<<dim3(cdiv(M, 512), std::min(N, 65535)), 256, 0, s>>>(c);
   BTA_LAUNCHED();
   return BTA_OK;
 }
