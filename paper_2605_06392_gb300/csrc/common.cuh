@@ -173,6 +173,18 @@ struct Gemv {
 };
 bta_status gemv_f64(const Gemv& g, cudaStream_t s);
 
+// The arrow's share of one block, T[a x a] -= C C^T and, where x is given, y[a] += C x, for
+// C of a x K (leading dimension a) and a <= kGramRows: one launch.  Batched like Gemm.
+constexpr int kGramRows = 16;
+struct Gram {
+  int a = 0, K = 0, batch = 0;
+  const double* const* C = nullptr;
+  double* const* T = nullptr;
+  const double* const* x = nullptr;   // entries may be null (no y)
+  double* const* y = nullptr;
+};
+bta_status gram_f64(const Gram& g, cudaStream_t s);
+
 // Split-precision (3xTF32) tensor-core GEMM (tc_gemm.cu): same contract as
 // gemm_f64 for a single problem; ws holds tc_gemm_ws_bytes(M, N, K) bytes;
 // *status (device, may be null) receives BTA_ERR_TIMEOUT if a bounded wait

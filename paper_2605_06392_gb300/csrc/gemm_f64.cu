@@ -305,6 +305,88 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_t_kernel(GemvDev g) {
   }
 }
 
+// The arrow's share of a block (Gram).  A 16 x 64 tile of gemm_f64 took K serial steps of
+// mostly padding on one SM's FP64 pipe (a = 9, K = 192: 48 us), and split over K it needed
+// a second launch.  Here a cluster of 8 CTAs shares K: a warp reads columns of C, R rows
+// of it to a lane group (R = 8 or 16, so 4 or 2 columns at once), and lane m of a group
+// accumulates row m of C C^T against the other rows, shuffled in, so that little but real
+// products reach the FP64 pipe.  The 64 warps' sums meet in shared memory and through the
+// cluster's in a fixed order.  a = 9, K = 192: 9.1 us; a = 12, K = 4800: 255 us in three
+// launches with C x before, 45 now.
+struct GramDev {
+  int a, K;
+  const double* C[kMaxBatch];
+  double* T[kMaxBatch];
+  const double* x[kMaxBatch];
+  double* y[kMaxBatch];
+};
+template <int R>
+__global__ void __cluster_dims__(kGemvCluster, 1, 1) __launch_bounds__(kGemvThreads)
+    gram_kernel(GramDev g) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
+  constexpr int kCols = 32 / R, kWarps = kGemvThreads / 32;
+  const int z = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = (int)cl.block_rank(), a = g.a;
+  const int m = lane % R, h = lane / R;
+  const double* __restrict__ C = g.C[z];
+  const double* __restrict__ x = g.x[z];
+  double acc[R + 1];   // row m of C C^T, then of C x
+#pragma unroll
+  for (int n = 0; n <= R; ++n) acc[n] = 0.0;
+  constexpr int kStep = kCols * kGemvCluster * kWarps;
+  const int first = (rank * kWarps + warp) * kCols + h;
+  for (int k0 = first - h; k0 < g.K; k0 += 4 * kStep) {   // one trip count for the warp
+    double c[4], v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = k0 + h + q * kStep;
+      const bool in = k < g.K;
+      c[q] = in && m < a ? C[m + (int64_t)k * a] : 0.0;
+      v[q] = in && x ? x[k] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (k0 + q * kStep >= g.K) break;   // the same in all lanes
+#pragma unroll
+      for (int n = 0; n < R; ++n)
+        if (n < a) acc[n] = fma(c[q], __shfl_sync(0xffffffffu, c[q], h * R + n), acc[n]);
+      if (x) acc[R] = fma(c[q], v[q], acc[R]);
+    }
+  }
+  __shared__ double part[kWarps][R + 1][R], sum[R + 1][R];
+#pragma unroll
+  for (int n = 0; n <= R; ++n) {
+    double t = acc[n];
+#pragma unroll
+    for (int o = R; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (h == 0) part[warp][n][m] = t;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < (R + 1) * R; e += kGemvThreads) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) t += part[w][e / R][e % R];
+    sum[e / R][e % R] = t;
+  }
+  cl.sync();
+  if (rank == 0) {
+    for (int e = threadIdx.x; e < (R + 1) * R; e += kGemvThreads) {
+      const int n = e / R, i = e % R;
+      double p[kGemvCluster];
+#pragma unroll
+      for (int r = 0; r < kGemvCluster; ++r) p[r] = cl.map_shared_rank(&sum[0][0], r)[e];
+      double t = 0.0;
+#pragma unroll
+      for (int r = 0; r < kGemvCluster; ++r) t += p[r];
+      if (i >= a) continue;
+      if (n < a) g.T[z][i + n * a] -= t;
+      else if (n == R && x) g.y[z][i] += t;
+    }
+  }
+  cl.sync();   // the sums stay until they have been read
+}
+
 // ---- measured tile choice ---------------------------------------------------
 // A product's tile shape is timed once per (shape, layout, problems in the
 // launch) on scratch buffers and the fastest kept; untimed products use the
@@ -540,6 +622,28 @@ bta_status gemv_f64(const Gemv& g, cudaStream_t s) {
       gemv_n_kernel<<<dim3(kGemvCluster * cdiv(g.M, 32), cnt), kGemvThreads, 0, s>>>(d);
     else
       gemv_t_kernel<<<dim3(cdiv((int64_t)g.M * 32, kGemvThreads), cnt), kGemvThreads, 0, s>>>(d);
+    BTA_LAUNCHED();
+  }
+  return BTA_OK;
+}
+
+bta_status gram_f64(const Gram& g, cudaStream_t s) {
+  if (g.batch <= 0) return BTA_OK;
+  if (g.a < 1 || g.a > kGramRows || !g.C || !g.T) return BTA_ERR_ARG;
+  GramDev d;
+  d.a = g.a; d.K = std::max(g.K, 0);
+  for (int z0 = 0; z0 < g.batch; z0 += kMaxBatch) {
+    const int cnt = std::min(kMaxBatch, g.batch - z0);
+    for (int z = 0; z < cnt; ++z) {
+      d.C[z] = g.C[z0 + z];
+      d.T[z] = g.T[z0 + z];
+      d.x[z] = g.x ? g.x[z0 + z] : nullptr;
+      d.y[z] = g.y ? g.y[z0 + z] : nullptr;
+      if (d.x[z] && !d.y[z]) return BTA_ERR_ARG;
+    }
+    const dim3 grid(kGemvCluster, cnt);
+    if (g.a <= 8) gram_kernel<8><<<grid, kGemvThreads, 0, s>>>(d);
+    else gram_kernel<16><<<grid, kGemvThreads, 0, s>>>(d);
     BTA_LAUNCHED();
   }
   return BTA_OK;

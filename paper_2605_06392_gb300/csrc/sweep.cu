@@ -434,11 +434,24 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
     if (!it[z].ws.tc) return BTA_ERR_ARG;
     return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s);
   };
-  // T -= L_Ci L_Ci^T
+  // T -= L_Ci L_Ci^T and v_T += L_Ci z_i
   auto tip_update = [&](const std::vector<int>& grp, int i) -> bta_status {
     const int a = it[grp[0]].q.a;
     auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
     auto T = ptrs(grp, tip);
+    if (a <= kGramRows) {
+      auto x = ptrs(grp, [&](int z) { return it[z].vec ? vec_of(it[z], i) : nullptr; });
+      auto y = ptrs(grp, [&](int z) { return it[z].ws.vT; });
+      Gram g; g.a = a; g.K = ld; g.batch = (int)grp.size();
+      g.C = cp(Ci); g.T = T.data(); g.x = cp(x); g.y = y.data();
+      return gram_f64(g, s);
+    }
+    for (int z : grp) {
+      if (!it[z].vec) continue;
+      Gemv h; h.M = a; h.K = ld; h.A = Cb(z, i); h.lda = a;
+      h.x = vec_of(it[z], i); h.y = it[z].ws.vT; h.beta = 1.0;
+      BTA_TRY(gemv_f64(h, s));
+    }
     auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });
     Gemm h; h.M = a; h.N = a; h.K = ld; h.batch = (int)grp.size();
     h.Ab = cp(Ci); h.lda = a; h.Bb = cp(Ci); h.ldb = a; h.transB = 1;
@@ -527,7 +540,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       BTA_SWEEP_MARK(s, 2, i);
     }
     const bool with_b = emu && i < n - 1;   // L_Ci as extra rows of L_Bi's product
-    for (const auto& grp : G.arrow) {  // L_Ci = C_i L_Di^{-T};  T -= L_Ci L_Ci^T
+    for (const auto& grp : G.arrow) {  // L_Ci = C_i L_Di^{-T}
       if (with_b && fused(grp[0])) continue;
       const int a = it[grp[0]].q.a, c = (int)grp.size();
       auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
@@ -540,7 +553,6 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       g.sk_wsb = SK.data(); g.sk_cap = blk;
       BTA_TRY(gemm_f64(g, s));
       BTA_TRY(copy_block_batch(c, cp(W), a, Ci.data(), a, a, ld, 1.0, s));
-      BTA_TRY(tip_update(grp, i));
     }
     if (i < n - 1) {  // L_Bi = Q[i+1, i] L_Di^{-T}
       if (low) BTA_TRY(assemble_b_items(it, G.all, i, s));
@@ -567,24 +579,16 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         BTA_TRY(big_product(g, it, G.all, precision, s));
       }
       if (!low && !over) BTA_TRY(copy_block_batch(M, cp(W), ld, Bi.data(), ld, ld, ld, 1.0, s));
-      if (with_b)
-        for (const auto& grp : G.arrow)
-          if (fused(grp[0])) BTA_TRY(tip_update(grp, i));
     }
-    if (!G.vec.empty()) {  // z_i = L_Di^{-1} t;  v_T += L_Ci z_i
+    if (!G.vec.empty()) {  // z_i = L_Di^{-1} t
       auto zi = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
       auto gv = ptrs(G.vec, [&](int z) { return it[z].ws.gv; });
       auto Di = ptrs(G.vec, [&](int z) { return D(z, i); });
       Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.triA = TRI_LOWER; g.batch = (int)G.vec.size();
       g.Ab = cp(Di); g.xb = cp(gv); g.yb = zi.data();
       BTA_TRY(gemv_f64(g, s));
-      for (int z : G.vec) {
-        if (it[z].q.a == 0) continue;
-        Gemv h; h.M = it[z].q.a; h.K = ld; h.A = Cb(z, i); h.lda = it[z].q.a;
-        h.x = vec_of(it[z], i); h.y = it[z].ws.vT; h.beta = 1.0;
-        BTA_TRY(gemv_f64(h, s));
-      }
     }
+    for (const auto& grp : G.arrow) BTA_TRY(tip_update(grp, i));
     BTA_SWEEP_MARK(s, 3, i);
   }
   if (i1 < n) return BTA_OK;
