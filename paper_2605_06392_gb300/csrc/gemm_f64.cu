@@ -437,12 +437,15 @@ bta_status gemm_f64(const Gemm& g, cudaStream_t s) {
     return u * count;
   };
   auto pick = [&](int count) {
-    if (g.M <= 16) return 0;   // 16 x 64 tiles
-    auto cost = [&](int t, double pen) {
-      const int64_t u = units(t, t, count);
-      return (double)((u + kSMs - 1) / kSMs) * t * t * (1.0 + pen);
+    auto cost = [&](int bm, int bn, double pen) {
+      const int64_t u = units(bm, bn, count);
+      return (double)((u + kSMs - 1) / kSMs) * bm * bn * (1.0 + pen);
     };
-    const double c64 = cost(64, 0.0), c32 = cost(32, 0.0), c16 = cost(16, 0.05);
+    const double c16 = cost(16, 16, 0.05);
+    // one row of tiles: 16 x 64 (0) only where its tiles fill the SMs as well (16 x 64 x
+    // 64: 18.4 us as one 16 x 64 tile, 7.8 as four)
+    if (g.M <= 16) return c16 < cost(16, 64, 0.0) ? 16 : 0;
+    const double c64 = cost(64, 64, 0.0), c32 = cost(32, 32, 0.0);
     int bm = 64;
     double best = c64;
     if (c32 < best) { bm = 32; best = c32; }
@@ -522,7 +525,7 @@ bta_status gemm_f64(const Gemm& g, cudaStream_t s) {
     }
     return BTA_OK;
   };
-  if (bm != 0 && autotune_on()) {
+  if (g.M > 16 && autotune_on()) {
     int dev = 0;
     BTA_CUDA_TRY(cudaGetDevice(&dev));
     const TuneKey key{dev, g.M, g.N, K, g.lda, g.ldb, g.transA, g.transB, g.triA, g.triB,
