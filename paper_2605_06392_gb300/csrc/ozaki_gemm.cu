@@ -19,7 +19,7 @@
 // the tensor core's FP32 accumulator; each 256 of K the accumulator is
 // reduced modulo p_i in FP32 (exactly).  So one FP64 product costs 14 BF16
 // products.  Splitting into 8 base-128 digits, with 36 digit products, cost
-// 2.6 times that: 4800^3 whole call 5.38 ms before, 2.63 ms now, at no larger
+// 2.6 times that: 4800^3 whole call 5.38 ms before, 2.61 ms now, at no larger
 // error (no digit products are dropped).
 //
 // Kernels: exponents of the rows (ozaki_exp_kernel), residue planes (residue_kernel),
@@ -836,6 +836,14 @@ __global__ void __launch_bounds__(kCrtThreads, 2)
   }
 }
 
+// The kernels on operands and results run in blocks of 128 threads at no more than 48
+// registers, one of which fits an SM's registers beside a CTA of crt_gemm_kernel (and 9 KB
+// its shared memory), so that one leg's conversions proceed behind another's products; the
+// smaller blocks also fill an SM more evenly (4800^3: residues 272 us with 256 threads, 252
+// with 128; b = 4800, 8 blocks gradient 176.0 / 174.7 ms).
+constexpr int kElemThreads = 128;
+constexpr int kElemRows = 16;   // an operand's block: 16 rows x 64 columns
+
 // ---- recovery ----------------------------------------------------------------
 
 // alpha and beta as integer modes (decided on the host: comparisons of
@@ -940,7 +948,7 @@ __device__ __forceinline__ double crt_value(const uint32_t (&r)[kNumMod], int ha
 // before the first is used; the padding of R makes the load beyond row M harmless.
 // Column bases are the same for a block, so a load's address is one 32-bit offset.
 // Bound by instruction issue (4800^3: 200 us with 96-bit fractions per residue, 179 now).
-__global__ void __launch_bounds__(256) crt_compose_kernel(ComposeArgs g) {
+__global__ void __launch_bounds__(kElemThreads) crt_compose_kernel(ComposeArgs g) {
   const unsigned m = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   await_prior();
   if (m >= (unsigned)g.M) return;
@@ -1032,33 +1040,34 @@ struct SplitArgs {
   int tile;      // of the products
 };
 
-// The 32 x 64 block of op(X) at (r0, k0), 8 elements a thread of 256: thread t holds
-// (r, k) = (t & 31, (t >> 5) + 8 i) with rows contiguous in memory, else ((t >> 6) + 4 i,
-// t & 63).  A block outside the triangle is not read, and one that lies wholly inside it
-// and the leading block takes 8 loads without tests between them: with the tests of the
-// general form in between, each load waited for the one before it (4800^3: exponents 127 ->
-// 61 us, residues 350 -> 272).
+// The block of op(X) at (r0, k0), 8 elements a thread: thread t holds (r, k) = (t & 15,
+// (t >> 4) + 8 i) with rows contiguous in memory, else ((t >> 6) + 2 i, t & 63).  A block
+// outside the triangle is not read, and one that lies wholly inside it and the leading block
+// takes 8 loads without tests between them: with the tests of the general form in between,
+// each load waited for the one before it (4800^3: exponents 127 us, 61 without; residues
+// 350, 272).
 template <int TR>
 __device__ __forceinline__ void load_block(const SplitOp& o, int K, int r0, int k0,
                                            double (&v)[8]) {
   const int t = threadIdx.x;
-  const int rr = TR ? t >> 6 : t & 31, kk = TR ? t & 63 : t >> 5;
-  const bool zero = (o.tri == TRI_LOWER && k0 > r0 + 31) || (o.tri == TRI_UPPER && k0 + 63 < r0);
-  const bool full = r0 + 32 <= min(o.rows, o.rc) && k0 + 64 <= min(K, o.kc) &&
-                    !(o.tri == TRI_LOWER && k0 + 63 > r0) && !(o.tri == TRI_UPPER && k0 < r0 + 31);
+  const int rr = TR ? t >> 6 : t & 15, kk = TR ? t & 63 : t >> 4;
+  const int r1 = r0 + kElemRows - 1, k1 = k0 + CK - 1;   // last row and column
+  const bool zero = (o.tri == TRI_LOWER && k0 > r1) || (o.tri == TRI_UPPER && k1 < r0);
+  const bool full = r1 < min(o.rows, o.rc) && k1 < min(K, o.kc) &&
+                    !(o.tri == TRI_LOWER && k1 > r0) && !(o.tri == TRI_UPPER && k0 < r1);
   if (zero) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = 0.0;
   } else if (full) {
     const double* x = TR ? o.X + (k0 + kk) + (int64_t)(r0 + rr) * o.ldx
                          : o.X + (r0 + rr) + (int64_t)(k0 + kk) * o.ldx;
-    const int64_t step = (int64_t)(TR ? 4 : 8) * o.ldx;
+    const int64_t step = (int64_t)(TR ? 2 : 8) * o.ldx;
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = x[i * step];
   } else {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int r = r0 + rr + (TR ? 4 * i : 0), k = k0 + kk + (TR ? 0 : 8 * i);
+      const int r = r0 + rr + (TR ? 2 * i : 0), k = k0 + kk + (TR ? 0 : 8 * i);
       v[i] = r < o.rows && k < K ? op_get<TR>(o, r, k) : 0.0;
     }
   }
@@ -1067,18 +1076,16 @@ __device__ __forceinline__ void load_block(const SplitOp& o, int K, int r0, int 
 // The row exponents: the biased exponent field's maximum over the 64 columns of block kb
 // of op(X)[r][k].  Up to kPartialK columns it goes to pm[kb][r], of which residue_kernel
 // takes the maximum (nothing to clear: two launches less on a short product's path);
-// above, to ex[r] by an atomic maximum (ex zeroed beforehand).  Block 256 threads over 32
-// rows x 64 columns, read in the memory order of X, 8 independent loads per thread.
-constexpr int kExpCols = 64;
+// above, to ex[r] by an atomic maximum (ex zeroed beforehand).
 constexpr int kPartialK = 1024;
-__global__ void __launch_bounds__(256) ozaki_exp_kernel(SplitArgs a) {
+__global__ void __launch_bounds__(kElemThreads) ozaki_exp_kernel(SplitArgs a) {
   const SplitOp o = blockIdx.z == 0 ? a.op[0] : a.op[1];
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * kExpCols;
+  const int r0 = blockIdx.x * kElemRows, k0 = blockIdx.y * CK;
   launch_next();
   if (r0 >= o.rows) return;
-  __shared__ int smax[32];
+  __shared__ int smax[kElemRows];
   const int t = threadIdx.x;
-  if (t < 32) smax[t] = 0;
+  if (t < kElemRows) smax[t] = 0;
   __syncthreads();
   double v[8];
   auto field = [](double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); };
@@ -1087,18 +1094,19 @@ __global__ void __launch_bounds__(256) ozaki_exp_kernel(SplitArgs a) {
     int e = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) e = max(e, field(v[i]));
-    atomicMax(&smax[t & 31], e);
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
+    if ((t & 16) == 0) atomicMax(&smax[t & 15], e);
   } else {
     load_block<1>(o, a.K, r0, k0, v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {   // a warp shares its row
       const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)field(v[i]));
-      if ((t & 31) == 0) atomicMax(&smax[(t >> 6) + 4 * i], e);
+      if ((t & 31) == 0) atomicMax(&smax[(t >> 6) + 2 * i], e);
     }
   }
   __syncthreads();
-  if (t >= 32) return;
-  if (a.eblocks) o.pm[(int64_t)blockIdx.x * o.rowsP + r0 + t] = smax[t];
+  if (t >= kElemRows) return;
+  if (a.eblocks) o.pm[(int64_t)blockIdx.y * o.rowsP + r0 + t] = smax[t];
   else if (r0 + t < o.rows && smax[t] > 0) atomicMax(&o.ex[r0 + t], smax[t]);
 }
 
@@ -1152,49 +1160,49 @@ __device__ __forceinline__ void residue_planes(const uint64_t (&d)[4][4], __nv_b
 }
 
 // Y[i][k / 64][r][k % 64] (i < kNumMod, r < rowsP, k < Kp) = residue of op(X)[r][k] modulo
-// p_i in BF16; zero in the padding.  A 64-wide K slab of a plane is contiguous, so that
-// this block writes 4 KB in a row to each plane, and a TMA load of the products reads 16
-// KB (not 128-byte pieces a row apart; 4800^3 call 3.05 ->
-// 2.95 ms).  Block 256 threads over 32 rows x 64 columns, staged through a swizzled shared tile: column c of
-// row q sits at c ^ ((q ^ (c >> 3)) & 15), which keeps both the transposing
-// writes (16 rows, one column) and the digit reads (2 rows x 8 column groups)
-// of every half-warp on 16 distinct 8-byte banks.
+// p_i in BF16; zero in the padding, unwritten where no product reads it.  A 64-wide K slab
+// of a plane is contiguous, so that a block writes 2 KB in a row to each plane, and a TMA
+// load of the products reads 16 KB (not 128-byte pieces a row apart: 4800^3 call 2.95 ms,
+// 3.05 so).  The block is staged through a swizzled shared tile: column c of row q sits at
+// c ^ ((q ^ (c >> 3)) & 15), which keeps both the transposing writes (16 rows, one column)
+// and the digit reads (2 rows x 8 column groups) of every half-warp on 16 distinct 8-byte
+// banks.
 __device__ __forceinline__ int split_swz(int q, int c) { return c ^ ((q ^ (c >> 3)) & 15); }
 
-__global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
+__global__ void __launch_bounds__(kElemThreads) residue_kernel(SplitArgs a) {
   const SplitOp o = blockIdx.z == 0 ? a.op[0] : a.op[1];
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
+  const int r0 = blockIdx.x * kElemRows, k0 = blockIdx.y * CK;
   if (r0 >= o.rowsP) return;
   // slabs outside the triangle of the products' tile are never read (crt_unit); the first
   // block of a row also writes the exponents
   const int t0 = r0 / a.tile * a.tile;
-  if (blockIdx.x > 0 && ((o.tri == TRI_LOWER && k0 >= t0 + a.tile) ||
-                         (o.tri == TRI_UPPER && k0 + 64 <= t0)))
+  if (blockIdx.y > 0 && ((o.tri == TRI_LOWER && k0 >= t0 + a.tile) ||
+                         (o.tri == TRI_UPPER && k0 + CK <= t0)))
     return;
-  __shared__ double tile[32][64];   // tile[r - r0][split_swz(r - r0, k - k0)]
-  __shared__ int s_er[8][32];
+  __shared__ double tile[kElemRows][CK];   // tile[r - r0][split_swz(r - r0, k - k0)]
+  __shared__ int s_er[8][kElemRows];
   const int t = threadIdx.x;
   double v[8];
   if (!o.trans) {
     load_block<0>(o, a.K, r0, k0, v);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) tile[t & 31][split_swz(t & 31, (t >> 5) + 8 * i)] = v[i];
+    for (int i = 0; i < 8; ++i) tile[t & 15][split_swz(t & 15, (t >> 4) + 8 * i)] = v[i];
   } else {
     load_block<1>(o, a.K, r0, k0, v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int rr = (t >> 6) + 4 * i;
+      const int rr = (t >> 6) + 2 * i;
       tile[rr][split_swz(rr, t & 63)] = v[i];
     }
   }
   await_prior();
   launch_next();
-  if (a.eblocks) {   // the rows' exponents: warp w takes every eighth partial maximum
-    const int r = r0 + (t & 31);
+  if (a.eblocks) {   // the rows' exponents: each eighth of the threads takes every eighth one
+    const int r = r0 + (t & 15);
     int e = 0;
     if (r < o.rows)
-      for (int b = t >> 5; b < a.eblocks; b += 8) e = max(e, o.pm[(int64_t)b * o.rowsP + r]);
-    s_er[t >> 5][t & 31] = e;
+      for (int b = t >> 4; b < a.eblocks; b += 8) e = max(e, o.pm[(int64_t)b * o.rowsP + r]);
+    s_er[t >> 4][t & 15] = e;
   }
   __syncthreads();
   const size_t plane = (size_t)o.rowsP * a.Kp;   // of one modulus
@@ -1206,7 +1214,7 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
   if (a.eblocks) {
 #pragma unroll
     for (int w = 0; w < 8; ++w) er = max(er, s_er[w][q]);
-    if (blockIdx.x == 0 && g == 0 && r < o.rows) o.ex[r] = er;
+    if (blockIdx.y == 0 && g == 0 && r < o.rows) o.ex[r] = er;
   } else if (r < o.rows) {
     er = o.ex[r];
   }
@@ -1219,7 +1227,7 @@ __global__ void __launch_bounds__(256) residue_kernel(SplitArgs a) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) d[j][e / 2] = pack2(x[j], y[j]);
   }
-  residue_planes<0>(d, o.Y + ((size_t)blockIdx.x * o.rowsP + r) * 64 + 8 * g, plane);
+  residue_planes<0>(d, o.Y + ((size_t)blockIdx.y * o.rowsP + r) * 64 + 8 * g, plane);
 }
 
 // 2D map over Y viewed as rowsAll = kNumMod * slabs * rowsP rows of 64 BF16, box 128 rows.
@@ -1279,7 +1287,7 @@ struct OzLayout {
     Mp = cdiv(M, tile) * tile;
     Np = cdiv(N, tile) * tile;
     Kp = cdiv(K, CK) * CK;
-    eblocks = K <= kPartialK ? cdiv(K, kExpCols) : 0;
+    eblocks = K <= kPartialK ? cdiv(K, CK) : 0;
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     a_off = 0;
     b_off = up((size_t)kNumMod * Mp * Kp * 2);
@@ -1335,10 +1343,12 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
                {g.B22.X, g.B22.ld, !g.B22.trans}}};
   const int nops = same ? 1 : 2;
   if (!L.eblocks) BTA_CUDA_TRY(cudaMemsetAsync(exA, 0, L.pa_off - L.ea_off, s));
-  ozaki_exp_kernel<<<dim3(cdiv(K, kExpCols), cdiv(std::max(M, N), 32), nops), 256, 0, s>>>(sa);
+  ozaki_exp_kernel<<<dim3(cdiv(std::max(M, N), kElemRows), cdiv(K, CK), nops), kElemThreads, 0,
+                     s>>>(sa);
   BTA_LAUNCHED();
-  BTA_CUDA_TRY(launch_after(residue_kernel, dim3(L.Kp / 64, std::max(L.Mp, L.Np) / 32, nops),
-                            dim3(256), 0, s, sa));
+  BTA_CUDA_TRY(launch_after(residue_kernel,
+                            dim3(std::max(L.Mp, L.Np) / kElemRows, L.Kp / CK, nops),
+                            dim3(kElemThreads), 0, s, sa));
   BTA_LAUNCHED();
   CUtensorMap mA, mB;
   CrtArgs q{};
@@ -1396,8 +1406,8 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   c.C2 = g.C2; c.ldc2 = g.ldc2;
   c.Cin2 = g.Cin2 ? g.Cin2 : g.C2; c.ldcin2 = g.Cin2 ? g.ldcin2 : g.ldc2;
   c.exA = exA; c.exB = same ? exA : exB; c.R = R;
-  BTA_CUDA_TRY(launch_after(crt_compose_kernel, dim3(cdiv(M, 512), std::min(N, 65535)), dim3(256),
-                            0, s, c));
+  BTA_CUDA_TRY(launch_after(crt_compose_kernel, dim3(cdiv(M, 2 * kElemThreads), std::min(N, 65535)),
+                            dim3(kElemThreads), 0, s, c));
   BTA_LAUNCHED();
   return BTA_OK;
 }
