@@ -398,8 +398,11 @@ bta_status assemble_b_items(const SweepItem* it, const std::vector<int>& idx, in
 // Algorithm 1 on a set of matrices
 // ----------------------------------------------------------------------------
 bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int precision, int i0,
-                              int i1) {
+                              int i1, cudaStream_t sv, cudaEvent_t ev) {
   BTA_TRY(check_set(it, m));
+  if (!sv) sv = s;
+  for (int z = 0; sv != s && z < m; ++z)
+    if (!ev || !it[z].q.B || it[z].q.a > kGramRows) return BTA_ERR_ARG;
   const int n = it[0].blocks(), ld = it[0].q.ld;
   const bool rev = it[0].rev;
   if (i1 < 0) i1 = n;
@@ -444,7 +447,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       auto y = ptrs(grp, [&](int z) { return it[z].ws.vT; });
       Gram g; g.a = a; g.K = ld; g.batch = (int)grp.size();
       g.C = cp(Ci); g.T = T.data(); g.x = cp(x); g.y = y.data();
-      return gram_f64(g, s);
+      return gram_f64(g, sv);
     }
     for (int z : grp) {
       if (!it[z].vec) continue;
@@ -458,6 +461,24 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
     h.Cb = T.data(); h.ldc = a; h.Cinb = cp(T); h.ldcin = a; h.alpha = -1.0; h.beta = 1.0;
     h.sk_wsb = SK.data(); h.sk_cap = blk;
     return gemm_f64(h, s);
+  };
+  auto vector_step = [&](int i) -> bta_status {
+    if (G.vec.empty()) return BTA_OK;
+    // t = r_i - L_B,i-1 z_{i-1} into gv (r_0 itself for the first block; into r_i where
+    // the legs join)
+    const int c = (int)G.vec.size();
+    auto ri = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
+    auto gv = ptrs(G.vec, [&](int z) { return i == i1 ? vec_of(it[z], i) : it[z].ws.gv; });
+    if (i == 0) {
+      BTA_TRY(copy_block_batch(c, cp(ri), ld, gv.data(), ld, ld, 1, 1.0, sv));
+    } else {
+      auto Bp = ptrs(G.vec, [&](int z) { return LB(z, i - 1); });
+      auto rp = ptrs(G.vec, [&](int z) { return vec_of(it[z], i - 1); });
+      Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.alpha = -1.0; g.beta = 1.0; g.batch = c;
+      g.Ab = cp(Bp); g.xb = cp(rp); g.yb = gv.data(); g.yinb = cp(ri);
+      BTA_TRY(gemv_f64(g, sv));
+    }
+    return BTA_OK;
   };
   for (int i = i0; i <= i1 && i < n; ++i) {
     // the range's end: a reverse leg's last coupling updates the block the legs share
@@ -501,23 +522,8 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         BTA_TRY(gemm_f64(g, s));
       }
     }
-    if (!G.vec.empty()) {
-      // t = r_i - L_B,i-1 z_{i-1} into gv (r_0 itself for the first block; into r_i where
-      // the legs join)
-      const int c = (int)G.vec.size();
-      auto ri = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
-      auto gv = ptrs(G.vec, [&](int z) { return join ? vec_of(it[z], i) : it[z].ws.gv; });
-      if (i == 0) {
-        BTA_TRY(copy_block_batch(c, cp(ri), ld, gv.data(), ld, ld, 1, 1.0, s));
-      } else {
-        auto Bp = ptrs(G.vec, [&](int z) { return LB(z, i - 1); });
-        auto rp = ptrs(G.vec, [&](int z) { return vec_of(it[z], i - 1); });
-        Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.alpha = -1.0; g.beta = 1.0; g.batch = c;
-        g.Ab = cp(Bp); g.xb = cp(rp); g.yb = gv.data(); g.yinb = cp(ri);
-        BTA_TRY(gemv_f64(g, s));
-      }
-    }
-    if (join) return BTA_OK;
+    if (join) return vector_step(i);
+    if (sv == s) BTA_TRY(vector_step(i));
     {  // L_Di^{-1} in place, log-det slots
       auto Di = ptrs(G.all, [&](int z) { return D(z, i); });
       auto W = ptrs(G.all, [&](int z) { return it[z].ws.pot; });
@@ -580,18 +586,27 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       }
       if (!low && !over) BTA_TRY(copy_block_batch(M, cp(W), ld, Bi.data(), ld, ld, ld, 1.0, s));
     }
+    if (sv != s) {
+      BTA_CUDA_TRY(cudaEventRecord(ev, s));
+      BTA_CUDA_TRY(cudaStreamWaitEvent(sv, ev, 0));
+      BTA_TRY(vector_step(i));
+    }
     if (!G.vec.empty()) {  // z_i = L_Di^{-1} t
       auto zi = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });
       auto gv = ptrs(G.vec, [&](int z) { return it[z].ws.gv; });
       auto Di = ptrs(G.vec, [&](int z) { return D(z, i); });
       Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.triA = TRI_LOWER; g.batch = (int)G.vec.size();
       g.Ab = cp(Di); g.xb = cp(gv); g.yb = zi.data();
-      BTA_TRY(gemv_f64(g, s));
+      BTA_TRY(gemv_f64(g, sv));
     }
     for (const auto& grp : G.arrow) BTA_TRY(tip_update(grp, i));
     BTA_SWEEP_MARK(s, 3, i);
   }
   if (i1 < n) return BTA_OK;
+  if (sv != s) {
+    BTA_CUDA_TRY(cudaEventRecord(ev, sv));
+    BTA_CUDA_TRY(cudaStreamWaitEvent(s, ev, 0));
+  }
   for (int z = 0; z < m; ++z) {
     const int a = it[z].q.a;
     if (a == 0) continue;

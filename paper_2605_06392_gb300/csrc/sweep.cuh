@@ -83,8 +83,14 @@ struct SweepItem {
 // range: the forward leg's step of that block, the tip and the shared block's x and Z must
 // be ordered after it, and the reverse leg's solve and selected inversion (from
 // block len - 2) after theirs.
+//
+// sv (optional, not for low-memory sweeps nor a > kGramRows; ev an event of its own): a
+// block's vector part and tip share go to this stream, after the block's factor on s; they
+// read finished parts of the factor only.  s waits for it before the tip; a reverse leg's
+// last vector part, which updates the shared block's, stays on sv.
 bta_status factor_sweep_multi(const SweepItem* items, int m, cudaStream_t s, int precision = 0,
-                              int i0 = 0, int i1 = -1);
+                              int i0 = 0, int i1 = -1, cudaStream_t sv = nullptr,
+                              cudaEvent_t ev = nullptr);
 bta_status upper_solve_multi(const SweepItem* items, int m, cudaStream_t s, int i_hi = -1,
                              int i_lo = 0);
 bta_status selinv_sweep_multi(const SweepItem* items, int m, cudaStream_t s, int precision = 0,
