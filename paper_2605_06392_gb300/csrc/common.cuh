@@ -143,6 +143,9 @@ struct Gemm {
   double* C2 = nullptr; int ldc2 = 0;
   const double* Cin2 = nullptr; int ldcin2 = 0;
   int c_rows = 0;
+  // M of the product before this one on the same workspace and stream, if that one had the
+  // same op(B) (operand, parts, N and K, unchanged since): its planes are used again.
+  int b_kept = 0;
   bool blocked() const {
     return A12.X || A21.X || A22.X || B12.X || B21.X || B22.X || C2 || a_rows || a_k || b_k ||
            b_cols || c_rows;

@@ -919,6 +919,28 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         BTA_TRY(gemm_f64(g, s));
       }
     }
+    // Z_D = L_Di^{-T} L_Di^{-1} (lower part); emulated it follows F_B, whose planes of L_Di
+    // serve it
+    auto inverse_gram = [&]() -> bta_status {
+      Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
+      g.Ab = cp(Di); g.lda = ld; g.transA = 1; g.triA = TRI_UPPER;
+      g.Bb = cp(Di); g.ldb = ld; g.triB = TRI_LOWER;
+      g.Cb = ZD.data(); g.ldc = ld; g.out_lower = 1;
+      if (!emu || !hasB) return big_product(g, it, G.all, precision, s);
+      for (size_t q = 0; q < G.all.size(); ++q) {
+        const int z = G.all[q];
+        Gemm h = g;
+        h.batch = 1;
+        h.Ab = h.Bb = nullptr;
+        h.Cb = nullptr;
+        h.A = h.B = Di[q];
+        h.C = ZD[q];
+        h.b_kept = ld + (fused(z) ? it[z].q.a : 0);
+        BTA_TRY(emulate(z, h));
+      }
+      return BTA_OK;
+    };
+    if (emu) BTA_TRY(inverse_gram());
     if (hasB) {
       auto Dn = ptrs(G.all, [&](int z) { return D(z, i + 1); });
       if (emu) {
@@ -959,13 +981,7 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         BTA_TRY(gemm_f64(g, s));
       }
     }
-    {  // Z_D = L_Di^{-T} L_Di^{-1} (lower part)
-      Gemm g; g.M = ld; g.N = ld; g.K = ld; g.batch = M;
-      g.Ab = cp(Di); g.lda = ld; g.transA = 1; g.triA = TRI_UPPER;
-      g.Bb = cp(Di); g.ldb = ld; g.triB = TRI_LOWER;
-      g.Cb = ZD.data(); g.ldc = ld; g.out_lower = 1;
-      BTA_TRY(big_product(g, it, G.all, precision, s));
-    }
+    if (!emu) BTA_TRY(inverse_gram());
     if (hasB) {  // Z_D -= Z_B^T F_B
       if (emu) {  // an arrow carried along extends K: Z_D -= [Z_B; Z_C]^T [F_B; F_C]
         for (size_t q = 0; q < G.all.size(); ++q) {
@@ -974,6 +990,7 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
           g.A = ZB[q]; g.lda = ld; g.transA = 1; g.B = W1[q]; g.ldb = ld;
           g.C = ZD[q]; g.ldc = ld; g.Cin = ZD[q]; g.ldcin = ld; g.alpha = -1.0; g.beta = 1.0;
           g.out_lower = 1;
+          g.b_kept = ld + (fused(z) ? it[z].q.a : 0);   // F_B's planes from Z_B's product
           if (fused(z)) {
             const int a = it[z].q.a;
             g.K = ld + a; g.a_k = ld; g.A12 = {Cb(z, i), a, 1};
