@@ -79,7 +79,8 @@ struct inla_model {
               evs6 = nullptr, ev5 = nullptr;
   cudaEvent_t evj = nullptr;    // join event of a multi-model graph
   // blocks of the reverse legs: both ends meet in the middle
-  int reverse_blocks() const { return n >= 3 ? (n - 1) / 2 : 0; }
+  // (mixed precision keeps the forward order: see group_program)
+  int reverse_blocks(int prec) const { return n >= 3 && prec != 1 ? (n - 1) / 2 : 0; }
 };
 
 // Several models evaluated by one CUDA graph (see inla_batch_value_and_grad).
@@ -154,7 +155,7 @@ bta_status ctx_alloc(inla_model* m, EvalCtx& c) {
   BTA_TRY(dmalloc(m, &c.RS, (size_t)kMaxK * resid_chunks(md)));
   BTA_TRY(dmalloc(m, &c.out, out_size(md.d)));
   BTA_TRY(dmalloc(m, &c.red, kRedDoubles));
-  const int legs = m->reverse_blocks() > 0 ? 4 : 2;
+  const int legs = m->reverse_blocks(0) > 0 ? 4 : 2;
   SweepWs* const ws[4] = {&c.wsc, &c.wsp, &c.wsc2, &c.wsp2};
   const size_t wsb = SweepWs::bytes(ld, a) / sizeof(double);
   double* wsbuf = nullptr;
@@ -202,7 +203,9 @@ bta_status ensure_ctx(inla_model* m, int count) {
 // leaves most of the GPU idle, and the serial diagonal steps of one leg overlap the wide
 // products of the others.  Per call, one leg per matrix / two: b = 1024, 50 blocks emulated
 // gradient 75.8 / 58.6 ms, value 55.2 / 38.7 ms; b = 4800, 8 blocks 215 / 205 ms; b = 64,
-// 4 blocks FP64 0.92 / 0.72 ms; the FP64-bound b = 1024 gradient 68.6 / 67.4 ms.
+// 4 blocks FP64 0.92 / 0.72 ms; the FP64-bound b = 1024 gradient 68.6 / 67.4 ms.  Mixed
+// precision keeps one forward leg per matrix: its products round to ~22 bits, so another
+// order would move a gradient by its own error (3e-9 where the results agree to 1e-12).
 // Each step issues one block of every leg, so the streams' operations, and the nodes of
 // a captured graph, are created in alternation: the driver submits a graph's kernels in
 // creation order into a bounded queue, and a whole sweep created first (~1600 launches a
@@ -218,7 +221,7 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
                          std::vector<IssueStep>& steps) {
   const ModelDev& md = m->md;
   const int grad = mode >= 1, nt = md.nt;
-  const int nb = m->reverse_blocks(), mid = nt - 1 - nb;
+  const int nb = m->reverse_blocks(prec), mid = nt - 1 - nb;
   auto sets = std::make_shared<GroupSets>();
   for (int e = 0; e < cnt; ++e) {
     EvalCtx& c = m->ctx[e];
