@@ -278,13 +278,14 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
     }
     return BTA_OK;
   });
-  // Q_c's vector parts on streams of their own: they only read finished blocks of the factor,
-  // and on s1 and s3 they lay between the dependent diagonal factors and before the selected
-  // inversion, which now follows the solve block by block.  Low-memory sweeps recompute L_B
-  // in workspaces that the next block needs, and a > kGramRows shares one with the arrow.
+  // Q_c's vector parts, and its arrow where no b x b product carries it, on streams of their
+  // own: they only read finished blocks of the factor, and on s1 and s3 they lay between the
+  // dependent diagonal factors and before the selected inversion, which now follows the solve
+  // block by block.  Low-memory sweeps recompute L_B in workspaces that the next block needs.
   // In line / on their own streams: b = 1024, 50 blocks emulated gradient 46.4 / 44.9 ms, value
-  // 29.0 / 28.3, mixed gradient 51.7 / 49.7; b = 64, 4 blocks 0.52 / 0.48 ms.
-  const bool side = !m->lowmem && md.a <= kGramRows;
+  // 29.0 / 28.3; b = 64, 4 blocks 0.52 / 0.48 ms, with the arrow 0.45; mixed 75.2 / 73.5 ms by
+  // the arrow.
+  const bool side = !m->lowmem;
   const cudaStream_t v1 = side ? m->s5 : m->s1, v3 = side ? m->s6 : m->s3;
   if (mode < 2)
     for (int i = 0; i <= mid; ++i)

@@ -402,7 +402,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
   BTA_TRY(check_set(it, m));
   if (!sv) sv = s;
   for (int z = 0; sv != s && z < m; ++z)
-    if (!ev || !it[z].q.B || it[z].q.a > kGramRows) return BTA_ERR_ARG;
+    if (!ev || !it[z].q.B) return BTA_ERR_ARG;
   const int n = it[0].blocks(), ld = it[0].q.ld;
   const bool rev = it[0].rev;
   if (i1 < 0) i1 = n;
@@ -453,14 +453,14 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       if (!it[z].vec) continue;
       Gemv h; h.M = a; h.K = ld; h.A = Cb(z, i); h.lda = a;
       h.x = vec_of(it[z], i); h.y = it[z].ws.vT; h.beta = 1.0;
-      BTA_TRY(gemv_f64(h, s));
+      BTA_TRY(gemv_f64(h, sv));
     }
     auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });
     Gemm h; h.M = a; h.N = a; h.K = ld; h.batch = (int)grp.size();
     h.Ab = cp(Ci); h.lda = a; h.Bb = cp(Ci); h.ldb = a; h.transB = 1;
     h.Cb = T.data(); h.ldc = a; h.Cinb = cp(T); h.ldcin = a; h.alpha = -1.0; h.beta = 1.0;
     h.sk_wsb = SK.data(); h.sk_cap = blk;
-    return gemm_f64(h, s);
+    return gemm_f64(h, sv);
   };
   auto vector_step = [&](int i) -> bta_status {
     if (G.vec.empty()) return BTA_OK;
@@ -477,6 +477,42 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
       Gemv g; g.M = ld; g.K = ld; g.lda = ld; g.alpha = -1.0; g.beta = 1.0; g.batch = c;
       g.Ab = cp(Bp); g.xb = cp(rp); g.yb = gv.data(); g.yinb = cp(ri);
       BTA_TRY(gemv_f64(g, sv));
+    }
+    return BTA_OK;
+  };
+  // The arrow in FP64 products, where none of b x b carries it: C_i -= L_C,i-1 L_B,i-1^T ...
+  auto arrow_update = [&](int i) -> bta_status {
+    for (const auto& grp : G.arrow) {
+      if (fused(grp[0])) continue;      // carried by the product above
+      const int a = it[grp[0]].q.a;
+      auto Cp = ptrs(grp, [&](int z) { return Cb(z, i - 1); });
+      auto Bp = ptrs(grp, [&](int z) { return LB(z, i - 1); });
+      auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
+      auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });   // W3 is free here
+      Gemm g; g.M = a; g.N = ld; g.K = ld; g.batch = (int)grp.size();
+      g.Ab = cp(Cp); g.lda = a; g.Bb = cp(Bp); g.ldb = ld; g.transB = 1;
+      g.Cb = Ci.data(); g.ldc = a; g.Cinb = cp(Ci); g.ldcin = a; g.alpha = -1.0; g.beta = 1.0;
+      g.sk_wsb = SK.data(); g.sk_cap = blk;
+      BTA_TRY(gemm_f64(g, sv));
+    }
+    return BTA_OK;
+  };
+  // ... and L_Ci = C_i L_Di^{-T}
+  auto arrow_factor = [&](int i) -> bta_status {
+    const bool with_b = emu && i < n - 1;   // L_Ci as extra rows of L_Bi's product
+    for (const auto& grp : G.arrow) {
+      if (with_b && fused(grp[0])) continue;
+      const int a = it[grp[0]].q.a, c = (int)grp.size();
+      auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
+      auto Di = ptrs(grp, [&](int z) { return D(z, i); });
+      auto W = ptrs(grp, [&](int z) { return it[z].ws.Wc1; });
+      auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });
+      Gemm g; g.M = a; g.N = ld; g.K = ld; g.batch = c;
+      g.Ab = cp(Ci); g.lda = a; g.Bb = cp(Di); g.ldb = ld; g.transB = 1; g.triB = TRI_UPPER;
+      g.Cb = W.data(); g.ldc = a;
+      g.sk_wsb = SK.data(); g.sk_cap = blk;
+      BTA_TRY(gemm_f64(g, sv));
+      BTA_TRY(copy_block_batch(c, cp(W), a, Ci.data(), a, a, ld, 1.0, sv));
     }
     return BTA_OK;
   };
@@ -508,22 +544,12 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
         g.alpha = -1.0; g.beta = 1.0; g.out_lower = 1;
         BTA_TRY(big_product(g, it, G.all, precision, s));
       }
-      for (const auto& grp : G.arrow) {  // C_i -= L_C,i-1 L_B,i-1^T
-        if (fused(grp[0])) continue;      // carried by the product above
-        const int a = it[grp[0]].q.a;
-        auto Cp = ptrs(grp, [&](int z) { return Cb(z, i - 1); });
-        auto Bp = ptrs(grp, [&](int z) { return LB(z, i - 1); });
-        auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
-        auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });   // W3 is free here
-        Gemm g; g.M = a; g.N = ld; g.K = ld; g.batch = (int)grp.size();
-        g.Ab = cp(Cp); g.lda = a; g.Bb = cp(Bp); g.ldb = ld; g.transB = 1;
-        g.Cb = Ci.data(); g.ldc = a; g.Cinb = cp(Ci); g.ldcin = a; g.alpha = -1.0; g.beta = 1.0;
-        g.sk_wsb = SK.data(); g.sk_cap = blk;
-        BTA_TRY(gemm_f64(g, s));
-      }
     }
-    if (join) return vector_step(i);
-    if (sv == s) BTA_TRY(vector_step(i));
+    if (join || sv == s) {
+      if (i > 0) BTA_TRY(arrow_update(i));
+      BTA_TRY(vector_step(i));
+    }
+    if (join) return BTA_OK;
     {  // L_Di^{-1} in place, log-det slots
       auto Di = ptrs(G.all, [&](int z) { return D(z, i); });
       auto W = ptrs(G.all, [&](int z) { return it[z].ws.pot; });
@@ -545,21 +571,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
                                    code.data(), precision, tw.data(), ts.data(), s));
       BTA_SWEEP_MARK(s, 2, i);
     }
-    const bool with_b = emu && i < n - 1;   // L_Ci as extra rows of L_Bi's product
-    for (const auto& grp : G.arrow) {  // L_Ci = C_i L_Di^{-T}
-      if (with_b && fused(grp[0])) continue;
-      const int a = it[grp[0]].q.a, c = (int)grp.size();
-      auto Ci = ptrs(grp, [&](int z) { return Cb(z, i); });
-      auto Di = ptrs(grp, [&](int z) { return D(z, i); });
-      auto W = ptrs(grp, [&](int z) { return it[z].ws.Wc1; });
-      auto SK = ptrs(grp, [&](int z) { return it[z].ws.W3; });
-      Gemm g; g.M = a; g.N = ld; g.K = ld; g.batch = c;
-      g.Ab = cp(Ci); g.lda = a; g.Bb = cp(Di); g.ldb = ld; g.transB = 1; g.triB = TRI_UPPER;
-      g.Cb = W.data(); g.ldc = a;
-      g.sk_wsb = SK.data(); g.sk_cap = blk;
-      BTA_TRY(gemm_f64(g, s));
-      BTA_TRY(copy_block_batch(c, cp(W), a, Ci.data(), a, a, ld, 1.0, s));
-    }
+    if (sv == s) BTA_TRY(arrow_factor(i));
     if (i < n - 1) {  // L_Bi = Q[i+1, i] L_Di^{-T}
       if (low) BTA_TRY(assemble_b_items(it, G.all, i, s));
       auto Bi = ptrs(G.all, [&](int z) { return low ? it[z].ws.W2 : B(z, i); });
@@ -589,7 +601,9 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
     if (sv != s) {
       BTA_CUDA_TRY(cudaEventRecord(ev, s));
       BTA_CUDA_TRY(cudaStreamWaitEvent(sv, ev, 0));
+      if (i > 0) BTA_TRY(arrow_update(i));
       BTA_TRY(vector_step(i));
+      BTA_TRY(arrow_factor(i));
     }
     if (!G.vec.empty()) {  // z_i = L_Di^{-1} t
       auto zi = ptrs(G.vec, [&](int z) { return vec_of(it[z], i); });

@@ -84,10 +84,10 @@ struct SweepItem {
 // be ordered after it, and the reverse leg's solve and selected inversion (from
 // block len - 2) after theirs.
 //
-// sv (optional, not for low-memory sweeps nor a > kGramRows; ev an event of its own): a
-// block's vector part and tip share go to this stream, after the block's factor on s; they
-// read finished parts of the factor only.  s waits for it before the tip; a reverse leg's
-// last vector part, which updates the shared block's, stays on sv.
+// sv (optional, not for low-memory sweeps; ev an event of its own): a block's vector part,
+// the arrow where no b x b product carries it, and the tip's share go to this stream, after
+// the block's factor on s; they read finished parts of the factor only.  s waits for it
+// before the tip; a reverse leg's last share, which updates the shared block's, stays on sv.
 bta_status factor_sweep_multi(const SweepItem* items, int m, cudaStream_t s, int precision = 0,
                               int i0 = 0, int i1 = -1, cudaStream_t sv = nullptr,
                               cudaEvent_t ev = nullptr);
