@@ -167,12 +167,11 @@ class ClockSampler:
 # ----------------------------------------------------------------------------
 FULL_NT = 192
 # DRAM bytes (read + write) of one launch of the emulated product kernel at
-# 4800 x 4800 x 4800 (composing C in its epilogue), from an ncu capture of that
-# launch (dram__bytes_read.sum 2.651 GB + dram__bytes_write.sum 0.201 GB;
-# `--metrics ... -k regex:ozaki_gemm128 -c 1` on `bench.py --mode gemm
-# --precision 2 --gemm-n 4800`).  The slices themselves are 0.75 GB: L2 absorbs
-# most tile re-reads.
-GEMM4800_DRAM_BYTES = 2.852e9
+# 4800 x 4800 x 4800 from an ncu capture of that launch (dram__bytes_read.sum
+# 2.535 GB + dram__bytes_write.sum 0.727 GB; `--metrics ... -k regex:crt_gemm`
+# on `bench.py --mode gemm --precision 2 --gemm-n 4800`).  The residue planes
+# of both operands are 1.31 GB, the residues of the result 0.66 GB.
+GEMM4800_DRAM_BYTES = 3.262e9
 
 
 def oracle_cut_problem(nt):

@@ -995,7 +995,7 @@ __device__ __forceinline__ double op_elem(const double* X, int ldx, int trans, i
 }
 
 // One operand to split: rows of op(X) (op(B)^T for the B side), their
-// exponent bounds ex[rowsP] and slices Y[S][rowsP][Kp].  op(X) may be a 2 x 2
+// exponent bounds ex[rowsP] and planes Y (residue_kernel).  op(X) may be a 2 x 2
 // block matrix cut after row rc and column kc: the leading block is (X, ldx,
 // trans, tri), the others P[0] (rows < rc, k >= kc), P[1] (rows >= rc,
 // k < kc) and P[2] (rows >= rc, k >= kc), each untriangular, zero when its
