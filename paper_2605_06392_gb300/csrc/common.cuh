@@ -1,6 +1,7 @@
 // Shared definitions for the BTA / INLA CUDA library (sm_103a, FP64 path).
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cstdio>
 #include <utility>
@@ -78,6 +79,19 @@ template <class... KArgs, class... Args>
 cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
                         Args&&... args) {
   return launch_prio_smem(kernel, grid, block, 0, s, std::forward<Args>(args)...);
+}
+
+// Raise a kernel's limit of dynamic shared memory on the current device.  The attribute
+// belongs to a device, so `done` (one per kernel) has a bit for each; devices beyond its
+// 64 set it on every call.
+inline bta_status allow_smem(std::atomic<uint64_t>& done, const void* kernel, int bytes) {
+  int dev = 0;
+  BTA_CUDA_TRY(cudaGetDevice(&dev));
+  const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+  if (done.load() & bit) return BTA_OK;
+  BTA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  done.fetch_or(bit);
+  return BTA_OK;
 }
 
 inline int pad_ld(int b) { return (b + kPad - 1) / kPad * kPad; }

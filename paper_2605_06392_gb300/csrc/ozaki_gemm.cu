@@ -1380,15 +1380,10 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   q.R = R;
   q.status = status;
   const int units = q.tiles * kNumMod;
-  static bool attr = false;
-  if (!attr) {
-    BTA_CUDA_TRY(cudaFuncSetAttribute(crt_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kCrtSmem));
-    BTA_CUDA_TRY(cudaFuncSetAttribute(crt_gemm_small_kernel,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem));
-    attr = true;
-  }
+  static std::atomic<uint64_t> allowed[2];
   if (tile == ST) {
+    BTA_TRY(allow_smem(allowed[0], reinterpret_cast<const void*>(&crt_gemm_small_kernel),
+                       kSmallSmem));
     q.group = q.mt;
     if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
     BTA_CUDA_TRY(launch_after(crt_gemm_small_kernel, dim3(units), dim3(kCrtThreads), kSmallSmem,
@@ -1397,6 +1392,7 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
     // A wave of pairs spans a near-square patch of tiles.  A pair takes several units
     // (the store of one overlaps the next) but at most ~300 slabs, ~75 us, so that the
     // launches of a concurrent sweep find free SMs.
+    BTA_TRY(allow_smem(allowed[1], reinterpret_cast<const void*>(&crt_gemm_kernel), kCrtSmem));
     q.slots = pair_slots();
     q.group = std::min(q.mt, std::max(1, (int)std::lround(std::sqrt((double)q.slots))));
     q.slots = std::min(q.slots, units);

@@ -1102,22 +1102,11 @@ bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* c
     const int cap = dag_max_ctas() > 0 ? dag_max_ctas() : max_ctas;
     if (cap > 0) grid = std::min(grid, std::max(2, cap));   // the chain and a bulk CTA
     grid = std::max(grid, std::min(g.total, cnt + 1));   // every chain, and a bulk CTA
-    static bool attr = false;   // above 48 KB of dynamic shared memory
-    if (!attr) {
-      BTA_CUDA_TRY(cudaFuncSetAttribute(potrf_dag_kernel<true>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        dag_smem<true>()));
-      BTA_CUDA_TRY(cudaFuncSetAttribute(potrf_dag_kernel<false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        dag_smem<false>()));
-      attr = true;
-    }
-    if (tc)
-      launch_prio_smem(potrf_dag_kernel<true>, dim3(grid), dim3(kDagAllThreads), dag_smem<true>(),
-                       s, g);
-    else
-      launch_prio_smem(potrf_dag_kernel<false>, dim3(grid), dim3(kDagAllThreads),
-                       dag_smem<false>(), s, g);
+    auto* const kernel = tc ? &potrf_dag_kernel<true> : &potrf_dag_kernel<false>;
+    const int smem = tc ? dag_smem<true>() : dag_smem<false>();
+    static std::atomic<uint64_t> allowed[2];   // above 48 KB of dynamic shared memory
+    BTA_TRY(allow_smem(allowed[tc ? 1 : 0], reinterpret_cast<const void*>(kernel), smem));
+    BTA_CUDA_TRY(launch_prio_smem(kernel, dim3(grid), dim3(kDagAllThreads), smem, s, g));
     BTA_LAUNCHED();
   }
   return BTA_OK;

@@ -381,12 +381,8 @@ bta_status tc_gemm_mixed(const Gemm& g, void* ws, int32_t* status, cudaStream_t 
   BTA_TRY(make_map(&mAlo, Alo, M, Kp));
   BTA_TRY(make_map(&mBhi, Bhi, N, Kp));
   BTA_TRY(make_map(&mBlo, Blo, N, Kp));
-  static bool attr_set = false;
-  if (!attr_set) {
-    BTA_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_tf32x3_kernel,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> allowed;
+  BTA_TRY(allow_smem(allowed, reinterpret_cast<const void*>(&tc_gemm_tf32x3_kernel), kSmemBytes));
   TcArgs a;
   a.M = M; a.N = N; a.K = K; a.alpha = g.alpha; a.beta = g.beta; a.C = g.C; a.ldc = g.ldc;
   a.amode = g.alpha == 1.0 ? 0 : g.alpha == -1.0 ? 1 : 2;
