@@ -1028,7 +1028,7 @@ int dag_max_ctas() {
   return v;
 }
 
-// Whether bulk tasks yield the SM to chain tasks (BTA_DAG_YIELD=0 disables).
+// Whether bulk tasks may yield the SM to chain tasks (BTA_DAG_YIELD=0 disables).
 int dag_yield() {
   static int v = [] {
     const char* e = getenv("BTA_DAG_YIELD");
@@ -1095,13 +1095,15 @@ bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* c
     g.counter = g.inst[0].st + 4 * p * p + p + 8;
     g.abort = g.counter + 16;
     g.smbusy = g.inst[0].st + 4 * p * p + p + 64;
-    g.yield = cnt <= 2 ? dag_yield() : 0;
     g.stall = g_dag_stall;
     g.wait_ns = g_dag_wait_ns;
     int grid = std::min(g.total, sm_count() * dag_ctas_per_sm());
     const int cap = dag_max_ctas() > 0 ? dag_max_ctas() : max_ctas;
     if (cap > 0) grid = std::min(grid, std::max(2, cap));   // the chain and a bulk CTA
     grid = std::max(grid, std::min(g.total, cnt + 1));   // every chain, and a bulk CTA
+    // Two CTAs fit an SM, so the chains' SMs hold at most 2 cnt of them: only with more do
+    // the bulk tasks have a CTA that does not wait for a chain to leave its SM.
+    g.yield = cnt <= 2 && grid > 2 * cnt ? dag_yield() : 0;
     auto* const kernel = tc ? &potrf_dag_kernel<true> : &potrf_dag_kernel<false>;
     const int smem = tc ? dag_smem<true>() : dag_smem<false>();
     static std::atomic<uint64_t> allowed[2];   // above 48 KB of dynamic shared memory

@@ -41,3 +41,36 @@ def test_kernel_attributes_on_every_device(fake, call):
     for dev in (0, 3, 0, 70):
         fake.device(dev)
         assert call(fake) == 0, dev
+
+
+# ---- the task graph's grid ----------------------------------------------------
+def _leaves(fake):
+    """(rows, matrices, CTAs, bulk tasks yield) of the task graphs launched."""
+    return [(32 * fake.head(i, 0), fake.head(i, 2), grid[0], fake.head(i, 10))
+            for name, grid, i in fake.launches() if "potrf_dag_kernel" in name]
+
+
+def _evaluate(fake, precision, count=1, grad=False, low_memory=False, **over):
+    """Task graphs of an evaluation of `count` thetas together."""
+    import numpy as np
+
+    import paper_2605_06392_gb300 as P
+    prob = workloads.make_problem("st_tiny", **over)
+    m = P.InlaModel(prob, low_memory=low_memory)
+    fake.reset()
+    m.value_and_grad(np.array([prob.theta] * count), grad=grad, use_graph=False, concurrent=count,
+                     precision=precision, stream=Stream())
+    got = _leaves(fake)
+    m.close()
+    assert got
+    return got
+
+
+@pytest.mark.parametrize("nx", [4, 8, 12, 16])
+@pytest.mark.parametrize("count", [1, 2])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_a_yielding_grid_has_a_free_cta(fake, precision, count, nx):
+    """Bulk tasks that yield wait for the chain on their SM, which waits for them: with two
+    CTAs an SM, at least one CTA must lie outside the chains' SMs."""
+    for rows, matrices, ctas, yields in _evaluate(fake, precision, count, nx=nx):
+        assert not yields or ctas > 2 * matrices, (rows, matrices, ctas)
