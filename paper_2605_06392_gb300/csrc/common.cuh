@@ -252,7 +252,8 @@ bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
 int potrf_hybrid_leaf(int precision);
 // The task-graph kernel (potrf_dag.cu) used by potrf_inv_batch for n <= 5120;
 // g_potrf_recursive = 1 selects the recursive launch sequence instead.
-// max_ctas > 0 caps the persistent grid (at least 2: the chain and a bulk CTA).
+// max_ctas > 0 caps the persistent grid at so many CTAs a matrix (at least 2: the chain
+// and a bulk CTA).
 // tc = 1: the 32 x 32 tile products emulated in FP64 from BF16 slices on the
 // tensor cores (the tensor-core modes); 0: FP64 FMAs.
 bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* const* scratch,

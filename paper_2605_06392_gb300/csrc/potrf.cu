@@ -229,11 +229,13 @@ bta_status level_product(const Gemm& g, const ProdCfg& c, cudaStream_t s) {
   return BTA_OK;
 }
 
-// Cap on the task graph's grid in the tensor-core modes: the other legs' products run on
+// Cap on the task graph's CTAs a matrix in the tensor-core modes: the other legs' products run on
 // the SMs the leaves leave free, and a CTA per 16 rows keeps the bulk tasks off the chain
 // (512 rows, 65 / 40 / 32 / 24 CTAs: 0.289 / 0.287 / 0.299 / 0.334 ms alone; the b = 1024
 // gradient of 50 blocks, 64 / 40 / 32 / 24: 46.7 / 43.6 / 43.5 / 45.0 ms, the uneven batch
-// 67.5 / 63.7 / 60.9 / 60.7 ms).  The FP64 mode, whose bulk tasks
+// 67.5 / 63.7 / 60.9 / 60.7 ms).  A set's matrices bring their tasks with them: with n / 16
+// for the whole set, 16 thetas at b = 600 left one CTA to 16 chains (72.5 ms a call of 6
+// blocks, 26.3 with n / 16 each; b = 1024 94.1 and 64.9).  The FP64 mode, whose bulk tasks
 // need the SMs, keeps them all.
 int leaf_ctas(int n) { return std::max(2, n / 16); }
 

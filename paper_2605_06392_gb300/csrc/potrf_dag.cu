@@ -1017,7 +1017,7 @@ int dag_ctas_per_sm() {
 }
 
 // Most CTAs of the persistent grid (BTA_DAG_MAX_CTAS, overriding the caller's
-// cap; 0: the caller's cap, or one per SM).  A leaf's critical path is its
+// cap; 0: the caller's cap for each matrix, or one per SM).  A leaf's critical path is its
 // chain on one CTA; CTAs beyond what keeps its bulk tasks off that path only
 // hold SMs that a concurrent sweep's products could use.
 int dag_max_ctas() {
@@ -1098,7 +1098,7 @@ bta_status potrf_dag_batch(int count, double* const* A, int n, int ld, double* c
     g.stall = g_dag_stall;
     g.wait_ns = g_dag_wait_ns;
     int grid = std::min(g.total, sm_count() * dag_ctas_per_sm());
-    const int cap = dag_max_ctas() > 0 ? dag_max_ctas() : max_ctas;
+    const int cap = dag_max_ctas() > 0 ? dag_max_ctas() : max_ctas * cnt;
     if (cap > 0) grid = std::min(grid, std::max(2, cap));   // the chain and a bulk CTA
     grid = std::max(grid, std::min(g.total, cnt + 1));   // every chain, and a bulk CTA
     // Two CTAs fit an SM, so the chains' SMs hold at most 2 cnt of them: only with more do

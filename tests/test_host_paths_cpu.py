@@ -74,3 +74,11 @@ def test_a_yielding_grid_has_a_free_cta(fake, precision, count, nx):
     CTAs an SM, at least one CTA must lie outside the chains' SMs."""
     for rows, matrices, ctas, yields in _evaluate(fake, precision, count, nx=nx):
         assert not yields or ctas > 2 * matrices, (rows, matrices, ctas)
+
+
+@pytest.mark.parametrize("count", [1, 4, 16])
+@pytest.mark.parametrize("precision", [1, 2])
+def test_every_matrix_of_a_set_brings_its_ctas(fake, precision, count):
+    """A set's bulk tasks grow with its matrices: so do the CTAs, up to the SMs."""
+    for rows, matrices, ctas, _ in _evaluate(fake, precision, count, nx=24, ny=25):
+        assert matrices == count and ctas >= min(152, count * rows // 16), (rows, ctas)
