@@ -235,10 +235,10 @@ bool ozaki_supported(const Gemm& g);
 bta_status potrf_inv(double* A, int n, int ld, double* scratch, double* logdet_parts,
                      int32_t* fail, int32_t fail_code, cudaStream_t s);
 // The same on `count` blocks of one size at once (host arrays of per-block
-// pointers and failure codes).
+// pointers and failure codes; max_ctas as for potrf_dag_batch).
 bta_status potrf_inv_batch(int count, double* const* A, int n, int ld, double* const* scratch,
                            double* const* logdet_parts, int32_t* const* fail,
-                           const int32_t* fail_code, cudaStream_t s);
+                           const int32_t* fail_code, cudaStream_t s, int max_ctas = 0);
 int potrf_inv_slots(int n);   // number of logdet slots potrf_inv writes
 // The same with the precision of the sweep: above potrf_hybrid_leaf(precision)
 // rows the block is split 2 x 2 recursively, the diagonal sub-blocks factored

@@ -235,7 +235,7 @@ bta_status level_product(const Gemm& g, const ProdCfg& c, cudaStream_t s) {
 // gradient of 50 blocks, 64 / 40 / 32 / 24: 46.7 / 43.6 / 43.5 / 45.0 ms, the uneven batch
 // 67.5 / 63.7 / 60.9 / 60.7 ms).  A set's matrices bring their tasks with them: with n / 16
 // for the whole set, 16 thetas at b = 600 left one CTA to 16 chains (72.5 ms a call of 6
-// blocks, 26.3 with n / 16 each; b = 1024 94.1 and 64.9).  The FP64 mode, whose bulk tasks
+// blocks, 25.8 with n / 16 each; b = 1024 93.6 and 63.8).  The FP64 mode, whose bulk tasks
 // need the SMs, keeps them all.
 int leaf_ctas(int n) { return std::max(2, n / 16); }
 
@@ -340,7 +340,9 @@ int potrf_hybrid_leaf(int precision) {
 
 namespace {
 // Blocks above this many rows are split at least once (tensor-core modes): a
-// 1024-row block is faster as two 512-row task graphs than as one.
+// 1024-row block is faster as two 512-row task graphs than as one.  Smaller ones are one
+// task graph with FP64 tile products, as in mode 0: emulated ones would be faster (b = 192:
+// 123 us a block, 150 in FP64), but hold an entry only to 2^-56 of its row's largest.
 int potrf_hybrid_top(int precision) {
   static const int tc = env_int("BTA_POTRF_SPLIT_TC", 512);
   return precision == 0 ? 0 : tc;
@@ -357,15 +359,11 @@ bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
   if (top <= 0 || top > leaf) top = leaf;   // the top-level split threshold
   bool tc_ok = precision == 0 || (tcws && tcstat && n <= 5120);
   for (int z = 0; tc_ok && precision != 0 && z < count; ++z) tc_ok = tcws[z] && tcstat[z];
-  if (precision != 0 && n <= std::min(top, leaf) && n / T <= 160 && !g_potrf_recursive) {
-    // one task graph, its tile products emulated like those of a larger block's leaves
-    // (b = 192: 150 -> 123 us a block)
-    PriorityScope prio(highest_priority());
-    return potrf_dag_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s,
-                           leaf_ctas(n), 1);
-  }
+  // (in the tensor-core modes beside the other legs' products, which a CTA per 8 rows leaves
+  // room for: b = 512, 6 blocks emulated value and gradient 3.45 ms on all SMs, 2.75 so)
   if (leaf < T || top < T || n <= top || n < 2 * T || !tc_ok || n / T > 160 || g_potrf_recursive)
-    return potrf_inv_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s);
+    return potrf_inv_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s,
+                           precision != 0 && n <= top ? n / 8 : 0);
   PriorityScope prio(highest_priority());
   ProdCfg pc;
   pc.precision = precision;
@@ -392,11 +390,11 @@ int g_potrf_recursive = 0;
 
 bta_status potrf_inv_batch(int count, double* const* A, int n, int ld, double* const* scratch,
                            double* const* logdet_parts, int32_t* const* fail,
-                           const int32_t* fail_code, cudaStream_t s) {
+                           const int32_t* fail_code, cudaStream_t s, int max_ctas) {
   if (n <= 0 || n % T || count < 0) return BTA_ERR_ARG;
   PriorityScope prio(highest_priority());   // the sweep's critical path
   if (count > 0 && n / T <= 160 && !g_potrf_recursive)
-    return potrf_dag_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s);
+    return potrf_dag_batch(count, A, n, ld, scratch, logdet_parts, fail, fail_code, s, max_ctas);
   for (int z0 = 0; z0 < count; z0 += kMaxBatch) {
     PB b;
     b.cnt = count - z0 < kMaxBatch ? count - z0 : kMaxBatch;

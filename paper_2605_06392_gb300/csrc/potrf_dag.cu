@@ -273,8 +273,13 @@ __device__ __forceinline__ void tile_syrk_lower(Tile L, Tile W) {
 // sums to an integer |S_L| < 2^21 over K = 32, exact in FP32; levels 0..5 are
 // added as 64-bit integers in units of level 5, levels 6 and 7 rounded to that
 // unit, and the FP64 result assembled by integer operations.  Levels from 8 on
-// are dropped, below the 56th bit of the operands' products.  ylower: Y is lower
-// triangular (its upper part is not read).
+// are dropped.  Error: with u, w the powers of two above a row's and a column's largest
+// entries, level L's unit is 2^(-14 - 7 L) u w.  The rounding to level 5's unit is off by
+// 2^-50 u w, the dropped levels by at most 7 2^17 units of level 8 (and 1 % more)
+// = 2^-50.2 u w, the 56-bit operands by 2^-51 u w: 2^-48.7 u w in all for 32 terms, where
+// the bound of FP64 FMAs is 2^-43 times the largest entries' product.  Unlike theirs it is
+// absolute in a row and column of a tile: small entries keep fewer bits.  ylower: Y is
+// lower triangular (its upper part is not read).
 constexpr int kOzPitch = 40;                      // bf16 a slice row: 80 bytes, conflict-free ldmatrix
 constexpr int kOzPlane = T * kOzPitch;            // one 32 x 32 slice
 constexpr int kOzTileSmem = 2 * 8 * kOzPlane * 2 + 2 * T * 4;   // both operands' slices, exponents

@@ -72,7 +72,9 @@ struct SweepItem {
 };
 // precision 0: every product in FP64; 1: the b x b off-diagonal Schur
 // products (and the selected-inversion products) in split precision on the
-// tensor cores, the diagonal-block factorisation, arrow and log-det in FP64.
+// tensor cores, the diagonal-block factorisation to FP64 accuracy (in FP64 up to 512
+// rows, above with emulated products: potrf_inv_batch_prec), arrow and log-det in
+// FP64; 2: the b x b products emulated in FP64, the diagonal factor as in 1.
 // Block range (optional): blocks i0 <= i < i1 of the factor sweep (i1 < 0:
 // to the end) and i_hi >= i >= i_lo of the solves and the selected inversion
 // (i_hi < 0: from the last block), the set-up with the first block and the tip with

@@ -82,3 +82,13 @@ def test_every_matrix_of_a_set_brings_its_ctas(fake, precision, count):
     """A set's bulk tasks grow with its matrices: so do the CTAs, up to the SMs."""
     for rows, matrices, ctas, _ in _evaluate(fake, precision, count, nx=24, ny=25):
         assert matrices == count and ctas >= min(152, count * rows // 16), (rows, ctas)
+
+
+# ---- diagonal factors in the tensor-core modes -------------------------------
+@pytest.mark.parametrize("b", [32, 64, 192, 480, 512])
+@pytest.mark.parametrize("precision", [1, 2])
+def test_blocks_up_to_512_rows_keep_fp64_tile_products(fake, b, precision):
+    """potrf_dag_kernel<false>: emulated tile products (<true>) begin above 512 rows."""
+    assert _factor(fake, 2, b, 0, precision) == 0
+    names = [n for n, _, _ in fake.launches() if "potrf_dag_kernel" in n]
+    assert len(names) == 2 and all("ILb0E" in n for n in names), names
