@@ -27,8 +27,9 @@ constexpr int kMaxTip = 32;
 
 // One CTA of 128 threads.  FP64 latency (72 clocks an operation, several hundred a
 // division or square root) bounds it, so the columns of an update go to different
-// threads and each pivot's reciprocal is taken once.  Measured a = 9: 35 us with one
-// thread, 10 us.
+// threads.  The solves divide by their pivots: products with reciprocals would round twice
+// (and save 6 us of a b = 64 gradient's 0.46 ms).  Measured a = 9, mode 0: 35 us with one
+// thread, 23 us.
 // mode 0: factor T in place (lower L_T, upper zeroed), logdet slot, and if
 //         r != null: z_T = L_T^{-1} (r_T - v_T)  (written to r); T2, vT2 (or null):
 //         another leg's shares, added to T and v_T
@@ -39,7 +40,6 @@ __global__ void __launch_bounds__(kTipThreads)
     tip_kernel(int mode, int a, double* T, double* r, const double* vT, const double* T2,
                const double* vT2, double* logdet_slot, int32_t* fail, int32_t fail_code) {
   __shared__ double L[kMaxTip][kMaxTip + 1];
-  __shared__ double rp[kMaxTip];   // reciprocal pivots
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int e = tid; e < a * a; e += kTipThreads)
     L[e % a][e / a] = T2 ? T[e] + T2[e] : T[e];
@@ -50,12 +50,9 @@ __global__ void __launch_bounds__(kTipThreads)
     for (int j = 0; j < a; ++j) {
       double d = L[j][j];
       if (!(d > 0.0) || !isfinite(d)) { bad = true; d = 1.0; }
-      const double piv = sqrt(d), inv = 1.0 / piv;   // every thread: the same value
+      const double piv = sqrt(d);   // every thread: the same value
       __syncthreads();
-      if (tid < a - j) {
-        L[j + tid][j] = tid == 0 ? piv : L[j + tid][j] * inv;
-        if (tid == 0) rp[j] = inv;
-      }
+      if (tid < a - j) L[j + tid][j] = tid == 0 ? piv : L[j + tid][j] / piv;
       if (warp == 0 && lane == j) ld = log(piv);
       __syncthreads();
       for (int k = j + 1 + warp; k < a; k += kTipThreads / 32)   // column k, lane = row
@@ -75,7 +72,7 @@ __global__ void __launch_bounds__(kTipThreads)
         double s = lane < a ? r[lane] - vT[lane] : 0.0;
         if (vT2 && lane < a) s -= vT2[lane];
         for (int k = 0; k < a; ++k) {
-          const double v = __shfl_sync(0xffffffffu, s, k) * rp[k];
+          const double v = __shfl_sync(0xffffffffu, s, k) / L[k][k];
           if (lane == k) s = v;
           else if (lane > k && lane < a) s = fma(-L[lane][k], v, s);
         }
@@ -84,13 +81,11 @@ __global__ void __launch_bounds__(kTipThreads)
     }
     return;
   }
-  if (tid < a) rp[tid] = 1.0 / L[tid][tid];
-  __syncthreads();
   if (mode == 1) {
     if (warp == 0) {
       double s = lane < a ? r[lane] : 0.0;
       for (int k = a - 1; k >= 0; --k) {
-        const double v = __shfl_sync(0xffffffffu, s, k) * rp[k];
+        const double v = __shfl_sync(0xffffffffu, s, k) / L[k][k];
         if (lane == k) s = v;
         else if (lane < k) s = fma(-L[k][lane], v, s);
       }
@@ -101,11 +96,11 @@ __global__ void __launch_bounds__(kTipThreads)
   // W = L^{-1} (lower): thread = column; then Z = W^T W
   __shared__ double W[kMaxTip][kMaxTip + 1];
   if (tid < a) {
-    for (int i = 0; i < a; ++i) W[i][tid] = i == tid ? rp[i] : 0.0;
+    for (int i = 0; i < a; ++i) W[i][tid] = i == tid ? 1.0 / L[i][i] : 0.0;
     for (int i = tid + 1; i < a; ++i) {
       double s = 0.0;
       for (int k = tid; k < i; ++k) s = fma(L[i][k], W[k][tid], s);
-      W[i][tid] = -s * rp[i];
+      W[i][tid] = -s / L[i][i];
     }
   }
   __syncthreads();
@@ -701,14 +696,13 @@ namespace {
 __global__ void tip_fwd_kernel(int a, const double* T, double* r, const double* vT,
                                const double* vT2) {
   const int lane = threadIdx.x;
-  double s = 0.0, inv = 0.0;
+  double s = 0.0;
   if (lane < a) {
     s = r[lane] - vT[lane];
     if (vT2) s -= vT2[lane];
-    inv = 1.0 / T[lane + lane * a];
   }
   for (int k = 0; k < a; ++k) {
-    const double v = __shfl_sync(0xffffffffu, s * inv, k);
+    const double v = __shfl_sync(0xffffffffu, s, k) / T[k + k * a];
     if (lane == k) s = v;
     else if (lane > k && lane < a) s = fma(-T[lane + k * a], v, s);
   }

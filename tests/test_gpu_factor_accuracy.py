@@ -50,3 +50,31 @@ def test_graded_blocks_up_to_512_rows_as_in_fp64(P, b, precision):
     ref = _factor(P, D)
     got = _factor(P, D, precision=precision)
     assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("a", [1, 7, 32])
+def test_tip_divides_by_its_pivots(P, a):
+    """Correctly rounded quotients in the tip's factor and solves (a rounded reciprocal
+    would cost a second rounding): a diagonal tip's solutions and a first column of L_T are
+    those of IEEE division and square root."""
+    import torch
+    rng = np.random.default_rng(a)
+    eye = np.eye(32)
+    for _ in range(8):
+        t = np.exp(rng.uniform(-9, 9, a))
+        r = np.concatenate([np.zeros(32), rng.standard_normal(a)])
+        _, _, q, z = _factor(P, eye, np.diag(t), r)
+        z_ref = r[32:] / np.sqrt(t)
+        assert np.array_equal(z[32:], z_ref)
+        x = torch.from_numpy(z).cuda()
+        P.bta_solve(q, x)
+        assert np.array_equal(x.cpu().numpy()[32:], z_ref / np.sqrt(t))
+        zl = torch.from_numpy(r).cuda()                  # the lower solve on its own
+        P.bta_solve(q, zl, lower=True)
+        assert np.array_equal(zl.cpu().numpy(), x.cpu().numpy())
+        T = np.diag(np.full(a, 1e3))
+        T[0, 0] = np.exp(rng.uniform(-1, 1))
+        T[1:, 0] = T[0, 1:] = rng.standard_normal(a - 1)
+        _, _, q, _ = _factor(P, eye, T)
+        L = q.T.cpu().numpy().reshape(a, a).T            # column-major
+        assert np.array_equal(L[1:, 0], T[1:, 0] / np.sqrt(T[0, 0]))
