@@ -16,6 +16,7 @@
 // and replayed.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <functional>
 #include <memory>
@@ -37,16 +38,20 @@ struct EvalCtx {
   double *PDc = nullptr, *PBc = nullptr, *PCc = nullptr, *PDp = nullptr, *PBp = nullptr;
   double *QD = nullptr, *QB = nullptr, *RS = nullptr;
   double* out = nullptr;
-  SweepWs wsc, wsp, wsc2, wsp2;   // forward and reverse legs
+  // forward legs of Q_c and Q_p, then the reverse ones (null until a call takes them)
+  SweepWs legs[4];
+  void* tc[3][4] = {};            // [precision][leg]: operand copies (null until used)
+  int group[3] = {};              // SweepWs::tcgroup of tc[precision]
   double* tip2 = nullptr;         // the reverse leg's share of Q_c's tip
   SelinvFuse fc, fp;
   double* dr = nullptr;         // mixed mode: refinement residual / correction
   double* red = nullptr;        // sums of the final combination
-  int have_factors = 0;         // last evaluation was value-only: factors still held
+  int have_factors = 0;         // last evaluation was value-only: factors still held ...
+  int reverse = 0;              // ... of so many blocks in the reverse legs
 };
 
 struct GraphKey {
-  int mode, count, precision;
+  int mode, count, precision, reverse;
   cudaGraphExec_t exec;
   int64_t kernels;
 };
@@ -78,9 +83,12 @@ struct inla_model {
   cudaEvent_t evv5 = nullptr, evv6 = nullptr, evjv = nullptr, evmv = nullptr, evs5 = nullptr,
               evs6 = nullptr, ev5 = nullptr;
   cudaEvent_t evj = nullptr;    // join event of a multi-model graph
+  int small[3] = {};            // [precision]: form of the workspaces (kFormGroup)
   // blocks of the reverse legs: both ends meet in the middle
   // (mixed precision keeps the forward order: see group_program)
-  int reverse_blocks(int prec) const { return n >= 3 && prec != 1 ? (n - 1) / 2 : 0; }
+  int reverse_blocks(int prec) const {
+    return n >= 3 && prec != 1 && !small[prec] ? (n - 1) / 2 : 0;
+  }
 };
 
 // Several models evaluated by one CUDA graph (see inla_batch_value_and_grad).
@@ -88,6 +96,7 @@ struct inla_batch {
   std::vector<inla_model*> models;
   cudaGraphExec_t exec[2][3] = {};   // [grad][precision]
   int64_t kernels[2][3] = {};
+  std::vector<int> reverse[2][3];   // of each model, in exec
   cudaEvent_t fork = nullptr;
 };
 
@@ -118,6 +127,20 @@ bool finite_theta(const double* th, int d) {
   for (int i = 0; i < d; ++i)
     if (!std::isfinite(th[i])) return false;
   return true;
+}
+
+// Free what was allocated since the model held `mark` buffers.
+void roll_back(inla_model* m, size_t mark) {
+  for (; m->allocs.size() > mark; m->allocs.pop_back()) cudaFree(m->allocs.back());
+}
+
+// Work blocks of a context's legs first and first + 1 (Q_c's and Q_p's).
+void leg_carve(const inla_model* m, EvalCtx& c, int first, double* buf) {
+  const size_t wsb = SweepWs::bytes(m->ld, m->a) / sizeof(double);
+  for (int q = 0; q < 2; ++q) {
+    c.legs[first + q].carve(buf + q * wsb, m->ld, m->a);
+    c.legs[first + q].tcstat = c.fail + 2;
+  }
 }
 
 // Allocate evaluation context c (buffers for Q_c, Q_p, x*, reductions).
@@ -155,20 +178,9 @@ bta_status ctx_alloc(inla_model* m, EvalCtx& c) {
   BTA_TRY(dmalloc(m, &c.RS, (size_t)kMaxK * resid_chunks(md)));
   BTA_TRY(dmalloc(m, &c.out, out_size(md.d)));
   BTA_TRY(dmalloc(m, &c.red, kRedDoubles));
-  const int legs = m->reverse_blocks(0) > 0 ? 4 : 2;
-  SweepWs* const ws[4] = {&c.wsc, &c.wsp, &c.wsc2, &c.wsp2};
-  const size_t wsb = SweepWs::bytes(ld, a) / sizeof(double);
-  double* wsbuf = nullptr;
-  BTA_TRY(dmalloc(m, &wsbuf, legs * wsb));
-  // tensor-core modes: operand copies of the tensor-core products, one per leg
-  const size_t tcb = sweep_tc_ws_bytes(ld, a);
-  uint8_t* tcbuf = nullptr;
-  BTA_TRY(dmalloc(m, &tcbuf, legs * tcb));
-  for (int q = 0; q < legs; ++q) {
-    ws[q]->carve(wsbuf + q * wsb, ld, a);
-    ws[q]->tc = tcbuf + q * tcb;
-    ws[q]->tcstat = c.fail + 2;
-  }
+  double* wsbuf = nullptr;   // every evaluation takes the forward legs
+  BTA_TRY(dmalloc(m, &wsbuf, 2 * SweepWs::bytes(ld, a) / sizeof(double)));
+  leg_carve(m, c, 0, wsbuf);
   BTA_TRY(dmalloc(m, &c.tip2, std::max(a * a, 1)));
   BTA_TRY(dmalloc(m, &c.dr, (size_t)nt * ld + a));
   c.fc.md = &m->md; c.fc.counts = 1; c.fc.PD = c.PDc; c.fc.PB = c.PBc; c.fc.PC = c.PCc;
@@ -182,9 +194,11 @@ bta_status ensure_ctx(inla_model* m, int count) {
   m->ctx.reserve(count);
   while ((int)m->ctx.size() < count) {
     m->ctx.emplace_back();
+    const size_t mark = m->allocs.size();
     bta_status st = ctx_alloc(m, m->ctx.back());
     if (st != BTA_OK) {
       m->ctx.pop_back();
+      roll_back(m, mark);
       return st;
     }
   }
@@ -192,9 +206,87 @@ bta_status ensure_ctx(inla_model* m, int count) {
   return BTA_OK;
 }
 
+// The workspaces of an evaluation in a precision: a context's legs take three work blocks
+// each, and in the tensor-core modes their products' operand copies (emulated: 84 bytes an
+// entry of a block, as much as ten blocks).  They are allocated when a call first needs them, outside
+// capture.  The smaller forms have one leg per matrix and hold the planes of seven moduli at
+// once (56 bytes an entry), or of four (44).  They are taken in turn where the one before does
+// not fit the device, so that a model whose matrices leave little room is evaluated all the
+// same; low-memory models whose full form would exceed kLowMemoryWork begin with the first of
+// them (b = 4800 emulated, 5 blocks: 3.5 GiB instead of 9.5, gradient 126 ms instead of 113).
+// BTA_SMALL_WORKSPACES = 1 or 2 asks for one.
+constexpr size_t kLowMemoryWork = (size_t)1 << 30;
+constexpr int kWorkForms = 3;
+constexpr int kFormGroup[kWorkForms] = {kOzakiModuli, 7, kOzakiSmallGroup};
+
+size_t work_bytes(const inla_model* m, int prec) {
+  const size_t legs = m->reverse_blocks(prec) > 0 ? 4 : 2;
+  return legs * (SweepWs::bytes(m->ld, m->a) +
+                 (prec ? sweep_tc_ws_bytes(m->ld, m->a, prec) : 0));
+}
+
+// Allocates what contexts 0..count-1 lack, or nothing.
+bta_status try_workspaces(inla_model* m, int count, int prec) {
+  const int legs = m->reverse_blocks(prec) > 0 ? 4 : 2;
+  const int group = kFormGroup[m->small[prec]];
+  const size_t tcb = prec ? sweep_tc_ws_bytes(m->ld, m->a, prec, group) : 0;
+  const size_t wsb = 2 * SweepWs::bytes(m->ld, m->a) / sizeof(double);
+  const size_t mark = m->allocs.size();
+  struct Got {
+    double* legs = nullptr;
+    uint8_t* tc[4] = {};
+  };
+  std::vector<Got> got(count);
+  bta_status st = BTA_OK;
+  for (int e = 0; e < count && st == BTA_OK; ++e) {
+    EvalCtx& c = m->ctx[e];
+    if (legs == 4 && !c.legs[2].W1) st = dmalloc(m, &got[e].legs, wsb);
+    // (where the emulated mode has its areas, the mixed mode's products fit into them)
+    if (prec == 1 && !c.tc[1][0] && c.tc[2][0] &&
+        tcb <= sweep_tc_ws_bytes(m->ld, m->a, 2, c.group[2]))
+      for (int q = 0; q < 2; ++q) got[e].tc[q] = static_cast<uint8_t*>(c.tc[2][q]);
+    for (int q = 0; q < legs && st == BTA_OK; ++q)
+      if (!c.tc[prec][q] && !got[e].tc[q]) st = dmalloc(m, &got[e].tc[q], tcb);
+  }
+  if (st != BTA_OK) {
+    roll_back(m, mark);
+    return st;
+  }
+  for (int e = 0; e < count; ++e) {
+    EvalCtx& c = m->ctx[e];
+    if (got[e].legs) leg_carve(m, c, 2, got[e].legs);
+    for (int q = 0; q < 4; ++q)
+      if (got[e].tc[q]) c.tc[prec][q] = got[e].tc[q];
+    if (!c.group[prec]) c.group[prec] = group;
+  }
+  return BTA_OK;
+}
+
+bta_status ensure_workspaces(inla_model* m, int count, int prec) {
+  const int form = m->small[prec];
+  bta_status st = try_workspaces(m, count, prec);
+  while (st == BTA_ERR_NOMEM && prec != 1 && m->small[prec] + 1 < kWorkForms) {
+    ++m->small[prec];
+    st = try_workspaces(m, count, prec);
+  }
+  if (st != BTA_OK) m->small[prec] = form;   // (fewer thetas go on in the larger form)
+  return st;
+}
+
+// The workspace of a context's leg in a precision.
+SweepWs leg_ws(const EvalCtx& c, int q, int prec) {
+  SweepWs ws = c.legs[q];
+  if (prec) {
+    ws.tc = c.tc[prec][q];
+    ws.tcgroup = c.group[prec];
+  }
+  return ws;
+}
+
 // The evaluation of contexts 0..cnt-1 as a list of issue steps.
 //   mode 0: f only; 1: f and gradient; 2: reverse pass of a preceding mode-0
 //   evaluation (the factors are still in place).
+//   nb: blocks of the reverse legs (reverse_blocks; mode 2: those of the factors held).
 // The conditional matrices Q_c of all contexts form one set and the priors
 // Q_p another; each set is swept with one batched launch per block step.  Each set
 // is eliminated from both ends towards the middle block (SweepItem: a forward and a
@@ -217,19 +309,18 @@ struct GroupSets {
   std::vector<SweepItem> jc, jp;   // reverse legs (empty below three blocks)
 };
 
-bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_t s0,
+bta_status group_program(inla_model* m, int mode, int cnt, int prec, int nb, cudaStream_t s0,
                          std::vector<IssueStep>& steps) {
   const ModelDev& md = m->md;
-  const int grad = mode >= 1, nt = md.nt;
-  const int nb = m->reverse_blocks(prec), mid = nt - 1 - nb;
+  const int grad = mode >= 1, nt = md.nt, mid = nt - 1 - nb;
   auto sets = std::make_shared<GroupSets>();
   for (int e = 0; e < cnt; ++e) {
     EvalCtx& c = m->ctx[e];
     SweepItem ic, ip;
     ic.q = c.qc; ic.vec = c.x; ic.slots = c.slots_c; ic.fail = c.fail;
-    ic.ws = c.wsc; ic.fuse = &c.fc;
+    ic.ws = leg_ws(c, 0, prec); ic.fuse = &c.fc;
     ip.q = c.qp; ip.vec = nullptr; ip.slots = c.slots_p; ip.fail = c.fail + 1;
-    ip.ws = c.wsp; ip.fuse = &c.fp;
+    ip.ws = leg_ws(c, 1, prec); ip.fuse = &c.fp;
     ic.md = ip.md = &md;
     ic.lay = ip.lay = &m->L;
     ic.coef = ip.coef = c.coefbuf;
@@ -238,12 +329,12 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
       ic.len = ip.len = mid + 1;
       jc.rev = jp.rev = 1;
       jc.len = jp.len = nb + 1;
-      jc.ws = c.wsc2;
-      jp.ws = c.wsp2;
+      jc.ws = leg_ws(c, 2, prec);
+      jp.ws = leg_ws(c, 3, prec);
       if (md.a > 0) {
         jc.tip = c.tip2;
         ic.tip2 = c.tip2;
-        ic.vT2 = c.wsc2.vT;
+        ic.vT2 = jc.ws.vT;
       }
       sets->jc.push_back(jc);
       sets->jp.push_back(jp);
@@ -444,9 +535,9 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, cudaStream_
 }
 
 // Record (issue, or capture) the evaluation of contexts 0..cnt-1.
-bta_status record_group(inla_model* m, int mode, int cnt, int prec, cudaStream_t s0) {
+bta_status record_group(inla_model* m, int mode, int cnt, int prec, int nb, cudaStream_t s0) {
   std::vector<IssueStep> steps;
-  BTA_TRY(group_program(m, mode, cnt, prec, s0, steps));
+  BTA_TRY(group_program(m, mode, cnt, prec, nb, s0, steps));
   for (auto& st : steps) BTA_TRY(st());
   return BTA_OK;
 }
@@ -472,6 +563,7 @@ bta_status worse(bta_status a, bta_status b) {
 bta_status run_group(inla_model* m, int mode, int cnt, int prec, int use_graph,
                      cudaStream_t stream) {
   const int d = m->d, no = out_size(d);
+  const int nb = mode < 2 ? m->reverse_blocks(prec) : m->ctx[0].reverse;
   if (mode < 2)
     for (int e = 0; e < cnt; ++e)
       BTA_CUDA_TRY(cudaMemcpyAsync(m->ctx[e].coefbuf + m->L.theta, m->htheta + (size_t)e * d,
@@ -479,20 +571,20 @@ bta_status run_group(inla_model* m, int mode, int cnt, int prec, int use_graph,
   if (use_graph) {
     GraphKey* gk = nullptr;
     for (auto& g : m->graphs)
-      if (g.mode == mode && g.count == cnt && g.precision == prec) gk = &g;
+      if (g.mode == mode && g.count == cnt && g.precision == prec && g.reverse == nb) gk = &g;
     if (!gk) {
       if (mode < 2) {
         // one eager evaluation first: it times the tile shapes of the
         // products the graph will hold, which then replays those choices
         TuneScope tune;
-        BTA_TRY(record_group(m, mode, cnt, prec, stream));
+        BTA_TRY(record_group(m, mode, cnt, prec, nb, stream));
         BTA_CUDA_TRY(cudaStreamSynchronize(stream));
       }
       const int64_t before = g_launches;
       cudaStream_t cap;
       BTA_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
       BTA_CUDA_TRY(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-      bta_status st = record_group(m, mode, cnt, prec, cap);
+      bta_status st = record_group(m, mode, cnt, prec, nb, cap);
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamEndCapture(cap, &graph);
       if (st != BTA_OK) {
@@ -506,14 +598,14 @@ bta_status run_group(inla_model* m, int mode, int cnt, int prec, int use_graph,
       cudaGraphDestroy(graph);
       cudaStreamDestroy(cap);
       BTA_CUDA_TRY(e);
-      m->graphs.push_back({mode, cnt, prec, exec, g_launches - before});
+      m->graphs.push_back({mode, cnt, prec, nb, exec, g_launches - before});
       gk = &m->graphs.back();
     }
     BTA_CUDA_TRY(cudaGraphLaunch(gk->exec, stream));
     m->launched += gk->kernels;
   } else {
     const int64_t before = g_launches;
-    BTA_TRY(record_group(m, mode, cnt, prec, stream));
+    BTA_TRY(record_group(m, mode, cnt, prec, nb, stream));
     m->launched += g_launches - before;
   }
   for (int e = 0; e < cnt; ++e)
@@ -527,6 +619,7 @@ bta_status run_group(inla_model* m, int mode, int cnt, int prec, int use_graph,
     const double* parts = m->hout + (size_t)e * no + 1 + d;
     st = worse(st, eval_status(parts, tcs));
     m->ctx[e].have_factors = mode == 0 ? 1 + prec : 0;   // remembers the factor's precision
+    m->ctx[e].reverse = nb;
   }
   m->last.assign(m->hout + (size_t)(cnt - 1) * no, m->hout + (size_t)cnt * no);
   return st;
@@ -656,6 +749,10 @@ static bta_status model_create_impl(const inla_model_spec* sp, inla_model* m) {
   // --- evaluation buffers: one context up front, more on demand
   m->L.init(k, md.d, nt);
   m->nslots = logdet_slots(nt, ld);
+  const char* env = std::getenv("BTA_SMALL_WORKSPACES");
+  const int form = env ? std::min(std::max(std::atoi(env), 0), kWorkForms - 1) : 0;
+  for (int prec : {0, 2})   // (the mixed mode has one form)
+    m->small[prec] = std::max(form, m->lowmem && work_bytes(m, prec) > kLowMemoryWork ? 1 : 0);
   BTA_TRY(ensure_ctx(m, 1));
   BTA_CUDA_TRY(cudaMallocHost(&m->hout, (size_t)kMaxBatch * out_size(md.d) * sizeof(double)));
   BTA_CUDA_TRY(cudaMallocHost(&m->htheta, (size_t)kMaxBatch * kMaxD * sizeof(double)));
@@ -735,13 +832,20 @@ bta_status bta_factor(bta_desc* q, double* rhs_inout, double* logdet, int32_t* f
   const int nsl = logdet_slots(q->n, q->ld);
   const size_t wsb = SweepWs::bytes(q->ld, q->a);
   const int ld = q->ld;
-  // tensor-core modes: operand copies of the b x b products (split TF32
-  // planes or BF16 residue planes, whichever is larger), 256-byte aligned
-  const size_t tcb = precision ? sweep_tc_ws_bytes(ld, q->a) : 0;
+  // tensor-core modes: operand copies of the b x b products, 256-byte aligned; the residue
+  // planes of fewer moduli at once where all of them do not fit the device
   const size_t head = (wsb + nsl * sizeof(double) + 255) / 256 * 256;
   uint8_t* buf = nullptr;
-  BTA_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&buf), head + tcb, stream));
   SweepWs ws;
+  cudaError_t e = cudaSuccess;
+  for (int group : {kOzakiModuli, kOzakiSmallGroup}) {
+    const size_t tcb = precision ? sweep_tc_ws_bytes(ld, q->a, precision, group) : 0;
+    e = cudaMallocAsync(reinterpret_cast<void**>(&buf), head + tcb, stream);
+    ws.tcgroup = group;
+    if (e != cudaErrorMemoryAllocation || precision != 2) break;
+    if (group != kOzakiSmallGroup) cudaGetLastError();
+  }
+  BTA_CUDA_TRY(e);
   ws.carve(reinterpret_cast<double*>(buf), ld, q->a);
   double* slots = reinterpret_cast<double*>(buf) + wsb / sizeof(double);
   if (precision) {
@@ -889,6 +993,7 @@ bta_status inla_value_and_grad(inla_model* m, const double* theta, int32_t batch
   int group = opts && opts->streams > 1 ? opts->streams : 1;
   group = std::min(group, std::min<int>(batch, kMaxBatch / 2));
   BTA_TRY(ensure_ctx(m, group));
+  BTA_TRY(ensure_workspaces(m, group, prec));
   const int mode = grad ? 1 : 0;
   const int d = m->d, no = out_size(d);
   bta_status st = BTA_OK;
@@ -1039,7 +1144,7 @@ static bta_status record_batch(inla_batch* b, int grad, int prec, cudaStream_t s
     BTA_CUDA_TRY(cudaStreamWaitEvent(m->s0, b->fork, 0));
     BTA_CUDA_TRY(cudaMemcpyAsync(m->ctx[0].coefbuf + m->L.theta, m->htheta,
                                  m->d * sizeof(double), cudaMemcpyHostToDevice, m->s0));
-    BTA_TRY(group_program(m, grad, 1, prec, m->s0, progs[k]));
+    BTA_TRY(group_program(m, grad, 1, prec, b->reverse[grad][prec][k], m->s0, progs[k]));
     longest = std::max(longest, progs[k].size());
   }
   for (size_t j = 0; j < longest; ++j)
@@ -1069,6 +1174,11 @@ bta_status inla_batch_value_and_grad(inla_batch* b, const double* theta, int32_t
     std::memcpy(m->htheta, theta + (size_t)i * ldt, m->d * sizeof(double));
   }
   if (!b->exec[g][prec]) {
+    b->reverse[g][prec].clear();
+    for (inla_model* m : b->models) {
+      BTA_TRY(ensure_workspaces(m, 1, prec));
+      b->reverse[g][prec].push_back(m->reverse_blocks(prec));
+    }
     {  // an eager run first times the products' tile shapes (see run_group)
       TuneScope tune;
       BTA_TRY(record_batch(b, g, prec, stream));
@@ -1103,6 +1213,7 @@ bta_status inla_batch_value_and_grad(inla_batch* b, const double* theta, int32_t
     BTA_CUDA_TRY(cudaMemcpy(&tcs, m->ctx[0].fail + 2, sizeof(int32_t), cudaMemcpyDeviceToHost));
     m->last.assign(m->hout, m->hout + no);
     m->ctx[0].have_factors = g ? 0 : 1 + prec;
+    m->ctx[0].reverse = b->reverse[g][prec][i];
     m->launched += b->kernels[g][prec] / nm;
     f[i] = m->hout[0];
     if (grad)

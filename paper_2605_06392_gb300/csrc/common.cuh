@@ -220,9 +220,13 @@ size_t tc_gemm_ws_bytes(int M, int N, int K);
 // (ozaki_gemm.cu); single problem, K <= kOzakiMaxK.
 constexpr int kOzakiMaxK = 5120;
 // marks (optional): events recorded around the tensor-core product kernel.
+// group: moduli whose operand planes the workspace holds at once; the products are taken
+// group by group, to the same bits.  A plane of each operand and of the result takes 2
+// bytes an entry: 84 bytes an entry of a square product with all 14, 44 with 4.
+constexpr int kOzakiModuli = 14, kOzakiSmallGroup = 4;
 bta_status ozaki_gemm(const Gemm& g, void* ws, int32_t* status, cudaStream_t s,
-                      const cudaEvent_t* marks = nullptr);
-size_t ozaki_ws_bytes(int M, int N, int K);
+                      const cudaEvent_t* marks = nullptr, int group = kOzakiModuli);
+size_t ozaki_ws_bytes(int M, int N, int K, int group = kOzakiModuli);
 bool ozaki_supported(const Gemm& g);
 
 // ----------------------------------------------------------------------------
@@ -244,7 +248,8 @@ int potrf_inv_slots(int n);   // number of logdet slots potrf_inv writes
 // rows the block is split 2 x 2 recursively, the diagonal sub-blocks factored
 // by the task-graph kernel and the products of each level run in FP64
 // (precision 0) or emulated FP64 (precision 1, 2; per-block workspace tcws of
-// ozaki_ws_bytes(n, n, n) bytes and status words tcstat).
+// potrf_tc_ws_bytes(n) bytes and status words tcstat).
+size_t potrf_tc_ws_bytes(int n);
 bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
                                 double* const* scratch, double* const* logdet_parts,
                                 int32_t* const* fail, const int32_t* fail_code, int precision,

@@ -8,13 +8,12 @@
 // that forbids allocation calls on its hot path, and code that cannot
 // afford the device-wide synchronisation that freeing memory may imply.
 // They pass in their inputs and outputs as usual; the temporary blocks the
-// sweep needs (three ld x ld work blocks, the diagonal-factor scratch, arrow
-// blocks, GEMV partials and the per-leaf log-determinant slots) live in the
-// static array below instead of a per-call allocation.
+// sweep needs (three ld x ld work blocks, an arrow block, a vector and the per-leaf
+// log-determinant slots) live in the static array below instead of a per-call allocation.
 //
 // Limits (checked, BTA_ERR_ARG beyond them): ld <= 256, a <= 32, and
 // n * (ld / 32) + 1 <= 16384 log-determinant slots (n <= 2047 at ld = 256).
-// The array holds 2.4 MB and, once reserved on a GPU, stays there until the
+// The array holds 1.8 MB and, once reserved on a GPU, stays there until the
 // process exits.
 //
 // Sharing: all calls on a device use the same array.  Calls that overlap on
@@ -41,8 +40,8 @@ constexpr int kNoAllocMaxLd = 256;
 constexpr int kNoAllocMaxA = 32;
 constexpr int kNoAllocMaxSlots = 16384;
 // Work area of one sweep at the maximum sizes, in doubles (see SweepWs):
-// 4 ld^2 + a ld + ld + a + 64, rounded up to a multiple of 32.
-constexpr size_t kWorkDoubles = 4 * (size_t)kNoAllocMaxLd * kNoAllocMaxLd +
+// 3 ld^2 + a ld + ld + a + 64, rounded up to a multiple of 32.
+constexpr size_t kWorkDoubles = 3 * (size_t)kNoAllocMaxLd * kNoAllocMaxLd +
                                 (size_t)kNoAllocMaxA * kNoAllocMaxLd + kNoAllocMaxLd +
                                 kNoAllocMaxA + 64 + 31;
 constexpr size_t kScratchDoubles = kWorkDoubles + kNoAllocMaxSlots;

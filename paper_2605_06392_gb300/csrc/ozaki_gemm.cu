@@ -45,7 +45,7 @@ using namespace tc;
 
 // ---- moduli ------------------------------------------------------------------
 // The 14 pairwise coprime numbers up to 511 with the largest product.
-constexpr int kNumMod = 14;
+constexpr int kNumMod = kOzakiModuli;
 constexpr int kMod[kNumMod] = {511, 509, 508, 505, 503, 501, 499,
                                493, 491, 487, 481, 479, 473, 467};
 constexpr int kMaxK56 = 4847;   // 2 K 2^112 <= P
@@ -408,12 +408,13 @@ struct CrtArgs {
   int lower;            // only tiles that reach the lower triangle
   int tri_a, tri_b;     // triangle of op(A) / op(B) (Tri): their zero K ranges are skipped
   int slots, per;       // pairs resident together; units per pair
+  int mod0, nmod;       // the moduli whose planes these are (ozaki_gemm: group)
   uint16_t* R;          // [kNumMod][Np][Mp] residues + kBias
   int32_t* status;
 };
 
 struct CrtUnit {
-  int mod, m0, n0, ks0, ks1;
+  int mod, m0, n0, ks0, ks1;   // mod: among the launch's moduli
 };
 
 // Unit u of CT x CT tiles: modulus-major, so that the resident pairs work on the planes of one
@@ -462,7 +463,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
                     const __grid_constant__ CUtensorMap mB, CrtArgs g) {
   const uint32_t rank = cluster_rank();
   // unit j of this pair: pairs launched together take consecutive units
-  const int pair = (int)blockIdx.x >> 1, total = g.tiles * kNumMod;
+  const int pair = (int)blockIdx.x >> 1, total = g.tiles * g.nmod;
   const int u0 = (pair / g.slots) * g.per * g.slots + pair % g.slots;
   if (u0 >= total) return;   // the same decision in both CTAs, before any set-up
   const int units = min(g.per, (total - u0 + g.slots - 1) / g.slots);
@@ -600,7 +601,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
     int e = 0;
     for (int j = 0; j < units && !failed; ++j) {
       const CrtUnit t = crt_unit<CT>(g, u0 + j * g.slots);
-      const CrtMod mod(t.mod);
+      const CrtMod mod(g.mod0 + t.mod);
       uint64_t acc[64];
 #pragma unroll
       for (int q = 0; q < 64; ++q) acc[q] = 0ull;
@@ -623,7 +624,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCrtThreads, 1)
       }
       if (failed) break;
       // a warp's lanes are 32 consecutive rows
-      crt_store(g.R + ((int64_t)t.mod * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp, acc);
+      crt_store(g.R + ((int64_t)(g.mod0 + t.mod) * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp,
+                acc);
     }
     if (failed && lane == 0) atomicExch(&s_abort, 1);
   }
@@ -792,7 +794,7 @@ __global__ void __launch_bounds__(kCrtThreads, 2)
     // ---- warps 0-7: thread = output row (TMEM lane) x 64 columns
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const int row = (warp & 3) * 32 + lane, col0 = (warp >> 2) * 64;
-    const CrtMod mod(t.mod);
+    const CrtMod mod(g.mod0 + t.mod);
     bool failed = false;
     uint64_t acc[32];
 #pragma unroll
@@ -816,7 +818,8 @@ __global__ void __launch_bounds__(kCrtThreads, 2)
       });
     }
     if (!failed)
-      crt_store(g.R + ((int64_t)t.mod * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp, acc);
+      crt_store(g.R + ((int64_t)(g.mod0 + t.mod) * g.Np + t.n0 + col0) * g.Mp + t.m0 + row, g.Mp,
+                acc);
     else if (lane == 0)
       atomicExch(&s_abort, 1);
   }
@@ -1038,6 +1041,7 @@ struct SplitArgs {
   int bits;   // of the integers F (see the file's head)
   int eblocks;   // partial maxima per row (0: ex holds the exponents)
   int tile;      // of the products
+  int mod0, nmod;   // the moduli whose planes are written
 };
 
 // The block of op(X) at (r0, k0), 8 elements a thread: thread t holds (r, k) = (t & 15,
@@ -1136,26 +1140,30 @@ __device__ __forceinline__ void fixed_digits(double v, int er, int bits, float (
 // congruent to F and |t| < 2^23 (|d3| <= 2^14, the others 2^13, |c| <= 255), so every
 // FP32 step is exact and the rounded quotient the nearest one (the error of t / p is
 // below 2^-24 |t| / p < 1 / (2 p)): |r| <= (p - 1) / 2, or p / 2 for the even modulus.
-template <int I>
+// All: of every modulus; else of nmod moduli from mod0 on (y: the plane of mod0).
+template <bool All, int I>
 __device__ __forceinline__ void residue_planes(const uint64_t (&d)[4][4], __nv_bfloat16* y,
-                                               size_t plane) {
+                                               size_t plane, int mod0, int nmod) {
   if constexpr (I < kNumMod) {
-    using Q = Modulus<I>;
-    const uint64_t c1 = pack2(Q::c1, Q::c1), c2 = pack2(Q::c2, Q::c2), c3 = pack2(Q::c3, Q::c3);
-    const uint64_t inv = pack2(Q::inv, Q::inv), np = pack2(-Q::p, -Q::p);
-    const uint64_t magic = pack2(kMagic, kMagic), nmagic = pack2(-kMagic, -kMagic);
-    uint32_t w[4];
+    if (All || (unsigned)(I - mod0) < (unsigned)nmod) {
+      using Q = Modulus<I>;
+      const uint64_t c1 = pack2(Q::c1, Q::c1), c2 = pack2(Q::c2, Q::c2), c3 = pack2(Q::c3, Q::c3);
+      const uint64_t inv = pack2(Q::inv, Q::inv), np = pack2(-Q::p, -Q::p);
+      const uint64_t magic = pack2(kMagic, kMagic), nmagic = pack2(-kMagic, -kMagic);
+      uint32_t w[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint64_t t = fma2(d[3][e], c3, fma2(d[2][e], c2, fma2(d[1][e], c1, d[0][e])));
-      const uint64_t k = add2(fma2(t, inv, magic), nmagic);
-      float r0, r1;
-      unpack2(fma2(k, np, t), r0, r1);
-      // at most 8 significant bits: the BF16 pattern is the upper half
-      w[e] = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
+      for (int e = 0; e < 4; ++e) {
+        const uint64_t t = fma2(d[3][e], c3, fma2(d[2][e], c2, fma2(d[1][e], c1, d[0][e])));
+        const uint64_t k = add2(fma2(t, inv, magic), nmagic);
+        float r0, r1;
+        unpack2(fma2(k, np, t), r0, r1);
+        // at most 8 significant bits: the BF16 pattern is the upper half
+        w[e] = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
+      }
+      *reinterpret_cast<uint4*>(y + (All ? I : I - mod0) * plane) =
+          make_uint4(w[0], w[1], w[2], w[3]);
     }
-    *reinterpret_cast<uint4*>(y + I * plane) = make_uint4(w[0], w[1], w[2], w[3]);
-    residue_planes<I + 1>(d, y, plane);
+    residue_planes<All, I + 1>(d, y, plane, mod0, nmod);
   }
 }
 
@@ -1169,6 +1177,7 @@ __device__ __forceinline__ void residue_planes(const uint64_t (&d)[4][4], __nv_b
 // banks.
 __device__ __forceinline__ int split_swz(int q, int c) { return c ^ ((q ^ (c >> 3)) & 15); }
 
+template <bool All>
 __global__ void __launch_bounds__(kElemThreads) residue_kernel(SplitArgs a) {
   const SplitOp o = blockIdx.z == 0 ? a.op[0] : a.op[1];
   const int r0 = blockIdx.x * kElemRows, k0 = blockIdx.y * CK;
@@ -1227,10 +1236,11 @@ __global__ void __launch_bounds__(kElemThreads) residue_kernel(SplitArgs a) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) d[j][e / 2] = pack2(x[j], y[j]);
   }
-  residue_planes<0>(d, o.Y + ((size_t)blockIdx.y * o.rowsP + r) * 64 + 8 * g, plane);
+  residue_planes<All, 0>(d, o.Y + ((size_t)blockIdx.y * o.rowsP + r) * 64 + 8 * g, plane, a.mod0,
+                         a.nmod);
 }
 
-// 2D map over Y viewed as rowsAll = kNumMod * slabs * rowsP rows of 64 BF16, box 128 rows.
+// 2D map over Y viewed as rowsAll = moduli * slabs * rowsP rows of 64 BF16, box 128 rows.
 bta_status make_map_bf16(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map,
                          const __nv_bfloat16* base, int rowsAll) {
   cuuint64_t dims[2] = {(cuuint64_t)CK, (cuuint64_t)rowsAll};
@@ -1283,19 +1293,19 @@ int crt_tile(int M, int N) {
 struct OzLayout {
   int Mp, Np, Kp, eblocks;
   size_t a_off, b_off, ea_off, eb_off, pa_off, pb_off, r_off, total;
-  OzLayout(int M, int N, int K, int tile) {
+  OzLayout(int M, int N, int K, int tile, int group) {
     Mp = cdiv(M, tile) * tile;
     Np = cdiv(N, tile) * tile;
     Kp = cdiv(K, CK) * CK;
     eblocks = K <= kPartialK ? cdiv(K, CK) : 0;
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     b_off = 0;   // B's part first: where it lies does not depend on M (Gemm::b_kept)
-    pb_off = up((size_t)kNumMod * Np * Kp * 2);
+    pb_off = up((size_t)group * Np * Kp * 2);
     eb_off = pb_off + up((size_t)eblocks * Np * 4);
     ea_off = eb_off + up((size_t)Np * 4);   // (one memset clears both ex)
     pa_off = ea_off + up((size_t)Mp * 4);
     a_off = pa_off + up((size_t)eblocks * Mp * 4);
-    r_off = a_off + up((size_t)kNumMod * Mp * Kp * 2);
+    r_off = a_off + up((size_t)group * Mp * Kp * 2);
     total = r_off + up((size_t)kNumMod * Mp * Np * 2) + 256;
   }
 };
@@ -1303,12 +1313,12 @@ struct OzLayout {
 // marks (optional): two events recorded on s around the tensor-core product
 // kernel's launch alone (the measurement entry point bta_gemm_emulated_timed).
 bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_t s,
-                        const cudaEvent_t* marks) {
+                        const cudaEvent_t* marks, int group) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
   BTA_TRY(tensor_map_encoder(&enc));
   const int M = g.M, N = g.N, K = g.K;
   const int tile = crt_tile(M, N);
-  const OzLayout L(M, N, K, tile);
+  const OzLayout L(M, N, K, tile, group);
   __nv_bfloat16* YA = reinterpret_cast<__nv_bfloat16*>(ws + L.a_off);
   __nv_bfloat16* YB = reinterpret_cast<__nv_bfloat16*>(ws + L.b_off);
   int* exA = reinterpret_cast<int*>(ws + L.ea_off);
@@ -1343,7 +1353,7 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
                {g.B22.X, g.B22.ld, !g.B22.trans}}};
   // op(B)'s planes from the product before (laid out alike), in a symmetric product op(A)'s
   // too (b = 4800, 8 blocks gradient 174.5 ms without, 171.1 with)
-  const bool kept = g.b_kept > 0 && crt_tile(g.b_kept, N) == tile &&
+  const bool kept = g.b_kept > 0 && group == kNumMod && crt_tile(g.b_kept, N) == tile &&
                     (!same || (L.Mp <= L.Np && !g.a_rows));
   const int nops = (same ? 1 : 2) - (kept ? 1 : 0);
   if (same && kept) {
@@ -1351,23 +1361,17 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
     exA = exB;
   }
   if (nops > 0) {
-    const int rows = nops > 1 ? std::max(M, N) : M, rowsP = nops > 1 ? std::max(L.Mp, L.Np) : L.Mp;
+    const int rows = nops > 1 ? std::max(M, N) : M;
     if (!L.eblocks) {
       if (kept) BTA_CUDA_TRY(cudaMemsetAsync(exA, 0, L.pa_off - L.ea_off, s));
       else BTA_CUDA_TRY(cudaMemsetAsync(exB, 0, L.pa_off - L.eb_off, s));
     }
     ozaki_exp_kernel<<<dim3(cdiv(rows, kElemRows), cdiv(K, CK), nops), kElemThreads, 0, s>>>(sa);
     BTA_LAUNCHED();
-    BTA_CUDA_TRY(launch_after(residue_kernel, dim3(rowsP / kElemRows, L.Kp / CK, nops),
-                              dim3(kElemThreads), 0, s, sa));
-    BTA_LAUNCHED();
   }
-  CUtensorMap mA, mB;
   CrtArgs q{};
   q.Mp = L.Mp; q.Np = L.Np; q.Ap = same && kept ? L.Np : L.Mp; q.Bp = same ? q.Ap : L.Np;
   q.nk = L.Kp / CK;
-  BTA_TRY(make_map_bf16(enc, &mA, YA, kNumMod * q.nk * q.Ap));
-  BTA_TRY(make_map_bf16(enc, &mB, same ? YA : YB, kNumMod * q.nk * q.Bp));
   q.mt = L.Mp / tile;
   q.nt = L.Np / tile;
   // tile row i holds columns up to i; a C2 row (row >= c_rows) needs every column, so
@@ -1379,29 +1383,46 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
   q.tri_b = g.triB;
   q.R = R;
   q.status = status;
-  const int units = q.tiles * kNumMod;
   static std::atomic<uint64_t> allowed[2];
-  if (tile == ST) {
+  if (tile == ST)
     BTA_TRY(allow_smem(allowed[0], reinterpret_cast<const void*>(&crt_gemm_small_kernel),
                        kSmallSmem));
-    q.group = q.mt;
-    if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
-    BTA_CUDA_TRY(launch_after(crt_gemm_small_kernel, dim3(units), dim3(kCrtThreads), kSmallSmem,
-                              s, mA, mB, q));
-  } else {
-    // A wave of pairs spans a near-square patch of tiles.  A pair takes several units
-    // (the store of one overlaps the next) but at most ~300 slabs, ~75 us, so that the
-    // launches of a concurrent sweep find free SMs.
+  else
     BTA_TRY(allow_smem(allowed[1], reinterpret_cast<const void*>(&crt_gemm_kernel), kCrtSmem));
-    q.slots = pair_slots();
-    q.group = std::min(q.mt, std::max(1, (int)std::lround(std::sqrt((double)q.slots))));
-    q.slots = std::min(q.slots, units);
-    q.per = std::max(1, std::min(cdiv(units, q.slots), 300 / q.nk));
-    if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
-    BTA_CUDA_TRY(launch_after(crt_gemm_kernel, dim3(2 * q.slots * cdiv(units, q.slots * q.per)),
-                              dim3(kCrtThreads), kCrtSmem, s, mA, mB, q));
+  // group by group: planes of its moduli, then their products (a group's residues wait for
+  // the products of the one before, whose planes they overwrite)
+  for (int m0 = 0; m0 < kNumMod; m0 += group) {
+    sa.mod0 = q.mod0 = m0;
+    sa.nmod = q.nmod = std::min(group, kNumMod - m0);
+    if (nops > 0) {
+      const int rowsP = nops > 1 ? std::max(L.Mp, L.Np) : L.Mp;
+      BTA_CUDA_TRY(launch_after(group == kNumMod ? residue_kernel<true> : residue_kernel<false>,
+                                dim3(rowsP / kElemRows, L.Kp / CK, nops), dim3(kElemThreads), 0,
+                                s, sa));
+      BTA_LAUNCHED();
+    }
+    CUtensorMap mA, mB;
+    BTA_TRY(make_map_bf16(enc, &mA, YA, q.nmod * q.nk * q.Ap));
+    BTA_TRY(make_map_bf16(enc, &mB, same ? YA : YB, q.nmod * q.nk * q.Bp));
+    const int units = q.tiles * q.nmod;
+    if (marks && m0 == 0) BTA_CUDA_TRY(cudaEventRecord(marks[0], s));
+    if (tile == ST) {
+      q.group = q.mt;
+      BTA_CUDA_TRY(launch_after(crt_gemm_small_kernel, dim3(units), dim3(kCrtThreads), kSmallSmem,
+                                s, mA, mB, q));
+    } else {
+      // A wave of pairs spans a near-square patch of tiles.  A pair takes several units
+      // (the store of one overlaps the next) but at most ~300 slabs, ~75 us, so that the
+      // launches of a concurrent sweep find free SMs.
+      q.slots = pair_slots();
+      q.group = std::min(q.mt, std::max(1, (int)std::lround(std::sqrt((double)q.slots))));
+      q.slots = std::min(q.slots, units);
+      q.per = std::max(1, std::min(cdiv(units, q.slots), 300 / q.nk));
+      BTA_CUDA_TRY(launch_after(crt_gemm_kernel, dim3(2 * q.slots * cdiv(units, q.slots * q.per)),
+                                dim3(kCrtThreads), kCrtSmem, s, mA, mB, q));
+    }
+    BTA_LAUNCHED();
   }
-  BTA_LAUNCHED();
   if (marks) BTA_CUDA_TRY(cudaEventRecord(marks[1], s));
   ComposeArgs c;
   c.M = M; c.N = N; c.Mp = L.Mp; c.Np = L.Np;
@@ -1425,9 +1446,9 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
 // An upper bound over every product of at most M x N x K: a sweep sizes one
 // workspace for all of its products.
 // (the larger tile's layout, and the partial maxima of a smaller K).
-size_t ozaki_ws_bytes(int M, int N, int K) {
-  const size_t full = OzLayout(M, N, K, CT).total;
-  return K > kPartialK ? std::max(full, OzLayout(M, N, kPartialK, CT).total) : full;
+size_t ozaki_ws_bytes(int M, int N, int K, int group) {
+  const size_t full = OzLayout(M, N, K, CT, group).total;
+  return K > kPartialK ? std::max(full, OzLayout(M, N, kPartialK, CT, group).total) : full;
 }
 
 bool ozaki_supported(const Gemm& g) {
@@ -1456,12 +1477,12 @@ bool ozaki_supported(const Gemm& g) {
 }
 
 bta_status ozaki_gemm(const Gemm& g, void* ws, int32_t* status, cudaStream_t s,
-                      const cudaEvent_t* marks) {
+                      const cudaEvent_t* marks, int group) {
   if (g.M <= 0 || g.N <= 0) return BTA_OK;
-  if (!ozaki_supported(g) || !ws) return BTA_ERR_ARG;
+  if (!ozaki_supported(g) || !ws || group < 1 || group > kNumMod) return BTA_ERR_ARG;
   uint8_t* w = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ws) + 255) &
                                           ~(uintptr_t)255);
-  return launch_ozaki(g, w, status, s, marks);
+  return launch_ozaki(g, w, status, s, marks, group);
 }
 
 }  // namespace bta

@@ -349,6 +349,12 @@ int potrf_hybrid_top(int precision) {
 }
 }  // namespace
 
+size_t potrf_tc_ws_bytes(int n) {   // the products of the first split, the largest
+  if (n <= 0 || n > kOzakiMaxK) return 0;
+  const int half = n - n / T / 2 * T;
+  return ozaki_ws_bytes(half, half, half);
+}
+
 bta_status potrf_inv_batch_prec(int count, double* const* A, int n, int ld,
                                 double* const* scratch, double* const* logdet_parts,
                                 int32_t* const* fail, const int32_t* fail_code, int precision,

@@ -251,7 +251,7 @@ size_t SweepWs::bytes(int ld, int a) {
   size_t m = (size_t)ld * ld;
   // a multiple of 256 bytes: a second workspace carved right after this one
   // keeps its blocks aligned for vector access
-  const size_t d = 4 * m + (size_t)a * ld + (size_t)ld + a + 64;
+  const size_t d = 3 * m + (size_t)a * ld + (size_t)ld + a + 64;
   return sizeof(double) * ((d + 31) / 32 * 32);
 }
 
@@ -260,8 +260,7 @@ void SweepWs::carve(double* base, int ld, int a) {
   W1 = base;
   W2 = W1 + m;
   W3 = W2 + m;
-  pot = W3 + m;
-  Wc1 = pot + m;
+  Wc1 = W3 + m;
   gv = Wc1 + (size_t)a * ld;
   vT = gv + ld;
 }
@@ -272,10 +271,12 @@ bool arrow_fused(int ld, int a, int precision) {
   return precision == 2 && a > 0 && ld + a <= kOzakiMaxK;
 }
 
-size_t sweep_tc_ws_bytes(int ld, int a) {
+size_t sweep_tc_ws_bytes(int ld, int a, int precision, int group) {
   const int e = a > 0 && ld + a <= kOzakiMaxK ? a : 0;
-  return std::max(tc_gemm_ws_bytes(ld, ld, ld),
-                  ld <= kOzakiMaxK ? ozaki_ws_bytes(ld + e, ld, ld + e) : (size_t)0);
+  const size_t big = precision == 1      ? tc_gemm_ws_bytes(ld, ld, ld)
+                     : ld <= kOzakiMaxK ? ozaki_ws_bytes(ld + e, ld, ld + e, group)
+                                         : 0;
+  return std::max(big, potrf_tc_ws_bytes(ld));
 }
 
 
@@ -332,7 +333,7 @@ bta_status big_product(const Gemm& g, const SweepItem* it, const std::vector<int
     one.A = g.Ab[z]; one.B = g.Bb[z]; one.C = g.Cb[z];
     one.Cin = g.Cinb ? g.Cinb[z] : g.Cb[z];
     if (precision == 2) {
-      BTA_TRY(ozaki_gemm(one, ws.tc, ws.tcstat, s));
+      BTA_TRY(ozaki_gemm(one, ws.tc, ws.tcstat, s, nullptr, ws.tcgroup));
     } else {
       BTA_TRY(tc_gemm_mixed(one, ws.tc, ws.tcstat, s));
     }
@@ -430,7 +431,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
   auto fused = [&](int z) { return emu && arrow_fused(ld, it[z].q.a, precision); };
   auto emulate = [&](int z, const Gemm& g) -> bta_status {
     if (!it[z].ws.tc) return BTA_ERR_ARG;
-    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s);
+    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s, nullptr, it[z].ws.tcgroup);
   };
   // T -= L_Ci L_Ci^T and v_T += L_Ci z_i
   auto tip_update = [&](const std::vector<int>& grp, int i) -> bta_status {
@@ -547,7 +548,7 @@ bta_status factor_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
     if (join) return BTA_OK;
     {  // L_Di^{-1} in place, log-det slots
       auto Di = ptrs(G.all, [&](int z) { return D(z, i); });
-      auto W = ptrs(G.all, [&](int z) { return it[z].ws.pot; });
+      auto W = ptrs(G.all, [&](int z) { return it[z].ws.W2; });
       auto sl = ptrs(G.all, [&](int z) { return it[z].slots + (int64_t)block_of(it[z], i) * p; });
       std::vector<int32_t*> fl;
       std::vector<int32_t> code;
@@ -851,7 +852,7 @@ bta_status selinv_sweep_multi(const SweepItem* it, int m, cudaStream_t s, int pr
   auto fused = [&](int z) { return emu && arrow_fused(ld, it[z].q.a, precision); };
   auto emulate = [&](int z, const Gemm& g) -> bta_status {
     if (!it[z].ws.tc) return BTA_ERR_ARG;
-    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s);
+    return ozaki_gemm(g, it[z].ws.tc, it[z].ws.tcstat, s, nullptr, it[z].ws.tcgroup);
   };
   for (int i = i_hi; i >= i_lo; --i) {
     BTA_SWEEP_MARK(s, 4, i);

@@ -5,14 +5,17 @@
 
 namespace bta {
 
-// Scratch for one sweep: three ld x ld blocks, the diagonal-factor scratch,
-// an a x ld arrow block, a solve vector and the arrow accumulator v_T.
+// Scratch for one sweep: three ld x ld blocks, an a x ld arrow block, a solve vector and
+// the arrow accumulator v_T.  W2 holds low-memory sweeps' assembled couplings, and before
+// a block's coupling is assembled (in the others throughout) its diagonal factor's scratch.
 struct SweepWs {
-  double *W1 = nullptr, *W2 = nullptr, *W3 = nullptr, *pot = nullptr;
+  double *W1 = nullptr, *W2 = nullptr, *W3 = nullptr;
   double *Wc1 = nullptr, *gv = nullptr, *vT = nullptr;   // gv: ld
-  // mixed precision only: operand copies of the tensor-core products and
-  // their status word (set by the owner, not by carve)
+  // tensor-core modes only: operand copies of the products (sweep_tc_ws_bytes), the moduli
+  // whose planes they hold at once (ozaki_gemm) and the products' status word (set by the
+  // owner, not by carve)
   void* tc = nullptr;
+  int tcgroup = kOzakiModuli;
   int32_t* tcstat = nullptr;
   static size_t bytes(int ld, int a);
   void carve(double* base, int ld, int a);
@@ -35,9 +38,9 @@ int logdet_slots(int n, int ld);   // n * (ld / 32) + 1 (tip)
 // 128), and its rank-a terms extend K, so that no FP64 product of the a x b
 // arrow blocks with a b x b block is left per block step.
 bool arrow_fused(int ld, int a, int precision);
-// Bytes of the tensor-core workspace (SweepWs::tc) of a sweep of block size
-// ld and arrow a in any precision, the arrow-extended products included.
-size_t sweep_tc_ws_bytes(int ld, int a);
+// Bytes of the tensor-core workspace (SweepWs::tc) of a sweep of block size ld and arrow a
+// in the given precision, the arrow-extended products and the diagonal factor's included.
+size_t sweep_tc_ws_bytes(int ld, int a, int precision, int group = kOzakiModuli);
 
 // One matrix of a set swept together, or one leg of it.  All matrices of a set share n and
 // ld; the arrow width may differ (Q_c with a > 0 next to the block-tridiagonal

@@ -25,6 +25,7 @@ class FakeCuda:
         self.lib.fake_live.restype = self.lib.fake_peak.restype = C.c_size_t
         self.lib.fake_launch_name.restype = C.c_char_p
         self.lib.fake_launch_grid.restype = C.c_uint
+        self.lib.fake_launch_stream.restype = C.c_size_t
 
     def install(self, monkeypatch):
         import torch
@@ -53,6 +54,10 @@ class FakeCuda:
         return [(self.lib.fake_launch_name(i).decode(),
                  tuple(self.lib.fake_launch_grid(i, d) for d in range(3)), i)
                 for i in range(self.lib.fake_launches())]
+
+    def streams(self):
+        """Streams that took launches since the last reset."""
+        return {self.lib.fake_launch_stream(i) for i in range(self.lib.fake_launches())}
 
     def head(self, i, k):
         """Int k of launch i's first argument (task-graph kernels)."""

@@ -21,6 +21,7 @@ struct Launch {
   std::string name;
   unsigned grid[3];
   size_t smem;
+  cudaStream_t stream;
   std::vector<int> head;   // first ints of the first argument (task-graph kernels)
 };
 struct State {
@@ -63,7 +64,7 @@ cudaError_t release(void* p) {
   return cudaSuccess;
 }
 
-cudaError_t launch(const void* f, dim3 g, size_t smem, void** args) {
+cudaError_t launch(const void* f, dim3 g, size_t smem, void** args, cudaStream_t stream) {
   State& s = st();
   if (!g.x || !g.y || !g.z || g.y > 65535 || g.z > 65535)
     return fail(cudaErrorInvalidConfiguration);
@@ -71,7 +72,7 @@ cudaError_t launch(const void* f, dim3 g, size_t smem, void** args) {
     auto it = s.smem.find({f, s.device});
     if (it == s.smem.end() || (size_t)it->second < smem) return fail(cudaErrorInvalidValue);
   }
-  Launch l{s.names[f], {g.x, g.y, g.z}, smem, {}};
+  Launch l{s.names[f], {g.x, g.y, g.z}, smem, stream, {}};
   if (l.name.find("potrf_dag_kernel") != std::string::npos)
     l.head.assign(static_cast<int*>(args[0]), static_cast<int*>(args[0]) + 16);
   s.launches.push_back(l);
@@ -98,6 +99,7 @@ size_t fake_peak() { return st().peak; }
 int fake_launches() { return (int)st().launches.size(); }
 const char* fake_launch_name(int i) { return st().launches[i].name.c_str(); }
 unsigned fake_launch_grid(int i, int d) { return st().launches[i].grid[d]; }
+size_t fake_launch_stream(int i) { return reinterpret_cast<size_t>(st().launches[i].stream); }
 int fake_launch_head(int i, int k) { return st().launches[i].head[k]; }
 
 // ---- registration and launches ---------------------------------------------
@@ -131,11 +133,11 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
   return cudaSuccess;
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3, void** args, size_t smem,
-                               cudaStream_t) {
-  return launch(reinterpret_cast<const void*>(k), g, smem, args);
+                               cudaStream_t s) {
+  return launch(reinterpret_cast<const void*>(k), g, smem, args, s);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
-  return launch(f, c->gridDim, c->dynamicSmemBytes, args);
+  return launch(f, c->gridDim, c->dynamicSmemBytes, args, c->stream);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {

@@ -92,3 +92,117 @@ def test_blocks_up_to_512_rows_keep_fp64_tile_products(fake, b, precision):
     assert _factor(fake, 2, b, 0, precision) == 0
     names = [n for n, _, _ in fake.launches() if "potrf_dag_kernel" in n]
     assert len(names) == 2 and all("ILb0E" in n for n in names), names
+
+
+# ---- workspaces ---------------------------------------------------------------
+def _pad(n, m):
+    return (n + m - 1) // m * m
+
+
+LD, A, NT = 2080, 4, 5
+BLOCK = 8 * LD * LD
+PLANE = _pad(LD + A, 256) * _pad(LD + A, 256)   # entries of a product's padded operand
+
+
+def _model(low=False):
+    import paper_2605_06392_gb300 as P
+    prob = workloads.make_problem("st_tiny", nx=65, ny=32, nt=NT, a=A, n_obs=400)
+    return prob, P.InlaModel(prob, low_memory=low)
+
+
+def _run(m, prob, precision, count=1, **kw):
+    import numpy as np
+    th = np.array([prob.theta] * count)
+    return m.value_and_grad(th, use_graph=False, precision=precision, concurrent=count,
+                            stream=Stream(), **kw)
+
+
+def _work_of(fake, precision, low):
+    """Bytes of a model that has been evaluated, beside its matrices' blocks."""
+    before = fake.live()
+    prob, m = _model(low)
+    _run(m, prob, precision)
+    work = fake.live() - before - 2 * (NT + (0 if low else NT - 1)) * BLOCK
+    m.close()
+    assert fake.live() == before
+    return work
+
+
+@pytest.mark.parametrize("precision,low,want", [
+    # legs of three blocks each; the products' planes: two operands' and the result's, of 14
+    # moduli (low memory: of 7, and one leg a matrix); TF32: high and low parts of two
+    (0, False, 4 * 3 * BLOCK),
+    (1, False, 2 * (3 * BLOCK + 16 * LD * LD)),
+    (2, False, 4 * (3 * BLOCK + 84 * PLANE)),
+    (0, True, 4 * 3 * BLOCK),
+    (2, True, 2 * (3 * BLOCK + 56 * PLANE)),
+])
+def test_workspaces_follow_legs_and_mode(fake, precision, low, want):
+    work = _work_of(fake, precision, low)
+    half = 84 * _pad(_pad(LD, 64) // 2, 256) ** 2       # the diagonal factor's products
+    if precision == 1:
+        want = max(want, 2 * (3 * BLOCK + half))
+    assert work <= want + 0.02 * want + (4 << 20), work / want
+
+
+def test_large_models_of_every_mode_fit_where_they_did(fake):
+    """b = 4800: an evaluation finds a form that fits into what two legs of four blocks and
+    40 bytes an entry once took."""
+    import paper_2605_06392_gb300 as P
+    prob = workloads.make_problem("coreg_production", nt=4, n_obs=600)
+    blk, once = 8 * 4800 ** 2, 2 * (4 * 8 * 4800 ** 2 + 40 * 4864 ** 2)
+    for precision, low in ((0, False), (1, False), (2, False), (0, True), (2, True)):
+        before = fake.live()
+        m = P.InlaModel(prob, low_memory=low)
+        fake.reset(limit=before + 2 * (4 + (0 if low else 3)) * blk + once + (48 << 20))
+        for grad in (False, True):
+            f, _ = m.value_and_grad(prob.theta, use_graph=False, precision=precision, grad=grad,
+                                    stream=Stream())
+        m.close()
+        assert fake.live() == before
+
+
+def test_out_of_memory_leaves_the_model_as_it_was(fake):
+    from paper_2605_06392_gb300._capi import BtaError
+    prob, m = _model()
+    _run(m, prob, 0)
+    live = fake.live()
+    fake.reset(limit=live + 80 * PLANE)             # less than the small form's 2 x 44
+    with pytest.raises(BtaError, match="memory"):
+        _run(m, prob, 2)
+    with pytest.raises(BtaError, match="memory"):
+        _run(m, prob, 0, count=2)                   # a second context does not fit either
+    assert fake.live() == live
+    _run(m, prob, 0)
+    fake.reset(limit=live + 90 * PLANE)
+    _run(m, prob, 2)                                # now the small form does
+    m.close()
+
+
+def test_reverse_pass_takes_the_order_of_its_factor(fake):
+    """A value by two legs a matrix, then by one (a set that finds no room for two): each
+    reverse pass runs in the order of the factors held, whatever a failed call tried since."""
+    import numpy as np
+
+    def legs(m):
+        fake.reset()
+        g = np.zeros(m.d)
+        assert fake.lib.inla_backward(m.handle, g.ctypes.data_as(C.POINTER(C.c_double)), 0,
+                                      None) == 0
+        return len(fake.streams() - {0})
+
+    from paper_2605_06392_gb300._capi import BtaError
+    prob, m = _model()
+    second = (2 * (2 * NT - 1) + 6) * BLOCK         # another context, without its planes
+    for room, streams in ((second + 60 * PLANE, 4), (second + 2 * 46 * PLANE, 2)):
+        _run(m, prob, 2, grad=False)
+        assert legs(m) == 4
+        _run(m, prob, 2, grad=False)
+        fake.reset(limit=fake.live() + room)
+        if streams == 4:
+            with pytest.raises(BtaError, match="memory"):
+                _run(m, prob, 2, count=2, grad=False)
+        else:
+            _run(m, prob, 2, count=2, grad=False)
+        assert legs(m) == streams
+    m.close()
