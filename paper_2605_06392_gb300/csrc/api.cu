@@ -15,6 +15,7 @@
 // The whole evaluation is captured once into a CUDA graph per (value / value+grad)
 // and replayed.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -1051,6 +1052,65 @@ bta_status bta_gemm_mixed(int32_t M, int32_t N, int32_t K, double alpha, const d
   return st;
 }
 
+// An emulated product in panels of the result, whose workspaces (84 bytes an entry, with
+// the operands' planes) then stay below 13 GiB: a result of 90000 columns as a whole would
+// take 227 GB for its residues.  Panels of 16384 rows and columns cost one more split of the
+// operands each, under 1 % of their products; where not even those fit the device, smaller
+// ones, at last with the planes of four moduli at once.  The bits do not depend on it.  A
+// result that overlaps an operand is not split: its panels would overwrite what others read.
+// kernel_ms (optional): the product kernels' time, which is waited for.
+static bta_status emulated_panels(const Gemm& g, int32_t* status, float* kernel_ms,
+                                  const cudaEvent_t* marks, cudaStream_t stream) {
+  auto span = [](const double* p, int rows, int cols, int ld) {
+    return std::make_pair(p, p + (int64_t)(cols - 1) * ld + rows);
+  };
+  const auto c = span(g.C, g.M, g.N, g.ldc);
+  auto clear = [&](std::pair<const double*, const double*> x) {
+    return x.second <= c.first || c.second <= x.first;
+  };
+  const bool split = clear(g.transA ? span(g.A, g.K, g.M, g.lda) : span(g.A, g.M, g.K, g.lda)) &&
+                     clear(g.transB ? span(g.B, g.N, g.K, g.ldb) : span(g.B, g.K, g.N, g.ldb));
+  struct Form {
+    int panel, group;
+  };
+  void* ws = nullptr;
+  Form form{};
+  cudaError_t e = cudaErrorMemoryAllocation;
+  for (Form f : {Form{16384, kOzakiModuli}, Form{4096, kOzakiModuli},
+                 Form{1024, kOzakiSmallGroup}}) {
+    if (!split) f.panel = INT_MAX;
+    e = cudaMallocAsync(&ws, ozaki_ws_bytes(std::min(g.M, f.panel), std::min(g.N, f.panel), g.K,
+                                            f.group), stream);
+    form = f;
+    if (e != cudaErrorMemoryAllocation) break;
+    cudaGetLastError();
+  }
+  if (e == cudaErrorMemoryAllocation) return BTA_ERR_NOMEM;
+  BTA_CUDA_TRY(e);
+  bta_status st = BTA_OK;
+  if (kernel_ms) *kernel_ms = 0.0f;
+  for (int64_t n0 = 0; n0 < g.N && st == BTA_OK; n0 += form.panel)
+    for (int64_t m0 = 0; m0 < g.M && st == BTA_OK; m0 += form.panel) {
+      Gemm q = g;
+      q.M = (int)std::min<int64_t>(form.panel, g.M - m0);
+      q.N = (int)std::min<int64_t>(form.panel, g.N - n0);
+      q.A += g.transA ? m0 * g.lda : m0;
+      q.B += g.transB ? n0 : n0 * g.ldb;
+      q.C += m0 + n0 * g.ldc;
+      q.Cin = q.C;
+      st = ozaki_gemm(q, ws, status, stream, marks, form.group);
+      float ms = 0.0f;
+      if (st == BTA_OK && kernel_ms) {
+        if (cudaEventSynchronize(marks[1]) != cudaSuccess ||
+            cudaEventElapsedTime(&ms, marks[0], marks[1]) != cudaSuccess)
+          st = BTA_ERR_CUDA;
+        *kernel_ms += ms;
+      }
+    }
+  cudaFreeAsync(ws, stream);
+  return st;
+}
+
 bta_status bta_gemm_emulated(int32_t M, int32_t N, int32_t K, double alpha, const double* A,
                              int32_t lda, int32_t transA, const double* B, int32_t ldb,
                              int32_t transB, double beta, double* Cm, int32_t ldc,
@@ -1062,11 +1122,8 @@ bta_status bta_gemm_emulated(int32_t M, int32_t N, int32_t K, double alpha, cons
   g.A = A; g.lda = lda; g.transA = transA ? 1 : 0;
   g.B = B; g.ldb = ldb; g.transB = transB ? 1 : 0;
   g.C = Cm; g.ldc = ldc; g.Cin = Cm; g.ldcin = ldc;
-  void* ws = nullptr;
-  BTA_CUDA_TRY(cudaMallocAsync(&ws, ozaki_ws_bytes(M, N, K), stream));
-  bta_status st = ozaki_gemm(g, ws, status, stream);
-  cudaFreeAsync(ws, stream);
-  return st;
+  if (M == 0 || N == 0) return BTA_OK;
+  return emulated_panels(g, status, nullptr, nullptr, stream);
 }
 
 bta_status bta_gemm_emulated_timed(int32_t M, int32_t N, int32_t K, double alpha,
@@ -1085,17 +1142,7 @@ bta_status bta_gemm_emulated_timed(int32_t M, int32_t N, int32_t K, double alpha
   cudaEvent_t marks[2] = {nullptr, nullptr};
   BTA_CUDA_TRY(cudaEventCreate(&marks[0]));
   BTA_CUDA_TRY(cudaEventCreate(&marks[1]));
-  void* ws = nullptr;
-  bta_status st = BTA_OK;
-  if (cudaMallocAsync(&ws, ozaki_ws_bytes(M, N, K), stream) != cudaSuccess) {
-    cudaGetLastError();
-    st = BTA_ERR_NOMEM;
-  }
-  if (st == BTA_OK) st = ozaki_gemm(g, ws, status, stream, marks);
-  if (ws) cudaFreeAsync(ws, stream);
-  if (st == BTA_OK && cudaEventSynchronize(marks[1]) == cudaSuccess &&
-      cudaEventElapsedTime(kernel_ms, marks[0], marks[1]) != cudaSuccess)
-    st = BTA_ERR_CUDA;
+  const bta_status st = emulated_panels(g, status, kernel_ms, marks, stream);
   cudaEventDestroy(marks[0]);
   cudaEventDestroy(marks[1]);
   return st;

@@ -76,3 +76,50 @@ def test_modes_share_a_model(P):
         assert f0 == f1 == f2
         assert np.array_equal(g0, g1) and np.array_equal(g0, g2)
     assert np.array_equal(th.grad.numpy(), first[2][1])
+
+
+@pytest.mark.parametrize("M,N,K,transA,transB", [(64, 16500, 96, False, False),
+                                                 (70, 16400, 1030, True, True),
+                                                 (16390, 130, 64, False, True)])
+def test_panels_of_a_large_product(P, M, N, K, transA, transB):
+    """Panels of 16384 rows and columns: the bits of products of the parts, whose operands'
+    rows and columns are the same."""
+    import torch
+    g = torch.Generator().manual_seed(M + N)
+    A = torch.randn((M, K) if transA else (K, M), generator=g, dtype=torch.float64).cuda()
+    B = torch.randn((K, N) if transB else (N, K), generator=g, dtype=torch.float64).cuda()
+    C0 = torch.randn((N, M), generator=g, dtype=torch.float64).cuda()
+    whole = C0.clone()
+    assert int(P.bta_gemm_emulated(A, B, whole, alpha=0.5, beta=-1.0, transA=transA,
+                                   transB=transB).item()) == 0
+    h = N // 2
+    for lo, hi in ((0, h), (h, N)) if N > M else ((0, N),):
+        r = (M // 2, M - M // 2) if M > N else (M,)
+        m0 = 0
+        for m in r:
+            a = A[m0:m0 + m] if transA else A[:, m0:m0 + m]
+            b = B[:, lo:hi] if transB else B[lo:hi]
+            c = C0[lo:hi, m0:m0 + m].contiguous()
+            P.bta_gemm_emulated(a.contiguous(), b.contiguous(), c, alpha=0.5, beta=-1.0,
+                                transA=transA, transB=transB)
+            torch.cuda.synchronize()
+            assert torch.equal(whole[lo:hi, m0:m0 + m], c)
+            m0 += m
+
+
+def test_slices_select_no_other_arithmetic(P):
+    """slices (6..8) states the accuracy asked for: one product serves all."""
+    import torch
+    g = torch.Generator().manual_seed(1)
+    A = torch.randn(300, 200, generator=g, dtype=torch.float64).cuda()
+    B = torch.randn(250, 300, generator=g, dtype=torch.float64).cuda()
+    out = []
+    for slices in (6, 7, 8):
+        C = torch.zeros(250, 200, dtype=torch.float64, device="cuda")
+        P.bta_gemm_emulated(A, B, C, slices=slices)
+        out.append(C.cpu())
+    ref = (B.cpu() @ A.cpu())
+    bound = 300 * 2.0 ** -55 * A.abs().amax(0)[None, :].cpu() * B.abs().amax(1)[:, None].cpu() \
+        + 304 * 2.0 ** -53 * (B.abs() @ A.abs()).cpu()
+    assert torch.equal(out[0], out[1]) and torch.equal(out[1], out[2])
+    assert bool(((out[2] - ref).abs() <= bound).all())

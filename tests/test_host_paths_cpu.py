@@ -206,3 +206,42 @@ def test_reverse_pass_takes_the_order_of_its_factor(fake):
             _run(m, prob, 2, count=2, grad=False)
         assert legs(m) == streams
     m.close()
+
+
+# ---- emulated products beyond one panel ---------------------------------------
+def _gemm(fake, M, N, K, transA=0, transB=0, A=1 << 40, B=1 << 42, Cm=1 << 44):
+    return fake.lib.bta_gemm_emulated(M, N, K, 1.0, C.c_void_p(A), K if transA else M, transA,
+                                      C.c_void_p(B), N if transB else K, transB, 0.0,
+                                      C.c_void_p(Cm), M, 8, None, None)
+
+
+@pytest.mark.parametrize("M,N,K", [(90000, 90000, 512), (1500000, 64, 5120), (64, 1500000, 5120)])
+def test_large_emulated_products_need_no_more_room(fake, M, N, K):
+    """Beside their operands such products took 16 bytes an operand entry and 8 a result's."""
+    room = 16 * (M + N) * K + 8 * M * N
+    fake.reset(limit=room)
+    assert _gemm(fake, M, N, K) == 0
+    assert fake.peak() <= room and fake.live() == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 200, 64), (5000, 3000, 256), (4096, 4096, 5120)])
+def test_emulated_products_under_a_full_device(fake, M, N, K):
+    assert _gemm(fake, M, N, K) == 0
+    once = max(16 * (M + N) * K + 8 * M * N, 32 << 20)
+    fake.reset(limit=once)
+    assert _gemm(fake, M, N, K) == 0
+    assert _gemm(fake, M, N, K, 1, 1) == 0
+    fake.reset(limit=1 << 20)
+    assert _gemm(fake, M, N, K) == -4
+    assert fake.lib.bta_gemm(8, 8, 8, 1.0, _ptr(1), 8, 0, _ptr(1), 8, 0, 0.0, _ptr(1), 8,
+                             None) == 0                          # no error left behind
+
+
+def test_a_result_in_place_of_an_operand_is_not_split(fake):
+    n = 4000
+    fake.reset()
+    assert _gemm(fake, n, n, n, Cm=1 << 40) == 0
+    whole = fake.peak()
+    fake.reset(limit=whole // 2)
+    assert _gemm(fake, n, n, n, Cm=1 << 40) == -4
+    assert _gemm(fake, n, n, n) == 0
