@@ -149,8 +149,12 @@ __global__ void __launch_bounds__(256) assemble_kernel(AsmArgs a, double* out) {
   const int c = blockIdx.x, t = a.t0 + blockIdx.y;
   const int ld = a.ld;
   double* colp = out + ((int64_t)blockIdx.y * ld + c) * ld;
-  double2* col2 = reinterpret_cast<double2*>(colp);
-  for (int r = threadIdx.x; r < ld / 2; r += blockDim.x) col2[r] = make_double2(0.0, 0.0);
+  if (reinterpret_cast<uintptr_t>(colp) % 16) {   // a caller's blocks on an 8-byte boundary
+    for (int r = threadIdx.x; r < ld; r += blockDim.x) colp[r] = 0.0;
+  } else {
+    double2* col2 = reinterpret_cast<double2*>(colp);
+    for (int r = threadIdx.x; r < ld / 2; r += blockDim.x) col2[r] = make_double2(0.0, 0.0);
+  }
   __syncthreads();
   if (c >= a.b) {
     if (a.diag && threadIdx.x == 0) colp[c] = 1.0;
