@@ -453,24 +453,10 @@ bta_status group_program(inla_model* m, int mode, int cnt, int prec, int nb, cud
           EvalCtx& c = m->ctx[e];
           BTA_TRY(launch_rhs(md, m->L, c.coefbuf, c.dr, m->s1));
           BTA_TRY(launch_qc_residual(md, m->L, c.coefbuf, c.x, c.dr, m->s1));
-          SweepItem dx = sets->ic[e], dj;
+          SweepItem dx = sets->ic[e];   // (the mixed mode has no reverse legs)
           dx.vec = c.dr;
-          if (nb > 0) {
-            dj = sets->jc[e];
-            dj.vec = c.dr;
-            BTA_CUDA_TRY(cudaEventRecord(m->evac, m->s1));
-            BTA_CUDA_TRY(cudaStreamWaitEvent(m->s3, m->evac, 0));
-            for (int i = 0; i < mid; ++i) {
-              BTA_TRY(lower_solve(dx, m->s1, i, i + 1));
-              if (i < nb) BTA_TRY(lower_solve(dj, m->s3, i, i + 1));
-            }
-            BTA_CUDA_TRY(cudaEventRecord(m->evjc, m->s3));
-            BTA_CUDA_TRY(cudaStreamWaitEvent(m->s1, m->evjc, 0));
-            BTA_TRY(lower_solve(dx, m->s1, mid, mid + 1));
-          } else {
-            BTA_TRY(lower_solve(dx, m->s1));
-          }
-          BTA_TRY(upper(&dx, &dj, 1));
+          BTA_TRY(lower_solve(dx, m->s1));
+          BTA_TRY(upper_solve_multi(&dx, 1, m->s1));
           BTA_TRY(launch_axpy((int64_t)md.nt * md.ld + md.a, 1.0, c.dr, c.x, m->s1));
         }
       }

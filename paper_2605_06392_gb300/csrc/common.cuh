@@ -275,7 +275,6 @@ bta_status copy_block_batch(int count, const double* const* src, int lds, double
 // dst = the symmetric n x n matrix whose lower triangle src holds (in place when src == dst)
 bta_status mirror_batch(int count, const double* const* src, int lds, double* const* dst, int ldd,
                         int n, cudaStream_t s);
-bta_status fill_value(double* p, int64_t n, double v, cudaStream_t s);
 bta_status sum_slots(const double* parts, int nparts, double* out, int accumulate,
                      cudaStream_t s);
 

@@ -278,8 +278,7 @@ __device__ __forceinline__ void tile_syrk_lower(Tile L, Tile W) {
 // 2^-50 u w, the dropped levels by at most 7 2^17 units of level 8 (and 1 % more)
 // = 2^-50.2 u w, the 56-bit operands by 2^-51 u w: 2^-48.7 u w in all for 32 terms, where
 // the bound of FP64 FMAs is 2^-43 times the largest entries' product.  Unlike theirs it is
-// absolute in a row and column of a tile: small entries keep fewer bits.  ylower: Y is
-// lower triangular (its upper part is not read).
+// absolute in a row and column of a tile: small entries keep fewer bits.
 constexpr int kOzPitch = 40;                      // bf16 a slice row: 80 bytes, conflict-free ldmatrix
 constexpr int kOzPlane = T * kOzPitch;            // one 32 x 32 slice
 constexpr int kOzTileSmem = 2 * 8 * kOzPlane * 2 + 2 * T * 4;   // both operands' slices, exponents
@@ -401,17 +400,11 @@ __device__ __forceinline__ void oz_combine(const __nv_bfloat16* xp, const __nv_b
 }
 
 // All compute threads; out must not alias X or Y.
-__device__ __forceinline__ void tile_mm_oz(Tile X, Tile Y, bool ytrans,
-                                           bool ylower, Tile out, double sign,
+__device__ __forceinline__ void tile_mm_oz(Tile X, Tile Y, bool ytrans, Tile out, double sign,
                                            bool accumulate, const OzTile& z) {
   const int warp = threadIdx.x >> 5;
   oz_split([&](int r, int k) { return at(X, r, k); }, z.xp, z.ex, warp);
-  oz_split(
-      [&](int n, int k) {
-        if (ylower && (ytrans ? k > n : n > k)) return 0.0;
-        return ytrans ? at(Y, n, k) : at(Y, k, n);
-      },
-      z.yp, z.ey, warp);
+  oz_split([&](int n, int k) { return ytrans ? at(Y, n, k) : at(Y, k, n); }, z.yp, z.ey, warp);
   compute_bar();
   oz_combine(z.xp, z.yp, z.ex, z.ey, out, sign, accumulate);
 }
@@ -928,7 +921,7 @@ __global__ void __launch_bounds__(kDagAllThreads, 2) potrf_dag_kernel(DagArgs g)
   // ---- compute warps
   auto mm = [&](Tile X, Tile Y, bool ytrans, Tile o,
                 double sign, bool acc) {
-    if constexpr (TC) tile_mm_oz(X, Y, ytrans, false, o, sign, acc, oz);
+    if constexpr (TC) tile_mm_oz(X, Y, ytrans, o, sign, acc, oz);
     else tile_mm(X, Y, ytrans, o, sign, acc);
   };
   for (int n = 0;; ++n) {
@@ -982,7 +975,7 @@ __global__ void __launch_bounds__(kDagAllThreads, 2) potrf_dag_kernel(DagArgs g)
     } else {
       switch (t.type) {
         case TK_S:
-          if constexpr (TC) tile_mm_oz(st[0], st[1], true, false, st[2], 1.0, false, oz);
+          if constexpr (TC) tile_mm_oz(st[0], st[1], true, st[2], 1.0, false, oz);
           else tile_mm_lt(st[0], st[1], st[2]);
           compute_bar();
           store_tile(Lt(I, t.i, t.k), T, st[2], false);

@@ -158,12 +158,6 @@ __global__ void __launch_bounds__(256) mirror_kernel(CopyDev d) {
   }
 }
 
-__global__ void fill_kernel(double* p, int64_t n, double v) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x)
-    p[e] = v;
-}
-
 __global__ void sum_kernel(const double* parts, int n, double* out, int acc) {
   if (threadIdx.x || blockIdx.x) return;
   double s = 0.0;
@@ -229,14 +223,6 @@ bta_status mirror_batch(int count, const double* const* src, int lds, double* co
     mirror_kernel<<<dim3(cdiv(n, 32), cdiv(n, 32), cnt), 256, 0, s>>>(d);
     BTA_LAUNCHED();
   }
-  return BTA_OK;
-}
-
-bta_status fill_value(double* p, int64_t n, double v, cudaStream_t s) {
-  if (n <= 0) return BTA_OK;
-  int grid = (int)std::min<int64_t>(cdiv(n, 256), 32 * sm_count());
-  fill_kernel<<<grid, 256, 0, s>>>(p, n, v);
-  BTA_LAUNCHED();
   return BTA_OK;
 }
 
@@ -689,19 +675,13 @@ bta_status bta_residual(const bta_desc& q, const double* x, double* d, cudaStrea
 }
 
 // ----------------------------------------------------------------------------
-// Lower solve alone (L z = r) with a factor: blocks i0 <= i < i1 of a leg, the set-up
-// with the first and the tip with a forward leg's last (see factor_sweep_multi)
+// Lower solve alone (L z = r) with a factor
 // ----------------------------------------------------------------------------
 namespace {
-// z_T = L_T^{-1} (r_T - v_T - v2_T) with the factored tip: one warp, lane = row.
-__global__ void tip_fwd_kernel(int a, const double* T, double* r, const double* vT,
-                               const double* vT2) {
+// z_T = L_T^{-1} (r_T - v_T) with the factored tip: one warp, lane = row.
+__global__ void tip_fwd_kernel(int a, const double* T, double* r, const double* vT) {
   const int lane = threadIdx.x;
-  double s = 0.0;
-  if (lane < a) {
-    s = r[lane] - vT[lane];
-    if (vT2) s -= vT2[lane];
-  }
+  double s = lane < a ? r[lane] - vT[lane] : 0.0;
   for (int k = 0; k < a; ++k) {
     const double v = __shfl_sync(0xffffffffu, s, k) / T[k + k * a];
     if (lane == k) s = v;
@@ -711,26 +691,20 @@ __global__ void tip_fwd_kernel(int a, const double* T, double* r, const double* 
 }
 }  // namespace
 
-bta_status lower_solve(const SweepItem& it, cudaStream_t s, int i0, int i1) {
-  const int n = it.blocks(), ld = it.q.ld, a = it.q.a;
-  const bool rev = it.rev;
-  if (i1 < 0) i1 = n;
-  if (i0 < 0 || i0 > i1 || i1 > n || !it.vec || (n > 1 && !it.q.B)) return BTA_ERR_ARG;
-  if (a > 0 && i0 == 0)
-    BTA_CUDA_TRY(cudaMemsetAsync(it.ws.vT, 0, a * sizeof(double), s));
-  for (int i = i0; i <= i1 && i < n; ++i) {
-    const bool join = i == i1;
-    if (join && !(rev && i1 == n - 1)) break;
+bta_status lower_solve(const SweepItem& it, cudaStream_t s) {
+  const int n = it.q.n, ld = it.q.ld, a = it.q.a;
+  if (it.rev || !it.vec || (n > 1 && !it.q.B)) return BTA_ERR_ARG;
+  if (a > 0) BTA_CUDA_TRY(cudaMemsetAsync(it.ws.vT, 0, a * sizeof(double), s));
+  for (int i = 0; i < n; ++i) {
     double* ri = vec_of(it, i);
     if (i == 0) {
       BTA_TRY(copy_block(ri, ld, it.ws.gv, ld, ld, 1, 1.0, s));
     } else {
       Gemv g; g.M = ld; g.K = ld; g.A = B_of(it, i - 1); g.lda = ld;
-      g.x = vec_of(it, i - 1); g.y = join ? ri : it.ws.gv; g.yin = ri;
+      g.x = vec_of(it, i - 1); g.y = it.ws.gv; g.yin = ri;
       g.alpha = -1.0; g.beta = 1.0;
       BTA_TRY(gemv_f64(g, s));
     }
-    if (join) return BTA_OK;
     Gemv g; g.M = ld; g.K = ld; g.A = D_of(it, i); g.lda = ld; g.triA = TRI_LOWER;
     g.x = it.ws.gv; g.y = ri;
     BTA_TRY(gemv_f64(g, s));
@@ -740,8 +714,8 @@ bta_status lower_solve(const SweepItem& it, cudaStream_t s, int i0, int i1) {
       BTA_TRY(gemv_f64(h, s));
     }
   }
-  if (i1 == n && a > 0) {
-    tip_fwd_kernel<<<1, 32, 0, s>>>(a, it.q.T, tip_vec(it), it.ws.vT, it.vT2);
+  if (a > 0) {
+    tip_fwd_kernel<<<1, 32, 0, s>>>(a, it.q.T, tip_vec(it), it.ws.vT);
     BTA_LAUNCHED();
   }
   return BTA_OK;

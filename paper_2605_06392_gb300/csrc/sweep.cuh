@@ -109,8 +109,8 @@ bta_status selinv_sums(const SweepItem* items, int m, cudaStream_t s);
 // d <- d - Q x for an assembled BTA matrix Q (D lower triangle referenced, B,
 // C, T as in bta_desc); x, d: n*ld + a.
 bta_status bta_residual(const bta_desc& q, const double* x, double* d, cudaStream_t s);
-// L z = r in place of item.vec with a factor (B kept), by block ranges as the factor's.
-bta_status lower_solve(const SweepItem& item, cudaStream_t s, int i0 = 0, int i1 = -1);
+// L z = r in place of item.vec with a forward factor (B kept).
+bta_status lower_solve(const SweepItem& item, cudaStream_t s);
 bta_status selinv_sweep(const bta_desc& q, const SweepWs& ws, const SelinvFuse* fuse,
                         cudaStream_t s);
 
