@@ -125,10 +125,13 @@ typedef struct {
                           2: emulated FP64 -- the same b x b products as in
                           mode 1, with the arrow's rows and rank-a terms
                           carried along, and the diagonal factor's inner and
-                          tile products, computed to FP64 accuracy on the
-                          BF16 tensor cores (as bta_gemm_emulated;
-                          products with K > 5120 fall back to FP64);
-                          everything else as in mode 0                        */
+                          tile products in blocks above 512 rows, computed to
+                          FP64 accuracy on the BF16 tensor cores (as
+                          bta_gemm_emulated; products with K > 5120 fall back
+                          to FP64); everything else as in mode 0.  A mode's
+                          workspaces are allocated by its first evaluation; in
+                          mode 2 smaller ones (one elimination order, the same
+                          products in groups) where the full ones do not fit   */
   int32_t use_graph;   /* 1: capture the evaluation in a CUDA graph, replay */
   int32_t streams;     /* thetas evaluated together for batch > 1 (1..16): their
                           matrices are swept in the same batched launches;
@@ -341,7 +344,9 @@ bta_status bta_gemm_mixed(int32_t M, int32_t N, int32_t K, double alpha, const d
  * rounding (slices = 8: the order of an FP64 GEMM's rounding bound); every
  * value gives the same product.  Requires 1 <= K <= 5120.  status as for
  * bta_gemm_mixed.  Allocates its operand residues with cudaMallocAsync on
- * the stream.
+ * the stream (28 bytes an entry of each operand and of the result; results of
+ * more than 16384 rows or columns are taken in panels, smaller ones where the
+ * device is full, to the same bits).
  */
 bta_status bta_gemm_emulated(int32_t M, int32_t N, int32_t K, double alpha, const double* A,
                              int32_t lda, int32_t transA, const double* B, int32_t ldb,

@@ -9,6 +9,7 @@
 //              forms (Phase B, x*^T Q_p x*) -> [grad] selected inversion of Q_p,
 //              Phase C sums
 //   streams 3, 4 : the reverse legs of Q_c and Q_p (three time blocks or more)
+//   streams 5, 6 : the vector's part of Q_c's legs, the sums over x
 //   stream 0 : join, final combination into f and grad.
 // Both matrices are eliminated from both ends towards the middle block (see SweepItem), so
 // four chains of dependent block steps run concurrently and fill each other's idle SMs.
@@ -209,8 +210,8 @@ bta_status ensure_ctx(inla_model* m, int count) {
 
 // The workspaces of an evaluation in a precision: a context's legs take three work blocks
 // each, and in the tensor-core modes their products' operand copies (emulated: 84 bytes an
-// entry of a block, as much as ten blocks).  They are allocated when a call first needs them, outside
-// capture.  The smaller forms have one leg per matrix and hold the planes of seven moduli at
+// entry of a block, as much as ten blocks).  They are allocated when a call first needs
+// them, outside capture.  The smaller forms have one leg per matrix and hold the planes of seven moduli at
 // once (56 bytes an entry), or of four (44).  They are taken in turn where the one before does
 // not fit the device, so that a model whose matrices leave little room is evaluated all the
 // same; low-memory models whose full form would exceed kLowMemoryWork begin with the first of

@@ -20,7 +20,8 @@
 // reduced modulo p_i in FP32 (exactly).  So one FP64 product costs 14 BF16
 // products.  Splitting into 8 base-128 digits, with 36 digit products, cost
 // 2.6 times that: 4800^3 whole call 5.38 ms before, 2.61 ms now, at no larger
-// error (no digit products are dropped).
+// error (no digit products are dropped: 8e-16 of the norm at K = 4847 and 5120, now 4e-17
+// and, with p = 55, 9e-17).
 //
 // Kernels: exponents of the rows (ozaki_exp_kernel), residue planes (residue_kernel),
 // the 14 products (crt_gemm_kernel, crt_gemm_small_kernel), and the recovery with alpha,
@@ -1444,8 +1445,8 @@ bta_status launch_ozaki(const Gemm& g, uint8_t* ws, int32_t* status, cudaStream_
 }  // namespace
 
 // An upper bound over every product of at most M x N x K: a sweep sizes one
-// workspace for all of its products.
-// (the larger tile's layout, and the partial maxima of a smaller K).
+// workspace for all of its products (the larger tile's layout, and the partial maxima of a
+// smaller K).
 size_t ozaki_ws_bytes(int M, int N, int K, int group) {
   const size_t full = OzLayout(M, N, K, CT, group).total;
   return K > kPartialK ? std::max(full, OzLayout(M, N, kPartialK, CT, group).total) : full;
