@@ -234,21 +234,20 @@ bta_status try_workspaces(inla_model* m, int count, int prec) {
   const size_t tcb = prec ? sweep_tc_ws_bytes(m->ld, m->a, prec, group) : 0;
   const size_t wsb = 2 * SweepWs::bytes(m->ld, m->a) / sizeof(double);
   const size_t mark = m->allocs.size();
-  struct Got {
+  struct Got {   // one buffer each for the reverse legs and the areas
     double* legs = nullptr;
-    uint8_t* tc[4] = {};
+    uint8_t* tc = nullptr;
   };
   std::vector<Got> got(count);
+  // (where the emulated mode has its areas, the mixed mode's products fit into them)
+  auto shared = [&](const EvalCtx& c) {
+    return prec == 1 && c.tc[2][0] && tcb <= sweep_tc_ws_bytes(m->ld, m->a, 2, c.group[2]);
+  };
   bta_status st = BTA_OK;
   for (int e = 0; e < count && st == BTA_OK; ++e) {
-    EvalCtx& c = m->ctx[e];
+    const EvalCtx& c = m->ctx[e];
     if (legs == 4 && !c.legs[2].W1) st = dmalloc(m, &got[e].legs, wsb);
-    // (where the emulated mode has its areas, the mixed mode's products fit into them)
-    if (prec == 1 && !c.tc[1][0] && c.tc[2][0] &&
-        tcb <= sweep_tc_ws_bytes(m->ld, m->a, 2, c.group[2]))
-      for (int q = 0; q < 2; ++q) got[e].tc[q] = static_cast<uint8_t*>(c.tc[2][q]);
-    for (int q = 0; q < legs && st == BTA_OK; ++q)
-      if (!c.tc[prec][q] && !got[e].tc[q]) st = dmalloc(m, &got[e].tc[q], tcb);
+    if (st == BTA_OK && !c.tc[prec][0] && !shared(c)) st = dmalloc(m, &got[e].tc, legs * tcb);
   }
   if (st != BTA_OK) {
     roll_back(m, mark);
@@ -257,9 +256,10 @@ bta_status try_workspaces(inla_model* m, int count, int prec) {
   for (int e = 0; e < count; ++e) {
     EvalCtx& c = m->ctx[e];
     if (got[e].legs) leg_carve(m, c, 2, got[e].legs);
-    for (int q = 0; q < 4; ++q)
-      if (got[e].tc[q]) c.tc[prec][q] = got[e].tc[q];
-    if (!c.group[prec]) c.group[prec] = group;
+    if (c.tc[prec][0]) continue;
+    for (int q = 0; q < legs; ++q)
+      c.tc[prec][q] = got[e].tc ? got[e].tc + q * tcb : prec ? c.tc[2][q] : nullptr;
+    c.group[prec] = group;
   }
   return BTA_OK;
 }
